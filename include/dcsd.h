@@ -388,6 +388,18 @@ dcsd_status dcsd_einsum_host(const char* spec, double alpha, const double* A, in
                              const long* size_b, const long* stride_b, double beta, double* C, int rank_c,
                              const long* size_c, const long* stride_c);
 
+/* dcsd_einsum_device -- the same contraction on the context's device and
+ * stream (device pointers), by one of the FP64 engines of the residual:
+ * a diagnostic that lets the engines be compared.
+ *   engine : 0 the one the library takes for these sizes, 1 the tiled
+ *            kernel of the FP64 CUDA cores.
+ * Asynchronous: the result is complete after the stream is synchronised.
+ * Errors: INVALID_ARG (as dcsd_einsum_host), CUDA. */
+dcsd_status dcsd_einsum_device(dcsd_ctx* ctx, int engine, const char* spec, double alpha, const double* A,
+                               int rank_a, const long* size_a, const long* stride_a, const double* B, int rank_b,
+                               const long* size_b, const long* stride_b, double beta, double* C, int rank_c,
+                               const long* size_c, const long* stride_c);
+
 /* dcsd_energy_noalloc -- Delta E_A, the value dcsd_energy returns as dEA,
  * for callers that cannot allocate device memory: code that is
  * capturing a CUDA graph, that hands all device memory to its own pool

@@ -24,7 +24,7 @@ PREC_FP64, PREC_BF16, PREC_BF16X3, PREC_MIXED, PREC_BF16X6 = 0, 1, 2, 3, 4
 EXPORTS = ["dcsd_init", "dcsd_residual", "dcsd_energy", "dcsd_solve", "dcsd_heff",
            "dcsd_destroy", "dcsd_last_error", "dcsd_kernel_launches", "dcsd_profile",
            "dcsd_energy_noalloc", "dcsd_selftest_conversions", "dcsd_vjp", "dcsd_lambda",
-           "dcsd_coupling_host", "dcsd_einsum_host", "dcsd_reserve", "dcsd_fcidump_header",
+           "dcsd_coupling_host", "dcsd_einsum_host", "dcsd_einsum_device", "dcsd_reserve", "dcsd_fcidump_header",
            "dcsd_fcidump_read", "dcsd_cholesky_host", "dcsd_fcidump_prepare", "dcsd_init_fcidump",
            "dcsd_fcidump_error"]
 PROF_CLASSES = ["ladder_tc", "tc_other", "pack", "fp64", "c4", "c5", "c6", "c7"]
@@ -98,6 +98,8 @@ def load():
     view = [P, C.c_int, P, P]
     lib.dcsd_einsum_host.argtypes = [C.c_char_p, C.c_double] + view + view + [C.c_double] + view
     lib.dcsd_einsum_host.restype = C.c_int
+    lib.dcsd_einsum_device.argtypes = [C.c_void_p, C.c_int, C.c_char_p, C.c_double] + view + view + [C.c_double] + view
+    lib.dcsd_einsum_device.restype = C.c_int
     lib.dcsd_reserve.argtypes = [P, C.c_int, C.c_int, C.c_int]
     lib.dcsd_reserve.restype = C.c_int
     lib.dcsd_fcidump_header.argtypes = [C.c_char_p, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_int)]
@@ -242,6 +244,24 @@ def dcsd_einsum_host(spec, alpha, a, b, beta, c):
     st = load().dcsd_einsum_host(spec.encode(), float(alpha), *view(a), *view(b), float(beta), *view(c))
     if st != 0:
         raise DcsdError(st, "dcsd_einsum_host failed for " + spec)
+
+
+def dcsd_einsum_device(ctx, engine, spec, alpha, a, b, beta, c):
+    """c = beta c + alpha einsum(spec)(a, b) on the device: a, b, c float64
+    CUDA tensors (any strides; c written in place); engine 0 chosen by size,
+    1 the tiled kernel of the FP64 CUDA cores."""
+    keep = []
+
+    def view(x):
+        if str(x.dtype) != "torch.float64" or not x.is_cuda:
+            raise TypeError("float64 CUDA tensors only")
+        n = max(1, x.dim())
+        sz, st = (C.c_long * n)(*x.shape), (C.c_long * n)(*x.stride())
+        keep.append((sz, st))
+        return [x.data_ptr(), x.dim(), C.cast(sz, C.c_void_p), C.cast(st, C.c_void_p)]
+
+    _check(load().dcsd_einsum_device(ctx, engine, spec.encode(), float(alpha), *view(a), *view(b), float(beta),
+                                     *view(c)), ctx)
 
 
 def dcsd_vjp(ctx, ref, method, precision, mem_kind, T, Rbar, Ebar, Wbar, Tbar, Bbar=None, Fa=None, Fb=None):

@@ -229,6 +229,8 @@ void free_ctx(Ctx* c) {
     }
     c->t2 = nullptr;
     c->R2 = nullptr;
+    if (c->gemm64_count) cudaFree(c->gemm64_count);
+    c->gemm64_count = nullptr;
     if (c->vvvv) cudaFree(c->vvvv);
     c->vvvv = nullptr;
     if (c->r2f) cudaFree(c->r2f);
@@ -401,6 +403,13 @@ extern "C" dcsd_status dcsd_init(dcsd_ctx** out, const dcsd_dims* d, const doubl
     c->splitk_elems = std::max<size_t>(1 << 20, std::min<size_t>(64ul << 20, 16 * (n * n + O * V)));
     A_(c->splitk_ws, c->splitk_elems);
     A_(c->scal, 64);
+    double* counters = nullptr;
+    A_(counters, kGemm64Counters / 2);
+    c->gemm64_count = (unsigned*)counters;
+    if (cudaMemsetAsync(counters, 0, kGemm64Counters * sizeof(unsigned), c->stream) != cudaSuccess) {
+        c->err = std::string("init: ") + cudaGetErrorString(cudaGetLastError());
+        return fail(DCSD_ERR_CUDA);
+    }
 #undef A_
     if (cudaMallocHost((void**)&c->hostbuf, 64 * sizeof(double)) != cudaSuccess) {
         c->err = "cudaMallocHost failed";
@@ -962,6 +971,12 @@ extern "C" dcsd_status dcsd_solve(dcsd_ctx* h, const dcsd_solve_opts* o, int mem
     const int nd = o->diis_n;
     if (nd > 0) DCSD_TRY(ensure_diis(c, nd, len));
     else DCSD_TRY(ensure_jacobi(c, len));
+    // One order of summation in every FP64 contraction of a solve.  The MIXED
+    // solve stops at the rounding noise of its BF16X6 residuals, and a change
+    // of 1e-16 in the amplitudes flips BF16 roundings that feed back: with
+    // another order the converged amplitudes moved by up to 6e-9 of their
+    // norm at (8, 90, 270).  The FP64 solve, its reference, keeps the order too.
+    const FmaChain chain(c, true);
     std::vector<double> Bm(16 * 16, 0.0);
     int nhist = 0, next = 0;
     // MIXED phases: 0 BF16, 1 BF16X6, 2 FP64

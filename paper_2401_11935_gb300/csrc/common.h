@@ -107,6 +107,8 @@ struct AdjRegion {
     double* adj = nullptr;
 };
 
+constexpr long kGemm64Counters = 4096;
+
 struct Ctx {
     int nc = 0, nv = 0, X = 0;
     int n = 0, O = 0, V = 0;      // n = nc+2+nv; union occ O = nc+2; union vir V = nv+2
@@ -148,6 +150,9 @@ struct Ctx {
     double* red = nullptr;        // reduction scratch
     double* splitk_ws = nullptr;  // split-K partial tiles of the FP64 contraction kernel
     size_t splitk_elems = 0;
+    // FP64 contractions in a fixed order of summation (see einsum64)
+    bool fma_chain = false;
+    unsigned* gemm64_count = nullptr;  // [kGemm64Counters] block arrivals of a split contraction (zero between launches)
     double* scal = nullptr;       // device scalars: [0]=W [1]=dEA [2..] misc
     double* c1 = nullptr;         // [2][O][V] two-determinant coefficients
     // tensor-core modes: FP32 accumulator shadowing R2.  While r2f_on, the
@@ -254,6 +259,14 @@ __device__ __forceinline__ float f64_to_f32(double x) {
     if (rem > 0x10000000u || (rem == 0x10000000u && (m23 & 1u))) ++bits;  // carry may reach infinity
     return __uint_as_float(bits);
 }
+
+// fixes the order of summation of FP64 contractions for a scope
+struct FmaChain {
+    Ctx* c;
+    bool before;
+    FmaChain(Ctx* c_, bool on) : c(c_), before(c_->fma_chain) { c->fma_chain = on; }
+    ~FmaChain() { c->fma_chain = before; }
+};
 
 // error helpers
 #define DCSD_CUDA(ctx, call)                                                  \

@@ -5,11 +5,12 @@
 // index letter as batch (A,B,C), m (A,C), n (B,C) or k (A,B), merges
 // adjacent modes and hands a GemmPlan to a shared-memory tiled FP64 kernel.
 // FP64 has no tcgen05 kind, so this path runs on the CUDA cores; it is the
-// parity path of the library and the fallback-free reference for the BF16
-// tensor-core engine (tc_gemm.cu) that shares the same planner.
+// parity path of the library, against which the BF16 tensor-core engine
+// (tc_gemm.cu, same planner) is measured.
 #include "common.h"
 
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 
@@ -219,9 +220,6 @@ bool plan_einsum(const char* spec, const TV& A, const TV& B, const TV& C,
 
 static unsigned grid_for(Ctx* c, long total);
 
-// ---------------------------------------------------------------------------
-// FP64 tiled GEMM over a GemmPlan
-// ---------------------------------------------------------------------------
 struct GemmArgs {
     const double* A;
     const double* B;
@@ -253,21 +251,166 @@ __device__ __forceinline__ void decomp2(long idx, int nmode, const long* size, c
     }
 }
 
+// ---------------------------------------------------------------------------
+// FP64 products on the CUDA cores
+// ---------------------------------------------------------------------------
+// The FP64 pipe retires 2 FMA per clock and SM, so what counts is that every
+// SM has products to do and that none is spent on padding; operand traffic is
+// no limit (a 16 x 16 tile reads 1 byte per FMA: 300 bytes per clock over the
+// chip).  Hence small tiles: T = 16 (one output per thread), or T = 8 with
+// four k-slices per output, summed through shared memory, where 16 x 16 tiles
+// would leave SMs idle; and a split of K over blocks when there are fewer
+// tiles than SMs, the last block of a tile adding the partial sums in order.
+// 64 x 64 tiles, which these replace, took 17 us per 16 k however few of
+// their rows were real: (M, N, K) = (108, 22, 484) 551 -> 17 us, (495, 495,
+// 131) 168 -> 73 us, (1464, 1464, 1464) 5.99 -> 5.19 ms (1.21 TFLOP/s, the FP64
+// pipe's rate).  Operands arrive by 8-byte cp.async (any strides), three
+// chunks of KC ahead.
+constexpr int kG64Stages = 4;
+
+struct Gemm64Args {
+    const double* A;
+    const double* B;
+    double* C;
+    double alpha, beta;
+    GemmPlan p;
+    int a_kfast, b_kfast;
+    int tilesN;
+    int nsplit;        // K splits (NB = 1 only): blockIdx.y = split
+    long kchunk;       // K per split
+    double* ws;        // [tile][split][T * T] partial sums
+    unsigned* count;   // [tile] arrivals (zero between launches)
+};
+
+__device__ __forceinline__ void cp_async8(double* dst, const double* src, bool ok) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(ok ? 8 : 0) : "memory");
+}
+
+template <int T, int SL>
+__global__ void __launch_bounds__(T* T* SL) k_gemm64(const Gemm64Args g) {
+    constexpr int NT = T * T * SL;      // threads: one output and one of SL k-slices each
+    constexpr int KC = 2 * NT / T;      // k per chunk: two elements of each operand per thread
+    constexpr int PT = T + 1;
+    __shared__ double As[kG64Stages][KC][PT], Bs[kG64Stages][KC][PT];
+    __shared__ long rA[T], rC[T], cB[T], cC[T];
+    __shared__ bool last;
+    const GemmPlan& p = g.p;
+    const int tid = threadIdx.x;
+    const int slice = tid / (T * T), out = tid % (T * T), tx = out % T, ty = out / T;
+    const long tile = blockIdx.x, m0 = tile / g.tilesN * T, n0 = tile % g.tilesN * T;
+    const long kb = g.nsplit > 1 ? blockIdx.y * g.kchunk : 0, ke = g.nsplit > 1 ? min(p.K, kb + g.kchunk) : p.K;
+    const long nbz = g.nsplit > 1 ? 1 : p.NB;
+    if (tid < T) {
+        rA[tid] = rC[tid] = -1;
+        if (m0 + tid < p.M) decomp2(m0 + tid, p.nm, p.m_size, p.m_sa, p.m_sc, rA[tid], rC[tid]);
+    } else if (tid < 2 * T) {
+        const int t = tid - T;
+        cB[t] = cC[t] = -1;
+        if (n0 + t < p.N) decomp2(n0 + t, p.nn, p.n_size, p.n_sb, p.n_sc, cB[t], cC[t]);
+    }
+    __syncthreads();
+    const bool live = m0 + ty < p.M && n0 + tx < p.N;
+    const bool rowlive = m0 + ty < p.M;
+    for (long bz = g.nsplit > 1 ? 0 : blockIdx.y; bz < nbz; bz += gridDim.y) {
+        long oA = 0, oB = 0, oC = 0;
+        {
+            long idx = bz;
+            for (int j = p.nb - 1; j >= 0; --j) {
+                long q = idx / p.b_size[j], r = idx - q * p.b_size[j];
+                oA += r * p.b_sa[j]; oB += r * p.b_sb[j]; oC += r * p.b_sc[j];
+                idx = q;
+            }
+        }
+        const long nch = (ke - kb + KC - 1) / KC;
+        auto load = [&](long c) {
+            if (c < nch) {
+                const int st = (int)(c % kG64Stages);
+                const long k0 = kb + c * KC;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int e = tid + NT * h;
+                    const int kk = g.a_kfast ? e % KC : e / T, mm = g.a_kfast ? e / KC : e % T;
+                    long ka = 0, kx = 0;
+                    const bool ok = k0 + kk < ke && rA[mm] >= 0;
+                    if (ok) decomp2(k0 + kk, p.nk, p.k_size, p.k_sa, p.k_sb, ka, kx);
+                    cp_async8(&As[st][kk][mm], ok ? g.A + oA + rA[mm] + ka : g.A, ok);
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int e = tid + NT * h;
+                    const int kk = g.b_kfast ? e % KC : e / T, nn = g.b_kfast ? e / KC : e % T;
+                    long ka = 0, kx = 0;
+                    const bool ok = k0 + kk < ke && cB[nn] >= 0;
+                    if (ok) decomp2(k0 + kk, p.nk, p.k_size, p.k_sa, p.k_sb, ka, kx);
+                    cp_async8(&Bs[st][kk][nn], ok ? g.B + oB + cB[nn] + kx : g.B, ok);
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        for (int c = 0; c < kG64Stages - 1; ++c) load(c);
+        double acc = 0.0;
+        for (long c = 0; c < nch; ++c) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(kG64Stages - 2) : "memory");
+            __syncthreads();
+            load(c + kG64Stages - 1);
+            const int st = (int)(c % kG64Stages);
+            if (rowlive) {
+                const int kn = (int)min((long)KC, ke - kb - c * KC);
+                if (kn == KC) {
+#pragma unroll
+                    for (int kk = 0; kk < KC / SL; ++kk)
+                        acc = fma(As[st][kk * SL + slice][ty], Bs[st][kk * SL + slice][tx], acc);
+                } else {
+                    for (int k = slice; k < kn; k += SL) acc = fma(As[st][k][ty], Bs[st][k][tx], acc);
+                }
+            }
+        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        if (SL > 1) {
+            double* red = &As[0][0][0];
+            red[tid] = acc;
+            __syncthreads();
+            if (slice == 0)
+#pragma unroll
+                for (int s = 1; s < SL; ++s) acc += red[s * T * T + out];
+        }
+        if (g.nsplit > 1) {
+            double* w = g.ws + tile * g.nsplit * (T * T);
+            if (slice == 0) w[(long)blockIdx.y * (T * T) + out] = acc;
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) {
+                const unsigned n = atomicAdd(g.count + tile, 1u);
+                last = n == (unsigned)g.nsplit - 1;
+                if (last) g.count[tile] = 0;
+            }
+            __syncthreads();
+            if (!last) return;
+            __threadfence();
+            if (slice != 0) return;
+            acc = 0.0;
+            for (int s = 0; s < g.nsplit; ++s) acc += __ldcg(w + (long)s * (T * T) + out);
+        }
+        if (slice == 0 && live) {
+            double* cp = g.C + oC + rC[ty] + cC[tx];
+            double v = g.alpha * acc;
+            if (g.beta != 0.0) v += g.beta * (*cp);
+            *cp = v;
+        }
+        __syncthreads();
+    }
+}
+
 constexpr int GBM = 64, GBN = 64, GBK = 16;
 
-// FP64 input in the product type (integer-unit conversion for FP32)
-template <typename T> __device__ __forceinline__ T cvt_in(double x);
-template <> __device__ __forceinline__ double cvt_in<double>(double x) { return x; }
-template <> __device__ __forceinline__ float cvt_in<float>(double x) { return f64_to_f32(x); }
-
-// T = double: FP64 products and accumulation.  T = float: FP32 products of
-// the FP64 inputs (each loaded element is converted once and reused across
-// the 64-wide tile), summed in FP32 over one k-tile of GBK and accumulated in
-// FP64 across k-tiles.
-template <typename T>
-__global__ void __launch_bounds__(256) k_gemm_t(GemmArgs g) {
-    __shared__ T As[GBK][GBM + 1];
-    __shared__ T Bs[GBK][GBN + 1];
+// FP32 products of the FP64 inputs (each loaded element is converted once and
+// reused across the 64-wide tile), summed in FP32 over one k-tile of GBK and
+// accumulated in FP64 across k-tiles.
+__global__ void __launch_bounds__(256) k_gemm32(GemmArgs g) {
+    __shared__ float As[GBK][GBM + 1];
+    __shared__ float Bs[GBK][GBN + 1];
     __shared__ long rA[GBM], rC[GBM], cB[GBN], cC[GBN];
     __shared__ long kA[GBK], kB[GBK];
     const GemmPlan& p = g.p;
@@ -315,24 +458,20 @@ __global__ void __launch_bounds__(256) k_gemm_t(GemmArgs g) {
                 if (g.a_kfast) { kk = e % GBK; mm = e / GBK; }
                 else { mm = e % GBM; kk = e / GBM; }
                 long ra = rA[mm], ka = kA[kk];
-                As[kk][mm] = (ra >= 0 && ka >= 0) ? cvt_in<T>(g.A[oA + ra + ka]) : (T)0;
+                As[kk][mm] = (ra >= 0 && ka >= 0) ? f64_to_f32(g.A[oA + ra + ka]) : 0.0f;
             }
             for (int e = tid; e < GBN * GBK; e += 256) {
                 int nn, kk;
                 if (g.b_kfast) { kk = e % GBK; nn = e / GBK; }
                 else { nn = e % GBN; kk = e / GBN; }
                 long cb = cB[nn], kb = kB[kk];
-                Bs[kk][nn] = (cb >= 0 && kb >= 0) ? cvt_in<T>(g.B[oB + cb + kb]) : (T)0;
+                Bs[kk][nn] = (cb >= 0 && kb >= 0) ? f64_to_f32(g.B[oB + cb + kb]) : 0.0f;
             }
             __syncthreads();
-            T part[4][4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) part[i][j] = sizeof(T) == 8 ? (T)acc[i][j] : (T)0;
+            float part[4][4] = {};
 #pragma unroll
             for (int kk = 0; kk < GBK; ++kk) {
-                T a[4], b[4];
+                float a[4], b[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
 #pragma unroll
@@ -345,8 +484,7 @@ __global__ void __launch_bounds__(256) k_gemm_t(GemmArgs g) {
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    acc[i][j] = sizeof(T) == 8 ? (double)part[i][j] : acc[i][j] + (double)part[i][j];
+                for (int j = 0; j < 4; ++j) acc[i][j] += (double)part[i][j];
         }
         if (g.nsplit > 1) {
 #pragma unroll
@@ -443,7 +581,7 @@ __global__ void __launch_bounds__(256) k_gemv64(GemmArgs g, int vec_is_b) {
 }
 
 static dcsd_status einsum_simt(Ctx* c, const char* spec, double alpha, const TV& A, const TV& B,
-                               double beta, const TV& C, bool fp32);
+                               double beta, const TV& C, bool fp32, int engine = 0);
 
 dcsd_status einsum64(Ctx* c, const char* spec, double alpha, const TV& A, const TV& B,
                      double beta, const TV& C) {
@@ -470,8 +608,9 @@ void record_einsum(Ctx* c, const char* spec, double alpha, const TV& A, const TV
     rec_push(c, std::move(op));
 }
 
+// engine 1: the tiled FP64 kernel also where a matrix-vector kernel would run
 static dcsd_status einsum_simt(Ctx* c, const char* spec, double alpha, const TV& A, const TV& B,
-                               double beta, const TV& C, bool fp32) {
+                               double beta, const TV& C, bool fp32, int engine) {
     if (c->rec) record_einsum(c, spec, alpha, A, B, beta, C, fp32 ? 1 : 0, 0);
     GemmArgs g;
     std::string err;
@@ -494,7 +633,7 @@ static dcsd_status einsum_simt(Ctx* c, const char* spec, double alpha, const TV&
     g.nsplit = 1;
     g.kchunk = g.p.K;
     g.ws = nullptr;
-    if (g.p.NB == 1 && (g.p.N == 1 || g.p.M == 1) && g.p.K >= 64) {
+    if (engine == 0 && g.p.NB == 1 && (g.p.N == 1 || g.p.M == 1) && g.p.K >= 64) {
         const int vec_is_b = g.p.N == 1 ? 1 : 0;
         const long outs = vec_is_b ? g.p.M : g.p.N;
         prof_begin(c, DCSD_PROF_FP64);
@@ -502,6 +641,67 @@ static dcsd_status einsum_simt(Ctx* c, const char* spec, double alpha, const TV&
             trace_begin(c, std::string("fp64-gemv ") + spec + " M=" + std::to_string(g.p.M) + " N=" +
                                std::to_string(g.p.N) + " K=" + std::to_string(g.p.K));
         k_gemv64<<<grid_for(c, outs * 32), 256, 0, c->stream>>>(g, vec_is_b);
+        trace_end(c);
+        prof_end(c, DCSD_PROF_FP64);
+        return launch_check(c, spec);
+    }
+    if (!fp32) {
+        Gemm64Args h;
+        h.A = g.A;
+        h.B = g.B;
+        h.C = g.C;
+        h.alpha = alpha;
+        h.beta = beta;
+        h.p = g.p;
+        h.a_kfast = g.a_kfast;
+        h.b_kfast = g.b_kfast;
+        auto tiles_of = [&](long t) { return ((g.p.M + t - 1) / t) * ((g.p.N + t - 1) / t); };
+        // two blocks per SM before the tiles grow, or K is split (a chunk of
+        // 64 k at least, the partial sums in the workspace)
+        int T = tiles_of(16) * std::min<long>(g.p.NB, 65535) >= 2l * c->num_sms ? 16 : 8;
+        long nt = tiles_of(T);
+        long ns = 1;
+        if (c->fma_chain) {
+            // fixed order of summation: one FMA chain per output, or, for few
+            // 64 x 64 tiles and a long K, chains over pieces of K added in order
+            const long t64 = tiles_of(64);
+            if (g.p.NB == 1 && t64 < c->num_sms && g.p.K >= 2048) {
+                ns = std::min<long>((8 * c->num_sms + t64 - 1) / t64, g.p.K / 256);
+                ns = std::min<long>(ns, (long)(c->splitk_elems / std::max<long>(1, g.p.M * g.p.N)));
+                ns = std::min<long>(ns, 65535);
+            }
+            h.kchunk = ns >= 2 ? ((g.p.K + ns - 1) / ns + 15) / 16 * 16 : g.p.K;
+            if (ns >= 2) {
+                const long real = (g.p.K + h.kchunk - 1) / h.kchunk;
+                auto fits = [&](long t) {
+                    return tiles_of(t) <= kGemm64Counters && tiles_of(t) * real * t * t <= (long)c->splitk_elems;
+                };
+                T = tiles_of(16) * real >= 2l * c->num_sms ? 16 : 8;
+                if (!fits(T)) T = 24 - T;
+                if (!fits(T)) h.kchunk = g.p.K;  // (tiles of 64 padded past the workspace)
+                nt = tiles_of(T);
+            }
+        } else {
+            if (g.p.NB == 1 && nt < 2l * c->num_sms && nt <= kGemm64Counters && g.p.K >= 128) {
+                ns = std::min<long>({(2l * c->num_sms + nt - 1) / nt, g.p.K / 64, (long)(c->splitk_elems / (nt * T * T))});
+                ns = std::max<long>(1, std::min<long>(ns, 65535));
+            }
+            h.kchunk = ((g.p.K + ns - 1) / ns + 63) / 64 * 64;
+        }
+        h.nsplit = (int)((g.p.K + h.kchunk - 1) / h.kchunk);
+        if (h.nsplit < 1) h.nsplit = 1;
+        h.tilesN = (int)((g.p.N + T - 1) / T);
+        h.ws = c->splitk_ws;
+        h.count = c->gemm64_count;
+        const dim3 grid((unsigned)nt, (unsigned)(h.nsplit > 1 ? h.nsplit : std::min<long>(g.p.NB, 65535)));
+        prof_begin(c, DCSD_PROF_FP64);
+        if (c->trace)
+            trace_begin(c, std::string("fp64 ") + spec + " M=" + std::to_string(g.p.M) + " N=" +
+                               std::to_string(g.p.N) + " K=" + std::to_string(g.p.K) + " B=" +
+                               std::to_string(g.p.NB) + " T=" + std::to_string(T) + " split=" + std::to_string(h.nsplit));
+        if (T == 16) k_gemm64<16, 1><<<grid, 256, 0, c->stream>>>(h);
+        else if (c->fma_chain) k_gemm64<8, 1><<<grid, 64, 0, c->stream>>>(h);
+        else k_gemm64<8, 4><<<grid, 256, 0, c->stream>>>(h);
         trace_end(c);
         prof_end(c, DCSD_PROF_FP64);
         return launch_check(c, spec);
@@ -525,11 +725,10 @@ static dcsd_status einsum_simt(Ctx* c, const char* spec, double alpha, const TV&
               (unsigned)(g.nsplit > 1 ? g.nsplit : std::min<long>(g.p.NB, 65535)));
     prof_begin(c, DCSD_PROF_FP64);
     if (c->trace)
-        trace_begin(c, std::string(fp32 ? "fp32 " : "fp64 ") + spec + " M=" + std::to_string(g.p.M) + " N=" +
+        trace_begin(c, std::string("fp32 ") + spec + " M=" + std::to_string(g.p.M) + " N=" +
                            std::to_string(g.p.N) + " K=" + std::to_string(g.p.K) + " B=" +
                            std::to_string(g.p.NB) + " split=" + std::to_string(g.nsplit));
-    if (fp32) k_gemm_t<float><<<grid, 256, 0, c->stream>>>(g);
-    else k_gemm_t<double><<<grid, 256, 0, c->stream>>>(g);
+    k_gemm32<<<grid, 256, 0, c->stream>>>(g);
     if (g.nsplit > 1) {
         long tot = g.p.M * g.p.N;
         k_splitk_reduce<<<grid_for(c, tot), 256, 0, c->stream>>>(g.p, g.nsplit, g.ws, g.C, alpha, beta);
@@ -1244,4 +1443,41 @@ extern "C" dcsd_status dcsd_einsum_host(const char* spec, double alpha, const do
         }
     }
     return DCSD_OK;
+}
+
+// one contraction on the device (diagnostic of the FP64 engines)
+extern "C" dcsd_status dcsd_einsum_device(dcsd_ctx* h, int engine, const char* spec, double alpha, const double* A,
+                                          int rank_a, const long* size_a, const long* stride_a, const double* B,
+                                          int rank_b, const long* size_b, const long* stride_b, double beta,
+                                          double* C, int rank_c, const long* size_c, const long* stride_c) {
+    using namespace dcsd;
+    if (!h) return DCSD_ERR_INVALID_ARG;
+    Ctx* c = &h->c;
+    if (!spec || !A || !B || !C || engine < 0 || engine > 1) {
+        c->err = "dcsd_einsum_device: NULL argument or unknown engine";
+        return DCSD_ERR_INVALID_ARG;
+    }
+    TV t[3];
+    const int rank[3] = {rank_a, rank_b, rank_c};
+    const long* size[3] = {size_a, size_b, size_c};
+    const long* stride[3] = {stride_a, stride_b, stride_c};
+    for (int x = 0; x < 3; ++x) {
+        if (rank[x] < 0 || rank[x] > kMaxRank || (rank[x] > 0 && (!size[x] || !stride[x]))) {
+            c->err = "dcsd_einsum_device: bad view";
+            return DCSD_ERR_INVALID_ARG;
+        }
+        t[x].rank = rank[x];
+        for (int i = 0; i < rank[x]; ++i) {
+            if (size[x][i] < 0) {
+                c->err = "dcsd_einsum_device: bad view";
+                return DCSD_ERR_INVALID_ARG;
+            }
+            t[x].size[i] = size[x][i];
+            t[x].stride[i] = stride[x][i];
+        }
+    }
+    t[0].p = (double*)A;
+    t[1].p = (double*)B;
+    t[2].p = C;
+    return einsum_simt(c, spec, alpha, t[0], t[1], beta, t[2], false, engine);
 }

@@ -46,6 +46,7 @@ dcsd_status init_constants(Ctx* c, int prec) {
     // J and the core part of K_ref, on the tensor cores)
     const bool rec = c->rec;
     const int nsplit = prec == DCSD_PREC_BF16X6 ? 3 : prec == DCSD_PREC_BF16X3 ? 2 : 1;
+    const FmaChain chain(c, true);
     auto ein = [&](const char* spec, const TV& A, const TV& Bm, double beta, const TV& C, bool tc) -> dcsd_status {
         if (!rec) return einsum64(c, spec, 1.0, A, Bm, beta, C);
         record_einsum(c, spec, 1.0, A, Bm, beta, C, tc ? 2 : 0, tc ? nsplit : 0);
