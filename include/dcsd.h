@@ -391,10 +391,12 @@ dcsd_status dcsd_einsum_host(const char* spec, double alpha, const double* A, in
 /* dcsd_einsum_device -- the same contraction on the context's device and
  * stream (device pointers), by one of the FP64 engines of the residual:
  * a diagnostic that lets the engines be compared.
- *   engine : 0 the one the library takes for these sizes, 1 the tiled
- *            kernel of the FP64 CUDA cores.
+ *   engine : 0 the one the library takes for these sizes, 1 the FP64 CUDA
+ *            cores, 2 the modular GEMMs on the tensor cores (unbatched
+ *            contractions only).
  * Asynchronous: the result is complete after the stream is synchronised.
- * Errors: INVALID_ARG (as dcsd_einsum_host), CUDA. */
+ * Errors: INVALID_ARG (as dcsd_einsum_host; engine 2 with a batched or empty
+ * contraction), CUDA. */
 dcsd_status dcsd_einsum_device(dcsd_ctx* ctx, int engine, const char* spec, double alpha, const double* A,
                                int rank_a, const long* size_a, const long* stride_a, const double* B, int rank_b,
                                const long* size_b, const long* stride_b, double beta, double* C, int rank_c,

@@ -249,7 +249,7 @@ def dcsd_einsum_host(spec, alpha, a, b, beta, c):
 def dcsd_einsum_device(ctx, engine, spec, alpha, a, b, beta, c):
     """c = beta c + alpha einsum(spec)(a, b) on the device: a, b, c float64
     CUDA tensors (any strides; c written in place); engine 0 chosen by size,
-    1 the tiled kernel of the FP64 CUDA cores."""
+    1 FP64 CUDA cores, 2 modular GEMMs on the tensor cores."""
     keep = []
 
     def view(x):

@@ -250,6 +250,7 @@ void free_ctx(Ctx* c) {
     }
     mtables_free(c);
     tc_free(c);
+    crt_free(c);
     vjp_free(c);
 }
 
@@ -365,6 +366,9 @@ extern "C" dcsd_status dcsd_init(dcsd_ctx** out, const dcsd_dims* d, const doubl
     const size_t n = c->n, O = c->O, V = c->V, X = c->X;
     const size_t OV = O * V, n1 = 2 * OV, n2 = 3 * OV * OV;
     c->big_elems = std::max({OV * OV, V * V * V, X * OV, O * O * O * V, (size_t)16});
+    // FP64 ladder and G pass: chunks of up to 2^25 integrals (256 MB), so that
+    // the amplitudes are packed for a few chunks only (one row a = V^3 at least)
+    c->lad_elems = std::max(c->big_elems, std::min(V * V * V * V, (size_t)1 << 25));
     auto fail = [&](dcsd_status s) {
         g_init_error = c->err;
         free_ctx(c);
@@ -395,8 +399,8 @@ extern "C" dcsd_status dcsd_init(dcsd_ctx** out, const dcsd_dims* d, const doubl
     A_(c->Wo, O * O * O * O);
     A_(c->Foc, 2 * O * O);
     A_(c->Fvi, 2 * V * V);
-    A_(c->big0, c->big_elems);
-    A_(c->big1, c->big_elems);
+    A_(c->big0, c->lad_elems);
+    A_(c->big1, c->lad_elems);
     A_(c->big2, c->big_elems);
     A_(c->big3, c->big_elems);
     A_(c->red, kRedDoubles);
@@ -422,9 +426,10 @@ extern "C" dcsd_status dcsd_init(dcsd_ctx** out, const dcsd_dims* d, const doubl
         c->err = std::string("input copy failed: ") + cudaGetErrorString(cudaGetLastError());
         return fail(DCSD_ERR_CUDA);
     }
+    if ((st = tc_init(c)) != DCSD_OK) return fail(st);
+    if ((st = crt_init(c)) != DCSD_OK) return fail(st);
     if ((st = init_constants(c)) != DCSD_OK) return fail(st);
     if ((st = mtables_build(c)) != DCSD_OK) return fail(st);
-    if ((st = tc_init(c)) != DCSD_OK) return fail(st);
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) {
         c->err = std::string("init: ") + cudaGetErrorString(cudaGetLastError());
         return fail(DCSD_ERR_CUDA);

@@ -107,6 +107,7 @@ struct AdjRegion {
     double* adj = nullptr;
 };
 
+struct CrtEngine;
 constexpr long kGemm64Counters = 4096;
 
 struct Ctx {
@@ -146,6 +147,7 @@ struct Ctx {
     double* big2 = nullptr;
     double* big3 = nullptr;
     size_t big_elems = 0;
+    size_t lad_elems = 0;         // elements of big0 and big1: the FP64 ladder's integral chunks
     double* abi[10] = {};         // device staging of ABI arrays for host mem_kind calls
     double* red = nullptr;        // reduction scratch
     double* splitk_ws = nullptr;  // split-K partial tiles of the FP64 contraction kernel
@@ -187,6 +189,8 @@ struct Ctx {
 
     MTables* mt[2] = {};          // per reference
     TcEngine* tc = nullptr;
+    CrtEngine* crt = nullptr;     // FP64 contractions on the tensor cores (crt_gemm.cu)
+    int* tc_err = nullptr;        // device error word of the tensor-core kernels (scal[22])
 
     // optional device-time accounting (dcsd_profile)
     bool prof_on = false;
@@ -393,6 +397,15 @@ dcsd_status init_constants(Ctx* c, int prec = DCSD_PREC_FP64);
 // one OP_EINSUM tape entry (engine 0 FP64, 1 FP32, 2 tensor cores with nsplit)
 void record_einsum(Ctx* c, const char* spec, double alpha, const TV& A, const TV& B, double beta, const TV& C,
                    int engine, int nsplit);
+
+// FP64 contractions by modular GEMMs on the tensor cores (crt_gemm.cu):
+// the engine's workspace is allocated by crt_init; crt_ready tells whether
+// it could be had.  einsum_crt takes unbatched plans (NB = 1).
+dcsd_status crt_init(Ctx* c);
+void crt_free(Ctx* c);
+bool crt_ready(const Ctx* c);
+dcsd_status einsum_crt(Ctx* c, const char* spec, const GemmPlan& plan, const double* A, const double* B, double* C,
+                       double alpha, double beta);
 
 // tensor-core engine (tc_gemm.cu)
 dcsd_status tc_init(Ctx* c);

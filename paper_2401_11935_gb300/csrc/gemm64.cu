@@ -4,9 +4,10 @@
 // over strided views (no explicit transposes): the planner classifies each
 // index letter as batch (A,B,C), m (A,C), n (B,C) or k (A,B), merges
 // adjacent modes and hands a GemmPlan to a shared-memory tiled FP64 kernel.
-// FP64 has no tcgen05 kind, so this path runs on the CUDA cores; it is the
-// parity path of the library, against which the BF16 tensor-core engine
-// (tc_gemm.cu, same planner) is measured.
+// FP64 has no tcgen05 kind: small contractions run on the FP64 CUDA cores
+// here, large ones as modular GEMMs on the tensor cores (crt_gemm.cu), to the
+// same accuracy.  Both are the parity path of the library, against which the
+// BF16 tensor-core engine (tc_gemm.cu, same planner) is measured.
 #include "common.h"
 
 #include <algorithm>
@@ -608,7 +609,26 @@ void record_einsum(Ctx* c, const char* spec, double alpha, const TV& A, const TV
     rec_push(c, std::move(op));
 }
 
-// engine 1: the tiled FP64 kernel also where a matrix-vector kernel would run
+// Whether an FP64 contraction goes to the modular GEMMs of the tensor cores:
+// a time model in microseconds of both.  Measured CUDA cores / modular:
+// (108, 484, 484) 66 / 62, (243, 55, 3025) 97 / 83, (495, 495, 131) 73 / 55,
+// (495, 495, 495) 240 / 62, (17568, 122, 12) 67 / 110, (132, 132, 132) 19 / 46,
+// (122, 12, 43920) 251 / 175.
+static bool crt_pays(const Ctx* c, const GemmPlan& p) {
+    if (!crt_ready(c) || p.NB != 1) return false;
+    const double M = (double)p.M, N = (double)p.N, K = (double)p.K;
+    auto up = [](double x, double m) { return std::ceil(x / m) * m; };
+    // CUDA cores: the tiles' products at the FP64 rate
+    const double T = up(M, 16) * up(N, 16) / 256 >= 2.0 * c->num_sms ? 16 : 8;
+    const double simt = 8.0 + 2.0 * up(M, T) * up(N, T) * K / 1.2e6;
+    // modular: four launches, residues of the operands, waves of tiles, output
+    const double tn = std::ceil(N / 256), bn = up(N / tn, 16), kb = std::ceil(K / 64);
+    const double waves = std::ceil(up(M, 128) / 128 * tn * 15 / c->num_sms);
+    const double crt = 30.0 + (M + N) * K / 1.2e5 + std::max(waves, 0.5) * (kb * 0.5 * bn / 256 + 1.5) + M * N / 1.1e5;
+    return crt < simt;
+}
+
+// engine: 0 chosen by size, 1 CUDA cores, 2 modular GEMM (FP64)
 static dcsd_status einsum_simt(Ctx* c, const char* spec, double alpha, const TV& A, const TV& B,
                                double beta, const TV& C, bool fp32, int engine) {
     if (c->rec) record_einsum(c, spec, alpha, A, B, beta, C, fp32 ? 1 : 0, 0);
@@ -633,7 +653,7 @@ static dcsd_status einsum_simt(Ctx* c, const char* spec, double alpha, const TV&
     g.nsplit = 1;
     g.kchunk = g.p.K;
     g.ws = nullptr;
-    if (engine == 0 && g.p.NB == 1 && (g.p.N == 1 || g.p.M == 1) && g.p.K >= 64) {
+    if (engine != 2 && g.p.NB == 1 && (g.p.N == 1 || g.p.M == 1) && g.p.K >= 64) {
         const int vec_is_b = g.p.N == 1 ? 1 : 0;
         const long outs = vec_is_b ? g.p.M : g.p.N;
         prof_begin(c, DCSD_PROF_FP64);
@@ -645,6 +665,8 @@ static dcsd_status einsum_simt(Ctx* c, const char* spec, double alpha, const TV&
         prof_end(c, DCSD_PROF_FP64);
         return launch_check(c, spec);
     }
+    if (!fp32 && (engine == 2 || (engine == 0 && !c->fma_chain && crt_pays(c, g.p))))
+        return einsum_crt(c, spec, g.p, A.p, B.p, C.p, alpha, beta);
     if (!fp32) {
         Gemm64Args h;
         h.A = g.A;
@@ -1453,7 +1475,7 @@ extern "C" dcsd_status dcsd_einsum_device(dcsd_ctx* h, int engine, const char* s
     using namespace dcsd;
     if (!h) return DCSD_ERR_INVALID_ARG;
     Ctx* c = &h->c;
-    if (!spec || !A || !B || !C || engine < 0 || engine > 1) {
+    if (!spec || !A || !B || !C || engine < 0 || engine > 2) {
         c->err = "dcsd_einsum_device: NULL argument or unknown engine";
         return DCSD_ERR_INVALID_ARG;
     }
@@ -1479,5 +1501,15 @@ extern "C" dcsd_status dcsd_einsum_device(dcsd_ctx* h, int engine, const char* s
     t[0].p = (double*)A;
     t[1].p = (double*)B;
     t[2].p = C;
+    GemmPlan p;
+    std::string err;
+    if (!plan_einsum(spec, t[0], t[1], t[2], p, err)) {
+        c->err = err;
+        return DCSD_ERR_INVALID_ARG;
+    }
+    if (engine == 2 && (p.NB != 1 || p.K < 1 || !crt_ready(c))) {
+        c->err = "dcsd_einsum_device: the modular engine takes unbatched, non-empty contractions";
+        return DCSD_ERR_INVALID_ARG;
+    }
     return einsum_simt(c, spec, alpha, t[0], t[1], beta, t[2], false, engine);
 }

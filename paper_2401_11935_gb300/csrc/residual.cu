@@ -356,14 +356,16 @@ dcsd_status residual_union(Ctx* c, int ref, int method, int prec) {
         // with stored four-index integrals, one contraction with them (the
         // reverse mode records the factorised form, equal to the threshold
         // of the factorisation)
-        const long ch = std::max<long>(1, std::min<long>(V, (long)(c->big_elems / (V * V * V))));
+        // (chunk sizes decide the split of K, hence the order of summation)
+        const size_t lad = c->fma_chain ? c->big_elems : c->lad_elems;
+        const long ch = std::max<long>(1, std::min<long>(V, (long)(lad / (V * V * V))));
         if (c->vvvv && !c->rec)
             DCSD_TRY(einsum64(c, "sijcd,acbd->sijab", 1.0, t2, view(c->vvvv, {V, V, V, V}), 1.0, R2));
         else
             DCSD_TRY(ladder64(c, t2, Bvv, R2, c->big0, ch, 0));
         // T1 corrections: G[s][ij][k][b] = sum_cd (kc|bd) t_s[ij][cd]; G[3] with
         // t_ab transposed in (c,d); H[s][ij][k][m] = sum_cd (kc|md) t_s[ij][cd]
-        const long kc = std::max<long>(1, std::min<long>(O, (long)(c->big_elems / (V * V * V))));
+        const long kc = std::max<long>(1, std::min<long>(O, (long)(lad / (V * V * V))));
         DCSD_TRY(gpass(c, t2, Bov, Bvv, G, c->big0, kc, 0));
     }
     DCSD_TRY(big("kmcd,sijcd->sijkm", 1.0, J, t2, 0.0, H));
@@ -500,5 +502,6 @@ dcsd_status residual_union(Ctx* c, int ref, int method, int prec) {
     else DCSD_TRY(apply_mterms(c, ref, fast));
     return DCSD_OK;
 }
+
 
 }  // namespace dcsd

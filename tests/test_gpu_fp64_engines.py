@@ -1,6 +1,12 @@
-"""The FP64 contraction kernels against sums in extended precision, at the
-edges of their tiles.  Error bound of a chain of K FMAs: K 2^-53 sum |a b|,
-with a factor two for the roundings of alpha and beta."""
+"""The FP64 contraction engines (FP64 CUDA cores; modular GEMMs on the tensor
+cores) against sums in extended precision, at the edges of their tiles.
+
+Error bound of the modular engine: the rows of A and B are scaled to integers
+of 2-norm in (2^57, 2^58] and (2^56, 2^57] and rounded (at most 1/2 per
+element), the integer product is exact, and one rounding to FP64 follows:
+|error| <= |a| |b| sqrt(K) / 2 (2^-57 + 2^-56) + 2^-53 |c| to first order.
+The FMA chain of the CUDA cores: K 2^-53 sum |a b|.  Both bounds take a
+factor two for the roundings of alpha and beta."""
 import numpy as np
 import pytest
 
@@ -23,9 +29,13 @@ def _exact(a, b):
     return np.asarray(a, dtype=np.longdouble) @ np.asarray(b, dtype=np.longdouble).T
 
 
-def _bound(a, b, alpha, c0, beta):
+def _bounds(a, b, alpha, c0, beta):
+    K = a.shape[1]
+    na, nb = np.linalg.norm(a, axis=1), np.linalg.norm(b, axis=1)
     ab = np.abs(a) @ np.abs(b).T
-    return 2 * 2.0 ** -53 * (abs(alpha) * (a.shape[1] + 1) * ab + abs(beta) * np.abs(c0))
+    tail = 2.0 ** -53 * (abs(alpha) * ab + abs(beta) * np.abs(c0))
+    crt = abs(alpha) * np.outer(na, nb) * np.sqrt(K) * 0.5 * (2.0 ** -57 + 2.0 ** -56)
+    return {1: 2 * (abs(alpha) * K * 2.0 ** -53 * ab + tail), 2: 2 * (crt + tail)}
 
 
 def _run(eng, engine, a, b, alpha, beta, c0, spec="mk,nk->mn"):
@@ -39,14 +49,15 @@ def _run(eng, engine, a, b, alpha, beta, c0, spec="mk,nk->mn"):
     return C.cpu().numpy()
 
 
-# edges of the 8 x 8 and 16 x 16 tiles and of their k-chunks, few tiles (K split), many tiles
+# tile edges: 4, 16 and 64 (packing, CUDA cores), 128 and 256 (tensor-core tiles), k-blocks of
+# 64, sums of 1024 k, norm blocks of 512 k, split k
 SHAPES = [(1, 1, 1), (3, 5, 2), (16, 16, 16), (17, 15, 33), (64, 64, 64), (65, 63, 65), (127, 16, 128), (128, 17, 63),
           (129, 255, 100), (130, 257, 31), (12, 12, 5000), (40, 300, 1024), (257, 33, 1025), (300, 530, 200),
           (9, 7, 20000), (513, 4, 513)]
 
 
 @pytest.mark.parametrize("M,N,K", SHAPES)
-@pytest.mark.parametrize("engine", [0, 1])
+@pytest.mark.parametrize("engine", [0, 1, 2])
 def test_contraction_error_bound(ctx, M, N, K, engine):
     rng = np.random.default_rng(M * 7 + N * 3 + K)
     a, b = rng.normal(size=(M, K)), rng.normal(size=(N, K))
@@ -56,10 +67,52 @@ def test_contraction_error_bound(ctx, M, N, K, engine):
         c0 = rng.normal(size=(M, N)) if beta else np.full((M, N), np.nan)
         ref = np.longdouble(alpha) * _exact(a, b) + (np.longdouble(beta) * c0 if beta else 0)
         err = np.abs(_run(ctx, engine, a, b, alpha, beta, c0) - ref)
-        assert (err <= _bound(a, b, alpha, c0 if beta else np.zeros((M, N)), beta)).all()
+        bound = _bounds(a, b, alpha, c0 if beta else np.zeros((M, N)), beta)
+        assert (err <= (np.maximum(bound[1], bound[2]) if engine == 0 else bound[engine])).all()
 
 
-@pytest.mark.parametrize("engine", [0, 1])
+@pytest.mark.parametrize("K", [64, 1024, 4096, 9000])
+def test_modular_sums_are_exact(ctx, K):
+    """Integers: every residue sum has to be exact, also where all products
+    have one sign (2^52 + 128 and 2^51 + 128 keep their unit bits at K = 1024
+    and have residues 128 modulo 256, so that the FP32 sums reach 2^24)."""
+    for va, vb in ((128, 128), (-128, 128), (127, 253), (2 ** 20 + 128, 3), (2 ** 52 + 128, 2 ** 51 + 128),
+                   (-2 ** 52 - 128, 2 ** 51 + 128), (2 ** 52 + 127, 2 ** 51 + 125)):
+        if K > 1024 and abs(va) > 2 ** 50:
+            continue  # the rounding to integers then acts
+        a, b = np.full((130, K), float(va)), np.full((24, K), float(vb))
+        c = _run(ctx, 2, a, b, 1.0, 0.0, np.zeros((130, 24)))
+        assert (c == float(va * vb * K)).all()
+    rng = np.random.default_rng(K)
+    a = rng.integers(-2 ** 18, 2 ** 18, (70, K)).astype(float)
+    b = rng.integers(-2 ** 18, 2 ** 18, (50, K)).astype(float)
+    ref = (a.astype(np.int64) @ b.astype(np.int64).T).astype(float)
+    assert (_run(ctx, 2, a, b, 1.0, 0.0, np.zeros((70, 50))) == ref).all()
+
+
+def test_modular_extreme_rows(ctx):
+    """Zero rows, subnormals, the largest magnitudes; Inf and NaN stay in
+    their rows and columns."""
+    rng = np.random.default_rng(1)
+    a, b = rng.normal(size=(20, 100)), rng.normal(size=(30, 100))
+    a[0] = 0.0
+    a[1] *= 1e-310
+    a[2] *= 1e300
+    a[3] *= 1e-200
+    b[4] *= 1e-5
+    a[5, 7] = np.inf
+    b[6, 3] = np.nan
+    c = _run(ctx, 2, a, b, 1.0, 0.0, np.zeros((20, 30)))
+    good = np.ones((20, 30), bool)
+    good[5] = good[:, 6] = False
+    assert not np.isfinite(c[~good]).any() and np.isfinite(c[good]).all()
+    a[5, 7] = b[6, 3] = 0.0
+    ref = _exact(a, b)
+    norm = np.outer(np.linalg.norm(a.astype(np.longdouble), axis=1), np.linalg.norm(b, axis=1))
+    assert (np.abs(c - ref)[good] <= (1e-14 * norm + 1e-322)[good]).all()
+
+
+@pytest.mark.parametrize("engine", [1, 2])
 @pytest.mark.parametrize("spec,sa,sb,sc", [
     ("Lac,Lbd->acbd", (9, 5, 7), (9, 6, 8), (5, 7, 6, 8)), ("ikac,kcjb->iajb", (4, 5, 9, 7), (5, 7, 3, 11), (4, 9, 3, 11)),
     ("klij,klab->ijab", (4, 5, 3, 2), (4, 5, 13, 17), (3, 2, 13, 17)), ("ijdc,kcbd->ijkb", (3, 3, 6, 6), (5, 6, 7, 6), (3, 3, 5, 7))])
