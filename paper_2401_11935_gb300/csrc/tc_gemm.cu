@@ -2,8 +2,8 @@
 //
 // C[m][n] = alpha * sum_k A[m][k] B[n][k] + beta * C with A, B in BF16,
 // K-major, staged in shared memory by TMA (128-byte swizzle) through a
-// 4-stage mbarrier pipeline and multiplied by tcgen05.mma (kind::f16,
-// M = 128, N = 128/256, K = 16 per instruction) into an FP32 accumulator in
+// 4- to 8-stage mbarrier pipeline and multiplied by tcgen05.mma (kind::f16,
+// M = 128, N = 64/128/256, K = 16 per instruction) into an FP32 accumulator in
 // tensor memory.  Warp roles: warp 0 issues TMA loads, warp 1 owns TMEM and
 // issues the MMAs (one thread), warps 2-5 drain TMEM with tcgen05.ld and
 // write the tile (FP64 C through arbitrary strides, or BF16 directly in the
@@ -31,7 +31,9 @@
 
 namespace dcsd {
 
-constexpr int TC_BM = 128, TC_BK = 64, TC_STAGES = 4;
+constexpr int TC_BM = 128, TC_BK = 64;
+// stages of the operand pipeline for tiles of BN columns (192 KB in all)
+__host__ __device__ constexpr int tc_stages(int BN) { return BN == 256 ? 4 : BN == 128 ? 6 : 8; }
 
 // x = hi + mid + lo with each part BF16 (8 significant bits each)
 __device__ __forceinline__ __nv_bfloat16 split_part(float x, int part) {
@@ -77,6 +79,15 @@ struct TcEpi {
     long O;
     const int* rowcode;     // mode 3: row -> (block << 20 | i << 10 | j); same-spin rows are pairs i < j
     const long* mrow;       // modes 0/4: row -> offset in C (replaces the m-mode decomposition)
+};
+
+// Operand parts of the split products of a GEMM: its k-steps run over the
+// products, nkb of 64 k each; product s takes part a[s] of A and b[s] of B
+// (parts are stored once, side by side, Kp elements apart: with the segments
+// of A and of B written out, a BF16X6 operand was packed and read twice over)
+struct TcParts {
+    int nkb;
+    int a[6], b[6];
 };
 
 // ladder consumer scatter of one accumulator element v = W(a,b) for the row
@@ -170,15 +181,16 @@ __device__ __forceinline__ void tile_mn(int mn, int tilesM, int tilesN, int grou
 template <int BN, bool MC>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcEpi epi,
-              int nkt, int tilesM, int tilesN, int kper, int group, int kblk, int* err) {
+              const TcParts parts, int nkt, int tilesM, int tilesN, int kper, int group, int kblk, int* err) {
     constexpr uint32_t A_BYTES = TC_BM * TC_BK * 2, B_BYTES = BN * TC_BK * 2;
     constexpr uint32_t STAGE = A_BYTES + B_BYTES;
+    constexpr int STAGES = tc_stages(BN);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t* staging = smem + TC_STAGES * STAGE;
+    uint8_t* staging = smem + STAGES * STAGE;
     uint64_t* full = (uint64_t*)(staging + kStageBytesMode2);
-    uint64_t* empty = full + TC_STAGES;
-    uint64_t* accf = empty + TC_STAGES;  // [2] MMA -> epilogue
+    uint64_t* empty = full + STAGES;
+    uint64_t* accf = empty + STAGES;  // [2] MMA -> epilogue
     uint64_t* acce = accf + 2;           // [2] epilogue -> MMA
     uint32_t* tslot = (uint32_t*)(acce + 2);
     volatile int* issued = (volatile int*)(tslot + 1);
@@ -196,7 +208,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int nmn = tilesMs * tilesN;
     const int ntiles = nmn * ((nkt + kper - 1) / kper);
     if (threadIdx.x == 0) {
-        for (int s = 0; s < TC_STAGES; ++s) {
+        for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], MC ? 2 : 1);
         }
@@ -228,24 +240,30 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 if (MC) tm = 2 * tm + crank;
                 const int m0 = tm * TC_BM, n0 = tn * BN;
                 const int kb = ks * kper, ke = min(nkt, kb + kper);
-                for (int kt = kb; kt < ke; ++kt, ++g) {
-                    const int s = g % TC_STAGES, round = g / TC_STAGES;
+                int seg = kb / parts.nkb, kq = kb - seg * parts.nkb;
+                for (int kt = kb; kt < ke; ++kt, ++g, ++kq) {
+                    const int s = g % STAGES, round = g / STAGES;
                     if (round > 0 && !mbar_wait(&empty[s], (round - 1) & 1)) {
                         atomicExch(err, 1);
                         ok = false;
                         break;
                     }
+                    if (kq == parts.nkb) {
+                        kq = 0;
+                        ++seg;
+                    }
+                    const int ka = parts.a[seg] * parts.nkb + kq, kz = parts.b[seg] * parts.nkb + kq;
                     mbar_expect_tx(&full[s], STAGE);
                     if (MC) {
-                        tma_load_3d(smem + s * STAGE, &tmA, &full[s], 0, m0, kt);
+                        tma_load_3d(smem + s * STAGE, &tmA, &full[s], 0, m0, ka);
                         tma_load_3d_mc(smem + s * STAGE + A_BYTES + crank * (B_BYTES / 2), &tmB, &full[s], 0,
-                                       n0 + crank * (BN / 2), kt, (uint16_t)0x3);
+                                       n0 + crank * (BN / 2), kz, (uint16_t)0x3);
                     } else if (kblk) {
-                        tma_load_3d(smem + s * STAGE, &tmA, &full[s], 0, m0, kt);
-                        tma_load_3d(smem + s * STAGE + A_BYTES, &tmB, &full[s], 0, n0, kt);
+                        tma_load_3d(smem + s * STAGE, &tmA, &full[s], 0, m0, ka);
+                        tma_load_3d(smem + s * STAGE + A_BYTES, &tmB, &full[s], 0, n0, kz);
                     } else {
-                        tma_load_2d(smem + s * STAGE, &tmA, &full[s], kt * TC_BK, m0);
-                        tma_load_2d(smem + s * STAGE + A_BYTES, &tmB, &full[s], kt * TC_BK, n0);
+                        tma_load_2d(smem + s * STAGE, &tmA, &full[s], ka * TC_BK, m0);
+                        tma_load_2d(smem + s * STAGE + A_BYTES, &tmB, &full[s], kz * TC_BK, n0);
                     }
                     *issued = g + 1;
                 }
@@ -253,9 +271,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if (MC) {
                 // every slot free in both CTAs: the peer's last MMA completions
                 // have arrived here and no multicast of this CTA is pending
-                const int g0 = max(0, g - TC_STAGES);
+                const int g0 = max(0, g - STAGES);
                 for (int gg = g0; gg < g; ++gg)
-                    if (!mbar_wait(&empty[gg % TC_STAGES], (gg / TC_STAGES) & 1)) atomicExch(err, 5);
+                    if (!mbar_wait(&empty[gg % STAGES], (gg / STAGES) & 1)) atomicExch(err, 5);
             }
         }
     } else if (warp == 1) {
@@ -275,7 +293,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 const uint32_t d = tmem + (uint32_t)(buf * BN);
                 const int kb = (tile / nmn) * kper, ke = min(nkt, kb + kper);
                 for (int kt = kb; kt < ke; ++kt, ++g) {
-                    const int s = g % TC_STAGES, round = g / TC_STAGES;
+                    const int s = g % STAGES, round = g / STAGES;
                     if (!mbar_wait(&full[s], round & 1)) {
                         atomicExch(err, 2);
                         ok = false;
@@ -297,7 +315,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 // let issued MMAs finish and drain copies that were not consumed
                 uint64_t* fin = &accf[j & 1];
                 mma_commit(fin);
-                for (int kt = *consumed; kt < *issued; ++kt) mbar_wait(&full[kt % TC_STAGES], (kt / TC_STAGES) & 1);
+                for (int kt = *consumed; kt < *issued; ++kt) mbar_wait(&full[kt % STAGES], (kt / STAGES) & 1);
             }
         }
     } else {
@@ -564,7 +582,9 @@ constexpr int SA_STAGES = 3;
 constexpr uint32_t SA_TILE = 128 * TC_BK * 2;  // one 128-row operand tile (16 KB)
 
 struct SaArgs {
-    int nkt;              // k-steps over the packed L (segments x L / 64)
+    int nkt;              // k-steps over the packed L (split products x L / 64)
+    int nkb;              // L / 64
+    int part_a[6], part_b[6];  // operand parts of the split products
     int nr, Vb, nblk;     // chunk rows, columns b, 128-wide c/d blocks
     int npair;            // (C, D) block pairs with C <= D
     long ntiles;          // npair x #(r, b'): b' >= r (ladder) or all (rect)
@@ -574,7 +594,7 @@ struct SaArgs {
     int V, Vp;
     long kbs;             // k-block stride of a V tile (vrows * 64)
     long segstride;       // elements between the segments of a V tile
-    int nseg, pat[6];
+    int nparts;           // parts of M+- written
     __nv_bfloat16* Vplus;
     __nv_bfloat16* Vminus;
 };
@@ -611,15 +631,15 @@ __device__ __forceinline__ void sa_tile(const SaArgs& a, long t, int& r, int& bb
 
 // Producer of the M+ and M- tiles of one chunk of a: tile (a, b, C, D) with
 // b >= a and C <= D, two accumulators acc1 = B_a[C] B_b[D]^T = M_ab[C][D] and
-// acc2 = B_b[C] B_a[D]^T (element (c,d) = (ad|bc)).  tmA / tmB: the packed
-// virtual-virtual DF factors [(x, y)][L] (y padded to YP rows per x), with
-// the A-side and the B-side split patterns, K-blocked.  Pipeline as in
+// acc2 = B_b[C] B_a[D]^T (element (c,d) = (ad|bc)).  tmX: the packed
+// virtual-virtual DF factors [part][(x, y)][L] (y padded to YP rows per x),
+// K-blocked; the k-steps of a split product take the parts of its two
+// operands from this one array.  Pipeline as in
 // k_tc_gemm: warp 0 loads four 16 KB tiles per stage, warp 1 issues the
 // MMAs, eight epilogue warps write M+- (BF16 split parts) at the compact
 // (c <= d) index of V tile row (r, b').
 __global__ void __launch_bounds__(kTcThreads, 1)
-    k_ladder_sa(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, SaArgs a,
-                int* err) {
+    k_ladder_sa(const __grid_constant__ CUtensorMap tmX, const SaArgs a, int* err) {
     constexpr uint32_t STAGE = 4 * SA_TILE;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -659,6 +679,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 int r, bb, C, D;
                 sa_tile(a, t, r, bb, C, D);
                 const int xa = (a.xa0 + r) * a.YP, xb = (a.xb0 + bb) * a.YP;
+                int seg = 0, kb = 0, za = a.part_a[0] * a.nkb, zb = a.part_b[0] * a.nkb;
                 for (int kt = 0; kt < a.nkt; ++kt, ++g) {
                     const int s = g % SA_STAGES, round = g / SA_STAGES;
                     if (round > 0 && !mbar_wait(&empty[s], (round - 1) & 1)) {
@@ -671,14 +692,19 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     uint8_t* st = smem + s * STAGE;
                     if (C == D) {
                         mbar_expect_tx(&full[s], 2 * SA_TILE);
-                        tma_load_3d(st, &tmA, &full[s], 0, xa + C * 128, kt);            // B_a[C]
-                        tma_load_3d(st + SA_TILE, &tmB, &full[s], 0, xb + D * 128, kt);  // B_b[C]
+                        tma_load_3d(st, &tmX, &full[s], 0, xa + C * 128, za + kb);            // B_a[C]
+                        tma_load_3d(st + SA_TILE, &tmX, &full[s], 0, xb + D * 128, zb + kb);  // B_b[C]
                     } else {
                         mbar_expect_tx(&full[s], STAGE);
-                        tma_load_3d(st, &tmA, &full[s], 0, xa + C * 128, kt);                // B_a[C]
-                        tma_load_3d(st + SA_TILE, &tmB, &full[s], 0, xb + D * 128, kt);      // B_b[D]
-                        tma_load_3d(st + 2 * SA_TILE, &tmA, &full[s], 0, xb + C * 128, kt);  // B_b[C]
-                        tma_load_3d(st + 3 * SA_TILE, &tmB, &full[s], 0, xa + D * 128, kt);  // B_a[D]
+                        tma_load_3d(st, &tmX, &full[s], 0, xa + C * 128, za + kb);                // B_a[C]
+                        tma_load_3d(st + SA_TILE, &tmX, &full[s], 0, xb + D * 128, zb + kb);      // B_b[D]
+                        tma_load_3d(st + 2 * SA_TILE, &tmX, &full[s], 0, xb + C * 128, za + kb);  // B_b[C]
+                        tma_load_3d(st + 3 * SA_TILE, &tmX, &full[s], 0, xa + D * 128, zb + kb);  // B_a[D]
+                    }
+                    if (++kb == a.nkb && ++seg < 6) {
+                        kb = 0;
+                        za = a.part_a[seg] * a.nkb;
+                        zb = a.part_b[seg] * a.nkb;
                     }
                     *issued = g + 1;
                 }
@@ -768,14 +794,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         pl[x] = v1 + v2;
                         mi[x] = v1 - v2;
                     }
-                    for (int sg = 0; sg < a.nseg; ++sg) {
+                    for (int sg = 0; sg < a.nparts; ++sg) {
                         uint32_t wp[4], wm[4];
 #pragma unroll
                         for (int x = 0; x < 4; ++x) {
-                            wp[x] = (uint32_t)__bfloat16_as_ushort(split_part(pl[2 * x], a.pat[sg])) |
-                                    ((uint32_t)__bfloat16_as_ushort(split_part(pl[2 * x + 1], a.pat[sg])) << 16);
-                            wm[x] = (uint32_t)__bfloat16_as_ushort(split_part(mi[2 * x], a.pat[sg])) |
-                                    ((uint32_t)__bfloat16_as_ushort(split_part(mi[2 * x + 1], a.pat[sg])) << 16);
+                            wp[x] = (uint32_t)__bfloat16_as_ushort(split_part(pl[2 * x], sg)) |
+                                    ((uint32_t)__bfloat16_as_ushort(split_part(pl[2 * x + 1], sg)) << 16);
+                            wm[x] = (uint32_t)__bfloat16_as_ushort(split_part(mi[2 * x], sg)) |
+                                    ((uint32_t)__bfloat16_as_ushort(split_part(mi[2 * x + 1], sg)) << 16);
                         }
                         *(uint4*)(a.Vplus + off + sg * a.segstride) = make_uint4(wp[0], wp[1], wp[2], wp[3]);
                         *(uint4*)(a.Vminus + off + sg * a.segstride) = make_uint4(wm[0], wm[1], wm[2], wm[3]);
@@ -1274,7 +1300,7 @@ struct Buf {
 struct TcEngine {
     PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
     int* d_err = nullptr;
-    int mc_clusters[2] = {0, 0};  // resident two-CTA clusters (BN 128, 256); 0 unknown, -1 none
+    int mc_clusters = 0;  // resident two-CTA clusters; 0 unknown, -1 none
     Buf pa, pb, pv, pt;  // generic A, generic B, ladder V tile, stacked amplitudes
     bool attr_set = false;
     // ladder row tables for the stacked amplitudes [aa pairs; bb pairs; ab; ab~]
@@ -1291,14 +1317,14 @@ struct TcEngine {
     long pc_clock = 0;
     // symmetric / antisymmetric ladder: amplitudes A- (same-spin pairs and
     // alpha-beta rows) and A+ (alpha-beta rows), the M+ and M- tiles of a
-    // chunk, the DF factors packed [(x, y)][L] with the A- and B-side split
-    // patterns, and the consumer row codes
-    Buf sam, sap, svp, svm, sxa, sxb;
+    // chunk, the DF factors packed [(x, y)][L], each with its split parts one
+    // after the other, and the consumer row codes
+    Buf sam, sap, svp, svm, sx;
     int* d_code_m = nullptr;
     int* d_code_p = nullptr;
     long sa_O = -1;
     bool sa_attr = false;
-    int sx_nsplit = 0;  // split of the packed DF factors in sxa / sxb (0: none; B never changes)
+    int sx_nsplit = 0;  // parts of the packed DF factors in sx (0: none; B never changes)
     // packed operands read from the DF factors B or from J, which never
     // change after initialisation: kept for the life of the context (key as
     // in pack_operand), up to kBCacheBytes in all
@@ -1343,7 +1369,7 @@ dcsd_status tc_init(Ctx* c) {
 void tc_free(Ctx* c) {
     TcEngine* e = c->tc;
     if (!e) return;
-    for (Buf* b : {&e->pa, &e->pb, &e->pv, &e->pt, &e->sam, &e->sap, &e->svp, &e->svm, &e->sxa, &e->sxb, &e->pbv})
+    for (Buf* b : {&e->pa, &e->pb, &e->pv, &e->pt, &e->sam, &e->sap, &e->svp, &e->svm, &e->sx, &e->pbv})
         if (b->p) cudaFree(b->p);
     for (auto& kv : e->bcache)
         if (kv.second.p) cudaFree(kv.second.p);
@@ -1501,57 +1527,86 @@ static dcsd_status make_map_kblk(Ctx* c, CUtensorMap* map, const __nv_bfloat16* 
     return DCSD_OK;
 }
 
-// C (epilogue epi) = A[M][Ktot] . B[N][Ktot]^T; the operands are K-major BF16
+// C (epilogue epi) = A[M][Ktot] . B[N][Ktot]^T (split: Ktot runs over the
+// split products, the operands hold nparts parts); the operands are K-major BF16
 // with row pitch `pitch` elements (0: Ktot), or K-blocked (kblocked: both
 // operands [Ktot / 64][rows][64])
 // mc (K-blocked operands, at least two m-tiles): clusters of two CTAs share
 // each B tile through TMA multicast (see k_tc_gemm)
 static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __nv_bfloat16* Bp, long N,
                                long Ktot, TcEpi& epi, int ksplit = 1, long pitch = 0, bool kblocked = false,
-                               bool mc = false) {
+                               bool mc = false, const TcParts* split = nullptr, int nparts = 1) {
     TcEngine* e = c->tc;
+    TcParts parts = {};
+    parts.nkb = (int)(Ktot / TC_BK);
+    if (split) parts = *split;
+    const long Kst = split ? (long)nparts * parts.nkb * TC_BK : Ktot;  // stored K
+    auto smem_of = [](int bn) {
+        return tc_stages(bn) * (TC_BM * TC_BK * 2 + (size_t)bn * TC_BK * 2) + kStageBytesMode2 + 2048;
+    };
+    const void* kern[2][3] = {
+        {(const void*)k_tc_gemm<64, false>, (const void*)k_tc_gemm<128, false>, (const void*)k_tc_gemm<256, false>},
+        {(const void*)k_tc_gemm<64, true>, (const void*)k_tc_gemm<128, true>, (const void*)k_tc_gemm<256, true>}};
+    mc = mc && kblocked && c->tc_multicast && M > TC_BM && c->num_sms >= 2;
+    auto config = [&](cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, unsigned grid, int bn) {
+        cfg = {};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(kTcThreads);
+        cfg.dynamicSmemBytes = smem_of(bn);
+        cfg.stream = c->stream;
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 2;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = mc ? 1 : 0;
+    };
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[1];
     if (!e->attr_set) {
-        size_t s256 = TC_STAGES * (TC_BM * TC_BK * 2 + 256 * TC_BK * 2) + kStageBytesMode2 + 2048;
-        size_t s128 = TC_STAGES * (TC_BM * TC_BK * 2 + 128 * TC_BK * 2) + kStageBytesMode2 + 2048;
-        DCSD_CUDA(c, cudaFuncSetAttribute(k_tc_gemm<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)s256));
-        DCSD_CUDA(c, cudaFuncSetAttribute(k_tc_gemm<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)s128));
-        DCSD_CUDA(c, cudaFuncSetAttribute(k_tc_gemm<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)s256));
-        DCSD_CUDA(c, cudaFuncSetAttribute(k_tc_gemm<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)s128));
+        for (int m = 0; m < 2; ++m)
+            for (int b = 0; b < 3; ++b)
+                DCSD_CUDA(c, cudaFuncSetAttribute(kern[m][b], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)smem_of(64 << b)));
         e->attr_set = true;
     }
-    const int BN = N >= 256 ? 256 : 128;
-    mc = mc && kblocked && c->tc_multicast && M > TC_BM && c->num_sms >= 2;
-    long max_clusters = c->num_sms / 2;
-    if (mc) {
-        if (e->mc_clusters[BN == 256 ? 1 : 0] == 0) {
-            cudaLaunchConfig_t q = {};
-            q.gridDim = dim3((unsigned)(2 * max_clusters));
-            q.blockDim = dim3(kTcThreads);
-            q.dynamicSmemBytes = TC_STAGES * (TC_BM * TC_BK * 2 + (size_t)BN * TC_BK * 2) + kStageBytesMode2 + 2048;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = 2;
-            at[0].val.clusterDim.y = 1;
-            at[0].val.clusterDim.z = 1;
-            q.attrs = at;
-            q.numAttrs = 1;
-            int nclu = 0;
-            const cudaError_t qe = BN == 256 ? cudaOccupancyMaxActiveClusters(&nclu, k_tc_gemm<256, true>, &q)
-                                             : cudaOccupancyMaxActiveClusters(&nclu, k_tc_gemm<128, true>, &q);
-            if (qe != cudaSuccess || nclu < 1) {
+    if (mc && e->mc_clusters == 0) {
+        // resident two-CTA clusters: every form takes one CTA per SM
+        int nclu = 1 << 20;
+        for (int b = 0; b < 3; ++b) {
+            int n1 = 0;
+            config(cfg, at, (unsigned)(c->num_sms / 2 * 2), 64 << b);
+            if (cudaOccupancyMaxActiveClusters(&n1, kern[1][b], &cfg) != cudaSuccess || n1 < 1) {
                 cudaGetLastError();
-                nclu = -1;  // clusters unavailable: the one-CTA kernel runs
+                n1 = -1;  // clusters unavailable: the one-CTA kernel runs
             }
-            e->mc_clusters[BN == 256 ? 1 : 0] = nclu;
+            nclu = std::min(nclu, n1);
         }
-        const int nclu = e->mc_clusters[BN == 256 ? 1 : 0];
-        if (nclu < 1) mc = false;
-        else max_clusters = std::min<long>(max_clusters, nclu);
+        e->mc_clusters = nclu;
     }
+    if (e->mc_clusters < 0) mc = false;
+    const long max_clusters = mc ? std::min<long>(c->num_sms / 2, e->mc_clusters) : 0;
+    // Columns per tile: 256, or fewer where that leaves SMs idle.  A k-step
+    // takes in 16 KB + 128 bytes per column at about 64 bytes per clock and SM,
+    // so narrow tiles cost up to twice as much per element but run on up to
+    // four times as many SMs.  (The sums over k do not depend on the width.)
+    // A BF16X6 ladder consumer at (10, 120, 360), M = 276, N = 1800, K = 8704:
+    // 118 us with 256 columns (16 CTAs in clusters), 63 us with 64.
+    int BN = 256;
+    {
+        const long tm = mc ? ((M + TC_BM - 1) / TC_BM + 1) / 2 : (M + TC_BM - 1) / TC_BM;
+        const long slots = mc ? max_clusters : c->num_sms;
+        double best = 1e300;
+        for (int bn = 256; bn >= 64; bn /= 2) {
+            const long nt = tm * ((N + bn - 1) / bn) * std::max(1, ksplit);
+            const double cost = (double)((nt + slots - 1) / slots) * (16384.0 + 128.0 * bn);
+            if (cost < 0.95 * best) {
+                best = cost;
+                BN = bn;
+            }
+        }
+    }
+    const int bsel = BN == 256 ? 2 : BN == 128 ? 1 : 0;
     CUtensorMap ma, mb;
     if (pitch != 0 && (pitch < Ktot || pitch % 8 != 0 || ((uintptr_t)Ap | (uintptr_t)Bp) % 16 != 0)) {
         c->err = "tensor-core GEMM: operand pitch or base not aligned";
@@ -1565,8 +1620,8 @@ static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __
         DCSD_TRY(make_map_kblk(c, &ma, Ap, M, Ktot, TC_BM));
         DCSD_TRY(make_map_kblk(c, &mb, Bp, N, Ktot, mc ? BN / 2 : BN));
     } else {
-        DCSD_TRY(make_map(c, &ma, Ap, M, Ktot, TC_BM, pitch));
-        DCSD_TRY(make_map(c, &mb, Bp, N, Ktot, BN, pitch));
+        DCSD_TRY(make_map(c, &ma, Ap, M, Kst, TC_BM, pitch));
+        DCSD_TRY(make_map(c, &mb, Bp, N, Kst, BN, pitch));
     }
     epi.M = M;
     epi.N = N;
@@ -1599,7 +1654,6 @@ static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __
     else if ((double)N * (double)Ktot * 2.0 <= l2q) group = 1;
     group = (int)std::max<long>(1, std::min<long>(group, tilesM));
     if (mc) group = (int)std::max<long>(1, std::min<long>((group + 1) / 2, tilesMs));
-    size_t smem = TC_STAGES * (TC_BM * TC_BK * 2 + (size_t)BN * TC_BK * 2) + kStageBytesMode2 + 2048;
     const int cls = c->ladder_phase ? DCSD_PROF_LADDER : DCSD_PROF_TC_OTHER;
     prof_begin(c, cls);
     if (c->trace) {
@@ -1610,37 +1664,19 @@ static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __
         trace_begin(c, label);
     }
     ++c->tc_seq;
-    if (mc) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = grid;
-        cfg.blockDim = dim3(kTcThreads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = c->stream;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 2;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        const int tm = (int)tilesM, tn = (int)tilesN, kb = 1;
-        cudaError_t le = BN == 256 ? cudaLaunchKernelEx(&cfg, k_tc_gemm<256, true>, ma, mb, epi, nkt, tm, tn, kper, group,
-                                                        kb, e->d_err)
-                                   : cudaLaunchKernelEx(&cfg, k_tc_gemm<128, true>, ma, mb, epi, nkt, tm, tn, kper, group,
-                                                        kb, e->d_err);
+    {
+        int tm = (int)tilesM, tn = (int)tilesN, kb = kblocked ? 1 : 0, nk = nkt, kp = kper;
+        int* derr = e->d_err;
+        void* args[] = {&ma, &mb, &epi, &parts, &nk, &tm, &tn, &kp, &group, &kb, &derr};
+        config(cfg, at, grid.x, BN);
+        const cudaError_t le = cudaLaunchKernelExC(&cfg, kern[mc ? 1 : 0][bsel], args);
         if (le != cudaSuccess) {
             trace_end(c);
             prof_end(c, cls);
-            c->err = std::string("tc_gemm (cluster launch): ") + cudaGetErrorString(le);
+            c->err = std::string("tc_gemm (launch): ") + cudaGetErrorString(le);
             cudaGetLastError();
             return DCSD_ERR_CUDA;
         }
-    } else if (BN == 256) {
-        k_tc_gemm<256, false><<<grid, kTcThreads, smem, c->stream>>>(ma, mb, epi, nkt, (int)tilesM, (int)tilesN, kper,
-                                                                     group, kblocked ? 1 : 0, e->d_err);
-    } else {
-        k_tc_gemm<128, false><<<grid, kTcThreads, smem, c->stream>>>(ma, mb, epi, nkt, (int)tilesM, (int)tilesN, kper,
-                                                                     group, kblocked ? 1 : 0, e->d_err);
     }
     trace_end(c);
     prof_end(c, cls);
@@ -1837,6 +1873,15 @@ dcsd_status einsum_tc_impl(Ctx* c, const char* spec, double alpha, const TV& A, 
     split_patterns(nsplit, nseg, pa, pb);
     const long Kp = round_up(p.K, TC_BK);
     const long Kt = nseg * Kp;
+    // each operand holds its parts hi (mid (lo)) once; the GEMM's k-steps pick
+    // the parts of the split products
+    const int np = std::max(1, nsplit), whole[6] = {0, 1, 2, 0, 0, 0};
+    TcParts parts;
+    parts.nkb = (int)(Kp / TC_BK);
+    for (int i = 0; i < 6; ++i) {
+        parts.a[i] = pa[i];
+        parts.b[i] = pb[i];
+    }
     // A long contraction onto few output tiles splits K over the SMs
     // (FP32 partial tiles, summed by a second kernel).  Rough time model:
     // 0.4 us per 64-deep k-step and tile wave plus operand packing at
@@ -1899,9 +1944,9 @@ dcsd_status einsum_tc_impl(Ctx* c, const char* spec, double alpha, const TV& A, 
     const double* nsrc = swapped ? A.p : B.p;
     const __nv_bfloat16* Apk = nullptr;
     const __nv_bfloat16* Bpk = nullptr;
-    DCSD_TRY(pack_operand(c, msrc, p.nm, p.m_size, p.m_sa, p.nk, p.k_size, p.k_sa, p.M, p.K, Kp, nseg, pa,
+    DCSD_TRY(pack_operand(c, msrc, p.nm, p.m_size, p.m_sa, p.nk, p.k_size, p.k_sa, p.M, p.K, Kp, np, whole,
                           e->pa, Apk));
-    DCSD_TRY(pack_operand(c, nsrc, p.nn, p.n_size, p.n_sb, p.nk, p.k_size, p.k_sb, p.N, p.K, Kp, nseg, pb,
+    DCSD_TRY(pack_operand(c, nsrc, p.nn, p.n_size, p.n_sb, p.nk, p.k_size, p.k_sb, p.N, p.K, Kp, np, whole,
                           e->pb, Bpk));
     TcEpi epi;
     std::memset(&epi, 0, sizeof(epi));
@@ -1923,7 +1968,7 @@ dcsd_status einsum_tc_impl(Ctx* c, const char* spec, double alpha, const TV& A, 
         epi.n_size[i] = i < p.nn ? p.n_size[i] : 1;
         epi.n_s[i] = i < p.nn ? p.n_sc[i] : 0;
     }
-    if (ksplit <= 1) return gemm_packed(c, Apk, p.M, Bpk, p.N, Kt, epi);
+    if (ksplit <= 1) return gemm_packed(c, Apk, p.M, Bpk, p.N, Kt, epi, 1, 0, false, false, &parts, np);
     // split K: partial tiles, then C (or its FP32 shadow) from their sum
     {
         const int nkt = (int)(Kt / TC_BK), kper = (nkt + ksplit - 1) / ksplit;
@@ -1942,7 +1987,7 @@ dcsd_status einsum_tc_impl(Ctx* c, const char* spec, double alpha, const TV& A, 
     red.N = p.N;
     epi.mode = 5;
     epi.C32 = e->wsk;
-    DCSD_TRY(gemm_packed(c, Apk, p.M, Bpk, p.N, Kt, epi, ksplit));
+    DCSD_TRY(gemm_packed(c, Apk, p.M, Bpk, p.N, Kt, epi, ksplit, 0, false, false, &parts, np));
     if (c->trace) trace_begin(c, "tc-splitk-reduce " + c->cur_spec);
     k_tc_splitk_reduce<<<(unsigned)std::max<long>(1, std::min<long>((p.M * p.N + 255) / 256, (long)c->num_sms * 8)),
                          256, 0, c->stream>>>(red, ksplit, e->wsk);
@@ -2054,6 +2099,7 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
     int nseg, pa[6], pb[6];
     split_patterns(nsplit, nseg, pa, pb);
     const long Vp = round_up(V, 8);
+    const int np = std::max(1, nsplit);  // parts of an operand: hi (mid (lo))
     const long KS = sa_koff(V, Vp), KSp = round_up(KS, TC_BK), KSt = nseg * KSp;
     const long XP = round_up(X, TC_BK), Xt = nseg * XP;
     const int nblk = (int)((Vp + 127) / 128);
@@ -2088,10 +2134,10 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
         e->sa_O = O;
     }
     // stacked A- and A+ amplitudes (the partial last k-block zeroed first)
-    DCSD_TRY(ensure(c, e->sam, (size_t)rowsM * KSt));
-    DCSD_TRY(ensure(c, e->sap, (size_t)rowsP * KSt));
+    DCSD_TRY(ensure(c, e->sam, (size_t)rowsM * KSp * np));
+    DCSD_TRY(ensure(c, e->sap, (size_t)rowsP * KSp * np));
     if (KS % TC_BK != 0)
-        for (int sg = 0; sg < nseg; ++sg) {
+        for (int sg = 0; sg < np; ++sg) {
             const long k0 = KS / TC_BK * TC_BK;
             DCSD_CUDA(c, cudaMemsetAsync(e->sam.p + (size_t)sg * rowsM * KSp + (size_t)k0 * rowsM, 0,
                                          sizeof(__nv_bfloat16) * rowsM * TC_BK, c->stream));
@@ -2114,8 +2160,8 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
         sp.Ap = e->sap.p;
         sp.rowsM = rowsM;
         sp.rowsP = rowsP;
-        sp.nseg = nseg;
-        for (int i = 0; i < 6; ++i) sp.pat[i] = pa[i];
+        sp.nseg = np;
+        for (int i = 0; i < np; ++i) sp.pat[i] = i;
         const long work = (2 * P + O * O) * ((long)sp.ntile * (sp.ntile + 1) / 2);
         prof_begin(c, DCSD_PROF_PACK);
         if (c->trace) trace_begin(c, "pack sa-amplitudes rows=" + std::to_string(rowsM + rowsP) + " K=" + std::to_string(KS));
@@ -2124,22 +2170,23 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
         prof_end(c, DCSD_PROF_PACK);
         DCSD_TRY(launch_check(c, "pack_sa"));
     }
-    // the DF factors B[L][x][nc + y] as [(x, y)][L] for every orbital x (the
-    // virtual rows serve the ladder, the occupied ones the G pass), y padded
-    // to YP, with the A- and B-side split patterns (B never changes: packed
-    // once per split)
+    // the DF factors B[L][x][nc + y] as [part][(x, y)][L] for every orbital x
+    // (the virtual rows serve the ladder, the occupied ones the G pass), y
+    // padded to YP (B never changes: the parts are packed once)
     const long xrows = n * YP;
-    DCSD_TRY(ensure(c, e->sxa, (size_t)xrows * Xt));
-    DCSD_TRY(ensure(c, e->sxb, (size_t)xrows * Xt));
-    if (e->sx_nsplit != nsplit) {
+    {
+        const __nv_bfloat16* old = e->sx.p;
+        DCSD_TRY(ensure(c, e->sx, (size_t)xrows * XP * np));
+        if (e->sx.p != old) e->sx_nsplit = 0;
+    }
+    if (e->sx_nsplit < np) {
         e->sx_nsplit = 0;
+        const int parts[3] = {0, 1, 2};
         long rsz[2] = {n, YP}, rs[2] = {n, 1};
         long ksz[1] = {X}, ks[1] = {n * n};
-        DCSD_TRY(pack(c, c->B + nc, 2, rsz, rs, 1, ksz, ks, xrows, X, XP, nseg, pa, e->sxa.p, V, 1l << 62, nullptr,
+        DCSD_TRY(pack(c, c->B + nc, 2, rsz, rs, 1, ksz, ks, xrows, X, XP, np, parts, e->sx.p, V, 1l << 62, nullptr,
                       0, xrows * XP, xrows * 64));
-        DCSD_TRY(pack(c, c->B + nc, 2, rsz, rs, 1, ksz, ks, xrows, X, XP, nseg, pb, e->sxb.p, V, 1l << 62, nullptr,
-                      0, xrows * XP, xrows * 64));
-        e->sx_nsplit = nsplit;
+        e->sx_nsplit = np;
     }
     // M+ and M- tiles of a chunk (zeroed when allocated: rows b' < r and the
     // k padding are never written, and must be finite).  Chunks of up to 16
@@ -2147,7 +2194,7 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
     const long chunk = std::max<long>(1, std::min<long>(V, 16));
     for (Buf* b : {&e->svp, &e->svm}) {
         const __nv_bfloat16* old = b->p;
-        DCSD_TRY(ensure(c, *b, (size_t)chunk * V * KSt));
+        DCSD_TRY(ensure(c, *b, (size_t)chunk * V * KSp * np));
         if (b->p != old) DCSD_CUDA(c, cudaMemsetAsync(b->p, 0, b->cap * sizeof(__nv_bfloat16), c->stream));
     }
     const size_t smem = SA_STAGES * 4 * (size_t)SA_TILE + 2048;
@@ -2155,9 +2202,8 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
         DCSD_CUDA(c, cudaFuncSetAttribute(k_ladder_sa, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         e->sa_attr = true;
     }
-    CUtensorMap ma, mb;
-    DCSD_TRY(make_map_kblk(c, &ma, e->sxa.p, xrows, Xt, 128));
-    DCSD_TRY(make_map_kblk(c, &mb, e->sxb.p, xrows, Xt, 128));
+    CUtensorMap mx;
+    DCSD_TRY(make_map_kblk(c, &mx, e->sx.p, xrows, XP * np, 128));
     // pass 0, the ladder: chunks of a (triangle b >= a), scatter into R2;
     // pass 1, the G intermediate G[s][i][j][k][b] = sum_cd t[ij][cd] (kc|bd)
     // (s = 3: t with (c,d) exchanged): chunks of occupied k against every b,
@@ -2174,6 +2220,7 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
             SaArgs sa;
             std::memset(&sa, 0, sizeof(sa));
             sa.nkt = (int)(Xt / TC_BK);
+            sa.nkb = (int)(XP / TC_BK);
             sa.nr = (int)nr;
             sa.Vb = (int)Vb;
             sa.nblk = nblk;
@@ -2187,8 +2234,11 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
             sa.Vp = (int)Vp;
             sa.kbs = vrows * 64;
             sa.segstride = vrows * KSp;
-            sa.nseg = nseg;
-            for (int i = 0; i < 6; ++i) sa.pat[i] = pb[i];
+            sa.nparts = np;
+            for (int i = 0; i < 6; ++i) {
+                sa.part_a[i] = pa[i];
+                sa.part_b[i] = pb[i];
+            }
             sa.Vplus = e->svp.p;
             sa.Vminus = e->svm.p;
             prof_begin(c, DCSD_PROF_LADDER);
@@ -2200,8 +2250,7 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
                 trace_begin(c, label);
             }
             ++c->tc_seq;
-            k_ladder_sa<<<(unsigned)std::min<long>(sa.ntiles, c->num_sms), kTcThreads, smem, c->stream>>>(ma, mb, sa,
-                                                                                                            e->d_err);
+            k_ladder_sa<<<(unsigned)std::min<long>(sa.ntiles, c->num_sms), kTcThreads, smem, c->stream>>>(mx, sa, e->d_err);
             trace_end(c);
             prof_end(c, DCSD_PROF_LADDER);
             DCSD_TRY(launch_check(c, "ladder_sa"));
@@ -2220,11 +2269,11 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
             ce.VV = V * V;
             for (int sp = 0; sp < nseg; ++sp) {
                 ce.rowcode = e->d_code_m;
-                DCSD_TRY(gemm_packed(c, e->sam.p + (size_t)sp * rowsM * KSp, rowsM,
-                                     e->svm.p + (size_t)sp * vrows * KSp, vrows, KSp, ce, 1, 0, true, true));
+                DCSD_TRY(gemm_packed(c, e->sam.p + (size_t)pa[sp] * rowsM * KSp, rowsM,
+                                     e->svm.p + (size_t)pb[sp] * vrows * KSp, vrows, KSp, ce, 1, 0, true, true));
                 ce.rowcode = e->d_code_p;
-                DCSD_TRY(gemm_packed(c, e->sap.p + (size_t)sp * rowsP * KSp, rowsP,
-                                     e->svp.p + (size_t)sp * vrows * KSp, vrows, KSp, ce, 1, 0, true, true));
+                DCSD_TRY(gemm_packed(c, e->sap.p + (size_t)pa[sp] * rowsP * KSp, rowsP,
+                                     e->svp.p + (size_t)pb[sp] * vrows * KSp, vrows, KSp, ce, 1, 0, true, true));
             }
         }
     }
