@@ -217,6 +217,11 @@ dcsd_status alloc(Ctx* c, double** p, size_t n) {
 }
 
 void free_ctx(Ctx* c) {
+    for (auto& g : c->graphs)
+        if (g.exec) cudaGraphExecDestroy(g.exec);
+    c->graphs.clear();
+    if (c->capture) cudaStreamDestroy(c->capture);
+    c->capture = nullptr;
     double** ptrs[] = {&c->B, &c->fock[0], &c->fock[1], &c->Kref[0][0], &c->Kref[0][1],
                        &c->Kref[1][0], &c->Kref[1][1], &c->t1, &c->R1, &c->t2s, &c->Bd, &c->Pbt, &c->fd,
                        &c->fsc, &c->Z, &c->J, &c->H, &c->G, &c->Wo, &c->Foc, &c->Fvi, &c->big0,
@@ -229,6 +234,8 @@ void free_ctx(Ctx* c) {
     }
     c->t2 = nullptr;
     c->R2 = nullptr;
+    if (c->pool) cudaFree(c->pool);
+    c->pool = nullptr;
     if (c->gemm64_count) cudaFree(c->gemm64_count);
     c->gemm64_count = nullptr;
     if (c->vvvv) cudaFree(c->vvvv);
@@ -407,6 +414,16 @@ extern "C" dcsd_status dcsd_init(dcsd_ctx** out, const dcsd_dims* d, const doubl
     c->splitk_elems = std::max<size_t>(1 << 20, std::min<size_t>(64ul << 20, 16 * (n * n + O * V)));
     A_(c->splitk_ws, c->splitk_elems);
     A_(c->scal, 64);
+    {
+        // intermediates of an FP64 residual side by side, for systems where
+        // that takes at most 256 MB (about 60 virtuals)
+        const size_t pool = 2 * X * n * n + 10 * X * OV + 2 * X * n * O + 16 * n * n + 16 * OV * OV + 7 * O * O * O * V +
+                            6 * O * O * O * O + V * V * V * V + O * V * V * V + 2 * V * V + 8 * OV + 4096;
+        if (pool <= (size_t)1 << 25) {
+            A_(c->pool, pool);
+            c->pool_elems = pool;
+        }
+    }
     double* counters = nullptr;
     A_(counters, kGemm64Counters / 2);
     c->gemm64_count = (unsigned*)counters;
@@ -506,7 +523,7 @@ static dcsd_status residual_common(Ctx* c, int ref, int method, int prec, int me
         }
     }
     DCSD_TRY(unpack_T(c, ref, Td[0], Td[1], Td[2], Td[3], Td[4]));
-    DCSD_TRY(residual_union(c, ref, method, prec));
+    DCSD_TRY(residual_run(c, ref, method, prec));
     if (R) {
         for (int k = 0; k < 5; ++k)
             if (!R[k]) {
@@ -1015,7 +1032,7 @@ extern "C" dcsd_status dcsd_solve(dcsd_ctx* h, const dcsd_solve_opts* o, int mem
         if (prec == DCSD_PREC_MIXED)
             prec = phase == 0 ? DCSD_PREC_BF16 : phase == 1 ? DCSD_PREC_BF16X6
                                                              : (outer ? DCSD_PREC_FP64 : DCSD_PREC_BF16X6);
-        dcsd_status s = residual_union(c, ref, o->method, prec);
+        dcsd_status s = residual_run(c, ref, o->method, prec);
         if (s != DCSD_OK) { status = s; break; }
         if (refining && !outer) {
             if ((s = axpy_view(c, -1.0, view(c->defect, {len}), 1.0, Rall)) != DCSD_OK) { status = s; break; }
@@ -1046,7 +1063,7 @@ extern "C" dcsd_status dcsd_solve(dcsd_ctx* h, const dcsd_solve_opts* o, int mem
             if (!c->defect && (s = alloc(c, &c->defect, len)) != DCSD_OK) { status = s; break; }
             double* defect = c->defect;
             DCSD_CUDA(c, cudaMemcpyAsync(defect, c->R1, len * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
-            if ((s = residual_union(c, ref, o->method, DCSD_PREC_BF16X6)) != DCSD_OK) { status = s; break; }
+            if ((s = residual_run(c, ref, o->method, DCSD_PREC_BF16X6)) != DCSD_OK) { status = s; break; }
             if ((s = axpy_view(c, 1.0, Rall, -1.0, view(defect, {len}))) != DCSD_OK) { status = s; break; }
             if ((s = axpy_view(c, -1.0, view(defect, {len}), 1.0, Rall)) != DCSD_OK) { status = s; break; }
             outer = false;

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <cstdint>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -110,6 +111,14 @@ struct AdjRegion {
 struct CrtEngine;
 constexpr long kGemm64Counters = 4096;
 
+// Memory that a launch reads or writes, for the dependencies of recorded launches
+struct Span {
+    const void* lo;
+    const void* hi;
+    bool write;
+};
+struct Dag;
+
 struct Ctx {
     int nc = 0, nv = 0, X = 0;
     int n = 0, O = 0, V = 0;      // n = nc+2+nv; union occ O = nc+2; union vir V = nv+2
@@ -154,6 +163,7 @@ struct Ctx {
     size_t splitk_elems = 0;
     // FP64 contractions in a fixed order of summation (see einsum64)
     bool fma_chain = false;
+    long chain_m = 0, chain_n = 0;  // extents that decide the split of K under fma_chain (0: the contraction's own)
     unsigned* gemm64_count = nullptr;  // [kGemm64Counters] block arrivals of a split contraction (zero between launches)
     double* scal = nullptr;       // device scalars: [0]=W [1]=dEA [2..] misc
     double* c1 = nullptr;         // [2][O][V] two-determinant coefficients
@@ -186,6 +196,23 @@ struct Ctx {
     // tensor-core ladder in symmetric / antisymmetric form over the (c <= d)
     // pairs (DCSD_LADDER_SA=0 selects the contraction over all (c, d))
     bool ladder_sa = true;
+
+    // CUDA graphs of residual_union, one per argument set (see residual_run)
+    struct Graph {
+        int key = -1;
+        cudaGraphExec_t exec = nullptr;
+        std::vector<uint64_t> state;  // what the recorded launches depend on
+        long long launches = 0;
+    };
+    std::vector<Graph> graphs;
+    cudaStream_t capture = nullptr;   // recording stream (the user's may be the legacy stream)
+    bool graphs_off = false;          // a recording failed: launches one by one
+    Dag* dag = nullptr;               // set while recording (see DagOp)
+    // intermediates of one residual in buffers of their own, taken one after
+    // the other, so that independent launches do not wait for a shared buffer
+    // (allocated for small systems)
+    double* pool = nullptr;
+    size_t pool_elems = 0, pool_used = 0;
 
     MTables* mt[2] = {};          // per reference
     TcEngine* tc = nullptr;
@@ -288,6 +315,32 @@ struct FmaChain {
         if (s_ != DCSD_OK) return s_;                                         \
     } while (0)
 
+// Recorded launches depend on the earlier ones whose memory they touch, not on
+// all of them.  A launcher declares what its launches read and write:
+//     const DagOp op(c, {rd(A), rd(B), wr(C)});  ... launches ...
+// They follow one another and start once every earlier launch that writes
+// what they read, or touches what they write, is done.  Launches outside any
+// DagOp come after everything before them and before everything after them.
+// Outside recording a DagOp does nothing.
+inline Span span_of(const TV& v, bool write) {
+    long n = 1;
+    for (int i = 0; i < v.rank; ++i) n += (v.size[i] - 1) * v.stride[i];
+    return {v.p, v.p + (n > 0 ? n : 0), write};
+}
+inline Span rd(const TV& v) { return span_of(v, false); }
+inline Span wr(const TV& v) { return span_of(v, true); }
+inline Span rd(const void* p, size_t bytes) { return {p, (const char*)p + bytes, false}; }
+inline Span wr(const void* p, size_t bytes) { return {p, (const char*)p + bytes, true}; }
+struct DagOp {
+    Ctx* c;
+    DagOp(Ctx* c_, std::initializer_list<Span> spans);
+    ~DagOp();
+    DagOp(const DagOp&) = delete;
+};
+// a piece of a scratch buffer of `size` units: another one for every recorded
+// launch (starting over when it is used up), the whole buffer otherwise
+size_t dag_slice(Ctx* c, int which, size_t need, size_t size);
+
 // ---------------------------------------------------------------------------
 // kernels (launchers return DCSD_OK or set ctx->err)
 // ---------------------------------------------------------------------------
@@ -299,6 +352,8 @@ dcsd_status einsum32(Ctx* c, const char* spec, double alpha, const TV& A,
                      const TV& B, double beta, const TV& C);
 // C (+)= alpha * A elementwise over identical index sets (4D max), any strides
 dcsd_status axpy_view(Ctx* c, double alpha, const TV& A, double beta, const TV& C);
+// C += (*alpha) A with alpha on the device; nothing where it is zero
+dcsd_status axpy_view_scalar(Ctx* c, const double* alpha, const TV& A, const TV& C);
 // sum_i A_i * B_i over identical shapes -> *out (device pointer), FP64
 dcsd_status dot_view(Ctx* c, const TV& A, const TV& B, double* out, double accumulate);
 dcsd_status fill(Ctx* c, double* p, size_t n, double val);
@@ -353,6 +408,11 @@ inline double method_fr_value(int m) { return m >= DCSD_FR_CCSD_T ? -1.0 : 1.0; 
 
 // residual orchestration (residual.cu)
 dcsd_status residual_union(Ctx* c, int ref, int method, int precision);
+// runs body, whose launches work on the context's own buffers only: launch by
+// launch the first time, then as a CUDA graph per key
+dcsd_status graph_run(Ctx* c, int key, const std::function<dcsd_status()>& body);
+// residual_union through graph_run
+dcsd_status residual_run(Ctx* c, int ref, int method, int precision);
 // reverse mode helpers (vjp.cu)
 // buffer for an intermediate: `normal` outside recording, a fresh arena block
 // (with a zeroed adjoint twin) while recording
@@ -367,11 +427,11 @@ inline bool recording(const Ctx* c) { return c->rec; }
 // that many operand splits.  One tape entry while recording; compute false
 // writes only that entry (a caller that produces the values another way).
 dcsd_status ladder64(Ctx* c, const TV& t2, const TV& Bvv, const TV& R2, double* chunkbuf, long chunk,
-                     int nsplit = 0, bool compute = true);
+                     int nsplit = 0, bool compute = true, long order_chunk = 0);
 // ladder T1-correction intermediate G[s][ij][k][b] = sum_cd t_s[ij][cd] (kc|bd)
 // (G[3] with t_ab exchanged in (c,d)) by chunks over k; one tape entry
 dcsd_status gpass(Ctx* c, const TV& t2, const TV& Bov, const TV& Bvv, const TV& G, double* chunkbuf, long chunk,
-                  int nsplit = 0, bool compute = true);
+                  int nsplit = 0, bool compute = true, long order_chunk = 0);
 void vjp_free(Ctx* c);
 // reverse mode in stages: record the FP64 residual at c->t1/c->t2, then any
 // number of reverse sweeps with union-layout seeds; the gradients of the
@@ -417,6 +477,8 @@ dcsd_status einsum_tc(Ctx* c, const char* spec, double alpha, const TV& A,
 
 // pp ladder + its T1 correction on tensor cores (R2 += ladder, G = correction)
 dcsd_status ladder_tc(Ctx* c, int nsplit, double* R2, double* G);
+// the engine's buffers and packed-operand states that recorded launches use
+void tc_state(const Ctx* c, std::vector<uint64_t>& s);
 // sources whose packed operands einsum_tc may reuse (NULL: none); clears the cache
 void pack_cache_set(Ctx* c, const double* src0, const double* src1);
 // the BF16 image of t2 with the parts of an nsplit-way split (see Ctx)

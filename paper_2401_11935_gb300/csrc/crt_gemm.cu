@@ -807,7 +807,10 @@ static dcsd_status crt_pass(Ctx* c, const char* spec, const GemmPlan& p, const d
     g.kper = (int)((g.nkb + ns - 1) / ns);
     g.nsplit = (g.nkb + g.kper - 1) / g.kper;
     g.group = (int)std::max<long>(1, std::min<long>(tilesMs, std::lround(std::sqrt((double)slots * g.BN / CG_BM / (mc ? 2 : 1)))));
-    uint8_t* w = e->ws;
+    // (recorded: a piece of the workspace of its own when it is large enough)
+    const size_t need = pass_bytes(M, N, K, g.nsplit);
+    const size_t at = need <= e->bytes / 2 ? dag_slice(c, 3, (need + 255) / 256 * 256, e->bytes) : 0;
+    uint8_t* w = e->ws + at;
     auto take = [&](size_t bytes) {
         uint8_t* r = w;
         w += (bytes + 255) / 256 * 256;
@@ -847,10 +850,21 @@ static dcsd_status crt_pass(Ctx* c, const char* spec, const GemmPlan& p, const d
     }
     const long N4 = (N + 3) / 4;
     g.planes = (uint32_t*)take((size_t)g.nsplit * kMods * 4 * N4 * M);
-    if ((size_t)(w - e->ws) > e->bytes) {
+    if ((size_t)(w - e->ws) > e->bytes || (size_t)(w - e->ws) > at + need) {
         c->err = std::string(spec) + ": modular GEMM workspace";
         return DCSD_ERR_INVALID_ARG;
     }
+    auto view_of = [](const double* p0, int na, const long* sa, const long* ta, int nb, const long* sb, const long* tb,
+                      bool write) {
+        long n = 1;
+        for (int i = 0; i < na; ++i) n += (sa[i] - 1) * ta[i];
+        for (int i = 0; i < nb; ++i) n += (sb[i] - 1) * tb[i];
+        return Span{p0, p0 + n, write};
+    };
+    const DagOp op(c, {view_of(Ap, p.nm, p.m_size, p.m_sa, p.nk, p.k_size, p.k_sa, false),
+                       view_of(Bp, p.nn, p.n_size, p.n_sb, p.nk, p.k_size, p.k_sb, false),
+                       view_of(Cp, p.nm, p.m_size, p.m_sc, p.nn, p.n_size, p.n_sc, true),
+                       wr(e->ws + at, (size_t)(w - e->ws) - at)});
     prof_begin(c, DCSD_PROF_FP64);
     auto label = [&](const char* what) {
         return std::string(what) + spec + " M=" + std::to_string(M) + " N=" + std::to_string(N) + " K=" +

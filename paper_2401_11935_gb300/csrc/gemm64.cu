@@ -279,6 +279,7 @@ struct Gemm64Args {
     int tilesN;
     int nsplit;        // K splits (NB = 1 only): blockIdx.y = split
     long kchunk;       // K per split
+    long kseg;         // > 0: a thread adds chains of kseg k in order (a multiple of 16; no split)
     double* ws;        // [tile][split][T * T] partial sums
     unsigned* count;   // [tile] arrivals (zero between launches)
 };
@@ -350,7 +351,8 @@ __global__ void __launch_bounds__(T* T* SL) k_gemm64(const Gemm64Args g) {
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
         for (int c = 0; c < kG64Stages - 1; ++c) load(c);
-        double acc = 0.0;
+        double acc = 0.0, total = 0.0;
+        long left = g.kseg;  // k left in the current chain
         for (long c = 0; c < nch; ++c) {
             asm volatile("cp.async.wait_group %0;" ::"n"(kG64Stages - 2) : "memory");
             __syncthreads();
@@ -358,7 +360,22 @@ __global__ void __launch_bounds__(T* T* SL) k_gemm64(const Gemm64Args g) {
             const int st = (int)(c % kG64Stages);
             if (rowlive) {
                 const int kn = (int)min((long)KC, ke - kb - c * KC);
-                if (kn == KC) {
+                if (SL == 1 && g.kseg > 0) {
+                    for (int h = 0; h < kn; h += 16) {
+                        if (kn - h >= 16) {
+#pragma unroll
+                            for (int kk = 0; kk < 16; ++kk) acc = fma(As[st][h + kk][ty], Bs[st][h + kk][tx], acc);
+                        } else {
+                            for (int k = h; k < kn; ++k) acc = fma(As[st][k][ty], Bs[st][k][tx], acc);
+                        }
+                        left -= 16;
+                        if (left == 0) {
+                            total += acc;
+                            acc = 0.0;
+                            left = g.kseg;
+                        }
+                    }
+                } else if (kn == KC) {
 #pragma unroll
                     for (int kk = 0; kk < KC / SL; ++kk)
                         acc = fma(As[st][kk * SL + slice][ty], Bs[st][kk * SL + slice][tx], acc);
@@ -369,6 +386,7 @@ __global__ void __launch_bounds__(T* T* SL) k_gemm64(const Gemm64Args g) {
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
+        if (SL == 1 && g.kseg > 0) acc = total + acc;
         if (SL > 1) {
             double* red = &As[0][0][0];
             red[tid] = acc;
@@ -656,6 +674,7 @@ static dcsd_status einsum_simt(Ctx* c, const char* spec, double alpha, const TV&
     if (engine != 2 && g.p.NB == 1 && (g.p.N == 1 || g.p.M == 1) && g.p.K >= 64) {
         const int vec_is_b = g.p.N == 1 ? 1 : 0;
         const long outs = vec_is_b ? g.p.M : g.p.N;
+        const DagOp op(c, {rd(A), rd(B), wr(C)});
         prof_begin(c, DCSD_PROF_FP64);
         if (c->trace)
             trace_begin(c, std::string("fp64-gemv ") + spec + " M=" + std::to_string(g.p.M) + " N=" +
@@ -683,13 +702,17 @@ static dcsd_status einsum_simt(Ctx* c, const char* spec, double alpha, const TV&
         int T = tiles_of(16) * std::min<long>(g.p.NB, 65535) >= 2l * c->num_sms ? 16 : 8;
         long nt = tiles_of(T);
         long ns = 1;
+        h.kseg = 0;
         if (c->fma_chain) {
             // fixed order of summation: one FMA chain per output, or, for few
-            // 64 x 64 tiles and a long K, chains over pieces of K added in order
-            const long t64 = tiles_of(64);
+            // 64 x 64 tiles and a long K, chains over pieces of K added in
+            // order, by a block each where the tiles do not fill the chip.
+            // (chain_m, chain_n: the extents that decide, see ladder64)
+            const long cm = c->chain_m > 0 ? c->chain_m : g.p.M, cn = c->chain_n > 0 ? c->chain_n : g.p.N;
+            const long t64 = ((cm + 63) / 64) * ((cn + 63) / 64);
             if (g.p.NB == 1 && t64 < c->num_sms && g.p.K >= 2048) {
                 ns = std::min<long>((8 * c->num_sms + t64 - 1) / t64, g.p.K / 256);
-                ns = std::min<long>(ns, (long)(c->splitk_elems / std::max<long>(1, g.p.M * g.p.N)));
+                ns = std::min<long>(ns, (long)(c->splitk_elems / std::max<long>(1, cm * cn)));
                 ns = std::min<long>(ns, 65535);
             }
             h.kchunk = ns >= 2 ? ((g.p.K + ns - 1) / ns + 15) / 16 * 16 : g.p.K;
@@ -700,7 +723,11 @@ static dcsd_status einsum_simt(Ctx* c, const char* spec, double alpha, const TV&
                 };
                 T = tiles_of(16) * real >= 2l * c->num_sms ? 16 : 8;
                 if (!fits(T)) T = 24 - T;
-                if (!fits(T)) h.kchunk = g.p.K;  // (tiles of 64 padded past the workspace)
+                if (!fits(T) || tiles_of(16) >= 2l * c->num_sms) {
+                    T = tiles_of(16) >= 2l * c->num_sms ? 16 : 8;
+                    h.kseg = h.kchunk;
+                    h.kchunk = g.p.K;
+                }
                 nt = tiles_of(T);
             }
         } else {
@@ -713,8 +740,11 @@ static dcsd_status einsum_simt(Ctx* c, const char* spec, double alpha, const TV&
         h.nsplit = (int)((g.p.K + h.kchunk - 1) / h.kchunk);
         if (h.nsplit < 1) h.nsplit = 1;
         h.tilesN = (int)((g.p.N + T - 1) / T);
-        h.ws = c->splitk_ws;
-        h.count = c->gemm64_count;
+        // (split: a piece of the partial sums and counters of its own)
+        const size_t wn = h.nsplit > 1 ? (size_t)nt * h.nsplit * T * T : 0, cn = h.nsplit > 1 ? (size_t)nt : 0;
+        h.ws = c->splitk_ws + dag_slice(c, 0, wn, c->splitk_elems);
+        h.count = c->gemm64_count + dag_slice(c, 1, cn, kGemm64Counters);
+        const DagOp op(c, {rd(A), rd(B), wr(C), wr(h.ws, 8 * wn), wr(h.count, 4 * cn)});
         const dim3 grid((unsigned)nt, (unsigned)(h.nsplit > 1 ? h.nsplit : std::min<long>(g.p.NB, 65535)));
         prof_begin(c, DCSD_PROF_FP64);
         if (c->trace)
@@ -743,6 +773,7 @@ static dcsd_status einsum_simt(Ctx* c, const char* spec, double alpha, const TV&
             g.ws = c->splitk_ws;
         }
     }
+    const DagOp op(c, {rd(A), rd(B), wr(C), wr(c->splitk_ws, 8 * c->splitk_elems)});
     dim3 grid((unsigned)((g.p.M + GBM - 1) / GBM), (unsigned)((g.p.N + GBN - 1) / GBN),
               (unsigned)(g.nsplit > 1 ? g.nsplit : std::min<long>(g.p.NB, 65535)));
     prof_begin(c, DCSD_PROF_FP64);
@@ -771,6 +802,7 @@ struct EwArgs {
     const double* A;
     double* C;
     double alpha, beta;
+    const double* alpha_dev;  // when set, alpha is read from here, and a zero leaves C as it is
 };
 
 // linear index -> (offset in A, offset in C); I = unsigned when the element
@@ -792,11 +824,13 @@ __device__ __forceinline__ void ew_offsets(const EwArgs& a, I idx, long& oa, lon
 
 template <typename I>
 __global__ void k_axpy_view(EwArgs a) {
+    const double alpha = a.alpha_dev ? *a.alpha_dev : a.alpha;
+    if (a.alpha_dev && alpha == 0.0) return;
     for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < a.total;
          e += (long)gridDim.x * blockDim.x) {
         long oa, oc;
         ew_offsets<I>(a, (I)e, oa, oc);
-        double v = a.alpha * a.A[oa];
+        double v = alpha * a.A[oa];
         if (a.beta != 0.0) v += a.beta * a.C[oc];
         a.C[oc] = v;
     }
@@ -844,6 +878,23 @@ static unsigned grid_for(Ctx* c, long total) {
     return (unsigned)std::max<long>(1, std::min(g, cap));
 }
 
+static dcsd_status axpy_launch(Ctx* c, double alpha, const double* alpha_dev, const TV& A, double beta, const TV& C) {
+    EwArgs a;
+    if (!ew_setup(c, A, C, a)) return DCSD_ERR_INVALID_ARG;
+    if (a.total == 0) return DCSD_OK;
+    a.A = A.p;
+    a.C = C.p;
+    a.alpha = alpha;
+    a.alpha_dev = alpha_dev;
+    a.beta = beta;
+    const DagOp op(c, {rd(A), wr(C), rd(alpha_dev, alpha_dev ? 8 : 0)});
+    if (c->trace) trace_begin(c, "axpy rank=" + std::to_string(a.rank) + " n=" + std::to_string(a.total));
+    if (a.total < (1l << 32)) k_axpy_view<unsigned><<<grid_for(c, a.total), 256, 0, c->stream>>>(a);
+    else k_axpy_view<unsigned long><<<grid_for(c, a.total), 256, 0, c->stream>>>(a);
+    trace_end(c);
+    return launch_check(c, "axpy_view");
+}
+
 dcsd_status axpy_view(Ctx* c, double alpha, const TV& A, double beta, const TV& C) {
     if (c->rec) {
         TapeOp op;
@@ -854,18 +905,11 @@ dcsd_status axpy_view(Ctx* c, double alpha, const TV& A, double beta, const TV& 
         op.C = C;
         rec_push(c, std::move(op));
     }
-    EwArgs a;
-    if (!ew_setup(c, A, C, a)) return DCSD_ERR_INVALID_ARG;
-    if (a.total == 0) return DCSD_OK;
-    a.A = A.p;
-    a.C = C.p;
-    a.alpha = alpha;
-    a.beta = beta;
-    if (c->trace) trace_begin(c, "axpy rank=" + std::to_string(a.rank) + " n=" + std::to_string(a.total));
-    if (a.total < (1l << 32)) k_axpy_view<unsigned><<<grid_for(c, a.total), 256, 0, c->stream>>>(a);
-    else k_axpy_view<unsigned long><<<grid_for(c, a.total), 256, 0, c->stream>>>(a);
-    trace_end(c);
-    return launch_check(c, "axpy_view");
+    return axpy_launch(c, alpha, nullptr, A, beta, C);
+}
+
+dcsd_status axpy_view_scalar(Ctx* c, const double* alpha, const TV& A, const TV& C) {
+    return axpy_launch(c, 0.0, alpha, A, 1.0, C);
 }
 
 // C[i0,i1,i2,i3] += sum_k alpha_k * A_k[i0,i1,i2,i3] for up to 4 strided views
@@ -930,6 +974,8 @@ dcsd_status axpy4(Ctx* c, int nv, const double* alpha, const TV* A, const TV& C)
     }
     a.C = C.p;
     const long nrow = C.size[0] * C.size[1];
+    const TV &X1 = A[nv > 1 ? 1 : 0], &X2 = A[nv > 2 ? 2 : 0], &X3 = A[nv > 3 ? 3 : 0];
+    const DagOp op(c, {rd(A[0]), rd(X1), rd(X2), rd(X3), wr(C)});
     if (c->trace) trace_begin(c, "axpy4 n=" + std::to_string(nrow * C.size[2] * C.size[3]));
     k_axpy4<<<(unsigned)std::max<long>(1, std::min<long>(nrow, (long)c->num_sms * 32)), 256, 0, c->stream>>>(a);
     trace_end(c);
@@ -1008,6 +1054,7 @@ dcsd_status ring_antisym_add(Ctx* c, const TV& X, const TV& R) {
     if (c->rec) record_axpy4(c, 4, al, views, R);
     const long nt = (V + 31) / 32, work = O * (O - 1) / 2 * (nt * (nt + 1) / 2);
     if (work == 0) return DCSD_OK;
+    const DagOp op(c, {rd(X), wr(R)});
     if (c->trace) trace_begin(c, "ring_antisym n=" + std::to_string(O * O * V * V));
     k_ring_antisym<<<(unsigned)std::max<long>(1, std::min<long>(work, (long)c->num_sms * 16)), 256, 0, c->stream>>>(
         X.p, R.p, (int)O, (int)V);
@@ -1060,6 +1107,7 @@ dcsd_status add_swapped(Ctx* c, const TV& X, const TV& R) {
     }
     const long nt = (V + 31) / 32, work = O * O * nt * nt;
     if (work == 0) return DCSD_OK;
+    const DagOp op(c, {rd(X), wr(R)});
     if (c->trace) trace_begin(c, "add_swapped n=" + std::to_string(O * O * V * V));
     k_add_swapped<<<(unsigned)std::max<long>(1, std::min<long>(work, (long)c->num_sms * 16)), 256, 0, c->stream>>>(
         X.p, R.p, (int)O, (int)V);
@@ -1199,12 +1247,14 @@ dcsd_status dot_view(Ctx* c, const TV& A, const TV& B, double* out, double accum
     if (!ew_setup(c, A, B, a)) return DCSD_ERR_INVALID_ARG;
     a.A = A.p;
     a.C = nullptr;
+    double* red = c->red + dag_slice(c, 2, kDotBlocks, kRedDoubles);
+    const DagOp op(c, {rd(A), rd(B), wr(out, 8), wr(red, 8ul * kDotBlocks)});
     if (c->trace) trace_begin(c, "dot n=" + std::to_string(a.total));
-    if (a.total < (1l << 32)) k_dot_partial<unsigned><<<kDotBlocks, 256, 0, c->stream>>>(a, B.p, c->red);
-    else k_dot_partial<unsigned long><<<kDotBlocks, 256, 0, c->stream>>>(a, B.p, c->red);
+    if (a.total < (1l << 32)) k_dot_partial<unsigned><<<kDotBlocks, 256, 0, c->stream>>>(a, B.p, red);
+    else k_dot_partial<unsigned long><<<kDotBlocks, 256, 0, c->stream>>>(a, B.p, red);
     trace_end(c);
     DCSD_TRY(launch_check(c, "dot_partial"));
-    k_dot_final<<<1, 256, 0, c->stream>>>(c->red, kDotBlocks, out, accumulate);
+    k_dot_final<<<1, 256, 0, c->stream>>>(red, kDotBlocks, out, accumulate);
     return launch_check(c, "dot_final");
 }
 
@@ -1367,6 +1417,8 @@ dcsd_status build_tau_mats(Ctx* c, int spin, double* Smat, double* Tmat) {
         op.B = view(Tmat, {(long)c->n, (long)c->n});
         rec_push(c, std::move(op));
     }
+    const size_t nn8 = 8ul * c->n * c->n;
+    const DagOp op(c, {rd(c->t1 + (long)spin * c->O * c->V, 8ul * c->O * c->V), wr(Smat, nn8), wr(Tmat, nn8)});
     k_tau_mats<<<grid_for(c, (long)c->n * c->n), 256, 0, c->stream>>>(
         c->n, c->nc, c->O, c->V, c->t1 + (long)spin * c->O * c->V, Smat, Tmat);
     return launch_check(c, "tau_mats");

@@ -1001,14 +1001,21 @@ dcsd_status apply_mterms(Ctx* c, int ref, bool fp32) {
     {
         const long nmat = 3l * c->O * c->O, tv = (c->V + 31) / 32;
         const long blocks = std::min<long>(nmat * tv * tv, (long)std::max(c->num_sms, 1) * 16);
+        const DagOp op(c, {rd(c->t2, 8ul * nmat * c->V * c->V), wr(c->t2s, 8ul * nmat * c->V * c->V)});
         trace_begin(c, "swap_vir");
         k_swap_vir<<<(unsigned)std::max<long>(1, blocks), 256, 0, c->stream>>>(nmat, c->V, c->t2, c->t2s);
         trace_end(c);
         DCSD_TRY(launch_check(c, "swap_vir"));
     }
     long n1 = 2l * c->O * c->V;
-    k_mterm_singles<<<(unsigned)std::max<long>(1, (n1 + 255) / 256), 256, 0, c->stream>>>(a);
-    DCSD_TRY(launch_check(c, "mterm_singles"));
+    const size_t b1 = 8ul * n1, b2 = 24ul * c->O * c->O * c->V * c->V;
+    {
+        const DagOp op(c, {rd(c->scal, 8), rd(c->t1, b1), rd(c->t2, b2), rd(c->t2s, b2), wr(c->c1, b1), wr(c->R1, b1)});
+        k_mterm_singles<<<(unsigned)std::max<long>(1, (n1 + 255) / 256), 256, 0, c->stream>>>(a);
+        DCSD_TRY(launch_check(c, "mterm_singles"));
+    }
+    const DagOp op2(c, {rd(c->scal, 8), rd(c->t1, b1), rd(c->t2, b2), rd(c->t2s, b2), rd(c->c1, b1), rd(c->R1, b1),
+                        wr(c->R2, b2)});
     const int maxx = std::max(g_max_xfac, 1);
     const size_t smem = (2ul * maxx + 4) * c->V * (fp32 ? sizeof(float) : sizeof(double));
     const unsigned grid = (unsigned)(3l * c->O * c->O);

@@ -92,6 +92,8 @@ dcsd_status add_fock_hh(Ctx* c, double* Wo, const double* F1, const double* F2) 
         rec_push(c, std::move(op));
     }
     const long total = (long)c->O * c->O * c->O * c->O;
+    const size_t OO8 = 8ul * c->O * c->O;
+    const DagOp op(c, {wr(Wo, 8ul * total), rd(F1, OO8), rd(F2, OO8)});
     k_add_fock_hh<<<(unsigned)std::max<long>(1, std::min<long>((total + 255) / 256, 4096)), 256, 0,
                     c->stream>>>(c->O, Wo, F1, F2);
     return launch_check(c, "add_fock_hh");
@@ -135,6 +137,7 @@ dcsd_status apply_c_condition(Ctx* c, int ref) {
         op.pos[2] = p.s2;
         rec_push(c, std::move(op));
     }
+    const DagOp op(c, {wr(c->t2 + p.e, 8), rd(c->t1 + p.s1, 8), rd(c->t1 + p.s2, 8)});
     k_c_condition<<<1, 1, 0, c->stream>>>(c->t2 + p.e, c->t1 + p.s1, c->t1 + p.s2);
     return launch_check(c, "c_condition");
 }
@@ -157,6 +160,8 @@ dcsd_status coupling_w(Ctx* c, int ref) {
         op.pos[2] = p.s2;
         rec_push(c, std::move(op));
     }
+    const DagOp op(c, {wr(c->scal, 8), wr(c->scal + 50, 16), rd(c->R2 + p.e, 8), rd(c->t1, 16ul * c->O * c->V),
+                       rd(c->R1, 16ul * c->O * c->V)});
     k_coupling_w<<<1, 1, 0, c->stream>>>(c->scal, c->R2 + p.e, c->t1, c->R1, p.s1, p.s2);
     return launch_check(c, "coupling_w");
 }
@@ -171,6 +176,116 @@ dcsd_status set_vvvv(Ctx* c, const double* host_vvvv) {
     }
     DCSD_CUDA(c, cudaMemcpy(c->vvvv, host_vvvv, nv4 * sizeof(double), cudaMemcpyHostToDevice));
     return DCSD_OK;
+}
+
+// ---------------------------------------------------------------------------
+// dependencies of recorded launches
+// ---------------------------------------------------------------------------
+struct Dag {
+    struct Node {
+        cudaGraphNode_t node;
+        std::vector<Span> spans;
+        std::vector<uint64_t> before;  // bit set of the nodes it comes after
+    };
+    std::vector<Node> nodes;                // since the last undeclared launch
+    std::vector<cudaGraphNode_t> barrier;   // what every node depends on at least
+    std::vector<cudaGraphNode_t> leaves;    // the stream's dependencies between two operations
+    std::vector<Span> spans;                // of the operation being recorded
+    std::vector<size_t> deps;
+    bool open = false, failed = false;
+    size_t slice[4] = {};
+};
+
+static bool capture_deps(Ctx* c, std::vector<cudaGraphNode_t>& out) {
+    cudaStreamCaptureStatus st;
+    const cudaGraphNode_t* d = nullptr;
+    size_t n = 0;
+    if (cudaStreamGetCaptureInfo(c->stream, &st, nullptr, nullptr, &d, nullptr, &n) != cudaSuccess ||
+        st != cudaStreamCaptureStatusActive)
+        return false;
+    out.assign(d, d + n);
+    return true;
+}
+
+static bool capture_deps_set(Ctx* c, std::vector<cudaGraphNode_t>& d) {
+    return cudaStreamUpdateCaptureDependencies(c->stream, d.data(), nullptr, d.size(), cudaStreamSetCaptureDependencies) ==
+           cudaSuccess;
+}
+
+DagOp::DagOp(Ctx* c_, std::initializer_list<Span> spans) : c(c_->dag && !c_->dag->open ? c_ : nullptr) {
+    if (!c) return;
+    Dag& g = *c->dag;
+    g.open = true;
+    std::vector<cudaGraphNode_t> now;
+    if (!capture_deps(c, now)) {
+        g.failed = true;
+        return;
+    }
+    if (now != g.leaves) {  // undeclared launches in between
+        g.nodes.clear();
+        g.barrier = now;
+    }
+    g.spans.clear();
+    for (const Span& s : spans)
+        if (s.lo < s.hi) g.spans.push_back(s);
+    // newest first; a node already behind a chosen one adds nothing
+    std::vector<uint64_t> seen((g.nodes.size() + 63) / 64, 0);
+    std::vector<cudaGraphNode_t> dep;
+    g.deps.clear();
+    for (size_t k = g.nodes.size(); k-- > 0;) {
+        if (seen[k / 64] >> (k % 64) & 1) continue;
+        bool hit = false;
+        for (const Span& a : g.nodes[k].spans)
+            for (const Span& b : g.spans)
+                if ((a.write || b.write) && a.lo < b.hi && b.lo < a.hi) hit = true;
+        if (!hit) continue;
+        g.deps.push_back(k);
+        dep.push_back(g.nodes[k].node);
+        for (size_t w = 0; w < g.nodes[k].before.size(); ++w) seen[w] |= g.nodes[k].before[w];
+    }
+    if (dep.empty()) dep = g.barrier;
+    if (!capture_deps_set(c, dep)) g.failed = true;
+}
+
+DagOp::~DagOp() {
+    if (!c) return;
+    Dag& g = *c->dag;
+    g.open = false;
+    std::vector<cudaGraphNode_t> now;
+    if (g.failed || !capture_deps(c, now)) {
+        g.failed = true;
+        return;
+    }
+    if (now.size() == 1 && (g.deps.empty() || now[0] != g.nodes[g.deps[0]].node || g.deps.size() != 1)) {
+        const size_t k = g.nodes.size();
+        Dag::Node n;
+        n.node = now[0];
+        n.spans = g.spans;
+        n.before.assign(k / 64 + 1, 0);
+        for (size_t d : g.deps) {
+            n.before[d / 64] |= 1ull << (d % 64);
+            for (size_t w = 0; w < g.nodes[d].before.size(); ++w) n.before[w] |= g.nodes[d].before[w];
+        }
+        g.nodes.push_back(std::move(n));
+    }
+    // between operations the stream depends on every node without a successor
+    std::vector<uint64_t> covered((g.nodes.size() + 63) / 64 + 1, 0);
+    g.leaves.clear();
+    for (size_t k = g.nodes.size(); k-- > 0;) {
+        if (!(covered[k / 64] >> (k % 64) & 1)) g.leaves.push_back(g.nodes[k].node);
+        for (size_t w = 0; w < g.nodes[k].before.size(); ++w) covered[w] |= g.nodes[k].before[w];
+    }
+    if (g.leaves.empty()) g.leaves = g.barrier;
+    if (!capture_deps_set(c, g.leaves) || !capture_deps(c, g.leaves)) g.failed = true;
+}
+
+size_t dag_slice(Ctx* c, int which, size_t need, size_t size) {
+    if (!c->dag) return 0;
+    size_t& at = c->dag->slice[which];
+    if (at + need > size) at = 0;
+    const size_t r = at;
+    at += need;
+    return r;
 }
 
 dcsd_status residual_union(Ctx* c, int ref, int method, int prec) {
@@ -214,6 +329,7 @@ dcsd_status residual_union(Ctx* c, int ref, int method, int prec) {
         return einsum64(c, spec, alpha, A, Bm, beta, C);
     };
 
+    c->pool_used = 0;  // intermediates of this evaluation
     // the A->B amplitude: its fixed value (fixed-reference methods), or the
     // C-condition (2D methods; zero in the CAS case)
     if (method_fr(method)) DCSD_TRY(set_fixed_amplitude(c, ref, method_fr_value(method)));
@@ -356,17 +472,20 @@ dcsd_status residual_union(Ctx* c, int ref, int method, int prec) {
         // with stored four-index integrals, one contraction with them (the
         // reverse mode records the factorised form, equal to the threshold
         // of the factorisation)
-        // (chunk sizes decide the split of K, hence the order of summation)
-        const size_t lad = c->fma_chain ? c->big_elems : c->lad_elems;
-        const long ch = std::max<long>(1, std::min<long>(V, (long)(lad / (V * V * V))));
+        // (in a solve the order of summation follows chunks of big_elems
+        // integrals; where those hold several rows the chunks keep that size)
+        const long v3 = V * V * V, och = (long)(c->big_elems / v3);
+        const bool keep = c->fma_chain && och > 1 && (V * V >= 2048 || X >= 2048);  // (shorter K is never split)
+        const long ch = std::max<long>(1, std::min<long>(V, keep ? och : (long)(c->lad_elems / v3)));
+        const long oc = c->fma_chain && !keep ? 1 : 0;
         if (c->vvvv && !c->rec)
             DCSD_TRY(einsum64(c, "sijcd,acbd->sijab", 1.0, t2, view(c->vvvv, {V, V, V, V}), 1.0, R2));
         else
-            DCSD_TRY(ladder64(c, t2, Bvv, R2, c->big0, ch, 0));
+            DCSD_TRY(ladder64(c, t2, Bvv, R2, c->rec ? c->big0 : scratch(c, c->big0, ch * v3), ch, 0, true, oc));
         // T1 corrections: G[s][ij][k][b] = sum_cd (kc|bd) t_s[ij][cd]; G[3] with
         // t_ab transposed in (c,d); H[s][ij][k][m] = sum_cd (kc|md) t_s[ij][cd]
-        const long kc = std::max<long>(1, std::min<long>(O, (long)(lad / (V * V * V))));
-        DCSD_TRY(gpass(c, t2, Bov, Bvv, G, c->big0, kc, 0));
+        const long kc = std::max<long>(1, std::min<long>(O, keep ? och : (long)(c->lad_elems / v3)));
+        DCSD_TRY(gpass(c, t2, Bov, Bvv, G, c->rec ? c->big0 : scratch(c, c->big0, kc * v3), kc, 0, true, oc));
     }
     DCSD_TRY(big("kmcd,sijcd->sijkm", 1.0, J, t2, 0.0, H));
     for (int b = 0; b < 3; ++b) {
@@ -478,6 +597,7 @@ dcsd_status residual_union(Ctx* c, int ref, int method, int prec) {
             op.type = OP_ECOMB;
             rec_push(c, std::move(op));
         }
+        const DagOp op(c, {wr(s + 1, 72)});
         k_energy_combine<<<1, 1, 0, c->stream>>>(s);
         DCSD_TRY(launch_check(c, "energy_combine"));
     }
@@ -503,5 +623,82 @@ dcsd_status residual_union(Ctx* c, int ref, int method, int prec) {
     return DCSD_OK;
 }
 
+
+// The residual is 200 to 400 launches, most of them a few microseconds: below
+// a few hundred thousand amplitudes the host's launch rate (6 us each) is the
+// limit, a graph's nodes follow each other in about 2 us, and nodes that do
+// not depend on each other (spins, blocks, energy) run side by side.  Everything that
+// residual_union enqueues works on the context's own buffers, so one recording
+// serves every later call with the same arguments as long as those buffers and
+// the packed operands kept in them are the same (state).  The first evaluation
+// runs launch by launch (it allocates), the second is recorded.
+dcsd_status graph_run(Ctx* c, int key, const std::function<dcsd_status()>& body) {
+    if (c->graphs_off || c->rec || c->trace || c->prof_on) return body();
+    auto state = [&]() {
+        std::vector<uint64_t> s;
+        tc_state(c, s);
+        for (const void* p : {(const void*)c->r2f, (const void*)c->t2img, (const void*)c->vvvv,
+                              (const void*)c->pack_cache_src[0], (const void*)c->pack_cache_src[1], (const void*)c->vbuf,
+                              (const void*)c->pairbuf})
+            s.push_back((uint64_t)(uintptr_t)p);
+        for (const auto& b : c->arena) s.push_back((uint64_t)(uintptr_t)b.fwd);
+        return s;
+    };
+    Ctx::Graph* g = nullptr;
+    for (auto& x : c->graphs)
+        if (x.key == key) g = &x;
+    if (!g) {
+        c->graphs.emplace_back();
+        g = &c->graphs.back();
+        g->key = key;
+    }
+    if (g->state != state()) {
+        if (g->exec) cudaGraphExecDestroy(g->exec);
+        g->exec = nullptr;
+        const dcsd_status st = body();
+        g->state = st == DCSD_OK ? state() : std::vector<uint64_t>();
+        return st;
+    }
+    if (!g->exec) {
+        if (!c->capture && cudaStreamCreateWithFlags(&c->capture, cudaStreamNonBlocking) != cudaSuccess) {
+            cudaGetLastError();
+            c->capture = nullptr;
+            c->graphs_off = true;
+            return body();
+        }
+        const long long l0 = c->launches;
+        const cudaStream_t user = c->stream;
+        cudaGraph_t graph = nullptr;
+        bool ok = cudaStreamBeginCapture(c->capture, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+        if (ok) {
+            Dag dag;
+            c->stream = c->capture;
+            c->dag = &dag;
+            const dcsd_status st = body();
+            c->dag = nullptr;
+            c->stream = user;
+            ok = cudaStreamEndCapture(c->capture, &graph) == cudaSuccess && st == DCSD_OK && graph && !dag.failed;
+        }
+        ok = ok && state() == g->state && cudaGraphInstantiate(&g->exec, graph, 0) == cudaSuccess;
+        if (graph) cudaGraphDestroy(graph);
+        g->launches = c->launches - l0;
+        c->launches = l0;
+        if (!ok) {
+            cudaGetLastError();
+            g->exec = nullptr;
+            c->graphs_off = true;
+            c->err.clear();
+            return body();
+        }
+    }
+    DCSD_CUDA(c, cudaGraphLaunch(g->exec, c->stream));
+    c->launches += g->launches;
+    return DCSD_OK;
+}
+
+dcsd_status residual_run(Ctx* c, int ref, int method, int prec) {
+    const int key = ((ref * 8 + method) * 8 + prec) * 2 + (c->fma_chain ? 1 : 0);
+    return graph_run(c, key, [=]() { return residual_union(c, ref, method, prec); });
+}
 
 }  // namespace dcsd

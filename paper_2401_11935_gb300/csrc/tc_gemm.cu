@@ -1329,7 +1329,7 @@ struct TcEngine {
     // change after initialisation: kept for the life of the context (key as
     // in pack_operand), up to kBCacheBytes in all
     static constexpr size_t kBCacheBytes = 8ul << 30;
-    std::vector<std::pair<std::string, Buf>> bcache;
+    std::map<std::string, Buf> bcache;
     size_t bcache_bytes = 0;
     Buf pbv;            // the ladder's B_vv [(b,d)][L] for the G pass
     int pbv_nsplit = 0; // its split (0: not packed)
@@ -1383,6 +1383,17 @@ void tc_free(Ctx* c) {
         if (b.p) cudaFree(b.p);
     delete e;
     c->tc = nullptr;
+}
+
+void tc_state(const Ctx* c, std::vector<uint64_t>& s) {
+    const TcEngine* e = c->tc;
+    for (const Buf* b : {&e->pa, &e->pb, &e->pv, &e->pt, &e->sam, &e->sap, &e->svp, &e->svm, &e->sx, &e->pbv})
+        s.push_back((uint64_t)(uintptr_t)b->p);
+    for (const void* p : {(const void*)e->d_pairoff, (const void*)e->d_rowcode, (const void*)e->d_growoff,
+                          (const void*)e->d_code_m, (const void*)e->d_code_p, (const void*)e->wsk})
+        s.push_back((uint64_t)(uintptr_t)p);
+    for (long v : {(long)e->sx_nsplit, (long)e->pbv_nsplit, (long)e->bcache.size(), e->tab_O, e->tab_V, e->sa_O})
+        s.push_back((uint64_t)v);
 }
 
 static long round_up(long x, long m) { return (x + m - 1) / m * m; }
@@ -1709,11 +1720,11 @@ static dcsd_status pack_operand(Ctx* c, const double* src, int nr, const long* r
         for (int i = 0; i < nr; ++i) key += "|r" + std::to_string(rsz[i]) + ":" + std::to_string(rs[i]);
         for (int i = 0; i < nk; ++i) key += "|k" + std::to_string(ksz[i]) + ":" + std::to_string(ks[i]);
         for (int i = 0; i < nseg; ++i) key += "|p" + std::to_string(pat[i]);
-        for (auto& kv : e->bcache)
-            if (kv.first == key) {
-                out = kv.second.p;
-                return DCSD_OK;
-            }
+        const auto hit = e->bcache.find(key);
+        if (hit != e->bcache.end()) {
+            out = hit->second.p;
+            return DCSD_OK;
+        }
         const size_t bytes = (size_t)rows * nseg * Kp * sizeof(__nv_bfloat16);
         if (e->bcache_bytes + bytes <= TcEngine::kBCacheBytes) {
             Buf b;
@@ -1723,7 +1734,7 @@ static dcsd_status pack_operand(Ctx* c, const double* src, int nr, const long* r
                 cudaFree(b.p);
                 return st;
             }
-            e->bcache.push_back({key, b});
+            e->bcache[key] = b;
             e->bcache_bytes += bytes;
             out = b.p;
             return DCSD_OK;

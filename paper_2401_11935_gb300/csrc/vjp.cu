@@ -30,7 +30,13 @@ namespace dcsd {
 // recording
 // ---------------------------------------------------------------------------
 double* scratch(Ctx* c, double* normal, size_t elems) {
-    if (!c->rec) return normal;
+    if (!c->rec) {
+        const size_t n = (elems + 31) & ~(size_t)31;
+        if (c->pool_used + n > c->pool_elems) return normal;
+        double* p = c->pool + c->pool_used;
+        c->pool_used += n;
+        return p;
+    }
     const size_t need = (std::max<size_t>(elems, 1) + 31) & ~(size_t)31;  // 256-byte granules
     for (auto& b : c->arena)
         if (b.cap - b.used >= need) {
@@ -68,6 +74,7 @@ dcsd_status copy_dev(Ctx* c, double* dst, const double* src, size_t n) {
         op.C = view(dst, {(long)n});
         rec_push(c, std::move(op));
     }
+    const DagOp op(c, {rd(src, n * sizeof(double)), wr(dst, n * sizeof(double))});
     DCSD_CUDA(c, cudaMemcpyAsync(dst, src, n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
     return DCSD_OK;
 }
@@ -79,6 +86,7 @@ dcsd_status zero_dev(Ctx* c, double* dst, size_t n) {
         op.C = view(dst, {(long)n});
         rec_push(c, std::move(op));
     }
+    const DagOp op(c, {wr(dst, n * sizeof(double))});
     DCSD_CUDA(c, cudaMemsetAsync(dst, 0, n * sizeof(double), c->stream));
     return DCSD_OK;
 }
@@ -105,8 +113,20 @@ struct PackCacheScope {
 
 // R2[s][ij][a][b] += sum_cd t2[s][ij][c][d] (ac|bd), (ac|bd) = sum_L B_L[a][c] B_L[b][d]
 // built for chunks of `chunk` values of a in `chunkbuf` (chunk * V^3 doubles)
+//
+// Under fma_chain the order of summation must not depend on the chunk, whose
+// size decides the split of K: it follows chunks of order_chunk values.
+struct ChainExtents {
+    Ctx* c;
+    ChainExtents(Ctx* c_, long m, long n) : c(c_) {
+        c->chain_m = m;
+        c->chain_n = n;
+    }
+    ~ChainExtents() { c->chain_m = c->chain_n = 0; }
+};
+
 dcsd_status ladder64(Ctx* c, const TV& t2, const TV& Bvv, const TV& R2, double* chunkbuf, long chunk,
-                     int nsplit, bool compute) {
+                     int nsplit, bool compute, long order_chunk) {
     const long V = c->V;
     if (c->rec) {
         TapeOp op;
@@ -126,8 +146,14 @@ dcsd_status ladder64(Ctx* c, const TV& t2, const TV& Bvv, const TV& R2, double* 
     for (long a0 = 0; a0 < V && st == DCSD_OK; a0 += chunk) {
         const long na = std::min(chunk, V - a0);
         TV Vc = view(chunkbuf, {na, V, V, V});  // [a][c][b][d] = (ac|bd)
-        st = contract(c, nsplit, "Lac,Lbd->acbd", 1.0, sub(Bvv, 1, a0, na), Bvv, 0.0, Vc);
-        if (st == DCSD_OK) st = contract(c, nsplit, "sijcd,acbd->sijab", 1.0, t2, Vc, 1.0, sub(R2, 3, a0, na));
+        {
+            const ChainExtents ext(c, order_chunk * V, order_chunk > 0 ? V * V : 0);
+            st = contract(c, nsplit, "Lac,Lbd->acbd", 1.0, sub(Bvv, 1, a0, na), Bvv, 0.0, Vc);
+        }
+        if (st == DCSD_OK) {
+            const ChainExtents ext(c, order_chunk > 0 ? t2.size[0] * t2.size[1] * t2.size[2] : 0, order_chunk * V);
+            st = contract(c, nsplit, "sijcd,acbd->sijab", 1.0, t2, Vc, 1.0, sub(R2, 3, a0, na));
+        }
     }
     c->rec = saved;
     return st;
@@ -136,7 +162,7 @@ dcsd_status ladder64(Ctx* c, const TV& t2, const TV& Bvv, const TV& R2, double* 
 // G[s][i][j][k][b] = sum_cd t2[s][ij][cd] (kc|bd) for s = aa, bb, ab and
 // G[3][i][j][k][b] = sum_cd t2ab[ij][dc] (kc|bd), by chunks of k
 dcsd_status gpass(Ctx* c, const TV& t2, const TV& Bov, const TV& Bvv, const TV& G, double* chunkbuf, long chunk,
-                  int nsplit, bool compute) {
+                  int nsplit, bool compute, long order_chunk) {
     const long O = c->O, V = c->V;
     if (c->rec) {
         TapeOp op;
@@ -158,11 +184,18 @@ dcsd_status gpass(Ctx* c, const TV& t2, const TV& Bov, const TV& Bvv, const TV& 
     for (long k0 = 0; k0 < O && st == DCSD_OK; k0 += chunk) {
         const long nk = std::min(chunk, O - k0);
         TV Ic = view(chunkbuf, {nk, V, V, V});  // [k][c][b][d] = (kc|bd)
-        st = contract(c, nsplit, "Lkc,Lbd->kcbd", 1.0, sub(Bov, 1, k0, nk), Bvv, 0.0, Ic);
-        if (st == DCSD_OK)
+        {
+            const ChainExtents ext(c, order_chunk * V, order_chunk > 0 ? V * V : 0);
+            st = contract(c, nsplit, "Lkc,Lbd->kcbd", 1.0, sub(Bov, 1, k0, nk), Bvv, 0.0, Ic);
+        }
+        if (st == DCSD_OK) {
+            const ChainExtents ext(c, order_chunk > 0 ? 3 * O * O : 0, order_chunk * V);
             st = contract(c, nsplit, "sijcd,kcbd->sijkb", 1.0, t2, Ic, 0.0, sub(sub(G, 0, 0, 3), 3, k0, nk));
-        if (st == DCSD_OK)
+        }
+        if (st == DCSD_OK) {
+            const ChainExtents ext(c, order_chunk > 0 ? O * O : 0, order_chunk * V);
             st = contract(c, nsplit, "ijdc,kcbd->ijkb", 1.0, t2ab, Ic, 0.0, sub(fix(G, 0, 3), 2, k0, nk));
+        }
     }
     c->rec = saved;
     return st;
@@ -223,16 +256,19 @@ dcsd_status scale_adj(Ctx* c, const TV& Cb, double beta) {
     return axpy_view(c, 0.0, Cb, beta, Cb);
 }
 
-dcsd_status read_scalar(Ctx* c, const double* dev, double* host) {
-    DCSD_CUDA(c, cudaMemcpyAsync(host, dev, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    DCSD_CUDA(c, cudaStreamSynchronize(c->stream));
-    return DCSD_OK;
-}
+__global__ void k_scale_scalar(double* s, double beta) { *s = beta * *s; }
 
-dcsd_status write_scalar(Ctx* c, double* dev, double v) {
-    DCSD_CUDA(c, cudaMemcpyAsync(dev, &v, sizeof(double), cudaMemcpyHostToDevice, c->stream));
-    DCSD_CUDA(c, cudaStreamSynchronize(c->stream));
-    return DCSD_OK;
+// s1' = s1 + (s2 + s5 - s6 + s3 + s7 - s8) / 2 + s4 + s9
+__global__ void k_ecomb_adj(double* s) {
+    const double g = s[1], h = 0.5 * g;
+    s[2] += h;
+    s[3] += h;
+    s[5] += h;
+    s[6] -= h;
+    s[7] += h;
+    s[8] -= h;
+    s[4] += g;
+    s[9] += g;
 }
 
 // Pair-row stack of a [3][O][O][V][V] array: rows 0..P-1 are the alpha-alpha
@@ -423,19 +459,19 @@ dcsd_status reverse_op(Ctx* c, const TapeOp& op) {
         case OP_DOT: {
             double* ob = adj_of(c, op.p[0]);
             if (!ob) return DCSD_OK;
-            double g = 0.0;
-            DCSD_TRY(read_scalar(c, ob, &g));
-            if (g != 0.0) {
-                if (adj_view(c, op.A, Ab)) DCSD_TRY(axpy_view(c, g, op.B, 1.0, Ab));
-                if (adj_view(c, op.B, Bb)) DCSD_TRY(axpy_view(c, g, op.A, 1.0, Bb));
-            }
-            return write_scalar(c, ob, op.beta * g);
+            if (adj_view(c, op.A, Ab)) DCSD_TRY(axpy_view_scalar(c, ob, op.B, Ab));
+            if (adj_view(c, op.B, Bb)) DCSD_TRY(axpy_view_scalar(c, ob, op.A, Bb));
+            const DagOp dag(c, {wr(ob, 8)});
+            k_scale_scalar<<<1, 1, 0, c->stream>>>(ob, op.beta);
+            return launch_check(c, "scale_scalar");
         }
         case OP_TAU: {
             double* Sb = adj_of(c, op.A.p);
             double* Tb = adj_of(c, op.B.p);
             double* t1b = adj_of(c, c->t1 + (long)op.iarg[0] * c->O * c->V);
             if (!Sb || !Tb || !t1b) return DCSD_OK;
+            const size_t nn8 = 8ul * c->n * c->n;
+            const DagOp dag(c, {rd(Sb, nn8), rd(Tb, nn8), wr(t1b, 8ul * c->O * c->V)});
             k_tau_adj<<<(unsigned)std::max(1, c->num_sms * 4), 256, 0, c->stream>>>(c->n, c->nc, c->O, c->V, Sb,
                                                                                     Tb, t1b);
             return launch_check(c, "tau_adj");
@@ -443,22 +479,19 @@ dcsd_status reverse_op(Ctx* c, const TapeOp& op) {
         case OP_FOCKHH: {
             double* Wb = adj_of(c, op.C.p);
             if (!Wb) return DCSD_OK;
+            double* F1b = adj_of(c, op.A.p);
+            double* F2b = adj_of(c, op.B.p);
+            const size_t O2 = 8ul * c->O * c->O;
+            const DagOp dag(c, {rd(Wb, O2 * c->O * c->O), wr(F1b, F1b ? O2 : 0), wr(F2b, F2b ? O2 : 0)});
             k_fockhh_adj<<<(unsigned)std::max(1, c->num_sms * 4), 256, 0, c->stream>>>(
-                c->O, Wb, adj_of(c, op.A.p), adj_of(c, op.B.p));
+                c->O, Wb, F1b, F2b);
             return launch_check(c, "fockhh_adj");
         }
         case OP_ECOMB: {
-            // s1' = s1 + (s2 + s5 - s6 + s3 + s7 - s8) / 2 + s4 + s9
             double* sb = adj_of(c, c->scal);
-            double h[10];
-            DCSD_CUDA(c, cudaMemcpyAsync(h, sb, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
-            DCSD_CUDA(c, cudaStreamSynchronize(c->stream));
-            const double g = h[1];
-            h[2] += 0.5 * g; h[3] += 0.5 * g; h[5] += 0.5 * g; h[6] -= 0.5 * g;
-            h[7] += 0.5 * g; h[8] -= 0.5 * g; h[4] += g; h[9] += g;
-            DCSD_CUDA(c, cudaMemcpyAsync(sb, h, sizeof(h), cudaMemcpyHostToDevice, c->stream));
-            DCSD_CUDA(c, cudaStreamSynchronize(c->stream));
-            return DCSD_OK;
+            const DagOp dag(c, {wr(sb, 80)});
+            k_ecomb_adj<<<1, 1, 0, c->stream>>>(sb);
+            return launch_check(c, "ecomb_adj");
         }
         case OP_CCOND: {
             // t2[e] = -t1[p] t1[q]: t1b[p] -= t1[q] t2b[e], t1b[q] -= t1[p] t2b[e], t2b[e] = 0
@@ -602,11 +635,8 @@ static VjpBufs vjp_layout(Ctx* c, double* base) {
     return v;
 }
 
-// Record the FP64 residual at the amplitudes already in c->t1/c->t2 and set
-// up the adjoint regions.  On return the tape holds the forward.
-dcsd_status vjp_record(Ctx* c, int ref, int method, int prec) {
-    const long n = c->n, O = c->O, V = c->V, X = c->X;
-    const size_t n1 = 2ul * O * V, n2 = 3ul * O * O * V * V, nn = (size_t)n * n;
+// Allocates the adjoint buffers
+static dcsd_status vjp_buffers(Ctx* c) {
     const size_t need = vjp_layout(c, nullptr).total;
     if (c->vbuf_elems < need) {
         if (c->vbuf) cudaFree(c->vbuf);
@@ -619,6 +649,15 @@ dcsd_status vjp_record(Ctx* c, int ref, int method, int prec) {
         }
         c->vbuf_elems = need;
     }
+    return DCSD_OK;
+}
+
+// Record the FP64 residual at the amplitudes already in c->t1/c->t2 and set
+// up the adjoint regions.  On return the tape holds the forward.
+dcsd_status vjp_record(Ctx* c, int ref, int method, int prec) {
+    const long n = c->n, O = c->O, V = c->V, X = c->X;
+    const size_t n1 = 2ul * O * V, n2 = 3ul * O * O * V * V, nn = (size_t)n * n;
+    DCSD_TRY(vjp_buffers(c));
     const VjpBufs v = vjp_layout(c, c->vbuf);
     c->regions.clear();
     c->regions.push_back({c->t1, n1, v.t1b});
@@ -670,8 +709,8 @@ dcsd_status vjp_sweep(Ctx* c, const double* R1bar_u, const double* R2bar_u, doub
         double* h = c->hostbuf + 40;  // pinned staging
         h[0] = Wbar;
         h[1] = Ebar;
+        // (the callers synchronise before the next sweep writes the staging)
         DCSD_CUDA(c, cudaMemcpyAsync(v.sb, h, 2 * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-        DCSD_CUDA(c, cudaStreamSynchronize(c->stream));
     }
     static const char* const kRevLabel[] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, "rev tau",
                                             "rev fockhh", "rev ecomb", "rev swap_vir", "rev mterms"};
@@ -699,7 +738,7 @@ dcsd_status vjp_run(Ctx* c, int ref, int method, int prec, const double* const* 
     const long n = c->n, X = c->X;
     const size_t nn = (size_t)n * n;
     DCSD_TRY(unpack_T(c, ref, Td[0], Td[1], Td[2], Td[3], Td[4]));
-    DCSD_TRY(vjp_record(c, ref, method, prec));
+    DCSD_TRY(vjp_buffers(c));
     const VjpBufs v = vjp_layout(c, c->vbuf);
     // the residual seeds in the union layout
     const double* s1 = nullptr;
@@ -715,8 +754,19 @@ dcsd_status vjp_run(Ctx* c, int ref, int method, int prec, const double* const* 
         s1 = u1;
         s2 = u2;
     }
-    DCSD_TRY(vjp_sweep(c, s1, s2, Ebar, Wbar));
+    c->hostbuf[40] = Wbar;
+    c->hostbuf[41] = Ebar;
+    auto both = [&]() -> dcsd_status {
+        DCSD_TRY(vjp_record(c, ref, method, prec));
+        return vjp_sweep(c, s1, s2, Ebar, Wbar);
+    };
+    // FP64: forward and sweep are about a thousand small launches, recorded as
+    // one graph (the seeds sit in fixed buffers); the tensor-core sweeps
+    // allocate pack caches as they go
+    const int key = 4096 + ((ref * 8 + method) * 8 + prec) * 2 + (Rb ? 1 : 0);
+    const dcsd_status st = prec == DCSD_PREC_FP64 ? graph_run(c, key, both) : both();
     c->tape.clear();
+    DCSD_TRY(st);
     DCSD_TRY(layout_union(c, ref, 1, v.t1b, v.t2b, Tb));
     if (Bb) DCSD_CUDA(c, cudaMemcpyAsync(Bb, v.Bbar, (size_t)X * nn * sizeof(double), cudaMemcpyDeviceToDevice,
                                          c->stream));
