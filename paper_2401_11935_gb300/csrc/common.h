@@ -475,6 +475,9 @@ void tc_free(Ctx* c);
 dcsd_status einsum_tc(Ctx* c, const char* spec, double alpha, const TV& A,
                       const TV& B, double beta, const TV& C, int nsplit);
 
+// whether einsum_tc sums an M x N x K and an M2 x N2 x K contraction in the same way
+bool tc_same_sums(const Ctx* c, long M, long N, long M2, long N2, long K, int nsplit);
+
 // pp ladder + its T1 correction on tensor cores (R2 += ladder, G = correction)
 dcsd_status ladder_tc(Ctx* c, int nsplit, double* R2, double* G);
 // the engine's buffers and packed-operand states that recorded launches use

@@ -1868,6 +1868,47 @@ dcsd_status einsum_tc(Ctx* c, const char* spec, double alpha, const TV& A, const
 constexpr long kAccBlocks = 64;
 constexpr double kAccWorkspaceBytes = 3e9;
 
+// How einsum_tc evaluates an M x N x K contraction
+struct TcChoice {
+    int ksplit;  // splits of K, summed by a second kernel
+    bool simt;   // the CUDA cores are faster
+};
+
+// A long contraction onto few output tiles splits K over the SMs
+// (FP32 partial tiles, summed by a second kernel).  Rough time model:
+// 0.4 us per 64-deep k-step and tile wave plus operand packing at
+// 3 TB/s, against 5 TFLOP/s of the FP32 CUDA-core kernel on its 64 x 64
+// tiles; the faster one runs.
+static TcChoice tc_choice(const Ctx* c, long M, long N, long K, int nsplit) {
+    const int nseg = nsplit >= 3 ? 6 : nsplit == 2 ? 3 : 1;
+    const long nkt = nseg * round_up(K, TC_BK) / TC_BK;
+    const long bn = N >= 256 ? 256 : 128;
+    const long tilesMN = ((M + TC_BM - 1) / TC_BM) * ((N + bn - 1) / bn);
+    TcChoice r{1, false};
+    if (tilesMN <= c->num_sms / 2 && nkt >= 64)
+        r.ksplit = (int)std::max<long>(1, std::min<long>(c->num_sms / tilesMN, nkt / 16));
+    // BF16X6, the refinement precision: FP32 partial sums over at most
+    // kAccBlocks k-blocks, summed in FP64, when the partials fit (the
+    // rounding error of an FP32 sum grows with its length, and the long
+    // small-output contractions would otherwise dominate its error)
+    if (nsplit >= 3) {
+        const long need = (nkt + kAccBlocks - 1) / kAccBlocks;
+        if (need >= 4 && need > r.ksplit && (double)need * (double)M * (double)N * 4.0 <= kAccWorkspaceBytes)
+            r.ksplit = (int)need;
+    }
+    const long kper = (nkt + r.ksplit - 1) / r.ksplit;
+    const long waves = (tilesMN * r.ksplit + c->num_sms - 1) / std::max(1, c->num_sms);
+    const double tc_us = (double)waves * (double)kper * 0.4 + (double)(M + N) * (double)K * 8.0 / 3e6;
+    const double simt_us = 2.0 * (double)round_up(M, 64) * (double)round_up(N, 64) * (double)K / 5e6;
+    r.simt = simt_us < tc_us;
+    return r;
+}
+
+bool tc_same_sums(const Ctx* c, long M, long N, long M2, long N2, long K, int nsplit) {
+    const TcChoice a = tc_choice(c, M, N, K, nsplit), b = tc_choice(c, M2, N2, K, nsplit);
+    return a.ksplit == b.ksplit && a.simt == b.simt;
+}
+
 dcsd_status einsum_tc_impl(Ctx* c, const char* spec, double alpha, const TV& A, const TV& B, double beta,
                            const TV& C, int nsplit) {
     GemmPlan p;
@@ -1893,34 +1934,10 @@ dcsd_status einsum_tc_impl(Ctx* c, const char* spec, double alpha, const TV& A, 
         parts.a[i] = pa[i];
         parts.b[i] = pb[i];
     }
-    // A long contraction onto few output tiles splits K over the SMs
-    // (FP32 partial tiles, summed by a second kernel).  Rough time model:
-    // 0.4 us per 64-deep k-step and tile wave plus operand packing at
-    // 3 TB/s, against 5 TFLOP/s of the FP32 CUDA-core kernel on its 64 x 64
-    // tiles; the faster one runs.
-    int ksplit = 1;
-    {
-        const long nkt = Kt / TC_BK;
-        const long bn = p.N >= 256 ? 256 : 128;
-        const long tilesMN = ((p.M + TC_BM - 1) / TC_BM) * ((p.N + bn - 1) / bn);
-        if (tilesMN <= c->num_sms / 2 && nkt >= 64)
-            ksplit = (int)std::max<long>(1, std::min<long>(c->num_sms / tilesMN, nkt / 16));
-        // BF16X6, the refinement precision: FP32 partial sums over at most
-        // kAccBlocks k-blocks, summed in FP64, when the partials fit (the
-        // rounding error of an FP32 sum grows with its length, and the long
-        // small-output contractions would otherwise dominate its error)
-        if (nsplit >= 3) {
-            const long need = (nkt + kAccBlocks - 1) / kAccBlocks;
-            if (need >= 4 && need > ksplit && (double)need * (double)p.M * (double)p.N * 4.0 <= kAccWorkspaceBytes)
-                ksplit = (int)need;
-        }
-        const long kper = (nkt + ksplit - 1) / ksplit;
-        const long waves = (tilesMN * ksplit + c->num_sms - 1) / std::max(1, c->num_sms);
-        const double tc_us = (double)waves * (double)kper * 0.4 + (double)(p.M + p.N) * (double)p.K * 8.0 / 3e6;
-        const double simt_us = 2.0 * (double)round_up(p.M, 64) * (double)round_up(p.N, 64) * (double)p.K / 5e6;
-        if (simt_us < tc_us)
-            return nsplit >= 3 ? einsum64(c, spec, alpha, A, B, beta, C) : einsum32(c, spec, alpha, A, B, beta, C);
-    }
+    const TcChoice choice = tc_choice(c, p.M, p.N, p.K, nsplit);
+    int ksplit = choice.ksplit;
+    if (choice.simt)
+        return nsplit >= 3 ? einsum64(c, spec, alpha, A, B, beta, C) : einsum32(c, spec, alpha, A, B, beta, C);
     // Row order within M (and N) is free: the packed operand and the
     // epilogue only have to agree.  Order each side's modes by decreasing
     // stride in C, so that its fastest mode is the one closest to C's
