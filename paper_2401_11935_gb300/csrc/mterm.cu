@@ -404,29 +404,44 @@ struct MArgs {
     const double* W;   // device scalar
 };
 
+// (four terms' factors are loaded before their products are added in order:
+// a term's loads otherwise wait for the previous term's)
 __device__ __forceinline__ double eval_class(const MArgs& a, int cls, const int q[4]) {
     const long O = a.O, V = a.V, nb = O * O * V * V;
     // code -> union position
     const int pos[8] = {q[0], q[1], q[2], q[3], a.nc, a.nc + 1, 0, 1};
     double sum = 0.0;
     const int o = c_off[a.ref][cls], n = c_cnt[a.ref][cls];
-    for (int k = 0; k < n; ++k) {
-        const MTerm& m = c_terms[a.ref][o + k];
-        double prod = (double)m.sign;
-        for (int f = 0; f < m.nf; ++f) {
-            const MFac& g = m.f[f];
-            const int x0 = pos[g.idx[0]], x1 = pos[g.idx[1]];
-            double val;
-            if (g.arr < 2) {
-                val = a.t1[((long)g.arr * O + x0) * V + x1];
-            } else {
-                const int x2 = pos[g.idx[2]], x3 = pos[g.idx[3]];
-                const double* base = g.arr < 5 ? a.t2 + (g.arr - 2) * nb : a.t2s + (g.arr - 5) * nb;
-                val = base[(((long)x0 * O + x1) * V + x2) * V + x3];
+    for (int k0 = 0; k0 < n; k0 += 4) {
+        double val[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const MTerm& m = c_terms[a.ref][o + min(k0 + u, n - 1)];
+#pragma unroll
+            for (int f = 0; f < 4; ++f) {
+                val[u][f] = 1.0;
+                if (f >= m.nf) continue;
+                const MFac& g = m.f[f];
+                const int x0 = pos[g.idx[0]], x1 = pos[g.idx[1]];
+                if (g.arr < 2) {
+                    val[u][f] = a.t1[((long)g.arr * O + x0) * V + x1];
+                } else {
+                    const int x2 = pos[g.idx[2]], x3 = pos[g.idx[3]];
+                    const double* base = g.arr < 5 ? a.t2 + (g.arr - 2) * nb : a.t2s + (g.arr - 5) * nb;
+                    val[u][f] = base[(((long)x0 * O + x1) * V + x2) * V + x3];
+                }
             }
-            prod *= val;
         }
-        sum += prod;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (k0 + u >= n) break;
+            const MTerm& m = c_terms[a.ref][o + k0 + u];
+            double prod = (double)m.sign;
+#pragma unroll
+            for (int f = 0; f < 4; ++f)
+                if (f < m.nf) prod *= val[u][f];
+            sum += prod;
+        }
     }
     return sum;
 }
@@ -590,37 +605,31 @@ template <> __device__ __forceinline__ float to_t<float>(double x) { return f64_
 __device__ __forceinline__ double to_f64(double x) { return x; }
 __device__ __forceinline__ double to_f64(float x) { return f32_to_f64(x); }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_mterm_doubles_sep(MArgs a, int maxx) {
-    extern __shared__ __align__(16) unsigned char mt_smem[];
-    const long O = a.O, V = a.V;
-    const long nb = O * O * V * V;
-    const int slot = blockIdx.x;
-    const int blk = slot / (int)(O * O), i = (slot / (int)O) % (int)O, j = slot % (int)O;
-    const int s1 = blk == 1 ? 1 : 0, s2 = blk == 0 ? 0 : 1;
-    double* Rrow = a.R2 + (long)slot * V * V;
-    bool rowok = occ_ok(a, s1, i) && occ_ok(a, s2, j);
-    if (blk != 2 && i == j) rowok = false;
-    if (!rowok) {
-        for (long e = threadIdx.x; e < V * V; e += blockDim.x) Rrow[e] = 0.0;
-        return;
-    }
-    const bool ai = i == a.occ_act[s1], aj = j == a.occ_act[s2];
-    const int cls_ff = blk * 16 + (ai << 3) + (aj << 2);
-    __shared__ FacDesc fac[kMaxClassTerms][2];
-    __shared__ double coefS[kMaxClassTerms];
-    __shared__ signed char grp[kMaxClassTerms];  // a-factor group of a separable term, -1 joint
-    __shared__ FacDesc xd[kMaxXFac], hd[kMaxHFac];
-    __shared__ double hc[kMaxHFac];
-    __shared__ int nx_s, nh_s;
-    T* F = (T*)mt_smem;           // [maxx][V]: F_d[a]
-    T* G = F + (long)maxx * V;    // [maxx][V]: G_d[b]
-    const int toff = c_off[a.ref][cls_ff], nterm = min(c_cnt[a.ref][cls_ff], kMaxClassTerms);
-    // (1) resolve each term's factors with this block's i, j; fold the
-    //     factors that hold neither a nor b into the coefficient
-    for (int k = threadIdx.x; k < nterm; k += blockDim.x) {
+// The terms of one block's class (a, b external) with its i, j substituted:
+// each term's factors as descriptors, factors without a and b folded into the
+// coefficient, terms grouped by their a-factor (separable) or as joint
+// factors, in order of first occurrence.
+struct ClassTerms {
+    FacDesc fac[kMaxClassTerms][2];
+    double coef[kMaxClassTerms];
+    short first[kMaxClassTerms];      // first term with the same a-factor / joint factor
+    signed char grp[kMaxClassTerms];  // group of a separable term, -1 - group of a joint one
+    signed char arr[kMaxClassTerms][2];
+    FacDesc xd[kMaxXFac], hd[kMaxHFac];
+    signed char xarr[kMaxXFac], harr[kMaxHFac];
+    double hc[kMaxHFac];
+    int nterm, nx, nh;                // nx > maxx: beyond the tables' bounds
+};
+
+__device__ __forceinline__ void resolve_class(const MArgs& a, int blk, int i, int j, bool ai, bool aj, int maxx,
+                                              ClassTerms& S) {
+    const long O = a.O, V = a.V, nb = O * O * V * V;
+    const int cls = blk * 16 + (ai << 3) + (aj << 2);
+    const int toff = c_off[a.ref][cls], nterm = min(c_cnt[a.ref][cls], kMaxClassTerms);
+    const int k = threadIdx.x;
+    if (k < nterm) {
         const MTerm& m = c_terms[a.ref][toff + k];
-        double S = (double)m.sign;
+        double c = (double)m.sign;
         int nf = 0;
         for (int f = 0; f < m.nf; ++f) {
             const MFac& g = m.f[f];
@@ -642,133 +651,229 @@ __global__ void __launch_bounds__(256) k_mterm_doubles_sep(MArgs a, int maxx) {
                                  : g.arr < 5 ? a.t2 + (long)(g.arr - 2) * nb + off
                                              : a.t2s + (long)(g.arr - 5) * nb + off;
             if (sa == 0 && sb == 0) {
-                S *= *base;
+                c *= *base;
             } else if (nf < 2) {
                 // order: the a-holding factor first
+                int at = nf;
                 if (sb == 0 && nf == 1) {
-                    fac[k][1] = fac[k][0];
-                    fac[k][0] = FacDesc{base, sa, sb};
-                } else {
-                    fac[k][nf] = FacDesc{base, sa, sb};
+                    S.fac[k][1] = S.fac[k][0];
+                    S.arr[k][1] = S.arr[k][0];
+                    at = 0;
                 }
+                S.fac[k][at] = FacDesc{base, sa, sb};
+                S.arr[k][at] = g.arr;
                 ++nf;
             }
         }
-        coefS[k] = S;
-        grp[k] = (signed char)(nf == 1 ? -1 : 0);
+        S.coef[k] = c;
+        S.grp[k] = (signed char)(nf == 1 ? -1 : 0);
+    }
+    if (k == 0) {
+        S.nterm = nterm;
+        S.nx = S.nh = 0;
     }
     __syncthreads();
-    // (2) group the terms (one thread, fixed order: deterministic sums)
-    if (threadIdx.x == 0) {
-        int nx = 0, nh = 0;
-        for (int k = 0; k < nterm; ++k) {
-            if (grp[k] < 0) {
-                const FacDesc& h = fac[k][0];
-                int m = 0;
-                while (m < nh && !(hd[m].base == h.base && hd[m].sa == h.sa && hd[m].sb == h.sb)) ++m;
-                if (m == nh) {
-                    if (nh == kMaxHFac) { nx = maxx + 1; break; }
-                    hd[nh] = h;
-                    hc[nh] = 0.0;
-                    ++nh;
+    // first term of the same kind with the same factor, then the rank of that
+    // term among the firsts
+    if (k < nterm) {
+        const FacDesc h = S.fac[k][0];
+        const bool joint = S.grp[k] < 0;
+        int q = 0;
+        while (q < k) {
+            const FacDesc& o = S.fac[q][0];
+            if ((S.grp[q] < 0) == joint && o.base == h.base && o.sa == h.sa && (!joint || o.sb == h.sb)) break;
+            ++q;
+        }
+        S.first[k] = (short)q;
+    }
+    __syncthreads();
+    int rank = 0;
+    bool joint = false;
+    if (k < nterm) {
+        joint = S.grp[k] < 0;
+        const int q = S.first[k];
+        for (int r = 0; r < q; ++r) rank += S.first[r] == r && (S.grp[r] < 0) == joint;
+    }
+    __syncthreads();
+    if (k < nterm) {
+        S.grp[k] = (signed char)(joint ? -1 - min(rank, 100) : min(rank, 100));
+        if (S.first[k] == k) {
+            if (joint) {
+                if (rank < kMaxHFac) {
+                    S.hd[rank] = S.fac[k][0];
+                    S.harr[rank] = S.arr[k][0];
                 }
-                hc[m] += coefS[k];
+                atomicMax(&S.nh, rank + 1);
             } else {
-                const FacDesc& x = fac[k][0];
-                int d = 0;
-                while (d < nx && !(xd[d].base == x.base && xd[d].sa == x.sa)) ++d;
-                if (d == nx) {
-                    if (nx == maxx) { nx = maxx + 1; break; }
-                    xd[nx++] = x;
+                if (rank < kMaxXFac) {
+                    S.xd[rank] = S.fac[k][0];
+                    S.xarr[rank] = S.arr[k][0];
                 }
-                grp[k] = (signed char)d;
+                atomicMax(&S.nx, rank + 1);
             }
         }
-        nx_s = nx;
-        nh_s = nh;
     }
     __syncthreads();
+    if (k < kMaxHFac && k < S.nh) {
+        double c = 0.0;
+        for (int q = 0; q < nterm; ++q)
+            if (S.grp[q] == -1 - k) c += S.coef[q];
+        S.hc[k] = c;
+    }
+    if (k == 0 && (S.nh > kMaxHFac || S.nx > kMaxXFac)) S.nx = maxx + 1;
+    __syncthreads();
+}
+
+// F_d[a] and G_d[b] of the groups, [nx][V] each: the a-factor and the sum of
+// the group's b-factors with their coefficients
+template <typename T>
+__device__ __forceinline__ void group_vectors(const ClassTerms& S, int nx, int V, T* F, T* G) {
+    for (int e = threadIdx.x; e < nx * V; e += blockDim.x) {
+        const int d = e / V, b = e - d * V;
+        F[e] = to_t<T>(S.xd[d].base[(long)b * S.xd[d].sa]);
+        T g = (T)0;
+        for (int k = 0; k < S.nterm; ++k)
+            if (S.grp[k] == d) g += to_t<T>(S.coef[k] * S.fac[k][1].base[(long)b * S.fac[k][1].sb]);
+        G[e] = g;
+    }
+}
+
+// One block per (spin block, i, j).  Bound by latency: a block's elements
+// need about ten loads from shared memory and one or two from t2 each, so the
+// rows are spread over the warps and every lane keeps the loads of several
+// columns in flight; the class is resolved by one thread per term, the group
+// vectors by one thread per element.  (A row of threads per a, with a serial
+// grouping of the terms by one thread, took 76 us at (4, 20, 60), 4.0 ms at
+// (20, 300, 900) and 14.3 ms at (30, 500, 1500) in FP32.)
+template <typename T>
+__global__ void __launch_bounds__(256) k_mterm_doubles_sep(MArgs a, int maxx) {
+    extern __shared__ __align__(16) unsigned char mt_smem[];
+    __shared__ ClassTerms S;
+    __shared__ T hcT[kMaxHFac];
+    const int O = a.O, V = a.V;
+    const int slot = blockIdx.x;
+    const int blk = slot / (O * O), i = (slot / O) % O, j = slot % O;
+    const int s1 = blk == 1 ? 1 : 0, s2 = blk == 0 ? 0 : 1;
+    double* Rrow = a.R2 + (long)slot * V * V;
+    bool rowok = occ_ok(a, s1, i) && occ_ok(a, s2, j);
+    if (blk != 2 && i == j) rowok = false;
+    if (!rowok) {
+        for (long e = threadIdx.x; e < (long)V * V; e += blockDim.x) Rrow[e] = 0.0;
+        return;
+    }
+    const bool ai = i == a.occ_act[s1], aj = j == a.occ_act[s2];
+    resolve_class(a, blk, i, j, ai, aj, maxx, S);
     // the host bounds both counts; a table outside them takes the per-term
     // evaluation for every element
-    const bool generic = nx_s > maxx;
-    const int nx = generic ? 0 : nx_s, nh = generic ? 0 : nh_s;
-    // (3) F_d[a] and G_d[b]
-    for (int b = threadIdx.x; b < V && !generic; b += blockDim.x) {
-        for (int d = 0; d < nx; ++d) {
-            F[(long)d * V + b] = to_t<T>(xd[d].base[(long)b * xd[d].sa]);
-            G[(long)d * V + b] = (T)0;
-        }
-        for (int k = 0; k < nterm; ++k)
-            if (grp[k] >= 0)
-                G[(long)grp[k] * V + b] += to_t<T>(coefS[k] * fac[k][1].base[(long)b * fac[k][1].sb]);
-    }
-    __syncthreads();
+    const bool generic = S.nx > maxx;
+    const int nx = generic ? 0 : S.nx, nh = generic ? 0 : S.nh;
+    T* F = (T*)mt_smem;           // [maxx][V]: F_d[a]
+    T* G = F + (long)maxx * V;    // [maxx][V]: G_d[b]
+    group_vectors<T>(S, nx, V, F, G);
     const double W = *a.W;
     const T Wt = to_t<T>(W);
     const double* t1a = a.t1;
-    const double* t1b = a.t1 + O * V;
+    const double* t1b = a.t1 + (long)O * V;
     const double* c1a = a.c1;
-    const double* c1b = a.c1 + O * V;
+    const double* c1b = a.c1 + (long)O * V;
     const double* tA = blk == 1 ? t1b : t1a;  // spin of a (s1)
     const double* cA = blk == 1 ? c1b : c1a;
     const double* tB = blk == 0 ? t1a : t1b;  // spin of b (s2)
     const double* cB = blk == 0 ? c1a : c1b;
-    // b-dependent factors of the antisymmetrised t1 c1 product, in T:
-    // cj[b] = c_jb, tj[b] = t_jb, ci[b] = c_ib, ti[b] = t_ib (spin of b)
+    // factors of the antisymmetrised t1 c1 product, in T: c_jb, t_jb, c_ib,
+    // t_ib (spin of b) and t_ia, c_ia, t_ja, c_ja (spin of a)
     T* cj = G + (long)maxx * V;
     T* tj = cj + V;
     T* ci = tj + V;
     T* ti = ci + V;
-    __shared__ T hcT[kMaxHFac];
+    T* xti = ti + V;
+    T* xci = xti + V;
+    T* xtj = xci + V;
+    T* xcj = xtj + V;
     for (int b = threadIdx.x; b < V; b += blockDim.x) {
         cj[b] = to_t<T>(cB[j * V + b]);
         tj[b] = to_t<T>(tB[j * V + b]);
         ci[b] = to_t<T>(cB[i * V + b]);
         ti[b] = to_t<T>(tB[i * V + b]);
+        xti[b] = to_t<T>(tA[i * V + b]);
+        xci[b] = to_t<T>(cA[i * V + b]);
+        xtj[b] = to_t<T>(tA[j * V + b]);
+        xcj[b] = to_t<T>(cA[j * V + b]);
     }
-    if (threadIdx.x < nh) hcT[threadIdx.x] = to_t<T>(hc[threadIdx.x]);
+    if (threadIdx.x < nh) hcT[threadIdx.x] = to_t<T>(S.hc[threadIdx.x]);
     __syncthreads();
     // the element's t1 c1 term (b-independent parts passed in)
     auto tc_of = [&](int b, T tia, T cia, T tja, T cja) -> T {
         if (blk == 2) return tia * cj[b] + tj[b] * cia;
         return tia * cj[b] - tja * ci[b] - ti[b] * cja + tj[b] * cia;
     };
-    // (4) elements with a and b external: separable form
     const bool zero_diag = blk != 2;
-    for (int x = 2; x < V; ++x) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // (1) elements with a and b external
+    constexpr int U = 4;  // columns per lane and pass
+    for (int x = 2 + warp; x < V; x += 8) {
         const bool okx = vir_ok(a, s1, x);
-        const T tia = to_t<T>(tA[i * V + x]), cia = to_t<T>(cA[i * V + x]);
-        const T tja = to_t<T>(tA[j * V + x]), cja = to_t<T>(cA[j * V + x]);
-        T fx[kMaxXFac];
-#pragma unroll
-        for (int d = 0; d < kMaxXFac; ++d) fx[d] = d < nx ? F[(long)d * V + x] : (T)0;
+        const T tia = xti[x], cia = xci[x], tja = xtj[x], cja = xcj[x];
         double* Rx = Rrow + (long)x * V;
-        for (int b = 2 + threadIdx.x; b < V; b += blockDim.x) {
-            if (!okx || (zero_diag && x == b)) {
-                Rx[b] = 0.0;
-                continue;
-            }
-            T c2 = (T)0;
-            if (!generic) {
-#pragma unroll
-                for (int d = 0; d < kMaxXFac; ++d)
-                    if (d < nx) c2 += fx[d] * G[(long)d * V + b];
-                for (int m = 0; m < nh; ++m)
-                    c2 += hcT[m] * to_t<T>(hd[m].base[(long)x * hd[m].sa + (long)b * hd[m].sb]);
-                // one update per element: a reduction (no load waited for)
-                atomicAdd(Rx + b, -to_f64(Wt * (c2 - tc_of(b, tia, cia, tja, cja))));
-            } else {
-                const int cls = blk * 16 + (ai << 3) + (aj << 2);
+        if (generic) {
+            const int cls = blk * 16 + (ai << 3) + (aj << 2);
+            for (int b = 2 + lane; b < V; b += 32) {
+                if (!okx || (zero_diag && x == b)) {
+                    Rx[b] = 0.0;
+                    continue;
+                }
                 const int q[4] = {i, j, x, b};
                 atomicAdd(Rx + b, -(W * (eval_class(a, cls, q) - to_f64(tc_of(b, tia, cia, tja, cja)))));
             }
+            continue;
+        }
+        T fx[kMaxXFac];
+#pragma unroll
+        for (int d = 0; d < kMaxXFac; ++d) fx[d] = d < nx ? F[d * V + x] : (T)0;
+        for (int b0 = 2 + lane; b0 < V; b0 += 32 * U) {
+            double h[2][U];
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int b = b0 + 32 * u;
+                    h[m][u] = m < nh && b < V ? S.hd[m].base[(long)x * S.hd[m].sa + (long)b * S.hd[m].sb] : 0.0;
+                }
+            T c2[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) c2[u] = (T)0;
+#pragma unroll
+            for (int d = 0; d < kMaxXFac; ++d)
+                if (d < nx)
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int b = b0 + 32 * u;
+                        c2[u] += fx[d] * G[d * V + (b < V ? b : 0)];
+                    }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int b = b0 + 32 * u;
+                if (b >= V) break;
+                if (!okx || (zero_diag && x == b)) {
+                    Rx[b] = 0.0;
+                    continue;
+                }
+                T c = c2[u];
+#pragma unroll
+                for (int m = 0; m < 2; ++m)
+                    if (m < nh) c += hcT[m] * to_t<T>(h[m][u]);
+                for (int m = 2; m < nh; ++m)
+                    c += hcT[m] * to_t<T>(S.hd[m].base[(long)x * S.hd[m].sa + (long)b * S.hd[m].sb]);
+                // one update per element: a reduction (no load waited for)
+                atomicAdd(Rx + b, -to_f64(Wt * (c - tc_of(b, tia, cia, tja, cja))));
+            }
         }
     }
-    // (5) elements with a or b an open orbital: per-term evaluation
-    for (int e2 = threadIdx.x; e2 < 4 * (int)V; e2 += blockDim.x) {
+    // (2) elements with a or b an open orbital: per-term evaluation
+    for (int e2 = threadIdx.x; e2 < 4 * V; e2 += blockDim.x) {
         int x, b;
-        if (e2 < 2 * (int)V) { x = e2 / (int)V; b = e2 % (int)V; }          // rows a = 0, 1
-        else { const int r = e2 - 2 * (int)V; b = r / (int)V; x = r % (int)V; if (x < 2) continue; }  // columns b = 0, 1
+        if (e2 < 2 * V) { x = e2 / V; b = e2 % V; }          // rows a = 0, 1
+        else { const int r = e2 - 2 * V; b = r / V; x = r % V; if (x < 2) continue; }  // columns b = 0, 1
         const long e = (long)x * V + b;
         const bool okx = vir_ok(a, s1, x), okb = vir_ok(a, s2, b);
         if (!okx || !okb || (zero_diag && x == b)) {
@@ -780,11 +885,9 @@ __global__ void __launch_bounds__(256) k_mterm_doubles_sep(MArgs a, int maxx) {
             Rrow[e] = 0.0;
             continue;
         }
-        const T tia = to_t<T>(tA[i * V + x]), cia = to_t<T>(cA[i * V + x]);
-        const T tja = to_t<T>(tA[j * V + x]), cja = to_t<T>(cA[j * V + x]);
         const int cls = blk * 16 + (ai << 3) + (aj << 2) + (aa << 1) + ab;
         const int q[4] = {i, j, x, b};
-        atomicAdd(Rrow + e, -(W * (eval_class(a, cls, q) - to_f64(tc_of(b, tia, cia, tja, cja)))));
+        atomicAdd(Rrow + e, -(W * (eval_class(a, cls, q) - to_f64(tc_of(b, xti[x], xci[x], xtj[x], xcj[x])))));
     }
 }
 
@@ -847,18 +950,23 @@ __device__ __forceinline__ void block_add(double v, double* target) {
     if ((threadIdx.x & 31) == 0 && v != 0.0) atomicAdd(target, v);
 }
 
-__global__ void __launch_bounds__(256) k_mterm_doubles_adj(MArgs a, MAdjPtrs d) {
-    const long O = a.O, V = a.V, VV = V * V, total = 3 * O * O * VV;
+// Element by element: all of them, or (open_only) those with a or b an open
+// orbital, 4 V - 4 per (block, i, j).
+__global__ void __launch_bounds__(256) k_mterm_doubles_adj(MArgs a, MAdjPtrs d, bool open_only) {
+    const long O = a.O, V = a.V, VV = V * V, per = open_only ? 4 * V - 4 : VV, total = 3 * O * O * per;
     const double W = *a.W;
     const double* t1a = a.t1;
     const double* t1b = a.t1 + O * V;
     const double* c1a = a.c1;
     const double* c1b = a.c1 + O * V;
     double wbar = 0.0;
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
-        const long slot = e / VV, ab = e - slot * VV;
+    for (long w = blockIdx.x * (long)blockDim.x + threadIdx.x; w < total; w += (long)gridDim.x * blockDim.x) {
+        const long slot = w / per, r = w - slot * per;
         const int blk = (int)(slot / (O * O)), i = (int)((slot / O) % O), j = (int)(slot % O);
-        const int x = (int)(ab / V), b = (int)(ab % V);
+        // open_only: rows a = 0, 1, then columns b = 0, 1 of the rows a >= 2
+        const int x = !open_only || r < 2 * V ? (int)(r / V) : 2 + (int)((r - 2 * V) >> 1);
+        const int b = !open_only || r < 2 * V ? (int)(r % V) : (int)(r & 1);
+        const long e = slot * VV + (long)x * V + b;
         const int s1 = blk == 1 ? 1 : 0, s2 = blk == 0 ? 0 : 1;
         bool ok = occ_ok(a, s1, i) && occ_ok(a, s2, j) && vir_ok(a, s1, x) && vir_ok(a, s2, b);
         if (blk != 2 && (i == j || x == b)) ok = false;
@@ -905,6 +1013,209 @@ __global__ void __launch_bounds__(256) k_mterm_doubles_adj(MArgs a, MAdjPtrs d) 
     block_add(wbar, d.scal);
 }
 
+// Adjoint of one block's elements with a and b external, in the separable
+// form of k_mterm_doubles_sep.  With g = R2_bar the sums over b of
+// g[a][b] {G_d, c_j, c_i, t_i, t_j}[b] give F_d_bar, the adjoints of the
+// a-side vectors and W_bar, the sums over a of g[a][b] {F_d, t_i, t_j, c_j,
+// c_i}[a] those of the b-side, each one update per vector element instead of
+// a dozen atomics per element (k_mterm_doubles_adj: 16.5 ms at (12, 160, 480)).
+// Bound by the FP64 pipe: 2 (nx + 4) FMAs per element.
+__device__ __forceinline__ double* adj_ptr(const MArgs& a, const MAdjPtrs& d, const FacDesc& f, int arr) {
+    return arr < 2 ? d.t1 + (f.base - a.t1) : arr < 5 ? d.t2 + (f.base - a.t2) : d.t2s + (f.base - a.t2s);
+}
+
+__device__ __forceinline__ void add_nonzero(double* p, double v) {
+    if (v != 0.0) atomicAdd(p, v);
+}
+
+__global__ void __launch_bounds__(256) k_mterm_rows_adj(MArgs a, MAdjPtrs d, int maxx) {
+    extern __shared__ __align__(16) unsigned char mt_smem[];
+    __shared__ ClassTerms S;
+    __shared__ double cbar[kMaxClassTerms];  // adjoints of the terms' coefficients
+    const int O = a.O, V = a.V;
+    const int slot = blockIdx.x;
+    const int blk = slot / (O * O), i = (slot / O) % O, j = slot % O;
+    const int s1 = blk == 1 ? 1 : 0, s2 = blk == 0 ? 0 : 1;
+    double* g = d.R2 + (long)slot * V * V;
+    bool rowok = occ_ok(a, s1, i) && occ_ok(a, s2, j);
+    if (blk != 2 && i == j) rowok = false;
+    if (!rowok) {  // the forward overwrote these elements
+        for (long e = threadIdx.x; e < (long)V * V; e += blockDim.x) g[e] = 0.0;
+        return;
+    }
+    const bool ai = i == a.occ_act[s1], aj = j == a.occ_act[s2];
+    resolve_class(a, blk, i, j, ai, aj, maxx, S);
+    const int nx = S.nx, nh = S.nh;
+    const double W = *a.W;
+    double* F = (double*)mt_smem;
+    double* G = F + (long)maxx * V;
+    // vectors of the t1 c1 product; same spin only: those of the exchanged pair
+    double* vb = G + (long)maxx * V;  // [4][V]: c_j, t_j, c_i, t_i over b
+    double* va = vb + 4 * V;          // [4][V]: t_i, c_i, t_j, c_j over a
+    const long OV = (long)O * V;
+    const double* tA = a.t1 + (blk == 1 ? OV : 0);
+    const double* cA = a.c1 + (blk == 1 ? OV : 0);
+    const double* tB = a.t1 + (blk == 0 ? 0 : OV);
+    const double* cB = a.c1 + (blk == 0 ? 0 : OV);
+    double* tAb = d.t1 + (blk == 1 ? OV : 0);
+    double* cAb = d.c1 + (blk == 1 ? OV : 0);
+    double* tBb = d.t1 + (blk == 0 ? 0 : OV);
+    double* cBb = d.c1 + (blk == 0 ? 0 : OV);
+    const bool same = blk != 2;
+    group_vectors<double>(S, nx, V, F, G);
+    for (int b = threadIdx.x; b < V; b += blockDim.x) {
+        vb[b] = cB[j * V + b];
+        vb[V + b] = tB[j * V + b];
+        vb[2 * V + b] = same ? cB[i * V + b] : 0.0;
+        vb[3 * V + b] = same ? tB[i * V + b] : 0.0;
+        va[b] = tA[i * V + b];
+        va[V + b] = cA[i * V + b];
+        va[2 * V + b] = same ? tA[j * V + b] : 0.0;
+        va[3 * V + b] = same ? cA[j * V + b] : 0.0;
+    }
+    if (threadIdx.x < kMaxClassTerms) cbar[threadIdx.x] = 0.0;
+    // same-spin diagonal: not an element (the forward overwrote it)
+    if (same)
+        for (int x = threadIdx.x; x < V; x += blockDim.x) g[(long)x * V + x] = 0.0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double wbar = 0.0;
+    double hsum[kMaxHFac] = {};  // sums of g H_m (joint factors)
+    // rows: sums over b
+    for (int x = 2 + warp; x < V; x += 8) {
+        double sd[kMaxXFac], st[4] = {};
+#pragma unroll
+        for (int k = 0; k < kMaxXFac; ++k) sd[k] = 0.0;
+        const double* gx = g + (long)x * V;
+        for (int b = 2 + lane; b < V; b += 32) {
+            const double v = gx[b];
+#pragma unroll
+            for (int k = 0; k < kMaxXFac; ++k)
+                if (k < nx) sd[k] = fma(v, G[k * V + b], sd[k]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (k < 2 || same) st[k] = fma(v, vb[k * V + b], st[k]);
+            if (v != 0.0)
+                for (int m = 0; m < nh; ++m) {
+                    const long o = (long)x * S.hd[m].sa + (long)b * S.hd[m].sb;
+                    const double h = S.hd[m].base[o];
+                    if (m < kMaxHFac) hsum[m] = fma(v, h, hsum[m]);
+                    add_nonzero(adj_ptr(a, d, S.hd[m], S.harr[m]) + o, -W * v * S.hc[m]);
+                }
+        }
+#pragma unroll
+        for (int k = 0; k < kMaxXFac; ++k)
+            if (k < nx) {
+                double v = sd[k];
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (lane == 0) {
+                    wbar -= v * F[k * V + x];
+                    add_nonzero(adj_ptr(a, d, S.xd[k], S.xarr[k]) + (long)x * S.xd[k].sa, -W * v);
+                }
+            }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (k < 2 || same) {
+                double v = st[k];
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                st[k] = v;
+            }
+        if (lane == 0) {
+            // tc = t_ia c_jb + c_ia t_jb (- t_ja c_ib - c_ja t_ib); tc_bar = W g
+            wbar += st[0] * va[x] + st[1] * va[V + x];
+            add_nonzero(tAb + i * V + x, W * st[0]);
+            add_nonzero(cAb + i * V + x, W * st[1]);
+            if (same) {
+                wbar -= st[2] * va[2 * V + x] + st[3] * va[3 * V + x];
+                add_nonzero(tAb + j * V + x, -W * st[2]);
+                add_nonzero(cAb + j * V + x, -W * st[3]);
+            }
+        }
+    }
+    // columns: sums over a
+    for (int b = 2 + threadIdx.x; b < V; b += blockDim.x) {
+        double sd[kMaxXFac], st[4] = {};
+#pragma unroll
+        for (int k = 0; k < kMaxXFac; ++k) sd[k] = 0.0;
+#pragma unroll 4
+        for (int x = 2; x < V; ++x) {
+            const double v = g[(long)x * V + b];
+#pragma unroll
+            for (int k = 0; k < kMaxXFac; ++k)
+                if (k < nx) sd[k] = fma(v, F[k * V + x], sd[k]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (k < 2 || same) st[k] = fma(v, va[k * V + x], st[k]);
+        }
+        add_nonzero(cBb + j * V + b, W * st[0]);
+        add_nonzero(tBb + j * V + b, W * st[1]);
+        if (same) {
+            add_nonzero(cBb + i * V + b, -W * st[2]);
+            add_nonzero(tBb + i * V + b, -W * st[3]);
+        }
+#pragma unroll
+        for (int k = 0; k < kMaxXFac; ++k)
+            if (k < nx) {
+                const double gb = -W * sd[k];  // adjoint of G_k[b]
+                for (int t = 0; t < S.nterm; ++t)
+                    if (S.grp[t] == k) {
+                        const long o = (long)b * S.fac[t][1].sb;
+                        add_nonzero(adj_ptr(a, d, S.fac[t][1], S.arr[t][1]) + o, gb * S.coef[t]);
+                        const double cb = gb * S.fac[t][1].base[o];
+                        if (cb != 0.0) atomicAdd(&cbar[t], cb);
+                    }
+            }
+    }
+#pragma unroll
+    for (int m = 0; m < kMaxHFac; ++m)
+        if (m < nh) {
+            double v = hsum[m];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) {
+                wbar -= v * S.hc[m];
+                for (int t = 0; t < S.nterm; ++t)
+                    if (S.grp[t] == -1 - m) atomicAdd(&cbar[t], -W * v);
+            }
+        }
+    block_add(wbar, d.scal);
+    __syncthreads();
+    // coefficients: product rule over their factors
+    if (threadIdx.x < S.nterm && cbar[threadIdx.x] != 0.0) {
+        const int t = threadIdx.x;
+        const int cls = blk * 16 + (ai << 3) + (aj << 2);
+        const MTerm& m = c_terms[a.ref][c_off[a.ref][cls] + t];
+        const long nb = (long)O * O * V * V;
+        const int pos[8] = {i, j, 0, 0, a.nc, a.nc + 1, 0, 1};
+        double val[4];
+        double* adr[4];
+        int n = 0;
+        for (int f = 0; f < m.nf; ++f) {
+            const MFac& q = m.f[f];
+            const int nslot = q.arr < 2 ? 2 : 4;
+            bool ext = false;
+            for (int r = 0; r < nslot; ++r) ext |= q.idx[r] == 2 || q.idx[r] == 3;
+            if (ext) continue;
+            const int x0 = pos[q.idx[0]], x1 = pos[q.idx[1]];
+            if (q.arr < 2) {
+                const long ix = ((long)q.arr * O + x0) * V + x1;
+                val[n] = a.t1[ix];
+                adr[n] = d.t1 + ix;
+            } else {
+                const long ix = (((long)x0 * O + x1) * V + pos[q.idx[2]]) * V + pos[q.idx[3]];
+                val[n] = q.arr < 5 ? a.t2[(q.arr - 2) * nb + ix] : a.t2s[(q.arr - 5) * nb + ix];
+                adr[n] = q.arr < 5 ? d.t2 + (q.arr - 2) * nb + ix : d.t2s + (q.arr - 5) * nb + ix;
+            }
+            ++n;
+        }
+        for (int f = 0; f < n; ++f) {
+            double prod = cbar[t] * (double)m.sign;
+            for (int h = 0; h < n; ++h)
+                if (h != f) prod *= val[h];
+            add_nonzero(adr[f], prod);
+        }
+    }
+}
+
 __global__ void __launch_bounds__(256) k_mterm_singles_adj(MArgs a, MAdjPtrs d) {
     const long total = 2l * a.O * a.V;
     const double W = *a.W;
@@ -948,7 +1259,16 @@ dcsd_status mterms_adjoint(Ctx* c, int ref, double* t1b, double* t2b, double* t2
     MAdjPtrs d{t1b, t2b, t2sb, c1b, R1b, R2b, scalb};
     const unsigned g = (unsigned)std::max(1, c->num_sms * 8);
     // doubles first: they add to c1_bar, which the singles then propagate
-    k_mterm_doubles_adj<<<g, 256, 0, c->stream>>>(a, d);
+    // (as many group vectors as fit 160 KB of shared memory, else element by element)
+    const int maxx = std::max(g_max_xfac, 1);
+    const size_t smem = (2ul * maxx + 8) * c->V * sizeof(double);
+    const bool rows = g_max_xfac <= kMaxXFac && g_max_hfac <= kMaxHFac && smem <= 160 * 1024;
+    if (rows) {
+        DCSD_CUDA(c, cudaFuncSetAttribute(k_mterm_rows_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_mterm_rows_adj<<<(unsigned)(3l * c->O * c->O), 256, smem, c->stream>>>(a, d, maxx);
+        DCSD_TRY(launch_check(c, "mterm_rows_adj"));
+    }
+    k_mterm_doubles_adj<<<g, 256, 0, c->stream>>>(a, d, rows);
     DCSD_TRY(launch_check(c, "mterm_doubles_adj"));
     k_mterm_singles_adj<<<g, 256, 0, c->stream>>>(a, d);
     return launch_check(c, "mterm_singles_adj");
@@ -1017,7 +1337,7 @@ dcsd_status apply_mterms(Ctx* c, int ref, bool fp32) {
     const DagOp op2(c, {rd(c->scal, 8), rd(c->t1, b1), rd(c->t2, b2), rd(c->t2s, b2), rd(c->c1, b1), rd(c->R1, b1),
                         wr(c->R2, b2)});
     const int maxx = std::max(g_max_xfac, 1);
-    const size_t smem = (2ul * maxx + 4) * c->V * (fp32 ? sizeof(float) : sizeof(double));
+    const size_t smem = (2ul * maxx + 8) * c->V * (fp32 ? sizeof(float) : sizeof(double));
     const unsigned grid = (unsigned)(3l * c->O * c->O);
     trace_begin(c, fp32 ? "mterm_doubles_sep32" : "mterm_doubles_sep64");
     if (g_max_xfac > kMaxXFac || g_max_hfac > kMaxHFac || smem > 160 * 1024) {
