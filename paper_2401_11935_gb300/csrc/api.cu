@@ -356,7 +356,7 @@ extern "C" dcsd_status dcsd_init(dcsd_ctx** out, const dcsd_dims* d, const doubl
         const char* vb = getenv("DCSD_VERBOSE");
         c->verbose = vb && vb[0] == '1';
         const char* mc = getenv("DCSD_TC_MULTICAST");
-        c->tc_multicast = !(mc && mc[0] == '0');
+        c->tc_pairs = !(mc && mc[0] == '0');
         const char* pg = getenv("DCSD_PACK_GENERIC");
         c->pack_generic = pg && pg[0] == '1';
         const char* ls = getenv("DCSD_LADDER_SA");

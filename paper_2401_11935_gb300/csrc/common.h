@@ -187,9 +187,9 @@ struct Ctx {
     int t2img_planes = 0;
     double* hostbuf = nullptr;    // pinned host staging for scalars
     int ladder_chunk = 8;         // virtual rows per V build chunk (FP64)
-    // the ladder contraction in clusters of two CTAs sharing each B tile by
-    // TMA multicast (DCSD_TC_MULTICAST=0 selects the one-CTA kernel)
-    bool tc_multicast = true;
+    // tensor-core GEMMs on pairs of SMs (DCSD_TC_MULTICAST=0 selects the
+    // one-CTA kernel)
+    bool tc_pairs = true;
     // operand packs: the tiled FP64 kernel only, without the t2 image and the
     // row kernel (DCSD_PACK_GENERIC=1; both give identical operands)
     bool pack_generic = false;

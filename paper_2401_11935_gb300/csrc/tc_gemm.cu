@@ -33,7 +33,9 @@ namespace dcsd {
 
 constexpr int TC_BM = 128, TC_BK = 64;
 // stages of the operand pipeline for tiles of BN columns (192 KB in all)
-__host__ __device__ constexpr int tc_stages(int BN) { return BN == 256 ? 4 : BN == 128 ? 6 : 8; }
+__host__ __device__ constexpr int tc_stages(int BN, bool pair) {
+    return pair ? (BN == 256 ? 6 : 8) : BN == 256 ? 4 : BN == 128 ? 6 : 8;
+}
 
 // x = hi + mid + lo with each part BF16 (8 significant bits each)
 __device__ __forceinline__ __nv_bfloat16 split_part(float x, int part) {
@@ -172,19 +174,20 @@ __device__ __forceinline__ void tile_mn(int mn, int tilesM, int tilesN, int grou
 // two TMEM accumulators of BN columns let the epilogue of one tile overlap
 // the MMAs of the next.
 //
-// MC: launched in clusters of two CTAs that take the two m-tiles of a pair
-// with the same n-tile.  Each CTA loads its own A tile and half of the B tile
-// (BN / 2 rows; tmB's box is that half) and multicasts the half to both, so
-// the pair fetches each B tile from L2 once.  A stage slot is free only when
-// both CTAs' MMAs have consumed it: the MMA completion is signalled on the
-// empty barrier of both CTAs (count 2), and every TMA issue waits for it.
-template <int BN, bool MC>
+// PAIR: a cluster of two CTAs works on one tile of 256 x BN (cta_group::2).
+// Each CTA loads its 128 rows of A and BN / 2 columns of B (tmB's box) and
+// drains its 128 rows of the accumulator; the CTA of rank 0 waits for the
+// bytes of both on its full barriers and issues the MMAs, whose completion
+// frees the stage in both.  What bounds the one-CTA form is shared memory: a
+// k-step of 64 writes and reads 16 KB + 128 BN bytes at 128 bytes a clock, 768
+// clocks for the 512 of MMAs at BN = 256; a pair's SM moves 64 KB, 512 clocks.
+template <int BN, bool PAIR>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcEpi epi,
               const TcParts parts, int nkt, int tilesM, int tilesN, int kper, int group, int kblk, int* err) {
-    constexpr uint32_t A_BYTES = TC_BM * TC_BK * 2, B_BYTES = BN * TC_BK * 2;
+    constexpr uint32_t A_BYTES = TC_BM * TC_BK * 2, B_BYTES = (PAIR ? BN / 2 : BN) * TC_BK * 2;
     constexpr uint32_t STAGE = A_BYTES + B_BYTES;
-    constexpr int STAGES = tc_stages(BN);
+    constexpr int STAGES = tc_stages(BN, PAIR);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* staging = smem + STAGES * STAGE;
@@ -198,35 +201,38 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // tiles enumerate (m tile, n tile, k split); split s covers the k-steps
-    // [s * kper, min(nkt, (s + 1) * kper)).  MC: the schedule runs over pairs
+    // [s * kper, min(nkt, (s + 1) * kper)).  PAIR: the schedule runs over pairs
     // of m-tiles (the pair's CTA of rank r takes m-tile 2 * pair + r; an
     // m-tile beyond the last one reads zeros and stores nothing)
-    const int crank = MC ? (int)cluster_rank() : 0;
-    const int tile0 = MC ? (int)blockIdx.x / 2 : (int)blockIdx.x;
-    const int tstep = MC ? (int)gridDim.x / 2 : (int)gridDim.x;
-    const int tilesMs = MC ? (tilesM + 1) / 2 : tilesM;
+    const int crank = PAIR ? (int)cluster_rank() : 0;
+    const int tile0 = PAIR ? (int)blockIdx.x / 2 : (int)blockIdx.x;
+    const int tstep = PAIR ? (int)gridDim.x / 2 : (int)gridDim.x;
+    const int tilesMs = PAIR ? (tilesM + 1) / 2 : tilesM;
     const int nmn = tilesMs * tilesN;
     const int ntiles = nmn * ((nkt + kper - 1) / kper);
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], MC ? 2 : 1);
+            mbar_init(&empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&accf[b], 1);
-            mbar_init(&acce[b], kEpiWarps);
+            mbar_init(&acce[b], PAIR ? 2 * kEpiWarps : kEpiWarps);
         }
         *issued = 0;
         *consumed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == 1) tmem_alloc(tslot, 2 * BN);
+    if (warp == 1) {
+        if (PAIR) tmem_alloc_pair(tslot, 2 * BN);
+        else tmem_alloc(tslot, 2 * BN);
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // MC: the peer's barriers are initialised before any multicast reaches them
-    if (MC) cluster_sync();
+    // the peer's barriers are initialised before anything reaches them
+    if (PAIR) cluster_sync();
     const uint32_t tmem = *tslot;
 
     if (warp == 0) {
@@ -237,7 +243,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 const int mn = tile % nmn, ks = tile / nmn;
                 int tm, tn;
                 tile_mn(mn, tilesMs, tilesN, group, tm, tn);
-                if (MC) tm = 2 * tm + crank;
+                if (PAIR) tm = 2 * tm + crank;
                 const int m0 = tm * TC_BM, n0 = tn * BN;
                 const int kb = ks * kper, ke = min(nkt, kb + kper);
                 int seg = kb / parts.nkb, kq = kb - seg * parts.nkb;
@@ -253,12 +259,23 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         ++seg;
                     }
                     const int ka = parts.a[seg] * parts.nkb + kq, kz = parts.b[seg] * parts.nkb + kq;
+                    if (PAIR) {
+                        // both CTAs' bytes complete on the leader's barrier
+                        if (crank == 0) mbar_expect_tx(&full[s], 2 * STAGE);
+                        const uint32_t bar = leader_addr(&full[s]);
+                        const int nb = n0 + crank * (BN / 2);
+                        if (kblk) {
+                            tma_load_3d_pair(smem + s * STAGE, &tmA, bar, 0, m0, ka);
+                            tma_load_3d_pair(smem + s * STAGE + A_BYTES, &tmB, bar, 0, nb, kz);
+                        } else {
+                            tma_load_2d_pair(smem + s * STAGE, &tmA, bar, ka * TC_BK, m0);
+                            tma_load_2d_pair(smem + s * STAGE + A_BYTES, &tmB, bar, kz * TC_BK, nb);
+                        }
+                        *issued = g + 1;
+                        continue;
+                    }
                     mbar_expect_tx(&full[s], STAGE);
-                    if (MC) {
-                        tma_load_3d(smem + s * STAGE, &tmA, &full[s], 0, m0, ka);
-                        tma_load_3d_mc(smem + s * STAGE + A_BYTES + crank * (B_BYTES / 2), &tmB, &full[s], 0,
-                                       n0 + crank * (BN / 2), kz, (uint16_t)0x3);
-                    } else if (kblk) {
+                    if (kblk) {
                         tma_load_3d(smem + s * STAGE, &tmA, &full[s], 0, m0, ka);
                         tma_load_3d(smem + s * STAGE + A_BYTES, &tmB, &full[s], 0, n0, kz);
                     } else {
@@ -268,18 +285,17 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     *issued = g + 1;
                 }
             }
-            if (MC) {
-                // every slot free in both CTAs: the peer's last MMA completions
-                // have arrived here and no multicast of this CTA is pending
+            if (PAIR) {
+                // every slot freed: the last MMA completions have arrived here
                 const int g0 = max(0, g - STAGES);
                 for (int gg = g0; gg < g; ++gg)
                     if (!mbar_wait(&empty[gg % STAGES], (gg / STAGES) & 1)) atomicExch(err, 5);
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (lane == 0 && crank == 0) {
             constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                                       ((uint32_t)(TC_BM >> 4) << 24);
+                                       ((uint32_t)((PAIR ? 2 * TC_BM : TC_BM) >> 4) << 24);
             int g = 0, j = 0;
             bool ok = true;
             for (int tile = tile0; tile < ntiles && ok; tile += tstep, ++j) {
@@ -302,19 +318,24 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     tc_fence_after();
                     const uint32_t a0 = smem_u32(smem + s * STAGE), b0 = a0 + A_BYTES;
 #pragma unroll
-                    for (int kk = 0; kk < TC_BK / 16; ++kk)
-                        mma_bf16(d, smem_desc(a0 + kk * 32), smem_desc(b0 + kk * 32), idesc,
-                                 (kt > kb || kk > 0) ? 1u : 0u);
-                    if (MC) mma_commit_mc(&empty[s], (uint16_t)0x3);
+                    for (int kk = 0; kk < TC_BK / 16; ++kk) {
+                        const uint32_t acc = (kt > kb || kk > 0) ? 1u : 0u;
+                        if (PAIR) mma_bf16_pair(d, smem_desc(a0 + kk * 32), smem_desc(b0 + kk * 32), idesc, acc);
+                        else mma_bf16(d, smem_desc(a0 + kk * 32), smem_desc(b0 + kk * 32), idesc, acc);
+                    }
+                    if (PAIR) mma_commit_pair(&empty[s]);
                     else mma_commit(&empty[s]);
                     *consumed = g + 1;
                 }
-                if (ok) mma_commit(&accf[buf]);
+                if (ok) {
+                    if (PAIR) mma_commit_pair(&accf[buf]);
+                    else mma_commit(&accf[buf]);
+                }
             }
             if (!ok) {
                 // let issued MMAs finish and drain copies that were not consumed
-                uint64_t* fin = &accf[j & 1];
-                mma_commit(fin);
+                if (PAIR) mma_commit_pair(&accf[j & 1]);
+                else mma_commit(&accf[j & 1]);
                 for (int kt = *consumed; kt < *issued; ++kt) mbar_wait(&full[kt % STAGES], (kt / STAGES) & 1);
             }
         }
@@ -329,7 +350,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const int mn = tile % nmn, ksp = tile / nmn;
             int tm, tn;
             tile_mn(mn, tilesMs, tilesN, group, tm, tn);
-            if (MC) tm = 2 * tm + crank;
+            if (PAIR) tm = 2 * tm + crank;
             const int m0 = tm * TC_BM, n0 = tn * BN;
             const bool ok = mbar_wait(&accf[buf], u & 1);
             tc_fence_after();
@@ -550,16 +571,20 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acce[buf]);
+            if (lane == 0) {
+                if (PAIR) mbar_arrive_cluster(leader_addr(&acce[buf]));
+                else mbar_arrive(&acce[buf]);
+            }
         }
     }
     tc_fence_before();
     __syncthreads();
     __syncwarp();
-    if (MC) cluster_sync();
+    if (PAIR) cluster_sync();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, 2 * BN);
+        if (PAIR) tmem_dealloc_pair(tmem, 2 * BN);
+        else tmem_dealloc(tmem, 2 * BN);
     }
 }
 
@@ -1300,7 +1325,7 @@ struct Buf {
 struct TcEngine {
     PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
     int* d_err = nullptr;
-    int mc_clusters = 0;  // resident two-CTA clusters; 0 unknown, -1 none
+    int pairs = 0;  // resident pairs of CTAs; 0 unknown, -1 none
     Buf pa, pb, pv, pt;  // generic A, generic B, ladder V tile, stacked amplitudes
     bool attr_set = false;
     // ladder row tables for the stacked amplitudes [aa pairs; bb pairs; ab; ab~]
@@ -1542,35 +1567,32 @@ static dcsd_status make_map_kblk(Ctx* c, CUtensorMap* map, const __nv_bfloat16* 
 // split products, the operands hold nparts parts); the operands are K-major BF16
 // with row pitch `pitch` elements (0: Ktot), or K-blocked (kblocked: both
 // operands [Ktot / 64][rows][64])
-// mc (K-blocked operands, at least two m-tiles): clusters of two CTAs share
-// each B tile through TMA multicast (see k_tc_gemm)
 static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __nv_bfloat16* Bp, long N,
                                long Ktot, TcEpi& epi, int ksplit = 1, long pitch = 0, bool kblocked = false,
-                               bool mc = false, const TcParts* split = nullptr, int nparts = 1) {
+                               const TcParts* split = nullptr, int nparts = 1) {
     TcEngine* e = c->tc;
     TcParts parts = {};
     parts.nkb = (int)(Ktot / TC_BK);
     if (split) parts = *split;
     const long Kst = split ? (long)nparts * parts.nkb * TC_BK : Ktot;  // stored K
-    auto smem_of = [](int bn) {
-        return tc_stages(bn) * (TC_BM * TC_BK * 2 + (size_t)bn * TC_BK * 2) + kStageBytesMode2 + 2048;
+    auto smem_of = [](int bn, bool pr) {
+        return tc_stages(bn, pr) * (TC_BM * TC_BK * 2 + (size_t)(pr ? bn / 2 : bn) * TC_BK * 2) + kStageBytesMode2 + 2048;
     };
     const void* kern[2][3] = {
         {(const void*)k_tc_gemm<64, false>, (const void*)k_tc_gemm<128, false>, (const void*)k_tc_gemm<256, false>},
         {(const void*)k_tc_gemm<64, true>, (const void*)k_tc_gemm<128, true>, (const void*)k_tc_gemm<256, true>}};
-    mc = mc && kblocked && c->tc_multicast && M > TC_BM && c->num_sms >= 2;
-    auto config = [&](cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, unsigned grid, int bn) {
+    auto config = [&](cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, unsigned grid, int bn, bool pr) {
         cfg = {};
         cfg.gridDim = dim3(grid);
         cfg.blockDim = dim3(kTcThreads);
-        cfg.dynamicSmemBytes = smem_of(bn);
+        cfg.dynamicSmemBytes = smem_of(bn, pr);
         cfg.stream = c->stream;
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = 2;
         at[0].val.clusterDim.y = 1;
         at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
-        cfg.numAttrs = mc ? 1 : 0;
+        cfg.numAttrs = pr ? 1 : 0;
     };
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[1];
@@ -1578,42 +1600,46 @@ static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __
         for (int m = 0; m < 2; ++m)
             for (int b = 0; b < 3; ++b)
                 DCSD_CUDA(c, cudaFuncSetAttribute(kern[m][b], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)smem_of(64 << b)));
+                                                  (int)smem_of(64 << b, m == 1)));
         e->attr_set = true;
     }
-    if (mc && e->mc_clusters == 0) {
-        // resident two-CTA clusters: every form takes one CTA per SM
-        int nclu = 1 << 20;
+    if (c->tc_pairs && e->pairs == 0) {
+        // resident pairs of CTAs: every form takes one CTA per SM
+        int nclu = c->num_sms / 2;
         for (int b = 0; b < 3; ++b) {
             int n1 = 0;
-            config(cfg, at, (unsigned)(c->num_sms / 2 * 2), 64 << b);
+            config(cfg, at, (unsigned)(c->num_sms / 2 * 2), 64 << b, true);
             if (cudaOccupancyMaxActiveClusters(&n1, kern[1][b], &cfg) != cudaSuccess || n1 < 1) {
                 cudaGetLastError();
                 n1 = -1;  // clusters unavailable: the one-CTA kernel runs
             }
             nclu = std::min(nclu, n1);
         }
-        e->mc_clusters = nclu;
+        e->pairs = nclu;
     }
-    if (e->mc_clusters < 0) mc = false;
-    const long max_clusters = mc ? std::min<long>(c->num_sms / 2, e->mc_clusters) : 0;
-    // Columns per tile: 256, or fewer where that leaves SMs idle.  A k-step
-    // takes in 16 KB + 128 bytes per column at about 64 bytes per clock and SM,
-    // so narrow tiles cost up to twice as much per element but run on up to
-    // four times as many SMs.  (The sums over k do not depend on the width.)
-    // A BF16X6 ladder consumer at (10, 120, 360), M = 276, N = 1800, K = 8704:
-    // 118 us with 256 columns (16 CTAs in clusters), 63 us with 64.
+    // One CTA or a pair per tile, and the columns per tile: the fewest clocks
+    // over the waves of tiles.  A k-step of 64 takes 256 + 2 BN clocks of shared
+    // memory in the one-CTA form and max(256 + BN, 2 BN) in a pair; narrow tiles
+    // cost more per element but run on up to four times as many SMs.  (The sums
+    // over k depend on neither.)  A BF16X6 ladder consumer at (10, 120, 360),
+    // M = 276, N = 1800, K = 8704: 118 us with 256 columns, 63 us with 64.
     int BN = 256;
+    bool pair = false;
     {
-        const long tm = mc ? ((M + TC_BM - 1) / TC_BM + 1) / 2 : (M + TC_BM - 1) / TC_BM;
-        const long slots = mc ? max_clusters : c->num_sms;
+        const long tm1 = (M + TC_BM - 1) / TC_BM;
         double best = 1e300;
-        for (int bn = 256; bn >= 64; bn /= 2) {
-            const long nt = tm * ((N + bn - 1) / bn) * std::max(1, ksplit);
-            const double cost = (double)((nt + slots - 1) / slots) * (16384.0 + 128.0 * bn);
-            if (cost < 0.95 * best) {
-                best = cost;
-                BN = bn;
+        for (int pr = 0; pr < 2; ++pr) {
+            if (pr && !(c->tc_pairs && e->pairs > 0 && tm1 > 1)) continue;
+            const long slots = pr ? e->pairs : c->num_sms;
+            for (int bn = 256; bn >= 64; bn /= 2) {
+                const long nt = (pr ? (tm1 + 1) / 2 : tm1) * ((N + bn - 1) / bn) * std::max(1, ksplit);
+                const double step = pr ? std::max(256 + bn, 2 * bn) : 256 + 2 * bn;
+                const double cost = (double)((nt + slots - 1) / slots) * step;
+                if (cost < 0.95 * best) {
+                    best = cost;
+                    BN = bn;
+                    pair = pr != 0;
+                }
             }
         }
     }
@@ -1629,10 +1655,10 @@ static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __
             return DCSD_ERR_INVALID_ARG;
         }
         DCSD_TRY(make_map_kblk(c, &ma, Ap, M, Ktot, TC_BM));
-        DCSD_TRY(make_map_kblk(c, &mb, Bp, N, Ktot, mc ? BN / 2 : BN));
+        DCSD_TRY(make_map_kblk(c, &mb, Bp, N, Ktot, pair ? BN / 2 : BN));
     } else {
         DCSD_TRY(make_map(c, &ma, Ap, M, Kst, TC_BM, pitch));
-        DCSD_TRY(make_map(c, &mb, Bp, N, Kst, BN, pitch));
+        DCSD_TRY(make_map(c, &mb, Bp, N, Kst, pair ? BN / 2 : BN, pitch));
     }
     epi.M = M;
     epi.N = N;
@@ -1649,11 +1675,11 @@ static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __
         c->err = "tensor-core GEMM too large";
         return DCSD_ERR_INVALID_ARG;
     }
-    // MC: the schedule runs over pairs of m-tiles, two CTAs per pair; as many
-    // clusters as can be resident at once (a persistent grid)
-    const long tilesMs = mc ? (tilesM + 1) / 2 : tilesM;
+    // a pair's schedule runs over pairs of m-tiles; as many clusters as can be
+    // resident at once (a persistent grid)
+    const long tilesMs = pair ? (tilesM + 1) / 2 : tilesM;
     const long ntiles_s = tilesMs * tilesN * ((nkt + kper - 1) / kper);
-    dim3 grid((unsigned)(mc ? 2 * std::min<long>(ntiles_s, max_clusters) : std::min<long>(ntiles, c->num_sms)));
+    dim3 grid((unsigned)(pair ? 2 * std::min<long>(ntiles_s, e->pairs) : std::min<long>(ntiles, c->num_sms)));
     // m-tile band height that minimises the A and B rows one wave of
     // num_sms tiles touches: g * BM + (num_sms / g) * BN
     // (an operand that fits in a quarter of L2 is kept there instead: all
@@ -1664,7 +1690,7 @@ static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __
     if ((double)M * (double)Ktot * 2.0 <= l2q || c->ladder_phase) group = (int)tilesM;
     else if ((double)N * (double)Ktot * 2.0 <= l2q) group = 1;
     group = (int)std::max<long>(1, std::min<long>(group, tilesM));
-    if (mc) group = (int)std::max<long>(1, std::min<long>((group + 1) / 2, tilesMs));
+    if (pair) group = (int)std::max<long>(1, std::min<long>((group + 1) / 2, tilesMs));
     const int cls = c->ladder_phase ? DCSD_PROF_LADDER : DCSD_PROF_TC_OTHER;
     prof_begin(c, cls);
     if (c->trace) {
@@ -1679,8 +1705,8 @@ static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __
         int tm = (int)tilesM, tn = (int)tilesN, kb = kblocked ? 1 : 0, nk = nkt, kp = kper;
         int* derr = e->d_err;
         void* args[] = {&ma, &mb, &epi, &parts, &nk, &tm, &tn, &kp, &group, &kb, &derr};
-        config(cfg, at, grid.x, BN);
-        const cudaError_t le = cudaLaunchKernelExC(&cfg, kern[mc ? 1 : 0][bsel], args);
+        config(cfg, at, grid.x, BN, pair);
+        const cudaError_t le = cudaLaunchKernelExC(&cfg, kern[pair ? 1 : 0][bsel], args);
         if (le != cudaSuccess) {
             trace_end(c);
             prof_end(c, cls);
@@ -1996,7 +2022,7 @@ dcsd_status einsum_tc_impl(Ctx* c, const char* spec, double alpha, const TV& A, 
         epi.n_size[i] = i < p.nn ? p.n_size[i] : 1;
         epi.n_s[i] = i < p.nn ? p.n_sc[i] : 0;
     }
-    if (ksplit <= 1) return gemm_packed(c, Apk, p.M, Bpk, p.N, Kt, epi, 1, 0, false, false, &parts, np);
+    if (ksplit <= 1) return gemm_packed(c, Apk, p.M, Bpk, p.N, Kt, epi, 1, 0, false, &parts, np);
     // split K: partial tiles, then C (or its FP32 shadow) from their sum
     {
         const int nkt = (int)(Kt / TC_BK), kper = (nkt + ksplit - 1) / ksplit;
@@ -2015,7 +2041,7 @@ dcsd_status einsum_tc_impl(Ctx* c, const char* spec, double alpha, const TV& A, 
     red.N = p.N;
     epi.mode = 5;
     epi.C32 = e->wsk;
-    DCSD_TRY(gemm_packed(c, Apk, p.M, Bpk, p.N, Kt, epi, ksplit, 0, false, false, &parts, np));
+    DCSD_TRY(gemm_packed(c, Apk, p.M, Bpk, p.N, Kt, epi, ksplit, 0, false, &parts, np));
     if (c->trace) trace_begin(c, "tc-splitk-reduce " + c->cur_spec);
     k_tc_splitk_reduce<<<(unsigned)std::max<long>(1, std::min<long>((p.M * p.N + 255) / 256, (long)c->num_sms * 8)),
                          256, 0, c->stream>>>(red, ksplit, e->wsk);
@@ -2298,10 +2324,10 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
             for (int sp = 0; sp < nseg; ++sp) {
                 ce.rowcode = e->d_code_m;
                 DCSD_TRY(gemm_packed(c, e->sam.p + (size_t)pa[sp] * rowsM * KSp, rowsM,
-                                     e->svm.p + (size_t)pb[sp] * vrows * KSp, vrows, KSp, ce, 1, 0, true, true));
+                                     e->svm.p + (size_t)pb[sp] * vrows * KSp, vrows, KSp, ce, 1, 0, true));
                 ce.rowcode = e->d_code_p;
                 DCSD_TRY(gemm_packed(c, e->sap.p + (size_t)pa[sp] * rowsP * KSp, rowsP,
-                                     e->svp.p + (size_t)pb[sp] * vrows * KSp, vrows, KSp, ce, 1, 0, true, true));
+                                     e->svp.p + (size_t)pb[sp] * vrows * KSp, vrows, KSp, ce, 1, 0, true));
             }
         }
     }
@@ -2474,7 +2500,7 @@ dcsd_status ladder_tc(Ctx* c, int nsplit, double* R2, double* G) {
                 // (the scatter epilogue adds)
                 for (int sp = 0; sp < nseg; ++sp)
                     DCSD_TRY(gemm_packed(c, e->pt.p + (size_t)sp * rows4 * K2p, rows4,
-                                         e->pv.p + (size_t)sp * vrows * K2p, vrows, K2p, ce, 1, 0, true, true));
+                                         e->pv.p + (size_t)sp * vrows * K2p, vrows, K2p, ce, 1, 0, true));
             } else {
                 ce.C = G + r0 * V;       // G[s][i][j][k][b], row (s,i,j) at the table's offset
                 ce.mrow = e->d_growoff;
@@ -2484,7 +2510,7 @@ dcsd_status ladder_tc(Ctx* c, int nsplit, double* R2, double* G) {
                 for (int sp = 0; sp < nseg; ++sp) {
                     ce.beta = sp == 0 ? 0.0 : 1.0;
                     DCSD_TRY(gemm_packed(c, e->pt.p + (size_t)sp * rows4 * K2p, rows4,
-                                         e->pv.p + (size_t)sp * vrows * K2p, vrows, K2p, ce, 1, 0, true, true));
+                                         e->pv.p + (size_t)sp * vrows * K2p, vrows, K2p, ce, 1, 0, true));
                 }
             }
         }
