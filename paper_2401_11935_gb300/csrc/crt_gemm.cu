@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     volatile int* issued = (volatile int*)(tslot + 1);
     volatile int* consumed = issued + 1;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int crank = MC ? (int)cluster_rank() : 0;
     const int tile0 = MC ? (int)blockIdx.x / 2 : (int)blockIdx.x;
     const int tstep = MC ? (int)gridDim.x / 2 : (int)gridDim.x;
@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             int it = 0;
             bool ok = true;
             for (int tile = tile0; tile < ntiles && ok; tile += tstep) {
@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                                    ((uint32_t)(CG_BM >> 4) << 24);
             int it = 0, j = 0;

@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     volatile int* issued = (volatile int*)(tslot + 1);
     volatile int* consumed = issued + 1;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     // tiles enumerate (m tile, n tile, k split); split s covers the k-steps
     // [s * kper, min(nkt, (s + 1) * kper)).  PAIR: the schedule runs over pairs
     // of m-tiles (the pair's CTA of rank r takes m-tile 2 * pair + r; an
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const uint32_t tmem = *tslot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             int g = 0;
             bool ok = true;
             for (int tile = tile0; tile < ntiles && ok; tile += tstep) {
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && crank == 0) {
+        if (crank == 0 && elect_one()) {
             constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                                        ((uint32_t)((PAIR ? 2 * TC_BM : TC_BM) >> 4) << 24);
             int g = 0, j = 0;
@@ -675,7 +675,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     uint32_t* tslot = (uint32_t*)(acce + 2);
     volatile int* issued = (volatile int*)(tslot + 1);
     volatile int* consumed = issued + 1;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < SA_STAGES; ++s) {
             mbar_init(&full[s], 1);
@@ -697,7 +697,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const uint32_t tmem = *tslot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             int g = 0;
             bool ok = true;
             for (long t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
@@ -736,7 +736,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) |
                                        ((uint32_t)(TC_BM >> 4) << 24);
             int g = 0, j = 0;
