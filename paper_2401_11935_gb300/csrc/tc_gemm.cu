@@ -846,6 +846,291 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
 }
 
+// The same tiles on pairs of SMs (cta_group::2): a pair takes the rows
+// r = 2 p + rank of two neighbouring a with one b, C and D.
+//   acc1 [c][d] = B_a[C] B_b[D]^T   (each CTA: its a's rows of C, half of D)
+//   acc2 [d][c] = B_a[D] B_b[C]^T   (its a's rows of D, half of C)
+// so the pair shares both tiles of b, and acc2 comes out transposed: the
+// epilogue turns it through shared memory, 64 rows d at a time.  On a diagonal
+// block acc2 = acc1.  A k-step of the one-CTA form writes and reads 64 KB of
+// shared memory for 512 clocks of MMAs, 1024 clocks at 128 bytes a clock; here
+// it is 48 KB, 768.  A stage is one product's k-step (24 KB).  A chunk of 16 a
+// at V = 380: 2.9 -> 2.1 ms with L = 1536, 1.94 -> 1.24 ms with L = 768, and at
+// V = 250 with 3456 packed L 2.3 -> 1.35 ms; a k-step now takes 500 clocks per
+// product.
+constexpr int SP_STAGES = 7;
+constexpr uint32_t SP_STAGE = SA_TILE + SA_TILE / 2;
+constexpr int SP_TPITCH = 68;  // floats per row c of the turned 64 rows d
+constexpr int SP_OPITCH = 40;  // BF16 per row c of a warp's 32 x 32 outputs
+constexpr size_t kSaPairSmem = SP_STAGES * (size_t)SP_STAGE + 128 * SP_TPITCH * sizeof(float) +
+                               kEpiWarps * 32 * SP_OPITCH * sizeof(__nv_bfloat16) + 2048;
+
+// pair tile t -> (p, b', C, D): (C, D) fastest, then p, then b' (>= 2 p)
+__device__ __forceinline__ void sa_pair_tile(const SaArgs& a, long t, int& p, int& bb, int& C, int& D) {
+    long u = t / a.npair;
+    int pr = (int)(t - u * a.npair);
+    const int np2 = (a.nr + 1) / 2;
+    const long tri = (long)np2 * (np2 + 1);  // b' < 2 np2: p in [0, b' / 2]
+    if (a.rect) {
+        bb = (int)(u / np2);
+        p = (int)(u % np2);
+    } else if (u < tri) {
+        bb = 0;
+        while (u >= bb / 2 + 1) {
+            u -= bb / 2 + 1;
+            ++bb;
+        }
+        p = (int)u;
+    } else {
+        u -= tri;
+        bb = 2 * np2 + (int)(u / np2);
+        p = (int)(u % np2);
+    }
+    C = 0;
+    while (pr >= a.nblk - C) {
+        pr -= a.nblk - C;
+        ++C;
+    }
+    D = C + pr;
+}
+
+__global__ void __launch_bounds__(kTcThreads, 1)
+    k_ladder_sa_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const SaArgs a,
+                     int* err) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    float* turn = (float*)(smem + SP_STAGES * SP_STAGE);  // [c][d]
+    __nv_bfloat16* outs = (__nv_bfloat16*)(turn + 128 * SP_TPITCH);
+    uint64_t* full = (uint64_t*)(outs + kEpiWarps * 32 * SP_OPITCH);
+    uint64_t* empty = full + SP_STAGES;
+    uint64_t* accf = empty + SP_STAGES;
+    uint64_t* acce = accf + 2;
+    uint32_t* tslot = (uint32_t*)(acce + 2);
+    volatile int* issued = (volatile int*)(tslot + 1);
+    volatile int* consumed = issued + 1;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
+    const int crank = (int)cluster_rank();
+    // the pair's j-th tile: turned by one place per wave of tiles, so that the
+    // diagonal blocks, half the work, are spread over the pairs
+    const long pid = blockIdx.x / 2, npid = gridDim.x / 2;
+    auto tile = [&](int j) { return j * npid + (pid + j) % npid; };
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < SP_STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&accf[b], 1);
+            mbar_init(&acce[b], 2 * kEpiWarps);
+        }
+        *issued = 0;
+        *consumed = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) tmem_alloc_pair(tslot, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    cluster_sync();
+    const uint32_t tmem = *tslot;
+
+    if (warp == 0) {
+        if (elect_one()) {
+            int g = 0, j = 0;
+            bool ok = true;
+            for (long t = tile(0); t < a.ntiles && ok; t = tile(++j)) {
+                int p, bb, C, D;
+                sa_pair_tile(a, t, p, bb, C, D);
+                const int r = min(2 * p + crank, a.nr - 1);  // (an odd chunk's last pair repeats a row)
+                const int xa = (a.xa0 + r) * a.YP, xb = (a.xb0 + bb) * a.YP + crank * 64;
+                int seg = 0, kb = 0, za = a.part_a[0] * a.nkb, zb = a.part_b[0] * a.nkb;
+                for (int kt = 0; kt < a.nkt && ok; ++kt) {
+                    for (int w = 0; w < (C == D ? 1 : 2); ++w, ++g) {
+                        const int s = g % SP_STAGES, round = g / SP_STAGES;
+                        if (round > 0 && !mbar_wait(&empty[s], (round - 1) & 1)) {
+                            atomicExch(err, 1);
+                            ok = false;
+                            break;
+                        }
+                        uint8_t* st = smem + s * SP_STAGE;
+                        if (crank == 0) mbar_expect_tx(&full[s], 2 * SP_STAGE);
+                        const uint32_t bar = leader_addr(&full[s]);
+                        // B_a[C] and half of B_b[D], or B_a[D] and half of B_b[C]
+                        tma_load_3d_pair(st, &tmA, bar, 0, xa + (w ? D : C) * 128, (w ? zb : za) + kb);
+                        tma_load_3d_pair(st + SA_TILE, &tmB, bar, 0, xb + (w ? C : D) * 128, (w ? za : zb) + kb);
+                        *issued = g + 1;
+                    }
+                    if (++kb == a.nkb && ++seg < 6) {
+                        kb = 0;
+                        za = a.part_a[seg] * a.nkb;
+                        zb = a.part_b[seg] * a.nkb;
+                    }
+                }
+            }
+            // every slot freed: the last MMA completions have arrived here
+            for (int gg = max(0, g - SP_STAGES); gg < g; ++gg)
+                if (!mbar_wait(&empty[gg % SP_STAGES], (gg / SP_STAGES) & 1)) atomicExch(err, 5);
+        }
+    } else if (warp == 1) {
+        if (crank == 0 && elect_one()) {
+            constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) |
+                                       ((uint32_t)(256 >> 4) << 24);
+            int g = 0, j = 0;
+            bool ok = true;
+            for (long t = tile(0); t < a.ntiles && ok; t = tile(++j)) {
+                const int buf = j & 1, u = j >> 1;
+                if (u > 0 && !mbar_wait(&acce[buf], (u - 1) & 1)) {
+                    atomicExch(err, 4);
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                int p_, bb_, C, D;
+                sa_pair_tile(a, t, p_, bb_, C, D);
+                const uint32_t d1 = tmem + (uint32_t)(buf * 256), d2 = d1 + 128;
+                for (int kt = 0; kt < a.nkt && ok; ++kt) {
+                    for (int w = 0; w < (C == D ? 1 : 2); ++w, ++g) {
+                        const int s = g % SP_STAGES, round = g / SP_STAGES;
+                        if (!mbar_wait(&full[s], round & 1)) {
+                            atomicExch(err, 2);
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint32_t base = smem_u32(smem + s * SP_STAGE);
+#pragma unroll
+                        for (int kk = 0; kk < TC_BK / 16; ++kk)
+                            mma_bf16_pair(w ? d2 : d1, smem_desc(base + kk * 32), smem_desc(base + SA_TILE + kk * 32),
+                                          idesc, (kt > 0 || kk > 0) ? 1u : 0u);
+                        mma_commit_pair(&empty[s]);
+                        *consumed = g + 1;
+                    }
+                }
+                if (ok) mma_commit_pair(&accf[buf]);
+            }
+            if (!ok) {
+                mma_commit_pair(&accf[j & 1]);
+                for (int kt = *consumed; kt < *issued; ++kt) mbar_wait(&full[kt % SP_STAGES], (kt / SP_STAGES) & 1);
+            }
+        }
+    } else {
+        // warps 2..9: TMEM lane quarter q = warp % 4, column half h.  What a
+        // thread computes is 32 d of one c; it goes through shared memory so
+        // that four lanes store 64 contiguous bytes.  Stored from the threads
+        // that computed it, 16 bytes a lane, it kept the L1's store path busy
+        // for longer than the MMAs of up to 24 k-steps.
+        const int q = warp & 3, h = (warp - 2) >> 2;
+        __nv_bfloat16* mine = outs + (warp - 2) * 32 * SP_OPITCH;
+        int j = 0;
+        for (long t = tile(0); t < a.ntiles; t = tile(++j)) {
+            const int buf = j & 1, u = j >> 1;
+            int p, bb, C, D;
+            sa_pair_tile(a, t, p, bb, C, D);
+            const int r = 2 * p + crank;
+            bool ok = mbar_wait(&accf[buf], u & 1);
+            tc_fence_after();
+            if (!ok) atomicExch(err, 3);
+            const uint32_t tb = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * 256);
+            const uint32_t tt = tb + (C == D ? 0u : 128u);
+            const int cl = 32 * q + lane;
+            const bool store = r < a.nr && (a.rect || bb >= r);
+            const long R = (long)r * a.Vb + bb;  // V tile row
+            long kc[4];                          // rows c of this lane's stores
+#pragma unroll
+            for (int x = 0; x < 4; ++x) kc[x] = sa_koff((long)C * 128 + 32 * q + 8 * x + (lane >> 2), a.Vp);
+#pragma unroll 1
+            for (int half = 0; half < 2; ++half) {
+                const int d0 = D * 128 + half * 64;
+                if (d0 >= a.Vp) break;
+                // (1) 64 rows d of acc2 (acc1 on a diagonal block) turned
+                if ((q >> 1) == half) {
+#pragma unroll 1
+                    for (int ch = 2 * h; ch < 2 * h + 2; ++ch) {
+                        uint32_t v[32];
+                        tmem_ld32(tt + (uint32_t)(ch * 32), v);
+                        float* tw = turn + ch * 32 * SP_TPITCH + 32 * (q & 1) + lane;
+#pragma unroll
+                        for (int x = 0; x < 32; ++x) tw[x * SP_TPITCH] = __uint_as_float(v[x]);
+                    }
+                }
+                asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+                // (2) lane = row c, 32 columns d
+                uint32_t r1[32];
+                float w2[32];
+                tmem_ld32(tb + (uint32_t)(half * 64 + h * 32), r1);
+                const float4* row = (const float4*)(turn + cl * SP_TPITCH + h * 32);
+#pragma unroll
+                for (int x = 0; x < 8; ++x) {
+                    const float4 f = row[x];
+                    w2[4 * x] = f.x;
+                    w2[4 * x + 1] = f.y;
+                    w2[4 * x + 2] = f.z;
+                    w2[4 * x + 3] = f.w;
+                }
+                // the turned rows are read before the next ones replace them
+                asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+                if (half == 1 || d0 + 64 >= a.Vp) {
+                    // both accumulators read: free the buffer
+                    tc_fence_before();
+                    if (lane == 0) mbar_arrive_cluster(leader_addr(&acce[buf]));
+                    __syncwarp();
+                }
+                const long dl = d0 + h * 32 + 8 * (lane & 3);
+                if (!store || d0 + h * 32 + 31 < C * 128 + 32 * q) continue;  // (all below the diagonal)
+                for (int sg = 0; sg < a.nparts; ++sg) {
+#pragma unroll
+                    for (int sign = 0; sign < 2; ++sign) {
+                        uint4* st = (uint4*)(mine + lane * SP_OPITCH);
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) {
+                            uint32_t w[4];
+#pragma unroll
+                            for (int y = 0; y < 4; ++y) {
+                                const int e = 8 * x + 2 * y;
+                                const float v0 = __uint_as_float(r1[e]), v1 = __uint_as_float(r1[e + 1]);
+                                w[y] = (uint32_t)__bfloat16_as_ushort(
+                                           split_part(sign ? v0 - w2[e] : v0 + w2[e], sg)) |
+                                       ((uint32_t)__bfloat16_as_ushort(
+                                            split_part(sign ? v1 - w2[e + 1] : v1 + w2[e + 1], sg))
+                                        << 16);
+                            }
+                            st[x] = make_uint4(w[0], w[1], w[2], w[3]);
+                        }
+                        __syncwarp();
+                        __nv_bfloat16* V = (sign ? a.Vminus : a.Vplus) + sg * a.segstride + R * 64;
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) {
+                            const long c = (long)C * 128 + 32 * q + 8 * x + (lane >> 2);
+                            const uint4 f = *(const uint4*)(mine + (8 * x + (lane >> 2)) * SP_OPITCH + 8 * (lane & 3));
+                            const long k = kc[x] + dl - (c & ~7l);
+                            if (c < a.V && dl >= (c & ~7l) && dl < a.Vp) *(uint4*)(V + (k >> 6) * a.kbs + (k & 63)) = f;
+                        }
+                        __syncwarp();
+                    }
+                }
+            }
+            // a wait that expired in one warp ends them all
+            int all_ok;
+            asm volatile(
+                "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbar.red.and.pred q, 1, %2, p;\n\t"
+                "selp.s32 %0, 1, 0, q;\n\t}\n"
+                : "=r"(all_ok)
+                : "r"((int)ok), "n"(32 * kEpiWarps)
+                : "memory");
+            if (!all_ok) break;
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    __syncwarp();
+    cluster_sync();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem, 512);
+    }
+}
+
 // Stacked S/A amplitudes from t2 (FP64): operand Am rows [same-spin pairs
 // i < j of blocks 0 and 1 (2P); alpha-beta (O^2)] with A-, operand Ap rows
 // [alpha-beta (O^2)] with A+, over the compact (c <= d) index, K-blocked
@@ -1563,6 +1848,88 @@ static dcsd_status make_map_kblk(Ctx* c, CUtensorMap* map, const __nv_bfloat16* 
     return DCSD_OK;
 }
 
+// One CTA or a pair per tile, and the columns per tile: the fewest clocks per
+// k-step over the waves of tiles.  A k-step of 64 occupies the shared memory
+// for 256 + 2 BN clocks in the one-CTA form and for max(256 + BN, 2 BN) in a
+// pair; the table has what a product of 8064 x 8064 x 8064 measured.  Narrow
+// tiles cost more per element but run on up to four times as many SMs.  (The
+// sums over k depend on neither.)  A BF16X6 ladder consumer at (10, 120, 360),
+// M = 276, N = 1800, K = 8704: 118 us with 256 columns, 63 us with 64.
+static double tc_tile_choice(const Ctx* c, long M, long N, long nsplits, int& BN, bool& pair) {
+    static const double step[2][3] = {{400, 464, 784}, {393, 418, 600}};  // 64, 128, 256 columns
+    const long tm1 = (M + TC_BM - 1) / TC_BM;
+    double best = 1e300;
+    for (int pr = 0; pr < 2; ++pr) {
+        if (pr && !(c->tc_pairs && c->tc->pairs > 0 && tm1 > 1)) continue;
+        const long slots = pr ? c->tc->pairs : c->num_sms;
+        for (int bn = 256; bn >= 64; bn /= 2) {
+            const long nt = (pr ? (tm1 + 1) / 2 : tm1) * ((N + bn - 1) / bn) * nsplits;
+            const double cost = (double)((nt + slots - 1) / slots) * step[pr][bn / 128];
+            if (cost < 0.95 * best) {
+                best = cost;
+                BN = bn;
+                pair = pr != 0;
+            }
+        }
+    }
+    return best;
+}
+
+static size_t tc_smem(int bn, bool pair) {
+    return tc_stages(bn, pair) * (TC_BM * TC_BK * 2 + (size_t)(pair ? bn / 2 : bn) * TC_BK * 2) + kStageBytesMode2 + 2048;
+}
+
+static const void* tc_kernel(int b, bool pair) {
+    static const void* const k[2][3] = {
+        {(const void*)k_tc_gemm<64, false>, (const void*)k_tc_gemm<128, false>, (const void*)k_tc_gemm<256, false>},
+        {(const void*)k_tc_gemm<64, true>, (const void*)k_tc_gemm<128, true>, (const void*)k_tc_gemm<256, true>}};
+    return k[pair ? 1 : 0][b];
+}
+
+static void tc_config(const Ctx* c, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, unsigned grid, size_t smem,
+                      bool pair) {
+    cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kTcThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c->stream;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pair ? 1 : 0;
+}
+
+// kernel attributes and the number of resident pairs, once per context
+static dcsd_status tc_setup(Ctx* c) {
+    TcEngine* e = c->tc;
+    if (e->attr_set) return DCSD_OK;
+    for (int m = 0; m < 2; ++m)
+        for (int b = 0; b < 3; ++b)
+            DCSD_CUDA(c, cudaFuncSetAttribute(tc_kernel(b, m == 1), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)tc_smem(64 << b, m == 1)));
+    DCSD_CUDA(c, cudaFuncSetAttribute(k_ladder_sa_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSaPairSmem));
+    // every form takes one CTA per SM
+    int nclu = c->num_sms / 2;
+    for (int b = 0; b < 4; ++b) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at[1];
+        int n1 = 0;
+        tc_config(c, cfg, at, (unsigned)(c->num_sms / 2 * 2), b < 3 ? tc_smem(64 << b, true) : kSaPairSmem, true);
+        if (cudaOccupancyMaxActiveClusters(&n1, b < 3 ? tc_kernel(b, true) : (const void*)k_ladder_sa_pair, &cfg) !=
+                cudaSuccess ||
+            n1 < 1) {
+            cudaGetLastError();
+            n1 = -1;  // clusters unavailable: the one-CTA kernels run
+        }
+        nclu = std::min(nclu, n1);
+    }
+    e->pairs = nclu;
+    e->attr_set = true;
+    return DCSD_OK;
+}
+
 // C (epilogue epi) = A[M][Ktot] . B[N][Ktot]^T (split: Ktot runs over the
 // split products, the operands hold nparts parts); the operands are K-major BF16
 // with row pitch `pitch` elements (0: Ktot), or K-blocked (kblocked: both
@@ -1575,74 +1942,12 @@ static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __
     parts.nkb = (int)(Ktot / TC_BK);
     if (split) parts = *split;
     const long Kst = split ? (long)nparts * parts.nkb * TC_BK : Ktot;  // stored K
-    auto smem_of = [](int bn, bool pr) {
-        return tc_stages(bn, pr) * (TC_BM * TC_BK * 2 + (size_t)(pr ? bn / 2 : bn) * TC_BK * 2) + kStageBytesMode2 + 2048;
-    };
-    const void* kern[2][3] = {
-        {(const void*)k_tc_gemm<64, false>, (const void*)k_tc_gemm<128, false>, (const void*)k_tc_gemm<256, false>},
-        {(const void*)k_tc_gemm<64, true>, (const void*)k_tc_gemm<128, true>, (const void*)k_tc_gemm<256, true>}};
-    auto config = [&](cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, unsigned grid, int bn, bool pr) {
-        cfg = {};
-        cfg.gridDim = dim3(grid);
-        cfg.blockDim = dim3(kTcThreads);
-        cfg.dynamicSmemBytes = smem_of(bn, pr);
-        cfg.stream = c->stream;
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 2;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = pr ? 1 : 0;
-    };
+    DCSD_TRY(tc_setup(c));
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[1];
-    if (!e->attr_set) {
-        for (int m = 0; m < 2; ++m)
-            for (int b = 0; b < 3; ++b)
-                DCSD_CUDA(c, cudaFuncSetAttribute(kern[m][b], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)smem_of(64 << b, m == 1)));
-        e->attr_set = true;
-    }
-    if (c->tc_pairs && e->pairs == 0) {
-        // resident pairs of CTAs: every form takes one CTA per SM
-        int nclu = c->num_sms / 2;
-        for (int b = 0; b < 3; ++b) {
-            int n1 = 0;
-            config(cfg, at, (unsigned)(c->num_sms / 2 * 2), 64 << b, true);
-            if (cudaOccupancyMaxActiveClusters(&n1, kern[1][b], &cfg) != cudaSuccess || n1 < 1) {
-                cudaGetLastError();
-                n1 = -1;  // clusters unavailable: the one-CTA kernel runs
-            }
-            nclu = std::min(nclu, n1);
-        }
-        e->pairs = nclu;
-    }
-    // One CTA or a pair per tile, and the columns per tile: the fewest clocks
-    // over the waves of tiles.  A k-step of 64 takes 256 + 2 BN clocks of shared
-    // memory in the one-CTA form and max(256 + BN, 2 BN) in a pair; narrow tiles
-    // cost more per element but run on up to four times as many SMs.  (The sums
-    // over k depend on neither.)  A BF16X6 ladder consumer at (10, 120, 360),
-    // M = 276, N = 1800, K = 8704: 118 us with 256 columns, 63 us with 64.
     int BN = 256;
     bool pair = false;
-    {
-        const long tm1 = (M + TC_BM - 1) / TC_BM;
-        double best = 1e300;
-        for (int pr = 0; pr < 2; ++pr) {
-            if (pr && !(c->tc_pairs && e->pairs > 0 && tm1 > 1)) continue;
-            const long slots = pr ? e->pairs : c->num_sms;
-            for (int bn = 256; bn >= 64; bn /= 2) {
-                const long nt = (pr ? (tm1 + 1) / 2 : tm1) * ((N + bn - 1) / bn) * std::max(1, ksplit);
-                const double step = pr ? std::max(256 + bn, 2 * bn) : 256 + 2 * bn;
-                const double cost = (double)((nt + slots - 1) / slots) * step;
-                if (cost < 0.95 * best) {
-                    best = cost;
-                    BN = bn;
-                    pair = pr != 0;
-                }
-            }
-        }
-    }
+    tc_tile_choice(c, M, N, std::max(1, ksplit), BN, pair);
     const int bsel = BN == 256 ? 2 : BN == 128 ? 1 : 0;
     CUtensorMap ma, mb;
     if (pitch != 0 && (pitch < Ktot || pitch % 8 != 0 || ((uintptr_t)Ap | (uintptr_t)Bp) % 16 != 0)) {
@@ -1705,8 +2010,8 @@ static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __
         int tm = (int)tilesM, tn = (int)tilesN, kb = kblocked ? 1 : 0, nk = nkt, kp = kper;
         int* derr = e->d_err;
         void* args[] = {&ma, &mb, &epi, &parts, &nk, &tm, &tn, &kp, &group, &kb, &derr};
-        config(cfg, at, grid.x, BN, pair);
-        const cudaError_t le = cudaLaunchKernelExC(&cfg, kern[pair ? 1 : 0][bsel], args);
+        tc_config(c, cfg, at, grid.x, tc_smem(BN, pair), pair);
+        const cudaError_t le = cudaLaunchKernelExC(&cfg, tc_kernel(bsel, pair), args);
         if (le != cudaSuccess) {
             trace_end(c);
             prof_end(c, cls);
@@ -2113,14 +2418,12 @@ static std::vector<std::pair<long, long>> ladder_chunks(long V, long Vp, long ro
 // #(r, b' >= r) tiles of nkx k-steps (two 128 x 128 MMAs per step, about one
 // 128 x 256 step), the consumers GEMMs of rowsM and rowsP rows against
 // nr * (V - r0) columns over nks k-steps
-static std::vector<std::pair<long, long>> ladder_chunks_sa(long V, long rowsM, long rowsP, long nks, long nkx,
-                                                           long npair, long nmax, int sms) {
-    auto waves = [&](long M, long N) {
-        const long bn = N >= 256 ? 256 : 128;
-        const long tiles = ((M + TC_BM - 1) / TC_BM) * ((N + bn - 1) / bn);
-        return (tiles + sms - 1) / sms;
-    };
-    const double launch = 64.0;
+static std::vector<std::pair<long, long>> ladder_chunks_sa(const Ctx* c, long V, long rowsM, long rowsP, long nks,
+                                                           long nkx, long npair, long nmax) {
+    int bn;
+    bool pr;
+    const bool pairs = c->tc_pairs && c->tc->pairs > 0;
+    const double launch = 64.0 * 768;
     std::vector<double> best(V + 1, 0.0);
     std::vector<long> pick(V + 1, 1);
     for (long r0 = V - 1; r0 >= 0; --r0) {
@@ -2128,10 +2431,14 @@ static std::vector<std::pair<long, long>> ladder_chunks_sa(long V, long rowsM, l
         const long Vb = V - r0;
         const long cap = std::min(4 * nmax, std::max(nmax, nmax * V / std::max<long>(1, Vb)));
         for (long nr = 1; nr <= std::min(cap, V - r0); ++nr) {
-            const long ptiles = npair * (nr * Vb - nr * (nr - 1) / 2);
-            const double cost = (double)((ptiles + sms - 1) / sms) * (double)nkx +
-                                (double)(waves(rowsM, nr * Vb) + waves(rowsP, nr * Vb)) * (double)nks + launch +
-                                best[r0 + nr];
+            // clocks of the producer's waves: 1024 per k-step, 768 in pairs
+            const long np2 = (nr + 1) / 2;
+            const long ptiles = pairs ? npair * (np2 * Vb - np2 * (np2 - 1)) : npair * (nr * Vb - nr * (nr - 1) / 2);
+            const long slots = pairs ? c->tc->pairs : c->num_sms;
+            const double prod = (double)((ptiles + slots - 1) / slots) * (double)nkx * (pairs ? 768.0 : 1024.0);
+            const double cons = (tc_tile_choice(c, rowsM, nr * Vb, 1, bn, pr) + tc_tile_choice(c, rowsP, nr * Vb, 1, bn, pr)) *
+                                (double)nks;
+            const double cost = prod + cons + launch + best[r0 + nr];
             if (cost < best[r0]) {
                 best[r0] = cost;
                 pick[r0] = nr;
@@ -2256,8 +2563,11 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
         DCSD_CUDA(c, cudaFuncSetAttribute(k_ladder_sa, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         e->sa_attr = true;
     }
-    CUtensorMap mx;
+    DCSD_TRY(tc_setup(c));
+    const bool pairs = c->tc_pairs && e->pairs > 0;
+    CUtensorMap mx, mh;  // boxes of 128 and of 64 rows
     DCSD_TRY(make_map_kblk(c, &mx, e->sx.p, xrows, XP * np, 128));
+    DCSD_TRY(make_map_kblk(c, &mh, e->sx.p, xrows, XP * np, 64));
     // pass 0, the ladder: chunks of a (triangle b >= a), scatter into R2;
     // pass 1, the G intermediate G[s][i][j][k][b] = sum_cd t[ij][cd] (kc|bd)
     // (s = 3: t with (c,d) exchanged): chunks of occupied k against every b,
@@ -2265,7 +2575,7 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
     DCSD_CUDA(c, cudaMemsetAsync(G, 0, sizeof(double) * 4 * O * O * O * V, c->stream));
     for (int pass = 0; pass < 2; ++pass) {
         std::vector<std::pair<long, long>> chunks;
-        if (pass == 0) chunks = ladder_chunks_sa(V, rowsM, rowsP, KSt / TC_BK, Xt / TC_BK, npair, chunk, c->num_sms);
+        if (pass == 0) chunks = ladder_chunks_sa(c, V, rowsM, rowsP, KSt / TC_BK, Xt / TC_BK, npair, chunk);
         else
             for (long k0 = 0; k0 < O; k0 += chunk) chunks.push_back({k0, std::min(chunk, O - k0)});
         for (const auto& ck : chunks) {
@@ -2280,7 +2590,9 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
             sa.nblk = nblk;
             sa.npair = npair;
             sa.rect = pass;
-            sa.ntiles = pass == 0 ? (long)npair * (nr * Vb - nr * (nr - 1) / 2) : (long)npair * nr * Vb;
+            const long np2 = (nr + 1) / 2;  // pairs of rows
+            if (pairs) sa.ntiles = (long)npair * (pass == 0 ? np2 * Vb - np2 * (np2 - 1) : np2 * Vb);
+            else sa.ntiles = (long)npair * (pass == 0 ? nr * Vb - nr * (nr - 1) / 2 : nr * Vb);
             sa.xa0 = (int)(pass == 0 ? nc + r0 : r0);
             sa.xb0 = (int)(pass == 0 ? nc + r0 : nc);
             sa.YP = (int)YP;
@@ -2304,7 +2616,15 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
                 trace_begin(c, label);
             }
             ++c->tc_seq;
-            k_ladder_sa<<<(unsigned)std::min<long>(sa.ntiles, c->num_sms), kTcThreads, smem, c->stream>>>(mx, sa, e->d_err);
+            if (pairs) {
+                cudaLaunchConfig_t cfg;
+                cudaLaunchAttribute at[1];
+                tc_config(c, cfg, at, (unsigned)(2 * std::min<long>(sa.ntiles, e->pairs)), kSaPairSmem, true);
+                DCSD_CUDA(c, cudaLaunchKernelEx(&cfg, k_ladder_sa_pair, mx, mh, (const SaArgs)sa, e->d_err));
+            } else {
+                k_ladder_sa<<<(unsigned)std::min<long>(sa.ntiles, c->num_sms), kTcThreads, smem, c->stream>>>(mx, sa,
+                                                                                                             e->d_err);
+            }
             trace_end(c);
             prof_end(c, DCSD_PROF_LADDER);
             DCSD_TRY(launch_check(c, "ladder_sa"));
