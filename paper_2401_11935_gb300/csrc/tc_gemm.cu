@@ -75,8 +75,6 @@ struct TcEpi {
     //         s = 0,1 (same spin): R[s][ij][a][b] += v, R[s][ij][b][a] -= v
     //         s = 2 (ab):           R[2][ij][a][b] += v
     //         s = 3 (ab, (c,d) exchanged): R[2][ij][b][a] += v  (b > a)
-    //         s = 4, 5 (ab, S+ and S- of the symmetric / antisymmetric form)
-    // mode 6: G-pass scatter of the symmetric / antisymmetric form (C = G)
     long a0, OO, VV;
     long O;
     const int* rowcode;     // mode 3: row -> (block << 20 | i << 10 | j); same-spin rows are pairs i < j
@@ -92,12 +90,19 @@ struct TcParts {
     int a[6], b[6];
 };
 
+// A launch over the ladder's contractions (n > 0): problem p is product p / 2
+// of the split, with A- and M- (p even) or A+ and M+ (p odd); all have the
+// same columns and k-steps.
+struct TcGroup {
+    int n;            // problems; 0: one contraction, as TcParts says
+    int first[13];    // first tile of every problem, and the end
+    int tm[2];        // m-tiles (or pairs of them) of an even / odd problem
+    long rows[2];     // their rows
+};
+
 // ladder consumer scatter of one accumulator element v = W(a,b) for the row
 // (blk, i, j); same-spin blocks hold the pair i < j only and also fill the
 // (j, i) row: R[ij][ab] = -R[ij][ba] = -R[ji][ab] = R[ji][ba]
-// Rows of the symmetric / antisymmetric form (blocks 4 and 5, alpha-beta):
-// S+ adds to R[ij][ab] and R[ij][ba], S- adds to R[ij][ab] and subtracts
-// from R[ij][ba] (S- vanishes at a = b).
 // Every target of a launch receives one update (the targets of different
 // rows and columns are distinct; a = b same-spin elements are skipped, their
 // four updates cancel), so the updates are reductions without a returned
@@ -113,14 +118,6 @@ __device__ __forceinline__ void ladder_scatter(T* R, int sblk, long ro1, long ro
         atomicAdd(R + ro2 + b * V + a, v);
     } else if (sblk == 2) {
         atomicAdd(R + ro1 + a * V + b, v);
-    } else if (sblk == 4) {
-        atomicAdd(R + ro1 + a * V + b, v);
-        if (b > a) atomicAdd(R + ro1 + b * V + a, v);
-    } else if (sblk == 5) {
-        if (b > a) {
-            atomicAdd(R + ro1 + a * V + b, v);
-            atomicAdd(R + ro1 + b * V + a, -v);
-        }
     } else if (b > a) {
         atomicAdd(R + ro1 + b * V + a, v);
     }
@@ -183,8 +180,9 @@ __device__ __forceinline__ void tile_mn(int mn, int tilesM, int tilesN, int grou
 // clocks for the 512 of MMAs at BN = 256; a pair's SM moves 64 KB, 512 clocks.
 template <int BN, bool PAIR>
 __global__ void __launch_bounds__(kTcThreads, 1)
-    k_tc_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcEpi epi,
-              const TcParts parts, int nkt, int tilesM, int tilesN, int kper, int group, int kblk, int* err) {
+    k_tc_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+              const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2, TcEpi epi,
+              const TcParts parts, const TcGroup grp, int nkt, int tilesM, int tilesN, int kper, int group, int kblk, int* err) {
     constexpr uint32_t A_BYTES = TC_BM * TC_BK * 2, B_BYTES = (PAIR ? BN / 2 : BN) * TC_BK * 2;
     constexpr uint32_t STAGE = A_BYTES + B_BYTES;
     constexpr int STAGES = tc_stages(BN, PAIR);
@@ -209,7 +207,20 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int tstep = PAIR ? (int)gridDim.x / 2 : (int)gridDim.x;
     const int tilesMs = PAIR ? (tilesM + 1) / 2 : tilesM;
     const int nmn = tilesMs * tilesN;
-    const int ntiles = nmn * ((nkt + kper - 1) / kper);
+    const int ntiles = grp.n ? grp.first[grp.n] : nmn * ((nkt + kper - 1) / kper);
+    // tile -> problem of a group, k split, m and n tile
+    auto locate = [&](int tile, int& prob, int& ks, int& tm, int& tn) {
+        prob = 0;
+        if (grp.n) {
+            while (tile >= grp.first[prob + 1]) ++prob;
+            ks = 0;
+            tile_mn(tile - grp.first[prob], grp.tm[prob & 1], tilesN, group, tm, tn);
+        } else {
+            ks = tile / nmn;
+            tile_mn(tile - ks * nmn, tilesMs, tilesN, group, tm, tn);
+        }
+        if (PAIR) tm = 2 * tm + crank;
+    };
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
@@ -240,13 +251,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             int g = 0;
             bool ok = true;
             for (int tile = tile0; tile < ntiles && ok; tile += tstep) {
-                const int mn = tile % nmn, ks = tile / nmn;
-                int tm, tn;
-                tile_mn(mn, tilesMs, tilesN, group, tm, tn);
-                if (PAIR) tm = 2 * tm + crank;
+                int prob, ks, tm, tn;
+                locate(tile, prob, ks, tm, tn);
+                const CUtensorMap *mA = prob & 1 ? &tmA2 : &tmA, *mB = prob & 1 ? &tmB2 : &tmB;
                 const int m0 = tm * TC_BM, n0 = tn * BN;
                 const int kb = ks * kper, ke = min(nkt, kb + kper);
-                int seg = kb / parts.nkb, kq = kb - seg * parts.nkb;
+                int seg = grp.n ? prob >> 1 : kb / parts.nkb, kq = grp.n ? 0 : kb - seg * parts.nkb;
                 for (int kt = kb; kt < ke; ++kt, ++g, ++kq) {
                     const int s = g % STAGES, round = g / STAGES;
                     if (round > 0 && !mbar_wait(&empty[s], (round - 1) & 1)) {
@@ -265,22 +275,22 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         const uint32_t bar = leader_addr(&full[s]);
                         const int nb = n0 + crank * (BN / 2);
                         if (kblk) {
-                            tma_load_3d_pair(smem + s * STAGE, &tmA, bar, 0, m0, ka);
-                            tma_load_3d_pair(smem + s * STAGE + A_BYTES, &tmB, bar, 0, nb, kz);
+                            tma_load_3d_pair(smem + s * STAGE, mA, bar, 0, m0, ka);
+                            tma_load_3d_pair(smem + s * STAGE + A_BYTES, mB, bar, 0, nb, kz);
                         } else {
-                            tma_load_2d_pair(smem + s * STAGE, &tmA, bar, ka * TC_BK, m0);
-                            tma_load_2d_pair(smem + s * STAGE + A_BYTES, &tmB, bar, kz * TC_BK, nb);
+                            tma_load_2d_pair(smem + s * STAGE, mA, bar, ka * TC_BK, m0);
+                            tma_load_2d_pair(smem + s * STAGE + A_BYTES, mB, bar, kz * TC_BK, nb);
                         }
                         *issued = g + 1;
                         continue;
                     }
                     mbar_expect_tx(&full[s], STAGE);
                     if (kblk) {
-                        tma_load_3d(smem + s * STAGE, &tmA, &full[s], 0, m0, ka);
-                        tma_load_3d(smem + s * STAGE + A_BYTES, &tmB, &full[s], 0, n0, kz);
+                        tma_load_3d(smem + s * STAGE, mA, &full[s], 0, m0, ka);
+                        tma_load_3d(smem + s * STAGE + A_BYTES, mB, &full[s], 0, n0, kz);
                     } else {
-                        tma_load_2d(smem + s * STAGE, &tmA, &full[s], ka * TC_BK, m0);
-                        tma_load_2d(smem + s * STAGE + A_BYTES, &tmB, &full[s], kz * TC_BK, n0);
+                        tma_load_2d(smem + s * STAGE, mA, &full[s], ka * TC_BK, m0);
+                        tma_load_2d(smem + s * STAGE + A_BYTES, mB, &full[s], kz * TC_BK, n0);
                     }
                     *issued = g + 1;
                 }
@@ -307,7 +317,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 }
                 tc_fence_after();
                 const uint32_t d = tmem + (uint32_t)(buf * BN);
-                const int kb = (tile / nmn) * kper, ke = min(nkt, kb + kper);
+                const int kb = grp.n ? 0 : (tile / nmn) * kper, ke = min(nkt, kb + kper);
                 for (int kt = kb; kt < ke; ++kt, ++g) {
                     const int s = g % STAGES, round = g / STAGES;
                     if (!mbar_wait(&full[s], round & 1)) {
@@ -347,10 +357,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         int j = 0;
         for (int tile = tile0; tile < ntiles; tile += tstep, ++j) {
             const int buf = j & 1, u = j >> 1;
-            const int mn = tile % nmn, ksp = tile / nmn;
-            int tm, tn;
-            tile_mn(mn, tilesMs, tilesN, group, tm, tn);
-            if (PAIR) tm = 2 * tm + crank;
+            int prob, ksp, tm, tn;
+            locate(tile, prob, ksp, tm, tn);
             const int m0 = tm * TC_BM, n0 = tn * BN;
             const bool ok = mbar_wait(&accf[buf], u & 1);
             tc_fence_after();
@@ -360,18 +368,22 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             const uint32_t tbase = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * BN);
             if (epi.mode == 5) {
-                // split-K partial: ws[(split * N + n) * M + m], lanes along m
+                // split-K partial: ws[(split * N + n) * M + m], lanes along m;
+                // in a group the problems' [n][m] follow one another
                 const long m = (long)m0 + 32 * q + lane;
-                float* ws = epi.C32 + (long)ksp * epi.N * epi.M + m;
+                const long M = grp.n ? grp.rows[prob & 1] : epi.M;
+                const long before = grp.n ? (prob >> 1) * (grp.rows[0] + grp.rows[1]) + (prob & 1 ? grp.rows[0] : 0)
+                                          : ksp * M;
+                float* ws = epi.C32 + before * epi.N + m;
 #pragma unroll 1
                 for (int ch = ch0; ch < ch1; ++ch) {
                     uint32_t r[32];
                     tmem_ld32(tbase + (uint32_t)(ch * 32), r);
-                    if (m >= epi.M) continue;
+                    if (m >= M) continue;
 #pragma unroll
                     for (int jj = 0; jj < 32; ++jj) {
                         const long nn = (long)n0 + ch * 32 + jj;
-                        if (nn < epi.N) ws[nn * epi.M] = __uint_as_float(r[jj]);
+                        if (nn < epi.N) ws[nn * M] = __uint_as_float(r[jj]);
                     }
                 }
             } else if (epi.mode == 2) {
@@ -448,39 +460,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                             else
                                 ladder_scatter<double>(epi.C, sblk, ro1, ro2, a, b, epi.V,
                                                        (double)__uint_as_float(r[jj]));
-                        }
-                        if (++bb == epi.Vb) { bb = 0; ++rr; }
-                    }
-                }
-            } else if (epi.mode == 6) {
-                // G-pass scatter of the symmetric / antisymmetric form: row m =
-                // (blk, i, j) as in mode 3, column n = (r, b) with k = a0 + r;
-                // G[s][i][j][k][b] at ((s O + i) O + j) O V + k V + b.  Blocks
-                // 0/1 add to their own G block, 4 (S+) adds to G[2] and G[3],
-                // 5 (S-) adds to G[2] and subtracts from G[3]
-                const long m = (long)m0 + 32 * q + lane;
-                const bool rowok = m < epi.M;
-                const int code = rowok ? epi.rowcode[m] : 0;
-                const int sblk = code >> 20, ri = (code >> 10) & 1023, rj = code & 1023;
-                const long OV = epi.O * epi.V;
-                const long g1 = (((long)(sblk < 2 ? sblk : 2) * epi.O + ri) * epi.O + rj) * OV;
-                const long g3 = ((3l * epi.O + ri) * epi.O + rj) * OV;
-#pragma unroll 1
-                for (int ch = ch0; ch < ch1; ++ch) {
-                    uint32_t r[32];
-                    tmem_ld32(tbase + (uint32_t)(ch * 32), r);
-                    if (!rowok) continue;
-                    const long nst = (long)n0 + ch * 32;
-                    long rr = nst / epi.Vb, bb = nst - rr * epi.Vb;
-#pragma unroll
-                    for (int jj = 0; jj < 32; ++jj) {
-                        if (nst + jj < epi.N) {
-                            const long off = (epi.a0 + rr) * epi.V + bb;
-                            // one update per target and launch: reductions
-                            const double v = (double)__uint_as_float(r[jj]);
-                            atomicAdd(epi.C + g1 + off, v);
-                            if (sblk == 4) atomicAdd(epi.C + g3 + off, v);
-                            else if (sblk == 5) atomicAdd(epi.C + g3 + off, -v);
                         }
                         if (++bb == epi.Vb) { bb = 0; ++rr; }
                     }
@@ -1131,6 +1110,106 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
 }
 
+// R2 (or G) += the consumers' contractions of one chunk, W[product][-, +][n][row]
+// with n = (r, b'): for the alpha-beta row (i, j) with S- and S+ of every
+// product in turn,
+//   R[ij][ab] += S-, += S+     R[ij][ba] += -S-, += S+   (a < b; a = b: S+ only)
+// and for a same-spin pair i < j
+//   R[ij][ab] = -R[ij][ba] = -R[ji][ab] = R[ji][ba] += S-.
+// G: G[2][ij][kb] += S-, += S+; G[3][ij][kb] += -S-, += S+; same spin: G[s] += S-.
+// A block takes 32 rows x 8 a x 8 b: W is read along the rows, R2 along its
+// last index.  (Scattered by the contractions' epilogues instead, each of 12
+// launches added 8 bytes to every line of R2 that it touched; and only what is
+// written apart can be computed in one launch.  At (12, 160, 480), six products:
+// 84 launches of 73 us on a part of the SMs each, 6.1 ms; now 8 of 160 us and
+// 0.9 ms of this kernel.  It is bound by the traffic of W and R2: at
+// (30, 500, 1500) 7 GB in 3.5 ms.)
+struct LadderJoin {
+    const float* W;
+    void* R;
+    const int* code;      // [2 P] block << 20 | i << 10 | j of the same-spin pairs
+    long rows[2];         // rows of the A- and the A+ problems
+    long pairs2, OO, N;   // 2 P, O^2, columns
+    int nsp, nr, Vb, mab; // products, chunk rows, columns b', blocks of alpha-beta rows
+    long a0, b0, O, V;
+};
+constexpr int LJ_M = 32, LJ_A = 8, LJ_B = 8, LJ_PITCH = LJ_A * LJ_B + 1;
+
+template <typename T, bool G, bool AB>
+__device__ __forceinline__ void ladder_join(const LadderJoin& a, float* lj) {
+    constexpr int NP = AB ? 2 : 1, NT = G ? NP : AB ? 2 : 4, TILE = LJ_M * LJ_PITCH;
+    const long m0 = (long)(AB ? blockIdx.x : blockIdx.x - a.mab) * LJ_M, nm = AB ? a.OO : a.pairs2;
+    const int r0 = blockIdx.y * LJ_A, b0 = blockIdx.z * LJ_B;
+    {
+        // lane = row, warp = b: the eight a of a tile are loads in flight together
+        const int m = threadIdx.x & 31, b = threadIdx.x >> 5;
+        const bool ok = m0 + m < nm && b0 + b < a.Vb;
+        for (int sp = 0; sp < a.nsp; ++sp) {
+#pragma unroll
+            for (int sg = 0; sg < NP; ++sg) {
+                const long before = sp * (a.rows[0] + a.rows[1]) + (sg ? a.rows[0] : 0);
+                const float* w = a.W + before * a.N + ((long)r0 * a.Vb + b0 + b) * a.rows[sg] + m0 + m +
+                                 (AB && sg == 0 ? a.pairs2 : 0);
+                float v[LJ_A];
+#pragma unroll
+                for (int k = 0; k < LJ_A; ++k)
+                    v[k] = ok && r0 + k < a.nr ? __ldcs(w + (long)k * a.Vb * a.rows[sg]) : 0.0f;
+#pragma unroll
+                for (int k = 0; k < LJ_A; ++k) lj[(sp * NP + sg) * TILE + m * LJ_PITCH + k * LJ_B + b] = v[k];
+            }
+        }
+    }
+    __syncthreads();
+    // the index that is contiguous in R (f) varies fastest over the lanes
+    const int f = threadIdx.x & 7, g = threadIdx.x >> 3 & 7, mt = threadIdx.x >> 6;
+    T* R = (T*)a.R;
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {  // R2: bit 0 (b, a), bit 1 (j, i); G: block 2 / 3
+        const bool swap = !G && (t & 1), minus = AB ? t == 1 : t == 1 || t == 2;
+        const int rr = swap ? f : g, bb = swap ? g : f;
+        const long ga = a.a0 + r0 + rr, gb = a.b0 + b0 + bb;
+        if (r0 + rr >= a.nr || b0 + bb >= a.Vb || (!G && (gb < ga || (gb == ga && (!AB || swap))))) continue;
+        const long ab = G ? ga * a.V + gb : swap ? gb * a.V + ga : ga * a.V + gb;
+        T v[LJ_M / 4];
+        long o[LJ_M / 4];
+#pragma unroll
+        for (int k = 0; k < LJ_M / 4; ++k) {
+            const long m = m0 + mt + 4 * k;
+            o[k] = -1;
+            if (m >= nm) continue;
+            long ij;
+            if (AB) {
+                ij = (G ? 2 + t : 2) * a.OO + m;
+            } else {
+                const int code = a.code[m], i = (code >> 10) & 1023, j = code & 1023;
+                ij = (code >> 20) * a.OO + (t & 2 ? j * a.O + i : i * a.O + j);
+            }
+            o[k] = ij * (G ? a.O : a.V) * a.V + ab;
+            v[k] = R[o[k]];
+        }
+        const float* w0 = lj + mt * LJ_PITCH + rr * LJ_B + bb;
+        for (int sp = 0; sp < a.nsp; ++sp, w0 += NP * TILE) {
+#pragma unroll
+            for (int k = 0; k < LJ_M / 4; ++k) {
+                const float* w = w0 + 4 * k * LJ_PITCH;
+                if (G || gb > ga) v[k] += minus ? -(T)w[0] : (T)w[0];
+                if (AB) v[k] += (T)w[TILE];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < LJ_M / 4; ++k)
+            if (o[k] >= 0) R[o[k]] = v[k];
+    }
+}
+
+template <typename T, bool G>
+__global__ void __launch_bounds__(256) k_ladder_join(const LadderJoin a) {
+    extern __shared__ float lj[];  // [product][-, +][row][r, b]
+    if (!G && (int)(blockIdx.z * LJ_B) + LJ_B <= (int)(blockIdx.y * LJ_A)) return;  // all b < a
+    if ((int)blockIdx.x < a.mab) ladder_join<T, G, true>(a, lj);
+    else ladder_join<T, G, false>(a, lj);
+}
+
 // Stacked S/A amplitudes from t2 (FP64): operand Am rows [same-spin pairs
 // i < j of blocks 0 and 1 (2P); alpha-beta (O^2)] with A-, operand Ap rows
 // [alpha-beta (O^2)] with A+, over the compact (c <= d) index, K-blocked
@@ -1628,10 +1707,9 @@ struct TcEngine {
     // symmetric / antisymmetric ladder: amplitudes A- (same-spin pairs and
     // alpha-beta rows) and A+ (alpha-beta rows), the M+ and M- tiles of a
     // chunk, the DF factors packed [(x, y)][L], each with its split parts one
-    // after the other, and the consumer row codes
+    // after the other
     Buf sam, sap, svp, svm, sx;
-    int* d_code_m = nullptr;
-    int* d_code_p = nullptr;
+    int* d_code_m = nullptr;  // same-spin pairs: block << 20 | i << 10 | j
     long sa_O = -1;
     bool sa_attr = false;
     int sx_nsplit = 0;  // parts of the packed DF factors in sx (0: none; B never changes)
@@ -1684,7 +1762,6 @@ void tc_free(Ctx* c) {
     for (auto& kv : e->bcache)
         if (kv.second.p) cudaFree(kv.second.p);
     if (e->d_code_m) cudaFree(e->d_code_m);
-    if (e->d_code_p) cudaFree(e->d_code_p);
     if (e->d_pairoff) cudaFree(e->d_pairoff);
     if (e->d_rowcode) cudaFree(e->d_rowcode);
     if (e->d_growoff) cudaFree(e->d_growoff);
@@ -1700,7 +1777,7 @@ void tc_state(const Ctx* c, std::vector<uint64_t>& s) {
     for (const Buf* b : {&e->pa, &e->pb, &e->pv, &e->pt, &e->sam, &e->sap, &e->svp, &e->svm, &e->sx, &e->pbv})
         s.push_back((uint64_t)(uintptr_t)b->p);
     for (const void* p : {(const void*)e->d_pairoff, (const void*)e->d_rowcode, (const void*)e->d_growoff,
-                          (const void*)e->d_code_m, (const void*)e->d_code_p, (const void*)e->wsk})
+                          (const void*)e->d_code_m, (const void*)e->wsk})
         s.push_back((uint64_t)(uintptr_t)p);
     for (long v : {(long)e->sx_nsplit, (long)e->pbv_nsplit, (long)e->bcache.size(), e->tab_O, e->tab_V, e->sa_O})
         s.push_back((uint64_t)v);
@@ -1848,22 +1925,22 @@ static dcsd_status make_map_kblk(Ctx* c, CUtensorMap* map, const __nv_bfloat16* 
     return DCSD_OK;
 }
 
-// One CTA or a pair per tile, and the columns per tile: the fewest clocks per
+// One CTA or a pair per tile (tm1 m-tiles, tm2 pairs of them), and the columns per
+// tile: the fewest clocks per
 // k-step over the waves of tiles.  A k-step of 64 occupies the shared memory
 // for 256 + 2 BN clocks in the one-CTA form and for max(256 + BN, 2 BN) in a
 // pair; the table has what a product of 8064 x 8064 x 8064 measured.  Narrow
 // tiles cost more per element but run on up to four times as many SMs.  (The
 // sums over k depend on neither.)  A BF16X6 ladder consumer at (10, 120, 360),
 // M = 276, N = 1800, K = 8704: 118 us with 256 columns, 63 us with 64.
-static double tc_tile_choice(const Ctx* c, long M, long N, long nsplits, int& BN, bool& pair) {
+static double tc_tile_choice(const Ctx* c, long tm1, long tm2, long N, long nsplits, int& BN, bool& pair) {
     static const double step[2][3] = {{400, 464, 784}, {393, 418, 600}};  // 64, 128, 256 columns
-    const long tm1 = (M + TC_BM - 1) / TC_BM;
     double best = 1e300;
     for (int pr = 0; pr < 2; ++pr) {
         if (pr && !(c->tc_pairs && c->tc->pairs > 0 && tm1 > 1)) continue;
         const long slots = pr ? c->tc->pairs : c->num_sms;
         for (int bn = 256; bn >= 64; bn /= 2) {
-            const long nt = (pr ? (tm1 + 1) / 2 : tm1) * ((N + bn - 1) / bn) * nsplits;
+            const long nt = (pr ? tm2 : tm1) * ((N + bn - 1) / bn) * nsplits;
             const double cost = (double)((nt + slots - 1) / slots) * step[pr][bn / 128];
             if (cost < 0.95 * best) {
                 best = cost;
@@ -1947,7 +2024,8 @@ static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __
     cudaLaunchAttribute at[1];
     int BN = 256;
     bool pair = false;
-    tc_tile_choice(c, M, N, std::max(1, ksplit), BN, pair);
+    const long tm1 = (M + TC_BM - 1) / TC_BM;
+    tc_tile_choice(c, tm1, (tm1 + 1) / 2, N, std::max(1, ksplit), BN, pair);
     const int bsel = BN == 256 ? 2 : BN == 128 ? 1 : 0;
     CUtensorMap ma, mb;
     if (pitch != 0 && (pitch < Ktot || pitch % 8 != 0 || ((uintptr_t)Ap | (uintptr_t)Bp) % 16 != 0)) {
@@ -2009,7 +2087,8 @@ static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __
     {
         int tm = (int)tilesM, tn = (int)tilesN, kb = kblocked ? 1 : 0, nk = nkt, kp = kper;
         int* derr = e->d_err;
-        void* args[] = {&ma, &mb, &epi, &parts, &nk, &tm, &tn, &kp, &group, &kb, &derr};
+        TcGroup grp = {};
+        void* args[] = {&ma, &mb, &ma, &mb, &epi, &parts, &grp, &nk, &tm, &tn, &kp, &group, &kb, &derr};
         tc_config(c, cfg, at, grid.x, tc_smem(BN, pair), pair);
         const cudaError_t le = cudaLaunchKernelExC(&cfg, tc_kernel(bsel, pair), args);
         if (le != cudaSuccess) {
@@ -2023,6 +2102,89 @@ static dcsd_status gemm_packed(Ctx* c, const __nv_bfloat16* Ap, long M, const __
     trace_end(c);
     prof_end(c, cls);
     return launch_check(c, "tc_gemm");
+}
+
+// FP32 workspace of split-K partial tiles and of the ladder's contractions
+static dcsd_status ensure_wsk(Ctx* c, size_t wsn) {
+    TcEngine* e = c->tc;
+    if (e->wsk_cap < wsn) {
+        if (e->wsk) cudaFree(e->wsk);
+        e->wsk = nullptr;
+        e->wsk_cap = 0;
+        DCSD_CUDA(c, cudaMalloc((void**)&e->wsk, wsn * sizeof(float)));
+        e->wsk_cap = wsn;
+    }
+    return DCSD_OK;
+}
+
+// W[product][-, +][n][row]: the ladder's contractions A-/+ x M-/+ of products
+// sp0 .. sp0 + nsp - 1 over one chunk's vrows columns, in one launch
+static dcsd_status gemm_ladder_group(Ctx* c, long rowsM, long rowsP, long vrows, long KSp, int np, const int* pa,
+                                     const int* pb, int nsp, float* W) {
+    TcEngine* e = c->tc;
+    const long rows[2] = {rowsM, rowsP};
+    long tm1 = 0, tm2 = 0;
+    for (long r : rows) {
+        const long t = (r + TC_BM - 1) / TC_BM;
+        tm1 += t;
+        tm2 += (t + 1) / 2;
+    }
+    int BN = 256;
+    bool pair = false;
+    tc_tile_choice(c, tm1, tm2, vrows, nsp, BN, pair);
+    CUtensorMap ma[2], mb[2];
+    const Buf* A[2] = {&e->sam, &e->sap};
+    const Buf* B[2] = {&e->svm, &e->svp};
+    for (int g = 0; g < 2; ++g) {
+        DCSD_TRY(make_map_kblk(c, &ma[g], A[g]->p, rows[g], KSp * np, TC_BM));
+        DCSD_TRY(make_map_kblk(c, &mb[g], B[g]->p, vrows, KSp * np, pair ? BN / 2 : BN));
+    }
+    TcParts parts = {};
+    parts.nkb = (int)(KSp / TC_BK);
+    TcGroup grp = {};
+    grp.n = 2 * nsp;
+    int tn = (int)((vrows + BN - 1) / BN);
+    for (int g = 0; g < 2; ++g) {
+        const long t = (rows[g] + TC_BM - 1) / TC_BM;
+        grp.tm[g] = (int)(pair ? (t + 1) / 2 : t);
+        grp.rows[g] = rows[g];
+    }
+    for (int p = 0; p < grp.n; ++p) {
+        parts.a[p / 2] = pa[p / 2];
+        parts.b[p / 2] = pb[p / 2];
+        grp.first[p + 1] = grp.first[p] + grp.tm[p & 1] * tn;
+    }
+    TcEpi epi;
+    std::memset(&epi, 0, sizeof(epi));
+    epi.mode = 5;
+    epi.C32 = W;
+    epi.N = vrows;
+    // all m-tiles of a column band in turn, so that M-/+ is read once
+    int tm = 1, nk = parts.nkb, kp = nk, kb = 1, group = 1 << 20;
+    int* derr = e->d_err;
+    void* args[] = {&ma[0], &mb[0], &ma[1], &mb[1], &epi, &parts, &grp, &nk, &tm, &tn, &kp, &group, &kb, &derr};
+    const long slots = pair ? e->pairs : c->num_sms;
+    const unsigned grid = (unsigned)std::min<long>(grp.first[grp.n], slots);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[1];
+    tc_config(c, cfg, at, pair ? 2 * grid : grid, tc_smem(BN, pair), pair);
+    prof_begin(c, DCSD_PROF_LADDER);
+    if (c->trace) {
+        const std::string label = "tc-ladder group=" + std::to_string(grp.n) + " M=" + std::to_string(rowsM + rowsP) +
+                                  " N=" + std::to_string(vrows) + " Kt=" + std::to_string(KSp);
+        if (c->trace_seq) fprintf(stderr, "[dcsd tc #%d] %s\n", c->tc_seq, label.c_str());
+        trace_begin(c, label);
+    }
+    ++c->tc_seq;
+    const cudaError_t le = cudaLaunchKernelExC(&cfg, tc_kernel(BN == 256 ? 2 : BN == 128 ? 1 : 0, pair), args);
+    trace_end(c);
+    prof_end(c, DCSD_PROF_LADDER);
+    if (le != cudaSuccess) {
+        c->err = std::string("ladder group (launch): ") + cudaGetErrorString(le);
+        cudaGetLastError();
+        return DCSD_ERR_CUDA;
+    }
+    return launch_check(c, "ladder group");
 }
 
 dcsd_status einsum_tc_impl(Ctx* c, const char* spec, double alpha, const TV& A, const TV& B, double beta,
@@ -2334,13 +2496,7 @@ dcsd_status einsum_tc_impl(Ctx* c, const char* spec, double alpha, const TV& A, 
         ksplit = (nkt + kper - 1) / kper;
     }
     const size_t wsn = (size_t)ksplit * p.M * p.N;
-    if (e->wsk_cap < wsn) {
-        if (e->wsk) cudaFree(e->wsk);
-        e->wsk = nullptr;
-        e->wsk_cap = 0;
-        DCSD_CUDA(c, cudaMalloc((void**)&e->wsk, wsn * sizeof(float)));
-        e->wsk_cap = wsn;
-    }
+    DCSD_TRY(ensure_wsk(c, wsn));
     TcEpi red = epi;
     red.M = p.M;
     red.N = p.N;
@@ -2415,11 +2571,12 @@ static std::vector<std::pair<long, long>> ladder_chunks(long V, long Vp, long ro
 
 // chunks of a for the symmetric / antisymmetric ladder (dynamic programming
 // over the tile waves): per chunk (r0, nr) the producer runs npair x
-// #(r, b' >= r) tiles of nkx k-steps (two 128 x 128 MMAs per step, about one
-// 128 x 256 step), the consumers GEMMs of rowsM and rowsP rows against
-// nr * (V - r0) columns over nks k-steps
-static std::vector<std::pair<long, long>> ladder_chunks_sa(const Ctx* c, long V, long rowsM, long rowsP, long nks,
-                                                           long nkx, long npair, long nmax) {
+// #(r, b' >= r) tiles of nkx k-steps, the consumers nsp products of rowsM and of
+// rowsP rows with nr * (V - r0) columns over nks k-steps each, in one launch
+static std::vector<std::pair<long, long>> ladder_chunks_sa(const Ctx* c, long V, long rowsM, long rowsP, long nsp,
+                                                           long nks, long nkx, long npair, long nmax) {
+    const long t0 = (rowsM + TC_BM - 1) / TC_BM, t1 = (rowsP + TC_BM - 1) / TC_BM;
+    const long tm1 = t0 + t1, tm2 = (t0 + 1) / 2 + (t1 + 1) / 2;
     int bn;
     bool pr;
     const bool pairs = c->tc_pairs && c->tc->pairs > 0;
@@ -2436,8 +2593,7 @@ static std::vector<std::pair<long, long>> ladder_chunks_sa(const Ctx* c, long V,
             const long ptiles = pairs ? npair * (np2 * Vb - np2 * (np2 - 1)) : npair * (nr * Vb - nr * (nr - 1) / 2);
             const long slots = pairs ? c->tc->pairs : c->num_sms;
             const double prod = (double)((ptiles + slots - 1) / slots) * (double)nkx * (pairs ? 768.0 : 1024.0);
-            const double cons = (tc_tile_choice(c, rowsM, nr * Vb, 1, bn, pr) + tc_tile_choice(c, rowsP, nr * Vb, 1, bn, pr)) *
-                                (double)nks;
+            const double cons = tc_tile_choice(c, tm1, tm2, nr * Vb, nsp, bn, pr) * (double)nks;
             const double cost = prod + cons + launch + best[r0 + nr];
             if (cost < best[r0]) {
                 best[r0] = cost;
@@ -2450,10 +2606,14 @@ static std::vector<std::pair<long, long>> ladder_chunks_sa(const Ctx* c, long V,
     return out;
 }
 
+// bytes of the ladder's contractions that are kept between the launch that
+// computes them and the one that adds them up
+constexpr size_t kLadderWork = 512ul << 20;
+
 // R2 += the ladder in symmetric / antisymmetric form (see sa_koff): per chunk
-// of a, k_ladder_sa builds the M+ and M- tiles and two consumer GEMMs
-// contract them with A- (same-spin pairs and alpha-beta rows) and A+
-// (alpha-beta rows), scattering into R2 (codes 0/1/5 and 4 of ladder_scatter).
+// of a, k_ladder_sa builds the M+ and M- tiles, one launch contracts them with
+// A- (same-spin pairs and alpha-beta rows) and A+ (alpha-beta rows), and
+// k_ladder_join adds the results to R2.
 static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
     TcEngine* e = c->tc;
     const long n = c->n, nc = c->nc, O = c->O, V = c->V, X = c->X;
@@ -2472,26 +2632,18 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
         c->err = "symmetric / antisymmetric ladder: sizes out of range";
         return DCSD_ERR_INVALID_ARG;
     }
-    // consumer row codes: A- rows [same-spin pairs; alpha-beta (block 5)],
-    // A+ rows [alpha-beta (block 4)]
     if (e->sa_O != O) {
-        std::vector<int> cm(rowsM), cp(rowsP);
-        long m = 0;
+        std::vector<int> cm;
         for (int sb = 0; sb < 2; ++sb)
             for (long i = 0; i < O; ++i)
-                for (long j = i + 1; j < O; ++j) cm[m++] = (sb << 20) | (int)(i << 10) | (int)j;
-        for (long i = 0; i < O; ++i)
-            for (long j = 0; j < O; ++j) {
-                cm[m++] = (5 << 20) | (int)(i << 10) | (int)j;
-                cp[i * O + j] = (4 << 20) | (int)(i << 10) | (int)j;
-            }
-        for (int** pp : {&e->d_code_m, &e->d_code_p})
-            if (*pp) { cudaFree(*pp); *pp = nullptr; }
+                for (long j = i + 1; j < O; ++j) cm.push_back((sb << 20) | (int)(i << 10) | (int)j);
+        if (e->d_code_m) cudaFree(e->d_code_m);
+        e->d_code_m = nullptr;
         e->sa_O = -1;
-        DCSD_CUDA(c, cudaMalloc((void**)&e->d_code_m, sizeof(int) * rowsM));
-        DCSD_CUDA(c, cudaMalloc((void**)&e->d_code_p, sizeof(int) * rowsP));
-        DCSD_CUDA(c, cudaMemcpy(e->d_code_m, cm.data(), sizeof(int) * rowsM, cudaMemcpyHostToDevice));
-        DCSD_CUDA(c, cudaMemcpy(e->d_code_p, cp.data(), sizeof(int) * rowsP, cudaMemcpyHostToDevice));
+        if (P > 0) {
+            DCSD_CUDA(c, cudaMalloc((void**)&e->d_code_m, sizeof(int) * cm.size()));
+            DCSD_CUDA(c, cudaMemcpy(e->d_code_m, cm.data(), sizeof(int) * cm.size(), cudaMemcpyHostToDevice));
+        }
         e->sa_O = O;
     }
     // stacked A- and A+ amplitudes (the partial last k-block zeroed first)
@@ -2561,6 +2713,10 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
     const size_t smem = SA_STAGES * 4 * (size_t)SA_TILE + 2048;
     if (!e->sa_attr) {
         DCSD_CUDA(c, cudaFuncSetAttribute(k_ladder_sa, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        const int jsm = 6 * 2 * LJ_M * LJ_PITCH * (int)sizeof(float);
+        for (const void* f : {(const void*)k_ladder_join<float, false>, (const void*)k_ladder_join<double, false>,
+                              (const void*)k_ladder_join<double, true>})
+            DCSD_CUDA(c, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, jsm));
         e->sa_attr = true;
     }
     DCSD_TRY(tc_setup(c));
@@ -2575,7 +2731,7 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
     DCSD_CUDA(c, cudaMemsetAsync(G, 0, sizeof(double) * 4 * O * O * O * V, c->stream));
     for (int pass = 0; pass < 2; ++pass) {
         std::vector<std::pair<long, long>> chunks;
-        if (pass == 0) chunks = ladder_chunks_sa(c, V, rowsM, rowsP, KSt / TC_BK, Xt / TC_BK, npair, chunk);
+        if (pass == 0) chunks = ladder_chunks_sa(c, V, rowsM, rowsP, nseg, KSp / TC_BK, Xt / TC_BK, npair, chunk);
         else
             for (long k0 = 0; k0 < O; k0 += chunk) chunks.push_back({k0, std::min(chunk, O - k0)});
         for (const auto& ck : chunks) {
@@ -2628,26 +2784,41 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
             trace_end(c);
             prof_end(c, DCSD_PROF_LADDER);
             DCSD_TRY(launch_check(c, "ladder_sa"));
-            // consumers: A- x M- and A+ x M+, one launch per split product
-            TcEpi ce;
-            std::memset(&ce, 0, sizeof(ce));
-            ce.mode = pass == 0 ? 3 : 6;
-            ce.alpha = 1.0;
-            ce.C = pass == 0 ? R2 : G;
-            ce.C32 = (pass == 0 && c->r2f_on && R2 == c->R2) ? c->r2f : nullptr;
-            ce.O = O;
-            ce.V = V;
-            ce.Vb = Vb;
-            ce.a0 = r0;
-            ce.OO = O * O;
-            ce.VV = V * V;
-            for (int sp = 0; sp < nseg; ++sp) {
-                ce.rowcode = e->d_code_m;
-                DCSD_TRY(gemm_packed(c, e->sam.p + (size_t)pa[sp] * rowsM * KSp, rowsM,
-                                     e->svm.p + (size_t)pb[sp] * vrows * KSp, vrows, KSp, ce, 1, 0, true));
-                ce.rowcode = e->d_code_p;
-                DCSD_TRY(gemm_packed(c, e->sap.p + (size_t)pa[sp] * rowsP * KSp, rowsP,
-                                     e->svp.p + (size_t)pb[sp] * vrows * KSp, vrows, KSp, ce, 1, 0, true));
+            // consumers: A- x M- and A+ x M+ of the split products, as many of
+            // them in a launch as the workspace holds
+            LadderJoin lj;
+            std::memset(&lj, 0, sizeof(lj));
+            lj.code = e->d_code_m;
+            lj.rows[0] = rowsM;
+            lj.rows[1] = rowsP;
+            lj.pairs2 = 2 * P;
+            lj.OO = O * O;
+            lj.N = vrows;
+            lj.nr = (int)nr;
+            lj.Vb = (int)Vb;
+            lj.mab = (int)((O * O + LJ_M - 1) / LJ_M);
+            lj.a0 = r0;
+            lj.b0 = pass == 0 ? r0 : 0;
+            lj.O = O;
+            lj.V = V;
+            const bool f32 = pass == 0 && c->r2f_on && R2 == c->R2;
+            lj.R = pass == 1 ? (void*)G : f32 ? (void*)c->r2f : (void*)R2;
+            const size_t each = (size_t)(rowsM + rowsP) * vrows;
+            const int most = (int)std::max<size_t>(1, std::min<size_t>(nseg, kLadderWork / (each * sizeof(float))));
+            DCSD_TRY(ensure_wsk(c, each * most));
+            lj.W = e->wsk;
+            for (int sp = 0; sp < nseg; sp += most) {
+                lj.nsp = std::min(most, nseg - sp);
+                DCSD_TRY(gemm_ladder_group(c, rowsM, rowsP, vrows, KSp, np, pa + sp, pb + sp, lj.nsp, e->wsk));
+                const dim3 grid((unsigned)(lj.mab + (2 * P + LJ_M - 1) / LJ_M), (unsigned)((nr + LJ_A - 1) / LJ_A),
+                                (unsigned)((Vb + LJ_B - 1) / LJ_B));
+                const size_t sm = (size_t)lj.nsp * 2 * LJ_M * LJ_PITCH * sizeof(float);
+                trace_begin(c, "ladder join");
+                if (pass == 1) k_ladder_join<double, true><<<grid, 256, sm, c->stream>>>(lj);
+                else if (f32) k_ladder_join<float, false><<<grid, 256, sm, c->stream>>>(lj);
+                else k_ladder_join<double, false><<<grid, 256, sm, c->stream>>>(lj);
+                trace_end(c);
+                DCSD_TRY(launch_check(c, "ladder join"));
             }
         }
     }
