@@ -338,16 +338,19 @@ __global__ void __launch_bounds__(256) k_crt_pack(const Operand oa, const Operan
 // ---------------------------------------------------------------------------
 // the modular GEMM
 // ---------------------------------------------------------------------------
-constexpr int CG_BM = 128, CG_BK = 64, CG_STAGES = 4;
-constexpr uint32_t CG_A = CG_BM * CG_BK * 2, CG_STAGE = CG_A + 256 * CG_BK * 2;
+constexpr int CG_BM = 128, CG_BK = 64;
+constexpr uint32_t CG_A = CG_BM * CG_BK * 2;
+// stages of 16 KB of A and up to 32 KB of B; in a pair half of B
+__host__ __device__ constexpr int cg_stages(bool pair) { return pair ? 6 : 4; }
+__host__ __device__ constexpr uint32_t cg_stage(bool pair) { return CG_A + (pair ? 128 : 256) * CG_BK * 2; }
 constexpr int kEpiWarps = 8, kThreads = 32 * (2 + kEpiWarps);
-constexpr size_t kCrtSmem = CG_STAGES * CG_STAGE + 2048;
+constexpr size_t kCrtSmem = 6 * cg_stage(true) + 2048;  // (= 4 * cg_stage(false) + 2048)
 
 struct GemmShape {
     long M, N;              // rows and columns
     int nkb, kper;          // 64-deep k-blocks, k-blocks per split
     int nsplit;
-    int tilesM, tilesN, BN; // n-tiles of BN columns (a multiple of 16, at most 256)
+    int tilesM, tilesN, BN; // n-tiles of BN columns (a multiple of 16, in a pair of 32; at most 256)
     int group;
     uint32_t* planes;       // [split][modulus][ceil(N / 4)][M] four residues (bytes) of consecutive n
 };
@@ -359,13 +362,17 @@ struct GemmShape {
 // exact, and kept modulo p in FP32 registers (four FP32 operations per
 // element, hidden behind the 16 k-blocks of MMAs), so a long k costs no
 // memory traffic; the residues leave as bytes.
-// MC: clusters of two CTAs on neighbouring m-tiles of one n-tile, each loading
-// half of the B tile and multicasting it to both: an SM takes in 64 bytes per
-// clock, less than a 128 x 256 tile's 48 KB per 64 k would need at full rate.
-template <bool MC>
+// PAIR: two CTAs on neighbouring m-tiles of one n-tile as a cta_group::2 pair,
+// as in k_tc_gemm: each loads its rows of A and half of B, and a k-block takes
+// 600 clocks instead of 784 with 256 columns.  (10, 120, 360): the ladder's
+// M = 2196, K = 14884 contraction of a chunk 373 -> 268 us, its integrals,
+// M = 14884, K = 360, 455 -> 405 us, with what electing the issuing lane gave.
+template <bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
     k_crt_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmShape g,
                int* err) {
+    constexpr int CG_STAGES = cg_stages(PAIR);
+    constexpr uint32_t CG_STAGE = cg_stage(PAIR);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t* full = (uint64_t*)(smem + CG_STAGES * CG_STAGE);
@@ -377,32 +384,35 @@ __global__ void __launch_bounds__(kThreads, 1)
     volatile int* consumed = issued + 1;
 
     const int warp = warp_id(), lane = threadIdx.x & 31;
-    const int crank = MC ? (int)cluster_rank() : 0;
-    const int tile0 = MC ? (int)blockIdx.x / 2 : (int)blockIdx.x;
-    const int tstep = MC ? (int)gridDim.x / 2 : (int)gridDim.x;
-    const int tilesMs = MC ? (g.tilesM + 1) / 2 : g.tilesM;
+    const int crank = PAIR ? (int)cluster_rank() : 0;
+    const int tile0 = PAIR ? (int)blockIdx.x / 2 : (int)blockIdx.x;
+    const int tstep = PAIR ? (int)gridDim.x / 2 : (int)gridDim.x;
+    const int tilesMs = PAIR ? (g.tilesM + 1) / 2 : g.tilesM;
     const int nmn = tilesMs * g.tilesN;
     const int ntiles = nmn * kMods * g.nsplit;
     const int BN = g.BN;
     if (threadIdx.x == 0) {
         for (int s = 0; s < CG_STAGES; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], MC ? 2 : 1);
+            mbar_init(&empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&accf[b], 1);
-            mbar_init(&acce[b], kEpiWarps);
+            mbar_init(&acce[b], PAIR ? 2 * kEpiWarps : kEpiWarps);
         }
         *issued = 0;
         *consumed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == 1) tmem_alloc(tslot, 512);
+    if (warp == 1) {
+        if (PAIR) tmem_alloc_pair(tslot, 512);
+        else tmem_alloc(tslot, 512);
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (MC) cluster_sync();
+    if (PAIR) cluster_sync();
     const uint32_t tmem = *tslot;
 
     // tile -> (m-tile, n-tile, modulus, split)
@@ -415,7 +425,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int rows = min(gr, tilesMs - band * gr);
         tm = band * gr + r % rows;
         tn = r / rows;
-        if (MC) tm = 2 * tm + crank;
+        if (PAIR) tm = 2 * tm + crank;
     };
 
     if (warp == 0) {
@@ -435,26 +445,30 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     const int z = mod * g.nkb + kt;
                     uint8_t* st = smem + s * CG_STAGE;
-                    mbar_expect_tx(&full[s], CG_A + (uint32_t)BN * CG_BK * 2);
-                    tma_load_3d(st, &tmA, &full[s], 0, tm * CG_BM, z);
-                    if (MC)
-                        tma_load_3d_mc(st + CG_A + crank * (BN / 2) * CG_BK * 2, &tmB, &full[s], 0,
-                                       tn * BN + crank * (BN / 2), z, (uint16_t)0x3);
-                    else
+                    if (PAIR) {
+                        // both CTAs' bytes complete on the leader's barrier
+                        if (crank == 0) mbar_expect_tx(&full[s], 2 * CG_A + (uint32_t)BN * CG_BK * 2);
+                        const uint32_t bar = leader_addr(&full[s]);
+                        tma_load_3d_pair(st, &tmA, bar, 0, tm * CG_BM, z);
+                        tma_load_3d_pair(st + CG_A, &tmB, bar, 0, tn * BN + crank * (BN / 2), z);
+                    } else {
+                        mbar_expect_tx(&full[s], CG_A + (uint32_t)BN * CG_BK * 2);
+                        tma_load_3d(st, &tmA, &full[s], 0, tm * CG_BM, z);
                         tma_load_3d(st + CG_A, &tmB, &full[s], 0, tn * BN, z);
+                    }
                     *issued = it + 1;
                 }
             }
-            if (MC) {
+            if (PAIR) {
                 // every slot free in both CTAs before the cluster may end
                 for (int i = max(0, it - CG_STAGES); i < it; ++i)
                     if (!mbar_wait(&empty[i % CG_STAGES], (i / CG_STAGES) & 1)) atomicExch(err, 5);
             }
         }
     } else if (warp == 1) {
-        if (elect_one()) {
+        if (crank == 0 && elect_one()) {
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                                   ((uint32_t)(CG_BM >> 4) << 24);
+                                   ((uint32_t)((PAIR ? 2 * CG_BM : CG_BM) >> 4) << 24);
             int it = 0, j = 0;
             bool ok = true;
             for (int tile = tile0; tile < ntiles && ok; tile += tstep) {
@@ -481,19 +495,25 @@ __global__ void __launch_bounds__(kThreads, 1)
                         tc_fence_after();
                         const uint32_t a0 = smem_u32(smem + s * CG_STAGE), b0 = a0 + CG_A;
 #pragma unroll
-                        for (int kk = 0; kk < CG_BK / 16; ++kk)
-                            mma_bf16(d, smem_desc(a0 + kk * 32), smem_desc(b0 + kk * 32), idesc,
-                                     (kt > k0 || kk > 0) ? 1u : 0u);
-                        if (MC) mma_commit_mc(&empty[s], (uint16_t)0x3);
+                        for (int kk = 0; kk < CG_BK / 16; ++kk) {
+                            const uint32_t acc = (kt > k0 || kk > 0) ? 1u : 0u;
+                            if (PAIR) mma_bf16_pair(d, smem_desc(a0 + kk * 32), smem_desc(b0 + kk * 32), idesc, acc);
+                            else mma_bf16(d, smem_desc(a0 + kk * 32), smem_desc(b0 + kk * 32), idesc, acc);
+                        }
+                        if (PAIR) mma_commit_pair(&empty[s]);
                         else mma_commit(&empty[s]);
                         *consumed = it + 1;
                     }
-                    if (ok) mma_commit(&accf[buf]);
+                    if (ok) {
+                        if (PAIR) mma_commit_pair(&accf[buf]);
+                        else mma_commit(&accf[buf]);
+                    }
                 }
             }
             if (!ok) {
                 // let issued MMAs finish and drain copies that were not consumed
-                mma_commit(&accf[j & 1]);
+                if (PAIR) mma_commit_pair(&accf[j & 1]);
+                else mma_commit(&accf[j & 1]);
                 for (int i = *consumed; i < *issued; ++i) mbar_wait(&full[i % CG_STAGES], (i / CG_STAGES) & 1);
             }
         }
@@ -534,7 +554,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&acce[buf]);
+                if (lane == 0) {
+                    if (PAIR) mbar_arrive_cluster(leader_addr(&acce[buf]));
+                    else mbar_arrive(&acce[buf]);
+                }
             }
             if (!ok) break;
             const long m = (long)tm * CG_BM + 32 * q + lane;
@@ -560,10 +583,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
     __syncthreads();
     __syncwarp();
-    if (MC) cluster_sync();
+    if (PAIR) cluster_sync();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, 512);
+        if (PAIR) tmem_dealloc_pair(tmem, 512);
+        else tmem_dealloc(tmem, 512);
     }
 }
 
@@ -796,17 +820,17 @@ static dcsd_status crt_pass(Ctx* c, const char* spec, const GemmPlan& p, const d
     g.nkb = (int)((K + 63) / 64);
     g.tilesM = (int)((M + CG_BM - 1) / CG_BM);
     g.tilesN = (int)((N + 255) / 256);
-    g.BN = (int)up((N + g.tilesN - 1) / g.tilesN, 16);
-    const bool mc = e->clusters > 0 && g.tilesM > 1;
-    const long tilesMs = mc ? (g.tilesM + 1) / 2 : g.tilesM;
-    const long slots = mc ? e->clusters : c->num_sms;
+    const bool pair = e->clusters > 0 && g.tilesM > 1;
+    g.BN = (int)up((N + g.tilesN - 1) / g.tilesN, pair ? 32 : 16);
+    const long tilesMs = pair ? (g.tilesM + 1) / 2 : g.tilesM;
+    const long slots = pair ? e->clusters : c->num_sms;
     const long t1 = tilesMs * g.tilesN * kMods;
     // few output tiles: k split over the idle SMs (a pass reduces the splits' residues)
     long ns = std::max<long>(1, std::min<long>({slots / t1, (long)g.nkb / 8, 8l}));
     while (ns > 1 && pass_bytes(M, N, K, ns) > e->bytes) --ns;
     g.kper = (int)((g.nkb + ns - 1) / ns);
     g.nsplit = (g.nkb + g.kper - 1) / g.kper;
-    g.group = (int)std::max<long>(1, std::min<long>(tilesMs, std::lround(std::sqrt((double)slots * g.BN / CG_BM / (mc ? 2 : 1)))));
+    g.group = (int)std::max<long>(1, std::min<long>(tilesMs, std::lround(std::sqrt((double)slots * g.BN / CG_BM / (pair ? 2 : 1)))));
     // (recorded: a piece of the workspace of its own when it is large enough)
     const size_t need = pass_bytes(M, N, K, g.nsplit);
     const size_t at = need <= e->bytes / 2 ? dag_slice(c, 3, (need + 255) / 256 * 256, e->bytes) : 0;
@@ -887,10 +911,10 @@ static dcsd_status crt_pass(Ctx* c, const char* spec, const GemmPlan& p, const d
     DCSD_TRY(launch_check(c, "crt_pack"));
     CUtensorMap ma, mb;
     DCSD_TRY(make_map(c, &ma, o[0].dst, M, (long)kMods * g.nkb, CG_BM));
-    DCSD_TRY(make_map(c, &mb, o[1].dst, N, (long)kMods * g.nkb, mc ? g.BN / 2 : g.BN));
+    DCSD_TRY(make_map(c, &mb, o[1].dst, N, (long)kMods * g.nkb, pair ? g.BN / 2 : g.BN));
     if (c->trace) trace_begin(c, label("crt-gemm "));
     const long nt = tilesMs * g.tilesN * kMods * g.nsplit;
-    if (mc) {
+    if (pair) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(2 * std::min<long>(nt, slots)));
         cfg.blockDim = dim3(kThreads);
