@@ -646,9 +646,15 @@ extern "C" dcsd_status dcsd_vjp(dcsd_ctx* h, int ref, int method, int precision,
         return DCSD_ERR_INVALID_ARG;
     }
     const size_t nn = (size_t)c->n * c->n, nB = (size_t)c->X * nn;
-    if (mem_kind == DCSD_MEM_DEVICE)
-        return vjp_run(c, ref, method, precision, T, nrb ? Rb : nullptr, dEA_bar, W_bar, Tb, B_bar, fock_a_bar,
-                       fock_b_bar);
+    auto waited = [&]() -> dcsd_status {  // did every wait of the tensor-core kernels end?
+        DCSD_TRY(sync_scalars(c, 23));
+        return tc_timeout(c) ? DCSD_ERR_TIMEOUT : DCSD_OK;
+    };
+    if (mem_kind == DCSD_MEM_DEVICE) {
+        DCSD_TRY(vjp_run(c, ref, method, precision, T, nrb ? Rb : nullptr, dEA_bar, W_bar, Tb, B_bar, fock_a_bar,
+                         fock_b_bar));
+        return waited();
+    }
     // host memory: stage through device buffers
     DCSD_TRY(ensure_abi(c));
     std::vector<double*> tmp;
@@ -683,6 +689,7 @@ extern "C" dcsd_status dcsd_vjp(dcsd_ctx* h, int ref, int method, int precision,
     if (fock_a_bar && !(Fad = dev(nn))) return DCSD_ERR_OOM;
     if (fock_b_bar && !(Fbd = dev(nn))) return DCSD_ERR_OOM;
     DCSD_TRY(vjp_run(c, ref, method, precision, Td, nrb ? Rd : nullptr, dEA_bar, W_bar, Tbd, Bd, Fad, Fbd));
+    DCSD_TRY(waited());
     for (int k = 0; k < 5; ++k)
         DCSD_CUDA(c, cudaMemcpyAsync(Tb[k], Tbd[k], abi_len(c, k) * sizeof(double), cudaMemcpyDeviceToHost,
                                      c->stream));
@@ -820,7 +827,8 @@ extern "C" dcsd_status dcsd_lambda(dcsd_ctx* h, const dcsd_solve_opts* o, int st
         Ctx* c;
         ~TapeClear() { c->tape.clear(); }
     } tc_guard{c};
-    DCSD_TRY(sync_scalars(c, 2));
+    DCSD_TRY(sync_scalars(c, 23));
+    if (tc_timeout(c)) return DCSD_ERR_TIMEOUT;
     res->W = c->hostbuf[0];
     res->dEA = c->hostbuf[1];
     res->E_S = res->dEA + res->W;
@@ -853,7 +861,8 @@ extern "C" dcsd_status dcsd_lambda(dcsd_ctx* h, const dcsd_solve_opts* o, int st
         DCSD_TRY(launch_check(c, "antisym_ss"));
         DCSD_CUDA(c, cudaMemsetAsync(gp + eAB, 0, sizeof(double), c->stream));
         DCSD_TRY(maxabs(c, gp, len, c->scal + 21));
-        DCSD_TRY(sync_scalars(c, 22));
+        DCSD_TRY(sync_scalars(c, 23));
+        if (tc_timeout(c)) return DCSD_ERR_TIMEOUT;
         const double gmax = c->hostbuf[21];
         res->max_r = gmax;
         if (c->verbose) fprintf(stderr, "[dcsd lambda] it %3d max|G| %.3e\n", it, gmax);

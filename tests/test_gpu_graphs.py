@@ -1,0 +1,69 @@
+"""Repeated calls on one context.  From the second call with the same method,
+reference and precision on, the residual and the FP64 reverse mode are replays
+of a recorded graph; each must give what a context that has done nothing else
+gives, bit for bit in the tensor-core precisions (their sums have one order)
+and to the rounding of FP64 sums in FP64 (the Frobenius norms agree to 1e-13:
+a few hundred roundings of 1.1e-16).  Also the ladder's contractions in one
+launch, with one and no same-spin pair and ragged edges of its 8 x 8 x 32
+blocks, against the FP64 residual."""
+import numpy as np
+import pytest
+
+from synth import make_system, random_amplitudes
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2401_11935_gb300 as P
+    return P
+
+
+def _res(eng, T, prec, method, ref):
+    R, W, dE = eng.residual(eng.to_device(T), ref=ref, method=method, precision=prec)
+    return [x.cpu().numpy() for x in R] + [np.array([W, dE])]
+
+
+def _same(a, b, prec):
+    for x, y in zip(a, b):
+        if prec == 0:
+            assert np.linalg.norm(x - y) <= 1e-13 * max(1.0, np.linalg.norm(y))
+        else:
+            assert np.array_equal(x, y)
+
+
+# (precision, method, ref, amplitudes): alternating, each at least three times
+CALLS = [(1, 0, 0, 0), (4, 0, 0, 1), (1, 0, 0, 1), (0, 1, 1, 0), (4, 0, 0, 0), (0, 1, 1, 1), (1, 0, 0, 0),
+         (2, 1, 0, 1), (0, 1, 1, 0), (4, 0, 0, 1), (2, 1, 0, 0), (1, 0, 0, 1), (2, 1, 0, 1)]
+
+
+@pytest.mark.parametrize("dims", [(3, 9, 16), (5, 37, 60)])
+def test_replayed_residuals_equal_first_calls(P, dims):
+    s = make_system(dims, seed=11)
+    T = {r: [random_amplitudes(s, seed=20 + k, ref=r, scale1=0.02, scale2=0.02) for k in range(2)] for r in (0, 1)}
+    first = {}
+    for call in set(CALLS):
+        eng = P.Engine.from_system(s)
+        first[call] = _res(eng, T[call[2]][call[3]], *call[:3])
+        eng.close()
+    eng = P.Engine.from_system(s)
+    for call in CALLS:
+        _same(_res(eng, T[call[2]][call[3]], *call[:3]), first[call], call[0])
+    eng.close()
+
+
+@pytest.mark.parametrize("dims", [(1, 21, 30), (2, 19, 30), (3, 131, 40)])
+@pytest.mark.parametrize("prec,tol", [(2, 2e-4), (4, 2e-5)])
+def test_ladder_block_edges(P, dims, prec, tol):
+    s = make_system(dims, seed=12)
+    T = random_amplitudes(s, seed=31, scale1=0.02, scale2=0.02)
+    eng = P.Engine.from_system(s)
+    R0, R = _res(eng, T, 0, 0, 0), _res(eng, T, prec, 0, 0)
+    eng.close()
+    rmax = max(float(np.abs(x).max()) for x in R0[:5])
+    # the split's precision, relative to max |R|, as for the full sizes
+    assert max(float(np.abs(a - b).max()) for a, b in zip(R[:5], R0[:5])) < tol * rmax
