@@ -38,13 +38,11 @@ METRIC = "2D-DCSD s/iteration & ladder TFLOP/s vs peak; mixed vs FP64 at 1e-6 Eh
 UNIT = "s/iteration"
 
 
-# dram__bytes_read.sum + dram__bytes_write.sum averaged over the 90 ladder
-# launches of one 30+2 / 500 / 1500 BF16 residual in symmetric / antisymmetric
-# form (28 M+- producers and 56 consumers for the ladder, 2 producers and 4
-# consumers for the G intermediate), from a one-pass ncu capture of this
-# benchmark; set to None whenever the ladder kernels change until a new
-# capture replaces it
-LADDER_DRAM_BYTES_PER_LAUNCH = 4.343e9
+# dram__bytes_read.sum + dram__bytes_write.sum averaged over the ladder launches
+# (M+- producers, grouped contractions, joins) of one 30+2 / 500 / 1500 BF16
+# residual, from a one-pass ncu capture; None whenever the ladder kernels change
+# until a new capture replaces it
+LADDER_DRAM_BYTES_PER_LAUNCH = None
 
 
 def ladder_flops(nc, nv, X):
@@ -390,7 +388,7 @@ def main():
                      "frac": (achieved / peak) if achieved else None, "peak_source": peak_src,
                      "algorithmic_flops_per_launch": lf / max(1.0, per_res_launches),
                      "avg_launch_ms": lad_ms / max(1, lad_n), "traffic": LADDER_DRAM_BYTES_PER_LAUNCH,
-                     "traffic_unit": "bytes per ladder launch (producer or consumer), DRAM read + write"},
+                     "traffic_unit": "bytes per ladder launch (producer, contractions or join), DRAM read + write"},
         "kernel_ms_per_step": {k: v[0] / args.steps for k, v in prof.items() if v[1]},
         "e2e": {"value": e2e, "unit": UNIT, "h2d_bytes_per_step": nbytes, "d2h_bytes_per_step": nbytes,
                 "note": "dcsd_solve(maxiter 1) with pinned host amplitudes: copy in, residual, update, copy out"},

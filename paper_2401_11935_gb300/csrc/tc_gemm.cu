@@ -2813,11 +2813,13 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
                 const dim3 grid((unsigned)(lj.mab + (2 * P + LJ_M - 1) / LJ_M), (unsigned)((nr + LJ_A - 1) / LJ_A),
                                 (unsigned)((Vb + LJ_B - 1) / LJ_B));
                 const size_t sm = (size_t)lj.nsp * 2 * LJ_M * LJ_PITCH * sizeof(float);
+                prof_begin(c, DCSD_PROF_LADDER);
                 trace_begin(c, "ladder join");
                 if (pass == 1) k_ladder_join<double, true><<<grid, 256, sm, c->stream>>>(lj);
                 else if (f32) k_ladder_join<float, false><<<grid, 256, sm, c->stream>>>(lj);
                 else k_ladder_join<double, false><<<grid, 256, sm, c->stream>>>(lj);
                 trace_end(c);
+                prof_end(c, DCSD_PROF_LADDER);
                 DCSD_TRY(launch_check(c, "ladder join"));
             }
         }
