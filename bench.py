@@ -38,11 +38,11 @@ METRIC = "2D-DCSD s/iteration & ladder TFLOP/s vs peak; mixed vs FP64 at 1e-6 Eh
 UNIT = "s/iteration"
 
 
-# dram__bytes_read.sum + dram__bytes_write.sum averaged over the ladder launches
-# (M+- producers, grouped contractions, joins) of one 30+2 / 500 / 1500 BF16
+# dram__bytes_read.sum + dram__bytes_write.sum averaged over the 84 ladder launches
+# (28 M+- producers, grouped contractions and joins each) of one 30+2 / 500 / 1500 BF16
 # residual, from a one-pass ncu capture; None whenever the ladder kernels change
 # until a new capture replaces it
-LADDER_DRAM_BYTES_PER_LAUNCH = None
+LADDER_DRAM_BYTES_PER_LAUNCH = 3.064e9
 
 
 def ladder_flops(nc, nv, X):
