@@ -1699,6 +1699,7 @@ struct TcEngine {
     long* d_growoff = nullptr;  // [rows] offset of the row's G[blk][i][j] slice
     float* wsk = nullptr;       // split-K partial tiles
     size_t wsk_cap = 0;
+    size_t wsk_refused = SIZE_MAX;  // the ladder asks for less than what could not be allocated
     static constexpr int kPackSlots = 4;
     Buf pc[kPackSlots];         // pack cache (see pack_operand)
     std::string pc_key[kPackSlots];
@@ -2804,8 +2805,15 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
             const bool f32 = pass == 0 && c->r2f_on && R2 == c->R2;
             lj.R = pass == 1 ? (void*)G : f32 ? (void*)c->r2f : (void*)R2;
             const size_t each = (size_t)(rowsM + rowsP) * vrows;
-            const int most = (int)std::max<size_t>(1, std::min<size_t>(nseg, kLadderWork / (each * sizeof(float))));
-            DCSD_TRY(ensure_wsk(c, each * most));
+            int most = (int)std::max<size_t>(1, std::min<size_t>(nseg, kLadderWork / (each * sizeof(float))));
+            for (;; most = (most + 1) / 2) {
+                if (most > 1 && each * most >= e->wsk_refused) continue;
+                const dcsd_status ws = ensure_wsk(c, each * most);
+                if (ws == DCSD_OK) break;
+                if (most == 1) return ws;
+                cudaGetLastError();
+                e->wsk_refused = each * most;
+            }
             lj.W = e->wsk;
             for (int sp = 0; sp < nseg; sp += most) {
                 lj.nsp = std::min(most, nseg - sp);
