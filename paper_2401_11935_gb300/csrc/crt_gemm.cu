@@ -7,23 +7,33 @@
 // FP32 accumulator.  So (Ozaki, Uchino and Imamura, "Ozaki Scheme II",
 // arXiv 2504.08009):
 //   1. every row of A and B (over k) is scaled by a power of two to integers
-//      with 2-norm below 2^58 and 2^57 (elements rounded to the nearest
+//      with 2-norm below 2^62 and 2^61 (elements rounded to the nearest
 //      integer, the only approximation);
-//   2. the integer rows are reduced modulo 15 pairwise coprime p_i <= 256;
+//   2. the integer rows are reduced modulo 16 pairwise coprime p_i <= 256;
 //   3. one tcgen05 GEMM per modulus gives C mod p_i exactly;
 //   4. C is put together by the Chinese remainder theorem: |C| <= |a| |b| <
-//      2^115 < P / 4 with P = prod p_i = 2^117.8, in integer arithmetic, then
+//      2^123 < P / 4 with P = prod p_i = 2^125.4, in integer arithmetic, then
 //      rounded once to FP64.
-// The rounding of step 1 gives an error of about 0.4 sqrt(K) 2^-57 of a
-// typical element, against 0.2 sqrt(K) 2^-52 of a chain of FP64 FMAs.
-// Non-finite inputs give NaN in the rows and columns that hold them.
+// The rounding of step 1 leaves an error relative to |a| |b|: in the units
+// where the norms' bounds are 1, at most 0.75 sqrt(K) 2^-61, 0.3 2^-61 in the
+// root mean square.  A chain of FMAs errs relative to S = sum_k |a_k b_k|,
+// which is far below |a| |b| where large elements of a meet small ones of b.
+// So one more GEMM, over the magnitudes rounded down to BF16, gives S; where it
+// is below 2^-7 in the same units (and not zero), the element is computed as a
+// chain of FMAs instead (k_crt_patch).  The others err by at most
+// 0.375 sqrt(K) 2^-53 S, 2e-17 S in the root mean square, as much as a chain
+// does for products of random sign.  Rows and columns with Inf or NaN go to
+// the chain, too.
 //
 // Measured (GB300), CUDA cores -> this path: (M, N, K) = (432, 2196, 14884)
-// 23.8 -> 1.08 ms, of which GEMM 0.37 (1.13 PFLOP/s of BF16), residues 0.43,
-// norms 0.18, output 0.04; (2196, 14884, 360) 19.2 -> 0.91 ms, of which output
-// 0.31 and GEMM 0.47 (short k); (1464, 1464, 1464) 5.19 -> 0.23 ms; error
-// against an extended-precision sum 0.1 to 0.35 of the CUDA cores'.  The whole
-// FP64 residual at (10, 120, 360): 445 -> 24.8 ms.
+// 23.6 -> 0.91 ms, of which GEMM 0.33 (1.46 PFLOP/s of BF16), residues 0.38,
+// norms 0.18; (2196, 14884, 360) 19.2 -> 0.98 ms, of which GEMM 0.43 (short
+// k) and output 0.41; (1464, 1464, 1464) 5.18 -> 0.20 ms.  The whole FP64
+// residual at (10, 120, 360): 445 -> 23.0 ms, of which the patch takes 1.4
+// (0.28 ms of a contraction whose i = j columns are zero in one operand where
+// the other is largest); before the sums of magnitudes and the patch, with 15
+// moduli, 21.1 ms.  Operands that fall by 12 decades along k, against each
+// other, take the CUDA cores' time and 7 to 20 % (50 to 90 us where it is short).
 #include "common.h"
 #include "tc_ptx.h"
 
@@ -42,11 +52,19 @@ namespace {
 // ---------------------------------------------------------------------------
 // moduli and derived constants
 // ---------------------------------------------------------------------------
-constexpr int kMods = 15;
-constexpr int kModulus[kMods] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197};
+constexpr int kMods = 16;
+constexpr int kModulus[kMods] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193};
+constexpr int kPlanes = kMods + 1;             // residues, and the magnitudes
 constexpr int kLimbs = 6;                      // 20-bit limbs of P and P / p_i
-constexpr int kBetaA = 58, kBetaB = 57;        // log2 bounds of the integer rows' 2-norms
+constexpr int kBetaA = 62, kBetaB = 61;        // log2 bounds of the integer rows' 2-norms
 constexpr int kSegBlocks = 16;                 // 64-deep k-blocks per exact FP32 sum (16 * 64 = 1024)
+
+// Sums of magnitudes as a byte per split of K: 0 for a zero sum, else S 2^13 +
+// 0.75 to the nearest integer, 1 to 255.  A result is kept where the splits'
+// sum is 0 (all products are zero) or at least 74: S >= (74 - 8 x 1.25) 2^-13 = 2^-7.
+constexpr float kSumScale = 8192.0f;
+constexpr int kSumKept = 74, kMaxSplit = 8;
+__device__ __forceinline__ bool sum_kept(int code) { return code == 0 || code >= kSumKept; }
 
 constexpr long sym_mod(long x, long p) {       // residue in [-(p - 1) / 2, p / 2]
     long r = x % p;
@@ -60,7 +78,7 @@ constexpr long sym_byte(long x, long p) {      // the same in [-128, 127]
 }
 
 struct Tables {
-    float p[kMods], inv_p[kMods];
+    float p[kPlanes], inv_p[kPlanes];          // (magnitudes: 0, which reduce_mod leaves as they are)
     // byte weights of a 64-bit integer, 2^(8 j) mod p (side B: times
     // (P / p_i)^-1), signed bytes; the start value -2^63 of a biased integer,
     // already offset by the FP32 pattern of kRint
@@ -94,7 +112,7 @@ constexpr Tables make_tables() {
         }
         for (int l = 0; l < kLimbs; ++l) t.limb[i][l] = (int)((Mi >> (20 * l)) & 0xFFFFF);
     }
-    for (int l = 0; l < kLimbs; ++l) t.plimb[l] = (int)((P >> (20 * l)) & 0xFFFFF);
+    for (int l = 0; l < kLimbs; ++l) t.plimb[l] = (int)((P >> (20 * l)) & (l + 1 < kLimbs ? 0xFFFFF : 0x7FFFFFFF));
     return t;
 }
 
@@ -126,7 +144,7 @@ struct Operand {
     unsigned long long* part_mx;  // [nchunk][rows] magnitudes' bit patterns
     int* shift;                 // [rows] power-of-two scale, kNonFinite where a row holds Inf or NaN
     long* coff;                 // [rows] offset in C
-    uint16_t* dst;              // [modulus][K / 64][rows][64] residues (BF16)
+    uint16_t* dst;              // [plane][K / 64][rows][64] residues and magnitudes (BF16)
     int nchunk, nkb;
     int kchunk;                 // k per partial norm
     int kbper;                  // k-blocks per block of the pack launch
@@ -233,7 +251,7 @@ __device__ __forceinline__ int row_shift(double ss, unsigned long long mx, long 
     return beta - L;
 }
 
-// x * 2^s rounded to the nearest integer (|result| < 2^59 by the row's scale)
+// x * 2^s rounded to the nearest integer (|result| <= 2^62 by the row's scale)
 __device__ __forceinline__ long long scaled_int(double x, int s) {
     const long long b = __double_as_longlong(x);
     const int ef = (int)((b >> 52) & 0x7FF);
@@ -255,11 +273,22 @@ __device__ __forceinline__ int byte_dot(unsigned bytes, unsigned weights, int ac
     return r;
 }
 
+// |v| 2^-beta rounded down to BF16, in the upper half of a word; at least
+// 2^(2 - beta) where the element is not zero, so that only sums whose products
+// are all zero vanish (the products stay normal in FP32: >= 2^-119)
+__device__ __forceinline__ unsigned magnitude(long long v, double x, int beta) {
+    if (x == 0.0) return 0u;
+    const float f = fmaxf(__ull2float_rz((unsigned long long)(v < 0 ? -v : v)), 4.0f);
+    return __float_as_uint(f) - ((unsigned)beta << 23);
+}
+
 // Residues of one operand: per 64 rows x 64 k, scale to integers, reduce
-// modulo every p_i, store BF16 K-blocked [modulus][k block][row][64].  Writes
-// 30 bytes per element read; two byte products and five FP32 operations
-// per element and modulus.
-__global__ void __launch_bounds__(256) k_crt_pack(const Operand oa, const Operand ob) {
+// modulo every p_i, store BF16 K-blocked [plane][k block][row][64], the
+// magnitudes after the residues.  Writes 34 bytes per element read; two byte
+// products and five FP32 operations per element and modulus.  Clears the
+// nclear words of the patch's flags as well.
+__global__ void __launch_bounds__(256) k_crt_pack(const Operand oa, const Operand ob, unsigned* clear, long nclear) {
+    for (long i = (long)blockIdx.x * 256 + threadIdx.x; i < nclear; i += (long)gridDim.x * 256) clear[i] = 0u;
     __shared__ double tile[64][65];
     __shared__ long roff[64], koff[64];
     __shared__ int sh[64];
@@ -315,10 +344,10 @@ __global__ void __launch_bounds__(256) k_crt_pack(const Operand oa, const Operan
             const long r = row0 + rl;
             if (r >= o.rows) break;
             const int s = sh[rl];
-            const unsigned long long v0 = (unsigned long long)(s == kNonFinite ? 0 : scaled_int(tile[rl][2 * lane], s)) ^
-                                          0x8000000000000000ull;
-            const unsigned long long v1 = (unsigned long long)(s == kNonFinite ? 0 : scaled_int(tile[rl][2 * lane + 1], s)) ^
-                                          0x8000000000000000ull;
+            const double e0 = s == kNonFinite ? 0.0 : tile[rl][2 * lane], e1 = s == kNonFinite ? 0.0 : tile[rl][2 * lane + 1];
+            const long long i0 = scaled_int(e0, s), i1 = scaled_int(e1, s);
+            const unsigned long long v0 = (unsigned long long)i0 ^ 0x8000000000000000ull;
+            const unsigned long long v1 = (unsigned long long)i1 ^ 0x8000000000000000ull;
             uint32_t* dst = (uint32_t*)(o.dst + ((long)kt * o.rows + r) * 64) + lane;
 #pragma unroll
             for (int i = 0; i < kMods; ++i) {
@@ -331,6 +360,7 @@ __global__ void __launch_bounds__(256) k_crt_pack(const Operand oa, const Operan
                 // integers of magnitude <= 128: the upper half of the FP32 word is the BF16 value
                 dst[(long)i * (plane / 2)] = __byte_perm(__float_as_uint(y0), __float_as_uint(y1), 0x7632);
             }
+            dst[(long)kMods * (plane / 2)] = __byte_perm(magnitude(i0, e0, o.beta), magnitude(i1, e1, o.beta), 0x7632);
         }
     }
 }
@@ -352,10 +382,10 @@ struct GemmShape {
     int nsplit;
     int tilesM, tilesN, BN; // n-tiles of BN columns (a multiple of 16, in a pair of 32; at most 256)
     int group;
-    uint32_t* planes;       // [split][modulus][ceil(N / 4)][M] four residues (bytes) of consecutive n
+    uint32_t* planes;       // [split][plane][ceil(N / 4)][M] four residues or sums (bytes) of consecutive n
 };
 
-// Persistent tcgen05 GEMM over (split, modulus, m-tile, n-tile).  The pipeline
+// Persistent tcgen05 GEMM over (split, plane, m-tile, n-tile).  The pipeline
 // is that of k_tc_gemm: warp 0 loads K-blocked tiles by TMA, warp 1 issues
 // the MMAs into one of two TMEM accumulators, eight warps drain the other.
 // The accumulator is drained every 1024 k, where its integer sum is still
@@ -366,7 +396,8 @@ struct GemmShape {
 // as in k_tc_gemm: each loads its rows of A and half of B, and a k-block takes
 // 600 clocks instead of 784 with 256 columns.  (10, 120, 360): the ladder's
 // M = 2196, K = 14884 contraction of a chunk 373 -> 268 us, its integrals,
-// M = 14884, K = 360, 455 -> 405 us, with what electing the issuing lane gave.
+// M = 14884, K = 360, 455 -> 405 us, with what electing the issuing lane gave
+// (both over 15 planes; 328 and 429 us over 17).
 template <bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
     k_crt_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmShape g,
@@ -389,7 +420,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int tstep = PAIR ? (int)gridDim.x / 2 : (int)gridDim.x;
     const int tilesMs = PAIR ? (g.tilesM + 1) / 2 : g.tilesM;
     const int nmn = tilesMs * g.tilesN;
-    const int ntiles = nmn * kMods * g.nsplit;
+    const int ntiles = nmn * kPlanes * g.nsplit;
     const int BN = g.BN;
     if (threadIdx.x == 0) {
         for (int s = 0; s < CG_STAGES; ++s) {
@@ -415,11 +446,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (PAIR) cluster_sync();
     const uint32_t tmem = *tslot;
 
-    // tile -> (m-tile, n-tile, modulus, split)
+    // tile -> (m-tile, n-tile, plane, split)
     auto locate = [&](int tile, int& tm, int& tn, int& mod, int& ks) {
         const int z = tile / nmn, mn = tile - z * nmn;
-        ks = z / kMods;
-        mod = z - ks * kMods;
+        ks = z / kPlanes;
+        mod = z - ks * kPlanes;
         const int gr = max(1, min(g.group, tilesMs));
         const int band = mn / (gr * g.tilesN), r = mn - band * gr * g.tilesN;
         const int rows = min(gr, tilesMs - band * gr);
@@ -562,22 +593,32 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!ok) break;
             const long m = (long)tm * CG_BM + 32 * q + lane;
             if (m >= g.M) continue;
-            uint32_t* out = g.planes + (long)(ks * kMods + mod) * N4 * g.M + m;
+            uint32_t* out = g.planes + (long)(ks * kPlanes + mod) * N4 * g.M + m;
             const long n4 = ((long)tn * BN + c0) >> 2;
+            // low byte of an FP32 word + kRint: the residue, or the sum's byte
+            // (two loops: one with the choice inside issued both and took 1.8
+            // times as long over a short k)
+            auto store = [&](auto byte) {
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (c < nch) {
+                for (int c = 0; c < 4; ++c)
+                    if (c < nch) {
 #pragma unroll
-                    for (int x = 0; x < 32; x += 4) {
-                        if (c * 32 + x >= half || n4 + c * 8 + x / 4 >= N4) continue;
-                        uint32_t w[4];
+                        for (int x = 0; x < 32; x += 4) {
+                            if (c * 32 + x >= half || n4 + c * 8 + x / 4 >= N4) continue;
+                            uint32_t w[4];
 #pragma unroll
-                        for (int y = 0; y < 4; ++y)
-                            w[y] = __float_as_uint(reduce_mod(acc[c][x + y], p, ip) + kRint);  // low byte: the residue
-                        const uint32_t lo = __byte_perm(w[0], w[1], 0x0040), hi = __byte_perm(w[2], w[3], 0x0040);
-                        out[(n4 + c * 8 + x / 4) * g.M] = __byte_perm(lo, hi, 0x5410);
+                            for (int y = 0; y < 4; ++y) w[y] = byte(acc[c][x + y]);
+                            const uint32_t lo = __byte_perm(w[0], w[1], 0x0040), hi = __byte_perm(w[2], w[3], 0x0040);
+                            out[(n4 + c * 8 + x / 4) * g.M] = __byte_perm(lo, hi, 0x5410);
+                        }
                     }
-                }
+            };
+            if (mod == kMods)
+                store([](float s) {
+                    return s == 0.0f ? 0u : __float_as_uint(fminf(255.0f, fmaf(s, kSumScale, 0.75f)) + kRint);
+                });
+            else
+                store([&](float r) { return __float_as_uint(reduce_mod(r, p, ip) + kRint); });
         }
     }
     tc_fence_before();
@@ -602,6 +643,8 @@ struct OutArgs {
     const long *off_m, *off_n;
     double* C;
     double alpha, beta;
+    unsigned* flags;        // [n / 16][m / 16] tiles with elements left to k_crt_patch
+    long tilesM;
 };
 
 // sum_i q_i (P / p_i) mod P in 20-bit limbs, as a double times 2^-e
@@ -669,6 +712,7 @@ __global__ void __launch_bounds__(128, 8) k_crt_out(const OutArgs a) {
         const uint32_t* src = a.planes + n4 * a.M + m;
         const long plane = N4 * a.M;
         uint32_t w[kMods], even[SPLIT ? kMods : 1], odd[SPLIT ? kMods : 1];
+        uint32_t sum = src[kMods * plane], sume = 0, sumo = 0;
 #pragma unroll
         for (int i = 0; i < kMods; ++i) w[i] = src[i * plane];
         if (SPLIT) {
@@ -677,9 +721,14 @@ __global__ void __launch_bounds__(128, 8) k_crt_out(const OutArgs a) {
                 even[i] = (w[i] ^ 0x80808080u) & 0x00FF00FFu;
                 odd[i] = ((w[i] ^ 0x80808080u) >> 8) & 0x00FF00FFu;
             }
+            sume = sum & 0x00FF00FFu;
+            sumo = (sum >> 8) & 0x00FF00FFu;
             for (int s = 1; s < a.nsplit; ++s) {
 #pragma unroll
-                for (int i = 0; i < kMods; ++i) w[i] = src[((long)s * kMods + i) * plane];
+                for (int i = 0; i < kMods; ++i) w[i] = src[((long)s * kPlanes + i) * plane];
+                sum = src[((long)s * kPlanes + kMods) * plane];
+                sume += sum & 0x00FF00FFu;
+                sumo += (sum >> 8) & 0x00FF00FFu;
 #pragma unroll
                 for (int i = 0; i < kMods; ++i) {
                     even[i] += (w[i] ^ 0x80808080u) & 0x00FF00FFu;
@@ -710,13 +759,136 @@ __global__ void __launch_bounds__(128, 8) k_crt_out(const OutArgs a) {
 #pragma unroll
             for (int l = 0; l < kLimbs; ++l) S[y][l] -= k * d_tab.plimb[l];
             const int sn = a.shift_n[n];
-            double v = (sm == kNonFinite || sn == kNonFinite) ? __longlong_as_double(0x7FF8000000000000ll)
-                                                              : crt_value(S[y], sm + sn);
+            const int code = (int)(SPLIT ? ((y & 1 ? sumo : sume) >> (8 * (y & 2))) & 0xFFFFu : (sum >> (8 * y)) & 0xFFu);
+            if (sm == kNonFinite || sn == kNonFinite || !sum_kept(code)) {
+                a.flags[(n4 >> 2) * a.tilesM + (m >> 4)] = 1u;
+                continue;
+            }
+            double v = crt_value(S[y], sm + sn);
             double* cp = a.C + om + a.off_n[n];
             v *= a.alpha;
             if (a.beta != 0.0) v = fma(a.beta, *cp, v);
             *cp = v;
         }
+    }
+}
+
+// The elements that k_crt_out left, by 16 x 16 tiles.  A tile with up to 64 of
+// them (a row or a column, a diagonal: exchange-antisymmetric amplitudes vanish
+// where a diagonal of the other operand is large): a warp per element, its lanes over k.  Else the
+// whole tile as FMAs of a chain per element.  K in pieces where few tiles are
+// to share the chip (kchunk; the last block of a tile adds the pieces in
+// order).  A block looks through the flags of its tiles 256 at a time.
+struct PatchArgs {
+    unsigned *flags, *count;  // [tile], count: arrivals of a tile's pieces
+    long ntiles;
+    int nsplit;
+    long kchunk;
+    double* ws;               // [tile][piece][256]
+};
+
+__global__ void __launch_bounds__(256) k_crt_patch(const Operand oa, const Operand ob, const OutArgs a,
+                                                   const PatchArgs g) {
+    constexpr int T = 16, KC = 32;
+    __shared__ double As[KC][T + 1], Bs[KC][T + 1];
+    __shared__ long ra[T], rb[T];
+    __shared__ int list[256], nlist, elem[256], nelem;
+    __shared__ double sums[256];
+    __shared__ bool last;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const long N4 = (a.N + 3) >> 2, plane = N4 * a.M;
+    const long kb = blockIdx.y * g.kchunk, ke = min(oa.K, kb + g.kchunk);
+    for (long r = 0; r * gridDim.x + blockIdx.x < g.ntiles; r += 256) {
+        const long mine = (r + tid) * gridDim.x + blockIdx.x;
+        if (tid == 0) nlist = 0;
+        __syncthreads();
+        if (mine < g.ntiles && g.flags[mine]) list[atomicAdd(&nlist, 1)] = (int)mine;
+        __syncthreads();
+        for (int i = 0; i < nlist; ++i) {
+            const long t = list[i], m0 = t % a.tilesM * T, n0 = t / a.tilesM * T, m = m0 + tx, n = n0 + ty;
+            if (tid < T) ra[tid] = m0 + tid < a.M ? mode_offset((unsigned)(oa.r0 + m0 + tid), oa.nr, oa.rsz, oa.rs) : -1;
+            else if (tid < 2 * T)
+                rb[tid - T] = n0 + tid - T < a.N ? mode_offset((unsigned)(ob.r0 + n0 + tid - T), ob.nr, ob.rsz, ob.rs) : -1;
+            else if (tid == 2 * T) nelem = 0;
+            bool wanted = false;
+            if (m < a.M && n < a.N) {
+                int code = 0;
+                for (int s = 0; s < a.nsplit; ++s)
+                    code += (a.planes[((long)s * kPlanes + kMods) * plane + (n >> 2) * a.M + m] >> (8 * (n & 3))) & 0xFFu;
+                wanted = a.shift_m[m] == kNonFinite || a.shift_n[n] == kNonFinite || !sum_kept(code);
+            }
+            __syncthreads();
+            if (wanted) elem[atomicAdd(&nelem, 1)] = tid;
+            __syncthreads();
+            double acc = 0.0;
+            if (nelem <= 64) {
+                for (int e = tid >> 5; e < nelem; e += 8) {
+                    const double *pa = oa.p + ra[elem[e] & 15], *pb = ob.p + rb[elem[e] >> 4];
+                    double s = 0.0;
+                    for (long k = kb + (tid & 31); k < ke; k += 32)
+                        s = fma(pa[mode_offset((unsigned)(oa.k0 + k), oa.nk, oa.ksz, oa.ks)],
+                                pb[mode_offset((unsigned)(ob.k0 + k), ob.nk, ob.ksz, ob.ks)], s);
+#pragma unroll
+                    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+                    if ((tid & 31) == 0) sums[elem[e]] = s;
+                }
+                __syncthreads();
+                if (wanted) acc = sums[tid];
+            } else {
+                double x[2], y[2];
+                auto fetch = [&](long k0) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int e = tid + 256 * h;
+                        const int ka = oa.kfast ? e & 31 : e >> 4, ma = oa.kfast ? e >> 5 : e & 15;
+                        const int kn = ob.kfast ? e & 31 : e >> 4, mn = ob.kfast ? e >> 5 : e & 15;
+                        x[h] = k0 + ka < ke && ra[ma] >= 0
+                                   ? oa.p[ra[ma] + mode_offset((unsigned)(oa.k0 + k0 + ka), oa.nk, oa.ksz, oa.ks)] : 0.0;
+                        y[h] = k0 + kn < ke && rb[mn] >= 0
+                                   ? ob.p[rb[mn] + mode_offset((unsigned)(ob.k0 + k0 + kn), ob.nk, ob.ksz, ob.ks)] : 0.0;
+                    }
+                };
+                fetch(kb);
+                for (long k0 = kb; k0 < ke; k0 += KC) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int e = tid + 256 * h;
+                        if (oa.kfast) As[e & 31][e >> 5] = x[h];
+                        else As[e >> 4][e & 15] = x[h];
+                        if (ob.kfast) Bs[e & 31][e >> 5] = y[h];
+                        else Bs[e >> 4][e & 15] = y[h];
+                    }
+                    __syncthreads();
+                    if (k0 + KC < ke) fetch(k0 + KC);
+                    const int kn = (int)min((long)KC, ke - k0);
+                    for (int k = 0; k < kn; ++k) acc = fma(As[k][tx], Bs[k][ty], acc);
+                    __syncthreads();
+                }
+            }
+            bool write = wanted;
+            if (g.nsplit > 1) {
+                double* w = g.ws + t * g.nsplit * 256;
+                w[blockIdx.y * 256 + tid] = acc;
+                __threadfence();
+                __syncthreads();
+                if (tid == 0) last = atomicAdd(g.count + t, 1u) == (unsigned)g.nsplit - 1;
+                __syncthreads();
+                write = wanted && last;
+                if (write) {
+                    __threadfence();
+                    acc = 0.0;
+                    for (int s = 0; s < g.nsplit; ++s) acc += __ldcg(w + s * 256 + tid);
+                }
+            }
+            if (write) {
+                double* cp = a.C + a.off_m[m] + a.off_n[n];
+                double v = acc * a.alpha;
+                if (a.beta != 0.0) v = fma(a.beta, *cp, v);
+                *cp = v;
+            }
+            __syncthreads();  // the tile's tables are free
+        }
+        __syncthreads();
     }
 }
 
@@ -748,7 +920,7 @@ dcsd_status crt_init(Ctx* c) {
     }
     e->encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
     const double V = c->V, OV = (double)c->O * c->V, rows = 4.0 * c->O * c->O;
-    const double want = 2.0 * kMods * 2.0 * ((V * V + rows) * (V * V + 64) + 2 * OV * (OV + 64)) + 15.0 * OV * OV;
+    const double want = 2.0 * kPlanes * 2.0 * ((V * V + rows) * (V * V + 64) + 2 * OV * (OV + 64)) + kPlanes * OV * OV;
     e->bytes = (size_t)std::min(2147483648.0, std::max(33554432.0, want)) / 1024 * 1024;
     if (cudaMalloc((void**)&e->ws, e->bytes) != cudaSuccess) {
         // without it every contraction stays on the CUDA cores
@@ -803,11 +975,13 @@ bool crt_ready(const Ctx* c) { return c->crt && c->crt->ws; }
 // k per partial norm: a multiple of 128, at most 32 pieces
 static int norm_chunk(long K) { return (int)std::max<long>(128, up((K + 31) / 32, 128)); }
 
-// bytes of a pass: residues of both operands, row tables, residues of the output
+static long patch_tiles(long M, long N) { return ((M + 15) / 16) * ((N + 15) / 16); }
+
+// bytes of a pass: residues of both operands, row tables, residues of the output, flags
 static size_t pass_bytes(long M, long N, long K, long nsplit) {
     const size_t nkb = (size_t)(K + 63) / 64, nch = (size_t)(K + norm_chunk(K) - 1) / norm_chunk(K);
-    return (size_t)(M + N) * (nkb * 64 * 2 * kMods + nch * 16 + 16) + (size_t)nsplit * kMods * 4 * ((N + 3) / 4) * M +
-           16 * 256;
+    return (size_t)(M + N) * (nkb * 64 * 2 * kPlanes + nch * 16 + 16) + (size_t)nsplit * kPlanes * 4 * ((N + 3) / 4) * M +
+           8 * (size_t)patch_tiles(M, N) + 16 * 256;
 }
 
 // one pass: rows [m0, m0 + M), columns [n0, n0 + N), k [k0, k0 + K)
@@ -824,9 +998,9 @@ static dcsd_status crt_pass(Ctx* c, const char* spec, const GemmPlan& p, const d
     g.BN = (int)up((N + g.tilesN - 1) / g.tilesN, pair ? 32 : 16);
     const long tilesMs = pair ? (g.tilesM + 1) / 2 : g.tilesM;
     const long slots = pair ? e->clusters : c->num_sms;
-    const long t1 = tilesMs * g.tilesN * kMods;
+    const long t1 = tilesMs * g.tilesN * kPlanes;
     // few output tiles: k split over the idle SMs (a pass reduces the splits' residues)
-    long ns = std::max<long>(1, std::min<long>({slots / t1, (long)g.nkb / 8, 8l}));
+    long ns = std::max<long>(1, std::min<long>({slots / t1, (long)g.nkb / 8, (long)kMaxSplit}));
     while (ns > 1 && pass_bytes(M, N, K, ns) > e->bytes) --ns;
     g.kper = (int)((g.nkb + ns - 1) / ns);
     g.nsplit = (g.nkb + g.kper - 1) / g.kper;
@@ -866,14 +1040,16 @@ static dcsd_status crt_pass(Ctx* c, const char* spec, const GemmPlan& p, const d
         x.nkb = g.nkb;
         x.kchunk = norm_chunk(K);
         x.nchunk = (int)((K + x.kchunk - 1) / x.kchunk);
-        x.dst = (uint16_t*)take((size_t)kMods * g.nkb * 64 * x.rows * 2);
+        x.dst = (uint16_t*)take((size_t)kPlanes * g.nkb * 64 * x.rows * 2);
         x.part_ss = (double*)take((size_t)x.nchunk * x.rows * 8);
         x.part_mx = (unsigned long long*)take((size_t)x.nchunk * x.rows * 8);
         x.shift = (int*)take((size_t)x.rows * 4);
         x.coff = (long*)take((size_t)x.rows * 8);
     }
     const long N4 = (N + 3) / 4;
-    g.planes = (uint32_t*)take((size_t)g.nsplit * kMods * 4 * N4 * M);
+    g.planes = (uint32_t*)take((size_t)g.nsplit * kPlanes * 4 * N4 * M);
+    const long ptiles = patch_tiles(M, N);
+    unsigned* flags = (unsigned*)take((size_t)ptiles * 8);
     if ((size_t)(w - e->ws) > e->bytes || (size_t)(w - e->ws) > at + need) {
         c->err = std::string(spec) + ": modular GEMM workspace";
         return DCSD_ERR_INVALID_ARG;
@@ -906,14 +1082,14 @@ static dcsd_status crt_pass(Ctx* c, const char* spec, const GemmPlan& p, const d
         o[s].blocks = rb * ((o[s].nkb + o[s].kbper - 1) / o[s].kbper);
     }
     if (c->trace) trace_begin(c, label("crt-pack "));
-    k_crt_pack<<<(unsigned)(o[0].blocks + o[1].blocks), 256, 0, c->stream>>>(o[0], o[1]);
+    k_crt_pack<<<(unsigned)(o[0].blocks + o[1].blocks), 256, 0, c->stream>>>(o[0], o[1], flags, 2 * ptiles);
     trace_end(c);
     DCSD_TRY(launch_check(c, "crt_pack"));
     CUtensorMap ma, mb;
-    DCSD_TRY(make_map(c, &ma, o[0].dst, M, (long)kMods * g.nkb, CG_BM));
-    DCSD_TRY(make_map(c, &mb, o[1].dst, N, (long)kMods * g.nkb, pair ? g.BN / 2 : g.BN));
+    DCSD_TRY(make_map(c, &ma, o[0].dst, M, (long)kPlanes * g.nkb, CG_BM));
+    DCSD_TRY(make_map(c, &mb, o[1].dst, N, (long)kPlanes * g.nkb, pair ? g.BN / 2 : g.BN));
     if (c->trace) trace_begin(c, label("crt-gemm "));
-    const long nt = tilesMs * g.tilesN * kMods * g.nsplit;
+    const long nt = tilesMs * g.tilesN * kPlanes * g.nsplit;
     if (pair) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(2 * std::min<long>(nt, slots)));
@@ -945,13 +1121,33 @@ static dcsd_status crt_pass(Ctx* c, const char* spec, const GemmPlan& p, const d
     a.C = Cp;
     a.alpha = alpha;
     a.beta = beta;
+    a.flags = flags;
+    a.tilesM = (M + 15) / 16;
     if (c->trace) trace_begin(c, label("crt-out "));
     dim3 grid((unsigned)((M + 127) / 128), (unsigned)std::min<long>(N4, 65535));
     if (g.nsplit > 1) k_crt_out<true><<<grid, 128, 0, c->stream>>>(a);
     else k_crt_out<false><<<grid, 128, 0, c->stream>>>(a);
     trace_end(c);
+    DCSD_TRY(launch_check(c, "crt_out"));
+    // the residues of A are not needed any more: pieces of the patch's sums
+    PatchArgs q;
+    q.flags = flags;
+    q.count = flags + ptiles;
+    q.ntiles = ptiles;
+    q.nsplit = 1;
+    q.ws = (double*)o[0].dst;
+    if (ptiles < 2l * c->num_sms) {
+        const long room = (long)((size_t)kPlanes * g.nkb * 64 * M * 2 / (2048ul * ptiles));
+        q.nsplit = (int)std::max<long>(1, std::min<long>({(2l * c->num_sms + ptiles - 1) / ptiles, K / 256, room}));
+    }
+    q.kchunk = up((K + q.nsplit - 1) / q.nsplit, 32);
+    q.nsplit = (int)((K + q.kchunk - 1) / q.kchunk);
+    if (c->trace) trace_begin(c, label("crt-patch "));
+    k_crt_patch<<<dim3((unsigned)std::min<long>(ptiles, 6l * c->num_sms), (unsigned)q.nsplit), 256, 0, c->stream>>>(
+        o[0], o[1], a, q);
+    trace_end(c);
     prof_end(c, DCSD_PROF_FP64);
-    return launch_check(c, "crt_out");
+    return launch_check(c, "crt_patch");
 }
 
 // C = alpha A B + beta C on the modular GEMM (NB = 1, crt_ready)

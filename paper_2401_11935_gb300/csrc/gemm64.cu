@@ -635,10 +635,14 @@ void record_einsum(Ctx* c, const char* spec, double alpha, const TV& A, const TV
 }
 
 // Whether an FP64 contraction goes to the modular GEMMs of the tensor cores:
-// a time model in microseconds of both.  Measured CUDA cores / modular:
-// (108, 484, 484) 66 / 62, (243, 55, 3025) 97 / 83, (495, 495, 131) 73 / 55,
-// (495, 495, 495) 240 / 62, (17568, 122, 12) 67 / 110, (132, 132, 132) 19 / 46,
-// (122, 12, 43920) 251 / 175.
+// a time model in microseconds of both, launches one by one.  Measured CUDA
+// cores / modular: (108, 484, 484) 63 / 46, (243, 55, 3025) 96 / 59,
+// (495, 495, 131) 71 / 47, (495, 495, 495) 239 / 53, (17568, 122, 12) 68 / 111,
+// (132, 132, 132) 17 / 40, (122, 12, 43920) 248 / 180, (60, 3000, 60) 29 / 45,
+// (1464, 1464, 1464) 5184 / 203, (2196, 14884, 360) 19200 / 983.  The model is
+// up to a third low on either side and decides all of these rightly; it misses
+// near the line only: (64, 64, 4096) 55 / 54, (256, 256, 256) 43 / 44,
+// (2000, 200, 50) 47 / 52.
 static bool crt_pays(const Ctx* c, const GemmPlan& p) {
     if (!crt_ready(c) || p.NB != 1) return false;
     const double M = (double)p.M, N = (double)p.N, K = (double)p.K;
@@ -646,9 +650,9 @@ static bool crt_pays(const Ctx* c, const GemmPlan& p) {
     // CUDA cores: the tiles' products at the FP64 rate
     const double T = up(M, 16) * up(N, 16) / 256 >= 2.0 * c->num_sms ? 16 : 8;
     const double simt = 8.0 + 2.0 * up(M, T) * up(N, T) * K / 1.2e6;
-    // modular: four launches, residues of the operands, waves of tiles, output
+    // modular: five launches, residues of the operands, waves of tiles over 17 planes, output
     const double tn = std::ceil(N / 256), bn = up(N / tn, 16), kb = std::ceil(K / 64);
-    const double waves = std::ceil(up(M, 128) / 128 * tn * 15 / c->num_sms);
+    const double waves = std::ceil(up(M, 128) / 128 * tn * 17 / c->num_sms);
     const double crt = 30.0 + (M + N) * K / 1.2e5 + std::max(waves, 0.5) * (kb * 0.5 * bn / 256 + 1.5) + M * N / 1.1e5;
     return crt < simt;
 }

@@ -137,3 +137,86 @@ def test_strided_views(ctx, engine, spec, sa, sb, sc, perm):
     assert np.abs(C.cpu().numpy() - ref).max() < 1e-12
     C.fill_(7.0)
     assert (big == 7.0).all()
+
+
+# What follows grades the elements along k: |a| |b| is then far above
+# S = sum |a_k b_k|, and an error relative to the norms would be a loss of
+# accuracy against the FMA chain.  Bound for every engine, in u = 2^-53: the
+# chain's K u S.  The modular engine keeps a result only where S is at least
+# 2^-7 in the units of its integers (2^-62 and 2^-61 of the norms' bounds, at
+# least half of which the norms are): sqrt(K) / 2 (2^-62 + 2^-61) <= 0.375 sqrt(K) u S.
+
+
+def _graded(rng, shape, decades):
+    return rng.normal(size=shape) * 10.0 ** (-decades * np.arange(shape[1]) / max(1, shape[1] - 1))
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 1, 2), (17, 15, 33), (64, 64, 484), (130, 257, 31), (129, 33, 1025), (12, 12, 5000),
+                                   (40, 300, 1024), (300, 530, 200)])
+@pytest.mark.parametrize("decades", [4, 8, 30])
+@pytest.mark.parametrize("engine", [0, 1, 2])
+def test_rows_graded_along_k(ctx, M, N, K, decades, engine):
+    rng = np.random.default_rng(M + 5 * N + 11 * K + decades)
+    a, b = _graded(rng, (M, K), decades), _graded(rng, (N, K), decades)[:, ::-1].copy()
+    for alpha, beta in ((1.0, 0.0), (-0.5, 1.0)):
+        c0 = rng.normal(size=(M, N)) if beta else np.full((M, N), np.nan)
+        ref = np.longdouble(alpha) * _exact(a, b) + (np.longdouble(beta) * c0 if beta else 0)
+        err = np.abs(_run(ctx, engine, a, b, alpha, beta, c0) - ref)
+        assert (err <= _bounds(a, b, alpha, c0 if beta else np.zeros((M, N)), beta)[1]).all()
+
+
+@pytest.mark.parametrize("spec", ["mk,nk->mn", "km,nk->nm", "mk,kn->mn"])
+def test_some_graded_rows_among_others(ctx, spec):
+    """A few graded rows, rows and columns of zeros, products that are all zero:
+    the elements computed again stand between others of their tiles."""
+    rng = np.random.default_rng(17)
+    M, N, K = 147, 290, 700
+    a, b = rng.normal(size=(M, K)), rng.normal(size=(N, K))
+    a[[0, 31, 100, 146]] = _graded(rng, (4, K), 12)
+    b[[5, 256, 289]] = _graded(rng, (3, K), 12)[:, ::-1]
+    a[7] = 0.0
+    b[44] = 0.0
+    a[20, ::2] = 0.0
+    b[21, 1::2] = 0.0
+    sa, rest = spec.split(",")
+    sb, sc = rest.split("->")
+    A, B = (a if sa == "mk" else a.T.copy()), (b if sb == "nk" else b.T.copy())
+    c = _run(ctx, 2, A, B, 1.0, 0.0, np.full((M, N) if sc == "mn" else (N, M), np.nan), spec)
+    c = c if sc == "mn" else c.T
+    assert (np.abs(c - _exact(a, b)) <= _bounds(a, b, 1.0, np.zeros((M, N)), 0.0)[1]).all()
+    assert (c[7] == 0).all() and (c[:, 44] == 0).all() and c[20, 21] == 0.0
+
+
+def test_small_products_beside_large_elements(ctx):
+    a, b = np.array([[1e9, 1e-9], [1.0, 1e-16]]), np.array([[0.0, 1.0], [1e-300, 1e-16]])
+    for engine in (0, 1, 2):
+        c = _run(ctx, engine, a, b, 1.0, 0.0, np.zeros((2, 2)))
+        assert c[0, 0] == 1e-9 and c[1, 0] == 1e-16
+        assert abs(c[0, 1] - 1e-25) <= 1e-40 and abs(c[1, 1] - 1e-32) <= 1e-47
+
+
+def test_infinities_as_in_a_chain(ctx):
+    rng = np.random.default_rng(2)
+    a, b = np.abs(rng.normal(size=(40, 90))), np.abs(rng.normal(size=(50, 90)))
+    a[3, 5], a[33, 8], b[17, 5], b[18, 0] = np.inf, -np.inf, 0.0, np.nan
+    with np.errstate(invalid="ignore"):
+        ref = a @ b.T
+    for engine in (0, 1, 2):
+        c = _run(ctx, engine, a, b, 1.0, 0.0, np.zeros((40, 50)))
+        assert (np.isnan(c) == np.isnan(ref)).all() and (np.isposinf(c) == np.isposinf(ref)).all()
+        assert (np.isneginf(c) == np.isneginf(ref)).all()
+        ok = np.isfinite(ref)
+        assert np.abs(c - ref)[ok].max() < 1e-11
+
+
+@pytest.mark.parametrize("K", [64, 1024])
+def test_modular_sums_at_the_integers_bounds(ctx, K):
+    """Elements that are integers of the modular engine as they stand (the
+    norms sqrt(K) 2^(61 - log2(K) / 2) and half of it are their bounds), with
+    residues 128 modulo 256: FP32 sums of 2^24 and results of 2^122."""
+    e = 61 - int(np.log2(K)) // 2
+    for sa, sb in ((1, 1), (-1, 1), (-1, -1)):
+        va, vb = sa * (2 ** e + 128), sb * (2 ** (e - 1) + 128)
+        assert float(va) == va and float(vb) == vb
+        c = _run(ctx, 2, np.full((130, K), float(va)), np.full((24, K), float(vb)), 1.0, 0.0, np.zeros((130, 24)))
+        assert (c == float(va * vb * K)).all()
