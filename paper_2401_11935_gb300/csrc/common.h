@@ -187,8 +187,9 @@ struct Ctx {
     int t2img_planes = 0;
     double* hostbuf = nullptr;    // pinned host staging for scalars
     int ladder_chunk = 8;         // virtual rows per V build chunk (FP64)
-    // tensor-core GEMMs on pairs of SMs (DCSD_TC_MULTICAST=0 selects the
-    // one-CTA kernel)
+    // tensor-core GEMMs, the modular ones too, on pairs of SMs
+    // (DCSD_TC_MULTICAST=0, a name from an earlier form, selects the one-CTA
+    // kernels; both give identical results)
     bool tc_pairs = true;
     // operand packs: the tiled FP64 kernel only, without the t2 image and the
     // row kernel (DCSD_PACK_GENERIC=1; both give identical operands)

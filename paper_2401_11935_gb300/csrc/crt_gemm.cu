@@ -994,7 +994,7 @@ static dcsd_status crt_pass(Ctx* c, const char* spec, const GemmPlan& p, const d
     g.nkb = (int)((K + 63) / 64);
     g.tilesM = (int)((M + CG_BM - 1) / CG_BM);
     g.tilesN = (int)((N + 255) / 256);
-    const bool pair = e->clusters > 0 && g.tilesM > 1;
+    const bool pair = c->tc_pairs && e->clusters > 0 && g.tilesM > 1;
     g.BN = (int)up((N + g.tilesN - 1) / g.tilesN, pair ? 32 : 16);
     const long tilesMs = pair ? (g.tilesM + 1) / 2 : g.tilesM;
     const long slots = pair ? e->clusters : c->num_sms;
@@ -1088,7 +1088,7 @@ static dcsd_status crt_pass(Ctx* c, const char* spec, const GemmPlan& p, const d
     CUtensorMap ma, mb;
     DCSD_TRY(make_map(c, &ma, o[0].dst, M, (long)kPlanes * g.nkb, CG_BM));
     DCSD_TRY(make_map(c, &mb, o[1].dst, N, (long)kPlanes * g.nkb, pair ? g.BN / 2 : g.BN));
-    if (c->trace) trace_begin(c, label("crt-gemm "));
+    if (c->trace) trace_begin(c, label(pair ? "crt-gemm-pairs " : "crt-gemm "));
     const long nt = tilesMs * g.tilesN * kPlanes * g.nsplit;
     if (pair) {
         cudaLaunchConfig_t cfg = {};
