@@ -159,10 +159,13 @@ typedef struct {
  * pointers).  Everything else a call may need -- the tensor-core operand
  * buffers and FP32 accumulator of the BF16* precisions, the DIIS history
  * of dcsd_solve, the defect vector of the MIXED solve, the staging buffers
- * of host-memory (mem_kind HOST) calls -- is allocated by dcsd_reserve
+ * of host-memory (mem_kind HOST) calls, the workspace of FP64 contractions
+ * on the tensor cores (at most 2 GB) -- is allocated by dcsd_reserve
  * ahead of time, or else by the first call that needs it (grow-only, kept
- * until dcsd_destroy).  dcsd_vjp and dcsd_lambda allocate their recorded
- * intermediates for the duration of the call.
+ * until dcsd_destroy; the workspace, without which those contractions run
+ * on the CUDA cores, is given back when another allocation finds no room).
+ * dcsd_vjp and dcsd_lambda allocate their recorded intermediates for the
+ * duration of the call.
  * Errors: INVALID_ARG (sizes < bounds, NULL pointers), OOM, CUDA, NO_DEVICE. */
 dcsd_status dcsd_init(dcsd_ctx** out, const dcsd_dims* d, const double* eps,
                       const double* fock_a, const double* fock_b,

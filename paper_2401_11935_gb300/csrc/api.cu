@@ -208,7 +208,7 @@ long abi_len(const Ctx* c, int k) {
 }
 
 dcsd_status alloc(Ctx* c, double** p, size_t n) {
-    if (cudaMalloc((void**)p, std::max<size_t>(n, 1) * sizeof(double)) != cudaSuccess) {
+    if (dev_malloc(c, (void**)p, std::max<size_t>(n, 1) * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         c->err = "cudaMalloc of " + std::to_string(n * sizeof(double)) + " bytes failed";
         return DCSD_ERR_OOM;
@@ -406,8 +406,16 @@ extern "C" dcsd_status dcsd_init(dcsd_ctx** out, const dcsd_dims* d, const doubl
     A_(c->Wo, O * O * O * O);
     A_(c->Foc, 2 * O * O);
     A_(c->Fvi, 2 * V * V);
-    A_(c->big0, c->lad_elems);
-    A_(c->big1, c->lad_elems);
+    if (cudaMalloc((void**)&c->big0, c->lad_elems * sizeof(double)) != cudaSuccess ||
+        cudaMalloc((void**)&c->big1, c->lad_elems * sizeof(double)) != cudaSuccess) {
+        // no room for the larger chunks
+        cudaGetLastError();
+        if (c->big0) cudaFree(c->big0);
+        c->big0 = c->big1 = nullptr;
+        c->lad_elems = c->big_elems;
+        A_(c->big0, c->lad_elems);
+        A_(c->big1, c->lad_elems);
+    }
     A_(c->big2, c->big_elems);
     A_(c->big3, c->big_elems);
     A_(c->red, kRedDoubles);
@@ -420,8 +428,12 @@ extern "C" dcsd_status dcsd_init(dcsd_ctx** out, const dcsd_dims* d, const doubl
         const size_t pool = 2 * X * n * n + 10 * X * OV + 2 * X * n * O + 16 * n * n + 16 * OV * OV + 7 * O * O * O * V +
                             6 * O * O * O * O + V * V * V * V + O * V * V * V + 2 * V * V + 8 * OV + 4096;
         if (pool <= (size_t)1 << 25) {
-            A_(c->pool, pool);
-            c->pool_elems = pool;
+            if (cudaMalloc((void**)&c->pool, pool * sizeof(double)) == cudaSuccess) {
+                c->pool_elems = pool;
+            } else {  // (they then share the buffers above)
+                cudaGetLastError();
+                c->pool = nullptr;
+            }
         }
     }
     double* counters = nullptr;
@@ -592,6 +604,7 @@ extern "C" dcsd_status dcsd_reserve(dcsd_ctx* h, int precision, int diis_n, int 
     if (host_staging) DCSD_TRY(ensure_abi(c));
     if (diis_n > 0) DCSD_TRY(ensure_diis(c, diis_n, len));
     else DCSD_TRY(ensure_jacobi(c, len));
+    crt_ready(c);  // (optional)
     int runs[2] = {-1, -1};
     if (precision == DCSD_PREC_MIXED) {
         runs[0] = DCSD_PREC_BF16;

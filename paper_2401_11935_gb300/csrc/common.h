@@ -460,11 +460,16 @@ void record_einsum(Ctx* c, const char* spec, double alpha, const TV& A, const TV
                    int engine, int nsplit);
 
 // FP64 contractions by modular GEMMs on the tensor cores (crt_gemm.cu):
-// the engine's workspace is allocated by crt_init; crt_ready tells whether
-// it could be had.  einsum_crt takes unbatched plans (NB = 1).
+// crt_ready allocates the engine's workspace when it is first asked and tells
+// whether it could be had.  einsum_crt takes unbatched plans (NB = 1).
 dcsd_status crt_init(Ctx* c);
 void crt_free(Ctx* c);
-bool crt_ready(const Ctx* c);
+bool crt_ready(Ctx* c);
+const void* crt_workspace(const Ctx* c);
+// cudaMalloc for everything a call cannot do without: where the device has no
+// room left, the modular GEMMs' workspace is given back first (their
+// contractions then stay on the CUDA cores, for the life of the context)
+cudaError_t dev_malloc(Ctx* c, void** p, size_t bytes);
 dcsd_status einsum_crt(Ctx* c, const char* spec, const GemmPlan& plan, const double* A, const double* B, double* C,
                        double alpha, double beta);
 

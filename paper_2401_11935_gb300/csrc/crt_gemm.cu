@@ -899,15 +899,18 @@ __global__ void __launch_bounds__(256) k_crt_patch(const Operand oa, const Opera
 // ---------------------------------------------------------------------------
 struct CrtEngine {
     PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-    uint8_t* ws = nullptr;  // workspace, allocated at initialisation
-    size_t bytes = 0;
+    uint8_t* ws = nullptr;  // workspace, allocated by the first contraction that pays
+    size_t bytes = 0, want = 0;
+    bool refused = false;   // it could not be allocated, or was given back
     int clusters = 0;       // resident two-CTA clusters (-1: none)
 };
 
 static long up(long x, long m) { return (x + m - 1) / m * m; }
 
 // Workspace: every contraction's operands, residues and outputs whole up to
-// 2 GB (larger ones run in pieces), at least 32 MB.
+// 2 GB (larger ones run in pieces), at least 32 MB.  It is optional: a context
+// whose calls stay in BF16 never has it, and without it every contraction
+// stays on the CUDA cores.
 dcsd_status crt_init(Ctx* c) {
     CrtEngine* e = new CrtEngine();
     c->crt = e;
@@ -921,13 +924,7 @@ dcsd_status crt_init(Ctx* c) {
     e->encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
     const double V = c->V, OV = (double)c->O * c->V, rows = 4.0 * c->O * c->O;
     const double want = 2.0 * kPlanes * 2.0 * ((V * V + rows) * (V * V + 64) + 2 * OV * (OV + 64)) + kPlanes * OV * OV;
-    e->bytes = (size_t)std::min(2147483648.0, std::max(33554432.0, want)) / 1024 * 1024;
-    if (cudaMalloc((void**)&e->ws, e->bytes) != cudaSuccess) {
-        // without it every contraction stays on the CUDA cores
-        cudaGetLastError();
-        e->ws = nullptr;
-        e->bytes = 0;
-    }
+    e->want = (size_t)std::min(2147483648.0, std::max(33554432.0, want)) / 1024 * 1024;
     DCSD_CUDA(c, cudaFuncSetAttribute(k_crt_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCrtSmem));
     DCSD_CUDA(c, cudaFuncSetAttribute(k_crt_gemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCrtSmem));
     cudaLaunchConfig_t cfg = {};
@@ -970,7 +967,34 @@ static dcsd_status make_map(Ctx* c, CUtensorMap* map, const uint16_t* p, long ro
     return DCSD_OK;
 }
 
-bool crt_ready(const Ctx* c) { return c->crt && c->crt->ws; }
+bool crt_ready(Ctx* c) {
+    CrtEngine* e = c->crt;
+    if (!e) return false;
+    if (!e->ws && !e->refused && !c->dag) {  // (nothing can be allocated while launches are recorded)
+        if (cudaMalloc((void**)&e->ws, e->want) == cudaSuccess) {
+            e->bytes = e->want;
+        } else {
+            cudaGetLastError();
+            e->ws = nullptr;
+            e->refused = true;
+        }
+    }
+    return e->ws != nullptr;
+}
+
+const void* crt_workspace(const Ctx* c) { return c->crt ? c->crt->ws : nullptr; }
+
+cudaError_t dev_malloc(Ctx* c, void** p, size_t bytes) {
+    cudaError_t st = cudaMalloc(p, bytes);
+    CrtEngine* e = c->crt;
+    if (st != cudaErrorMemoryAllocation || !e || !e->ws) return st;
+    cudaGetLastError();
+    cudaFree(e->ws);  // (waits for the launches that use it)
+    e->ws = nullptr;
+    e->bytes = 0;
+    e->refused = true;
+    return cudaMalloc(p, bytes);
+}
 
 // k per partial norm: a multiple of 128, at most 32 pieces
 static int norm_chunk(long K) { return (int)std::max<long>(128, up((K + 31) / 32, 128)); }

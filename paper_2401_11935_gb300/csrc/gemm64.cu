@@ -643,8 +643,8 @@ void record_einsum(Ctx* c, const char* spec, double alpha, const TV& A, const TV
 // up to a third low on either side and decides all of these rightly; it misses
 // near the line only: (64, 64, 4096) 55 / 54, (256, 256, 256) 43 / 44,
 // (2000, 200, 50) 47 / 52.
-static bool crt_pays(const Ctx* c, const GemmPlan& p) {
-    if (!crt_ready(c) || p.NB != 1) return false;
+static bool crt_pays(Ctx* c, const GemmPlan& p) {
+    if (p.NB != 1) return false;
     const double M = (double)p.M, N = (double)p.N, K = (double)p.K;
     auto up = [](double x, double m) { return std::ceil(x / m) * m; };
     // CUDA cores: the tiles' products at the FP64 rate
@@ -654,7 +654,7 @@ static bool crt_pays(const Ctx* c, const GemmPlan& p) {
     const double tn = std::ceil(N / 256), bn = up(N / tn, 16), kb = std::ceil(K / 64);
     const double waves = std::ceil(up(M, 128) / 128 * tn * 17 / c->num_sms);
     const double crt = 30.0 + (M + N) * K / 1.2e5 + std::max(waves, 0.5) * (kb * 0.5 * bn / 256 + 1.5) + M * N / 1.1e5;
-    return crt < simt;
+    return crt < simt && crt_ready(c);
 }
 
 // engine: 0 chosen by size, 1 CUDA cores, 2 modular GEMM (FP64)

@@ -168,7 +168,7 @@ dcsd_status coupling_w(Ctx* c, int ref) {
 
 dcsd_status set_vvvv(Ctx* c, const double* host_vvvv) {
     const size_t V = c->V, nv4 = V * V * V * V;
-    if (!c->vvvv && cudaMalloc((void**)&c->vvvv, nv4 * sizeof(double)) != cudaSuccess) {
+    if (!c->vvvv && dev_malloc(c, (void**)&c->vvvv, nv4 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         c->vvvv = nullptr;
         c->err = "cudaMalloc of the stored (ac|bd) integrals failed";
@@ -414,7 +414,7 @@ dcsd_status residual_union(Ctx* c, int ref, int method, int prec) {
     } r2f_guard{c};
     if (fast) {
         if (!c->r2f) {
-            if (cudaMalloc((void**)&c->r2f, sizeof(float) * 3 * O * O * V * V) != cudaSuccess) {
+            if (dev_malloc(c, (void**)&c->r2f, sizeof(float) * 3 * O * O * V * V) != cudaSuccess) {
                 cudaGetLastError();
                 c->r2f = nullptr;
                 c->err = "cudaMalloc of the FP32 residual accumulator failed";
@@ -639,7 +639,7 @@ dcsd_status graph_run(Ctx* c, int key, const std::function<dcsd_status()>& body)
         tc_state(c, s);
         for (const void* p : {(const void*)c->r2f, (const void*)c->t2img, (const void*)c->vvvv,
                               (const void*)c->pack_cache_src[0], (const void*)c->pack_cache_src[1], (const void*)c->vbuf,
-                              (const void*)c->pairbuf})
+                              (const void*)c->pairbuf, crt_workspace(c)})
             s.push_back((uint64_t)(uintptr_t)p);
         for (const auto& b : c->arena) s.push_back((uint64_t)(uintptr_t)b.fwd);
         return s;

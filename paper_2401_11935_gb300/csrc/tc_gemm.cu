@@ -1729,7 +1729,7 @@ static dcsd_status ensure(Ctx* c, Buf& b, size_t elems) {
     if (b.p) cudaFree(b.p);
     b.p = nullptr;
     b.cap = 0;
-    if (cudaMalloc((void**)&b.p, elems * sizeof(__nv_bfloat16)) != cudaSuccess) {
+    if (dev_malloc(c, (void**)&b.p, elems * sizeof(__nv_bfloat16)) != cudaSuccess) {
         cudaGetLastError();
         c->err = "cudaMalloc of BF16 operand buffer failed";
         return DCSD_ERR_OOM;
@@ -2112,7 +2112,7 @@ static dcsd_status ensure_wsk(Ctx* c, size_t wsn) {
         if (e->wsk) cudaFree(e->wsk);
         e->wsk = nullptr;
         e->wsk_cap = 0;
-        DCSD_CUDA(c, cudaMalloc((void**)&e->wsk, wsn * sizeof(float)));
+        DCSD_CUDA(c, dev_malloc(c, (void**)&e->wsk, wsn * sizeof(float)));
         e->wsk_cap = wsn;
     }
     return DCSD_OK;
@@ -2273,7 +2273,7 @@ dcsd_status t2_image(Ctx* c, int nsplit) {
         if (c->t2img) cudaFree(c->t2img);
         c->t2img = nullptr;
         c->t2img_cap = 0;
-        DCSD_CUDA(c, cudaMalloc((void**)&c->t2img, need * sizeof(uint16_t)));
+        DCSD_CUDA(c, dev_malloc(c, (void**)&c->t2img, need * sizeof(uint16_t)));
         c->t2img_cap = need;
     }
     if (c->trace) trace_begin(c, "t2 image planes=" + std::to_string(np));
@@ -2642,7 +2642,7 @@ static dcsd_status ladder_sa_pass(Ctx* c, int nsplit, double* R2, double* G) {
         e->d_code_m = nullptr;
         e->sa_O = -1;
         if (P > 0) {
-            DCSD_CUDA(c, cudaMalloc((void**)&e->d_code_m, sizeof(int) * cm.size()));
+            DCSD_CUDA(c, dev_malloc(c, (void**)&e->d_code_m, sizeof(int) * cm.size()));
             DCSD_CUDA(c, cudaMemcpy(e->d_code_m, cm.data(), sizeof(int) * cm.size(), cudaMemcpyHostToDevice));
         }
         e->sa_O = O;
@@ -2874,9 +2874,9 @@ dcsd_status ladder_tc(Ctx* c, int nsplit, double* R2, double* G) {
             if (*pp) { cudaFree(*pp); *pp = nullptr; }
         if (e->d_rowcode) { cudaFree(e->d_rowcode); e->d_rowcode = nullptr; }
         e->tab_O = e->tab_V = -1;
-        DCSD_CUDA(c, cudaMalloc((void**)&e->d_pairoff, sizeof(long) * pairoff.size()));
-        DCSD_CUDA(c, cudaMalloc((void**)&e->d_growoff, sizeof(long) * rows4));
-        DCSD_CUDA(c, cudaMalloc((void**)&e->d_rowcode, sizeof(int) * rows4));
+        DCSD_CUDA(c, dev_malloc(c, (void**)&e->d_pairoff, sizeof(long) * pairoff.size()));
+        DCSD_CUDA(c, dev_malloc(c, (void**)&e->d_growoff, sizeof(long) * rows4));
+        DCSD_CUDA(c, dev_malloc(c, (void**)&e->d_rowcode, sizeof(int) * rows4));
         DCSD_CUDA(c, cudaMemcpy(e->d_pairoff, pairoff.data(), sizeof(long) * pairoff.size(), cudaMemcpyHostToDevice));
         DCSD_CUDA(c, cudaMemcpy(e->d_growoff, growoff.data(), sizeof(long) * rows4, cudaMemcpyHostToDevice));
         DCSD_CUDA(c, cudaMemcpy(e->d_rowcode, code.data(), sizeof(int) * rows4, cudaMemcpyHostToDevice));

@@ -46,8 +46,8 @@ double* scratch(Ctx* c, double* normal, size_t elems) {
         }
     ArenaBlock nb;
     nb.cap = std::max(need, (size_t)32 << 20);
-    if (cudaMalloc((void**)&nb.fwd, nb.cap * sizeof(double)) != cudaSuccess ||
-        cudaMalloc((void**)&nb.adj, nb.cap * sizeof(double)) != cudaSuccess ||
+    if (dev_malloc(c, (void**)&nb.fwd, nb.cap * sizeof(double)) != cudaSuccess ||
+        dev_malloc(c, (void**)&nb.adj, nb.cap * sizeof(double)) != cudaSuccess ||
         cudaMemsetAsync(nb.adj, 0, nb.cap * sizeof(double), c->stream) != cudaSuccess) {
         cudaGetLastError();
         if (nb.fwd) cudaFree(nb.fwd);
@@ -348,7 +348,7 @@ static bool ladder_reverse_pairs(Ctx* c, const TapeOp& op, const TV& R2b, bool w
         if (c->pairbuf) cudaFree(c->pairbuf);
         c->pairbuf = nullptr;
         c->pairbuf_elems = 0;
-        if (cudaMalloc((void**)&c->pairbuf, need * sizeof(double)) != cudaSuccess) {
+        if (dev_malloc(c, (void**)&c->pairbuf, need * sizeof(double)) != cudaSuccess) {
             cudaGetLastError();
             return false;
         }
@@ -659,7 +659,7 @@ static dcsd_status vjp_buffers(Ctx* c) {
         if (c->vbuf) cudaFree(c->vbuf);
         c->vbuf = nullptr;
         c->vbuf_elems = 0;
-        if (cudaMalloc((void**)&c->vbuf, need * sizeof(double)) != cudaSuccess) {
+        if (dev_malloc(c, (void**)&c->vbuf, need * sizeof(double)) != cudaSuccess) {
             cudaGetLastError();
             c->err = "reverse mode: cudaMalloc of the adjoint buffers failed";
             return DCSD_ERR_OOM;

@@ -163,3 +163,59 @@ def test_autograd_gives_B_and_fock_gradients(P, method):
     with pytest.raises(ValueError):
         eng.residual_autograd(Tt, inputs=(fa.detach().clone(), fb, Bt))
     eng.close()
+
+
+def _used(f):
+    import torch
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    x = f()
+    torch.cuda.synchronize()
+    return x, before - torch.cuda.mem_get_info()[0]
+
+
+def test_modular_workspace_only_where_fp64_uses_it(P):
+    """At (4, 100, 60) the workspace is 2 GB (15 bytes V^4 and more): a context
+    that evaluates BF16 residuals has none, the first FP64 residual takes it."""
+    from synth import random_amplitudes
+    s = make_system((4, 100, 60), seed=5)
+    T = random_amplitudes(s, seed=6, scale1=0.02, scale2=0.02)
+    eng, init = _used(lambda: P.Engine.from_system(s))
+    Td = eng.to_device(T)
+    R, bf16 = _used(lambda: eng.residual(Td, precision=P.PREC_BF16))
+    R, fp64 = _used(lambda: eng.residual(Td, precision=P.PREC_FP64))
+    eng.close()
+    assert fp64 >= 2 ** 31 - 2 ** 20 and init + bf16 < 2 ** 31, (init, bf16, fp64)
+
+
+def test_modular_workspace_is_given_back(P):
+    """With 300 MB of the device left, the DIIS history of a solve (0.8 GB) takes the
+    place of the workspace; recorded residuals that used it are not replayed."""
+    import torch
+    from synth import random_amplitudes
+    s = make_system((10, 120, 60), seed=5)
+    T = random_amplitudes(s, seed=6, scale1=0.02, scale2=0.02)
+    eng = P.Engine.from_system(s)
+    Td = eng.to_device(T)
+    first = None
+    for _ in range(3):
+        R, W, dE = eng.residual(Td, precision=P.PREC_FP64)
+        R = [x.cpu().numpy() for x in R]
+        first = first or R
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - 300 * 2 ** 20, dtype=torch.uint8, device="cuda")
+    try:
+        from paper_2401_11935_gb300 import _lib as L
+        Ts = eng.to_device(T)
+        opts = L.dcsd_solve_opts(1, 0, 0, 1, 8, 1e-12, 1e-5, 1, 0.0)
+        L.dcsd_solve(eng.ctx, opts, L.MEM_DEVICE, [x.data_ptr() for x in Ts])
+        del Ts
+        for _ in range(3):
+            R, W, dE = eng.residual(Td, precision=P.PREC_FP64)
+            for x, y in zip(R, first):  # (another engine: a few hundred roundings of 2^-53)
+                assert np.linalg.norm(x.cpu().numpy() - y) <= 1e-13 * max(1.0, np.linalg.norm(y))
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    eng.close()
