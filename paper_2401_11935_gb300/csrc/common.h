@@ -110,6 +110,7 @@ struct AdjRegion {
 
 struct CrtEngine;
 constexpr long kGemm64Counters = 4096;
+constexpr int kGraphAttempts = 4;  // recordings of one argument set that may fail
 
 // Memory that a launch reads or writes, for the dependencies of recorded launches
 struct Span {
@@ -204,10 +205,10 @@ struct Ctx {
         cudaGraphExec_t exec = nullptr;
         std::vector<uint64_t> state;  // what the recorded launches depend on
         long long launches = 0;
+        int failures = 0;             // recordings that failed since the state changed
     };
     std::vector<Graph> graphs;
     cudaStream_t capture = nullptr;   // recording stream (the user's may be the legacy stream)
-    bool graphs_off = false;          // a recording failed: launches one by one
     Dag* dag = nullptr;               // set while recording (see DagOp)
     // intermediates of one residual in buffers of their own, taken one after
     // the other, so that independent launches do not wait for a shared buffer

@@ -632,67 +632,74 @@ dcsd_status residual_union(Ctx* c, int ref, int method, int prec) {
 // serves every later call with the same arguments as long as those buffers and
 // the packed operands kept in them are the same (state).  The first evaluation
 // runs launch by launch (it allocates), the second is recorded.
-dcsd_status graph_run(Ctx* c, int key, const std::function<dcsd_status()>& body) {
-    if (c->graphs_off || c->rec || c->trace || c->prof_on) return body();
-    auto state = [&]() {
-        std::vector<uint64_t> s;
-        tc_state(c, s);
-        for (const void* p : {(const void*)c->r2f, (const void*)c->t2img, (const void*)c->vvvv,
-                              (const void*)c->pack_cache_src[0], (const void*)c->pack_cache_src[1], (const void*)c->vbuf,
-                              (const void*)c->pairbuf, crt_workspace(c)})
-            s.push_back((uint64_t)(uintptr_t)p);
-        for (const auto& b : c->arena) s.push_back((uint64_t)(uintptr_t)b.fwd);
-        return s;
-    };
-    Ctx::Graph* g = nullptr;
-    for (auto& x : c->graphs)
-        if (x.key == key) g = &x;
-    if (!g) {
-        c->graphs.emplace_back();
-        g = &c->graphs.back();
-        g->key = key;
+static std::vector<uint64_t> graph_state(const Ctx* c) {
+    std::vector<uint64_t> s;
+    tc_state(c, s);
+    for (const void* p : {(const void*)c->r2f, (const void*)c->t2img, (const void*)c->vvvv,
+                          (const void*)c->pack_cache_src[0], (const void*)c->pack_cache_src[1], (const void*)c->vbuf,
+                          (const void*)c->pairbuf, crt_workspace(c)})
+        s.push_back((uint64_t)(uintptr_t)p);
+    for (const auto& b : c->arena) s.push_back((uint64_t)(uintptr_t)b.fwd);
+    return s;
+}
+
+static Ctx::Graph& graph_of(Ctx* c, int key) {
+    for (auto& g : c->graphs)
+        if (g.key == key) return g;
+    c->graphs.emplace_back();
+    c->graphs.back().key = key;
+    return c->graphs.back();
+}
+
+// records body's launches, which must not allocate, as g.exec
+static bool graph_record(Ctx* c, Ctx::Graph& g, const std::function<dcsd_status()>& body) {
+    if (!c->capture && cudaStreamCreateWithFlags(&c->capture, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaGetLastError();
+        c->capture = nullptr;
+        return false;
     }
-    if (g->state != state()) {
-        if (g->exec) cudaGraphExecDestroy(g->exec);
-        g->exec = nullptr;
+    const long long l0 = c->launches;
+    const cudaStream_t user = c->stream;
+    cudaGraph_t graph = nullptr;
+    bool ok = cudaStreamBeginCapture(c->capture, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+    if (ok) {
+        Dag dag;
+        c->stream = c->capture;
+        c->dag = &dag;
         const dcsd_status st = body();
-        g->state = st == DCSD_OK ? state() : std::vector<uint64_t>();
+        c->dag = nullptr;
+        c->stream = user;
+        ok = cudaStreamEndCapture(c->capture, &graph) == cudaSuccess && st == DCSD_OK && graph && !dag.failed;
+    }
+    ok = ok && graph_state(c) == g.state && cudaGraphInstantiate(&g.exec, graph, 0) == cudaSuccess;
+    if (graph) cudaGraphDestroy(graph);
+    g.launches = c->launches - l0;
+    c->launches = l0;
+    if (!ok) {
+        cudaGetLastError();
+        g.exec = nullptr;
+        c->err.clear();
+    }
+    return ok;
+}
+
+dcsd_status graph_run(Ctx* c, int key, const std::function<dcsd_status()>& body) {
+    if (c->rec || c->trace || c->prof_on) return body();
+    Ctx::Graph& g = graph_of(c, key);
+    if (g.state != graph_state(c)) {
+        if (g.exec) cudaGraphExecDestroy(g.exec);
+        g.exec = nullptr;
+        g.failures = 0;
+        const dcsd_status st = body();
+        g.state = st == DCSD_OK ? graph_state(c) : std::vector<uint64_t>();
         return st;
     }
-    if (!g->exec) {
-        if (!c->capture && cudaStreamCreateWithFlags(&c->capture, cudaStreamNonBlocking) != cudaSuccess) {
-            cudaGetLastError();
-            c->capture = nullptr;
-            c->graphs_off = true;
-            return body();
-        }
-        const long long l0 = c->launches;
-        const cudaStream_t user = c->stream;
-        cudaGraph_t graph = nullptr;
-        bool ok = cudaStreamBeginCapture(c->capture, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-        if (ok) {
-            Dag dag;
-            c->stream = c->capture;
-            c->dag = &dag;
-            const dcsd_status st = body();
-            c->dag = nullptr;
-            c->stream = user;
-            ok = cudaStreamEndCapture(c->capture, &graph) == cudaSuccess && st == DCSD_OK && graph && !dag.failed;
-        }
-        ok = ok && state() == g->state && cudaGraphInstantiate(&g->exec, graph, 0) == cudaSuccess;
-        if (graph) cudaGraphDestroy(graph);
-        g->launches = c->launches - l0;
-        c->launches = l0;
-        if (!ok) {
-            cudaGetLastError();
-            g->exec = nullptr;
-            c->graphs_off = true;
-            c->err.clear();
-            return body();
-        }
-    }
-    DCSD_CUDA(c, cudaGraphLaunch(g->exec, c->stream));
-    c->launches += g->launches;
+    // (a recording fails where its graph finds no memory: launch by launch
+    // this time, and another attempt at the next calls)
+    if (!g.exec && g.failures < kGraphAttempts && !graph_record(c, g, body)) ++g.failures;
+    if (!g.exec) return body();
+    DCSD_CUDA(c, cudaGraphLaunch(g.exec, c->stream));
+    c->launches += g.launches;
     return DCSD_OK;
 }
 

@@ -67,3 +67,46 @@ def test_ladder_block_edges(P, dims, prec, tol):
     rmax = max(float(np.abs(x).max()) for x in R0[:5])
     # the split's precision, relative to max |R|, as for the full sizes
     assert max(float(np.abs(a - b).max()) for a, b in zip(R[:5], R0[:5])) < tol * rmax
+
+
+def test_recording_without_memory_is_tried_again(P):
+    """No room for the recorded graphs: the calls run launch by launch and are
+    right; with memory free again the following ones are recorded (a graph
+    at this size takes 4 to 8 MB)."""
+    import torch
+    s = make_system((4, 20, 60), seed=11)
+    T = random_amplitudes(s, seed=20, scale1=0.02, scale2=0.02)
+    eng = P.Engine.from_system(s)
+    Td = eng.to_device(T)
+    keys = [(m, r) for m in (0, 1) for r in (0, 1)]
+
+    def run():
+        out = {}
+        for m, r in keys:
+            R, W, dE = eng.residual(Td, ref=r, method=m, precision=0)
+            out[m, r] = [x.cpu().numpy() for x in R] + [np.array([W, dE])]
+        torch.cuda.synchronize()
+        return out
+
+    first = run()  # launch by launch; loads the kernels
+    filler = []
+    try:
+        for size in (2 ** 30, 2 ** 24, 2 ** 21):
+            while True:
+                try:
+                    free = torch.cuda.mem_get_info()[0]
+                    filler.append(torch.empty(max(size, (free - size) // size * size), dtype=torch.uint8, device="cuda"))
+                except torch.OutOfMemoryError:
+                    break
+        full = run()
+    finally:
+        filler.clear()
+        torch.cuda.empty_cache()
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    again = run()
+    assert before - torch.cuda.mem_get_info()[0] >= 2 ** 22
+    for out in (full, again, run()):
+        for k in keys:
+            _same(out[k], first[k], 0)
+    eng.close()
