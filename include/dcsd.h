@@ -182,7 +182,12 @@ dcsd_status dcsd_init(dcsd_ctx** out, const dcsd_dims* d, const double* eps,
  * not released before dcsd_destroy.  The tensor-core buffers are sized by
  * running one CCSD residual at zero amplitudes in each of those precisions
  * (their sizes depend only on the dimensions); the context's amplitude
- * buffers are overwritten.  Synchronises the context stream.  Not part of
+ * buffers are overwritten.  The launches of those residuals are recorded here
+ * as CUDA graphs, too, one for each method and reference (1.5 ms and 2 to
+ * 8 MB of device memory each for 100 to 400 launches, 12 to 60 graphs;
+ * without a reservation the second call of a kind records its own).  A call
+ * of another kind that allocates, such as a reverse sweep, may make the next
+ * residual record again.  Synchronises the context stream.  Not part of
  * the paper's method: memory management of this library.
  * Errors: INVALID_ARG (bad precision, diis_n outside 0..16, host_staging
  * not 0/1), OOM, CUDA, TIMEOUT. */

@@ -620,6 +620,15 @@ extern "C" dcsd_status dcsd_reserve(dcsd_ctx* h, int precision, int diis_n, int 
     }
     DCSD_TRY(sync_scalars(c, 23));
     if (tc_timeout(c)) return DCSD_ERR_TIMEOUT;
+    // every buffer is there: record what residuals, energies and solves launch
+    residual_prepare(c, DCSD_PREC_FP64, false);  // (energies)
+    if (precision == DCSD_PREC_FP64 || precision == DCSD_PREC_MIXED) residual_prepare(c, DCSD_PREC_FP64, true);
+    for (int r : runs) {
+        if (r < 0) continue;
+        residual_prepare(c, r, false);
+        if (r == DCSD_PREC_BF16X6) residual_prepare(c, r, true);
+    }
+    DCSD_CUDA(c, cudaStreamSynchronize(c->stream));
     return DCSD_OK;
 }
 

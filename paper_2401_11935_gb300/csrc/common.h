@@ -110,6 +110,7 @@ struct AdjRegion {
 
 struct CrtEngine;
 constexpr long kGemm64Counters = 4096;
+constexpr size_t kGraphNodes = 4096;  // launches of a recorded graph at most
 constexpr int kGraphAttempts = 4;  // recordings of one argument set that may fail
 
 // Memory that a launch reads or writes, for the dependencies of recorded launches
@@ -415,6 +416,10 @@ dcsd_status residual_union(Ctx* c, int ref, int method, int precision);
 dcsd_status graph_run(Ctx* c, int key, const std::function<dcsd_status()>& body);
 // residual_union through graph_run
 dcsd_status residual_run(Ctx* c, int ref, int method, int precision);
+// records the graphs of residual_run for every method and reference without
+// running them, with the FP64 sums of a residual or of a solve (chain); what
+// the launches need must have been allocated
+void residual_prepare(Ctx* c, int precision, bool chain);
 // reverse mode helpers (vjp.cu)
 // buffer for an intermediate: `normal` outside recording, a fresh arena block
 // (with a zeroed adjoint twin) while recording
@@ -487,6 +492,8 @@ bool tc_same_sums(const Ctx* c, long M, long N, long M2, long N2, long K, int ns
 
 // pp ladder + its T1 correction on tensor cores (R2 += ladder, G = correction)
 dcsd_status ladder_tc(Ctx* c, int nsplit, double* R2, double* G);
+// whether the ladder's operands are packed again for each precision
+bool tc_repacks(const Ctx* c);
 // the engine's buffers and packed-operand states that recorded launches use
 void tc_state(const Ctx* c, std::vector<uint64_t>& s);
 // sources whose packed operands einsum_tc may reuse (NULL: none); clears the cache

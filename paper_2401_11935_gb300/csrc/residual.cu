@@ -671,12 +671,19 @@ static bool graph_record(Ctx* c, Ctx::Graph& g, const std::function<dcsd_status(
         c->stream = user;
         ok = cudaStreamEndCapture(c->capture, &graph) == cudaSuccess && st == DCSD_OK && graph && !dag.failed;
     }
-    ok = ok && graph_state(c) == g.state && cudaGraphInstantiate(&g.exec, graph, 0) == cudaSuccess;
+    // (a graph takes 10 to 30 KB of the device per launch; where there are
+    // thousands of them they are large ones, which gain nothing)
+    size_t nodes = 0;
+    ok = ok && graph_state(c) == g.state && cudaGraphGetNodes(graph, nullptr, &nodes) == cudaSuccess;
+    if (nodes > kGraphNodes) g.failures = kGraphAttempts;
+    ok = ok && nodes <= kGraphNodes && cudaGraphInstantiate(&g.exec, graph, 0) == cudaSuccess &&
+         cudaGraphUpload(g.exec, c->stream) == cudaSuccess;
     if (graph) cudaGraphDestroy(graph);
     g.launches = c->launches - l0;
     c->launches = l0;
     if (!ok) {
         cudaGetLastError();
+        if (g.exec) cudaGraphExecDestroy(g.exec);
         g.exec = nullptr;
         c->err.clear();
     }
@@ -703,9 +710,39 @@ dcsd_status graph_run(Ctx* c, int key, const std::function<dcsd_status()>& body)
     return DCSD_OK;
 }
 
+// (FP64 sums occur in FP64 and BF16X6 only: the order asked for makes no
+// difference to the others)
+static int residual_key(const Ctx* c, int ref, int method, int prec) {
+    const bool chain = c->fma_chain && (prec == DCSD_PREC_FP64 || prec == DCSD_PREC_BF16X6);
+    return ((ref * 8 + method) * 8 + prec) * 2 + (chain ? 1 : 0);
+}
+
+// The classic ladder packs B for one split at a time, so a recording of one
+// precision would not outlive a call of another: there every launch is made
+static bool residual_records(const Ctx* c, int prec) { return prec == DCSD_PREC_FP64 || !tc_repacks(c); }
+
 dcsd_status residual_run(Ctx* c, int ref, int method, int prec) {
-    const int key = ((ref * 8 + method) * 8 + prec) * 2 + (c->fma_chain ? 1 : 0);
-    return graph_run(c, key, [=]() { return residual_union(c, ref, method, prec); });
+    if (!residual_records(c, prec)) return residual_union(c, ref, method, prec);
+    return graph_run(c, residual_key(c, ref, method, prec), [=]() { return residual_union(c, ref, method, prec); });
+}
+
+void residual_prepare(Ctx* c, int prec, bool chain) {
+    if (c->rec || c->trace || c->prof_on || !residual_records(c, prec)) return;
+    const FmaChain order(c, chain);
+    for (int method = DCSD_CCSD; method <= DCSD_FR_DCSD_T; ++method)
+        for (int ref = 0; ref < 2; ++ref) {
+            Ctx::Graph& g = graph_of(c, residual_key(c, ref, method, prec));
+            std::vector<uint64_t> now = graph_state(c);
+            if (g.exec && g.state == now) continue;
+            if (g.exec) cudaGraphExecDestroy(g.exec);
+            g.exec = nullptr;
+            g.failures = 0;
+            g.state = std::move(now);
+            if (!graph_record(c, g, [=]() { return residual_union(c, ref, method, prec); })) {
+                if (g.failures >= kGraphAttempts) return;  // (too many launches)
+                g.failures = kGraphAttempts;               // (no attempt in the middle of a later call)
+            }
+        }
 }
 
 }  // namespace dcsd

@@ -1773,6 +1773,8 @@ void tc_free(Ctx* c) {
     c->tc = nullptr;
 }
 
+bool tc_repacks(const Ctx* c) { return c->tc->pbv_nsplit != 0; }
+
 void tc_state(const Ctx* c, std::vector<uint64_t>& s) {
     const TcEngine* e = c->tc;
     for (const Buf* b : {&e->pa, &e->pb, &e->pv, &e->pt, &e->sam, &e->sap, &e->svp, &e->svm, &e->sx, &e->pbv})

@@ -219,3 +219,64 @@ def test_modular_workspace_is_given_back(P):
         del filler
         torch.cuda.empty_cache()
     eng.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1, 3, 4])
+def test_reserved_contexts_record_nothing_later(P, precision):
+    """After a reservation, repeated residuals of every method and reference,
+    energies and solves leave the device's free memory as it is (a graph
+    recorded by one of them would take 2 to 8 MB)."""
+    import torch
+    from paper_2401_11935_gb300 import _lib as L
+    s = make_system((4, 20, 60), seed=5)
+    precs = [1, 4] if precision == 3 else [precision]
+
+    def work(eng, T, R):
+        t, r = [x.data_ptr() for x in T], [x.data_ptr() for x in R]
+        for _ in range(3):
+            for method in range(6):
+                for ref in (0, 1):
+                    for p in precs:
+                        L.dcsd_residual(eng.ctx, ref, method, p, L.MEM_DEVICE, t, r)
+            L.dcsd_energy(eng.ctx, 0, 1, L.MEM_DEVICE, t)
+            L.dcsd_solve(eng.ctx, L.dcsd_solve_opts(1, 0, precision, 4, 8, 1e-12, 1e-5, 0, 0.0), L.MEM_DEVICE, t)
+        torch.cuda.synchronize()
+
+    e0 = P.Engine.from_system(s)  # (loads the kernels)
+    T, R = _pointers(e0)
+    work(e0, T, R)
+    e0.close()
+    e1 = P.Engine.from_system(s)
+    _, taken = _used(lambda: e1.reserve(precision, diis_n=8))
+    g0 = torch.cuda.mem_get_info()[0]
+    work(e1, T, R)
+    assert torch.cuda.mem_get_info()[0] == g0 and taken >= 12 * 2 ** 20
+    e1.close()
+
+
+def test_reservation_in_a_fresh_process(P):
+    """Recorded before anything has run or been loaded: the graphs give the
+    residuals of a context without a reservation."""
+    import subprocess
+    import sys
+    code = """
+import numpy as np, torch, time
+import paper_2401_11935_gb300 as P
+from synth import make_system, random_amplitudes
+s = make_system((5, 37, 60), seed=11)
+T = [random_amplitudes(s, seed=20, ref=r, scale1=0.02, scale2=0.02) for r in (0, 1)]
+a = P.Engine.from_system(s)
+a.reserve(P.PREC_MIXED, diis_n=4)
+b = P.Engine.from_system(s)
+for prec in (0, 1, 4):
+    for method in range(6):
+        for ref in (0, 1):
+            x, y = (e.residual(e.to_device(T[ref]), ref=ref, method=method, precision=prec) for e in (a, b))
+            for u, v in zip(x[0], y[0]):
+                n = float(torch.linalg.norm(u - v))
+                assert n == 0.0 if prec == 1 else n <= 1e-13 * max(1.0, float(torch.linalg.norm(v))), (prec, method, ref, n)
+            assert abs(x[1] - y[1]) < 1e-13 and abs(x[2] - y[2]) < 1e-13
+print("equal")
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "equal" in r.stdout, r.stderr[-2000:]
