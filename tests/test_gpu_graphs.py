@@ -110,3 +110,47 @@ def test_recording_without_memory_is_tried_again(P):
         for k in keys:
             _same(out[k], first[k], 0)
     eng.close()
+
+
+# (amplitudes, cotangents or None, Ebar, Wbar): every input changes from call to call
+SWEEPS = [(0, 0, 0.3, -0.8), (1, 1, -0.4, 1.1), (0, None, 1.0, 0.0), (1, None, 0.0, 1.0), (1, 0, 0.0, 0.0),
+          (0, 1, 2.0, 0.5), (1, None, -1.5, 0.25), (0, 0, 0.3, -0.8)]
+
+
+@pytest.mark.parametrize("dims", [(3, 9, 16), (6, 60, 40), (6, 90, 30)])
+def test_replayed_reverse_sweeps_equal_first_calls(P, dims):
+    """FP64 reverse mode on one context, with other inputs each time and other
+    calls in between that use or grow the same buffers, against contexts that
+    have done nothing else: small tiles, pool and modular engine, no pool.  The
+    gradients are sums of at most a few thousand terms that are not all larger
+    than the result: to 1e-11 of their norm."""
+    s = make_system(dims, seed=13)
+    T = [random_amplitudes(s, seed=40 + k, scale1=0.02, scale2=0.02) for k in range(2)]
+    rng = np.random.default_rng(3)
+    Rb = [[rng.normal(size=x.shape) for x in T[0]] for _ in range(2)]
+
+    def sweep(eng, call, prec=0):
+        t, r, eb, wb = call
+        Tb, Bb, fa, fb = eng.vjp(eng.to_device(T[t]), Rbar=None if r is None else eng.to_device(Rb[r]), Ebar=eb, Wbar=wb,
+                                 want_B=True, want_fock=True, precision=prec)
+        return [x.cpu().numpy() for x in Tb] + [Bb.cpu().numpy(), fa.cpu().numpy(), fb.cpu().numpy()]
+
+    def same(a, b, tol):
+        for x, y in zip(a, b):
+            assert np.linalg.norm(x - y) <= tol * np.linalg.norm(y)
+
+    first = {}
+    for call in set(SWEEPS):
+        eng = P.Engine.from_system(s)
+        first[call] = sweep(eng, call)
+        if call == SWEEPS[0]:
+            x6 = sweep(eng, call, 4)
+        eng.close()
+    eng = P.Engine.from_system(s)
+    for k, call in enumerate(SWEEPS + SWEEPS):
+        same(sweep(eng, call), first[call], 1e-11)
+        if k % 3 == 1:
+            _res(eng, T[k % 2], 0, 0, 0)
+        if k in (5, 9):
+            same(sweep(eng, SWEEPS[0], 4), x6, 1e-5)
+    eng.close()
