@@ -738,6 +738,12 @@ __device__ __forceinline__ void group_vectors(const ClassTerms& S, int nx, int V
     }
 }
 
+// The group vectors and those of the t1 c1 product, 2 x 9 + 8 of V elements, in
+// shared memory: up to 216 KB beside the 4 KB of ClassTerms, V <= 1063 in FP64 and
+// 2126 in FP32.  Beyond that every element is evaluated term by term: at
+// (8, 880, 16) 57 ms in FP64 instead of 8.6.
+constexpr size_t kSepSmem = 216 * 1024;
+
 // One block per (spin block, i, j).  Bound by latency: a block's elements
 // need about ten loads from shared memory and one or two from t2 each, so the
 // rows are spread over the warps and every lane keeps the loads of several
@@ -1339,8 +1345,9 @@ dcsd_status apply_mterms(Ctx* c, int ref, bool fp32) {
     const int maxx = std::max(g_max_xfac, 1);
     const size_t smem = (2ul * maxx + 8) * c->V * (fp32 ? sizeof(float) : sizeof(double));
     const unsigned grid = (unsigned)(3l * c->O * c->O);
-    trace_begin(c, fp32 ? "mterm_doubles_sep32" : "mterm_doubles_sep64");
-    if (g_max_xfac > kMaxXFac || g_max_hfac > kMaxHFac || smem > 160 * 1024) {
+    const bool sep = g_max_xfac <= kMaxXFac && g_max_hfac <= kMaxHFac && smem <= kSepSmem;
+    trace_begin(c, !sep ? "mterm_doubles (per term)" : fp32 ? "mterm_doubles_sep32" : "mterm_doubles_sep64");
+    if (!sep) {
         k_mterm_doubles<<<grid, 256, 0, c->stream>>>(a);  // per-term form (large V)
     } else if (fp32) {
         DCSD_CUDA(c, cudaFuncSetAttribute(k_mterm_doubles_sep<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
