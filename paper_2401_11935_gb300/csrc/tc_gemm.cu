@@ -10,9 +10,11 @@
 // packed operand layout of a following GEMM).
 //
 // Precision: operands are rounded to BF16 (nsplit = 1) or split x = hi + lo
-// with hi, lo BF16 (nsplit = 2) and multiplied as hi*hi + hi*lo + lo*hi by
-// concatenating three segments along K (A: [hi|hi|lo], B: [hi|lo|hi]); the
-// accumulation is FP32 in TMEM, the result is added to the FP64 residual.
+// with hi, lo BF16 (nsplit = 2; hi, mid, lo and six products with nsplit = 3)
+// and multiplied as hi*hi + hi*lo + lo*hi.  Each operand holds its parts once,
+// side by side; the k-steps of a GEMM run over the products and take the parts
+// that each names (TcParts).  The accumulation is FP32 in TMEM, the result is
+// added to the FP64 residual.
 //
 // Every mbarrier wait is bounded (about two seconds of wall time); on
 // expiry the kernel records an error flag, waits (bounded) for its own
@@ -506,19 +508,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     // two halves of 16 columns: all loads of a half, then its stores
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        if (epi.mode == 4) {
-                            float oldf[16];
-#pragma unroll
-                            for (int jj = 0; jj < 16; ++jj) {
-                                const long co = cb[h * 16 + jj];
-                                oldf[jj] = co >= 0 ? epi.C32[roff + co] : 0.0f;
-                            }
-#pragma unroll
-                            for (int jj = 0; jj < 16; ++jj) {
-                                const long co = cb[h * 16 + jj];
-                                if (co >= 0) epi.C32[roff + co] = fmaf(alpha, __uint_as_float(r[h * 16 + jj]), oldf[jj]);
-                            }
-                        } else if (epi.mode == 0) {
+                        if (epi.mode == 0) {
                             double old[16];
                             if (epi.beta != 0.0) {
 #pragma unroll
@@ -2374,7 +2364,12 @@ struct TcChoice {
 // (FP32 partial tiles, summed by a second kernel).  Rough time model:
 // 0.4 us per 64-deep k-step and tile wave plus operand packing at
 // 3 TB/s, against 5 TFLOP/s of the FP32 CUDA-core kernel on its 64 x 64
-// tiles; the faster one runs.
+// tiles; the faster one runs.  This describes one-CTA tiles of 128 or 256
+// columns and the FP32 kernel: the pairs and narrow tiles that gemm_packed picks are faster
+// (a k-step of 256 columns takes 0.31 us in a pair), and in BF16X6 the other
+// side is an FP64 contraction, slower than 5 TFLOP/s unless it is modular.
+// The line has not been moved with them: it decides how a sum is split and
+// rounded, and a MIXED solve follows the rounding of its BF16 parts.
 static TcChoice tc_choice(const Ctx* c, long M, long N, long K, int nsplit) {
     const int nseg = nsplit >= 3 ? 6 : nsplit == 2 ? 3 : 1;
     const long nkt = nseg * round_up(K, TC_BK) / TC_BK;
