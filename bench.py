@@ -40,8 +40,8 @@ UNIT = "s/iteration"
 
 # dram__bytes_read.sum + dram__bytes_write.sum averaged over the 84 ladder launches
 # (28 M+- producers, grouped contractions and joins each) of one 30+2 / 500 / 1500 BF16
-# residual, from a one-pass ncu capture; None whenever the ladder kernels change
-# until a new capture replaces it
+# residual, counted by ncu in one pass for the ladder kernels as they are; set it to
+# None, or to a count from the tile shapes that says so, when they change
 LADDER_DRAM_BYTES_PER_LAUNCH = 3.064e9
 
 
