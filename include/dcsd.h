@@ -89,12 +89,17 @@ typedef enum { DCSD_MEM_HOST = 0, DCSD_MEM_DEVICE = 1 } dcsd_mem_kind;
  * orbital-energy denominators, DIIS, energies, residual norm and the 2x2
  * effective Hamiltonian are always FP64. */
 typedef enum {
-    DCSD_PREC_FP64 = 0,   /* FP64 on CUDA cores                              */
+    DCSD_PREC_FP64 = 0,   /* FP64: CUDA cores, or for large contractions     */
+                          /* exact modular products on the tensor cores (*)  */
     DCSD_PREC_BF16 = 1,   /* BF16 operands on tcgen05 tensor cores, FP32 acc */
     DCSD_PREC_BF16X3 = 2, /* split operands hi+mid, 3 BF16 products          */
     DCSD_PREC_MIXED = 3,  /* dcsd_solve only: BF16, BF16X6, FP64 (see below) */
     DCSD_PREC_BF16X6 = 4  /* split hi+mid+lo, 6 BF16 products (FP32-class)  */
 } dcsd_precision;
+/* (*) Both compute an element c = sum_k a_k b_k of a contraction over K
+ * indices within the bound of a chain of FMAs, K 2^-53 sum |a_k b_k|, for
+ * elements of any relative size; infinite and NaN inputs give what they
+ * give in a chain.  dcsd_solve uses the CUDA cores only. */
 
 typedef struct dcsd_ctx dcsd_ctx;
 
@@ -296,7 +301,7 @@ dcsd_status dcsd_profile(dcsd_ctx* ctx, int enable, int reset, double* ms,
  *   B_bar             : out or NULL, [naux][n][n] (both triangles: the
  *                       gradient with respect to the array as stored).
  *   fock_a_bar, fock_b_bar : out or NULL, [n][n].
- * precision: DCSD_PREC_FP64 (CUDA cores) or a tensor-core precision, in
+ * precision: DCSD_PREC_FP64 or a tensor-core precision, in
  * which the forward and the adjoint contractions run on the tensor cores
  * with that operand split (the adjoint of a BF16X6 residual is accurate to
  * its FP32-class accuracy).

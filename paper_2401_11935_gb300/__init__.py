@@ -130,7 +130,7 @@ class Engine:
         of <Rbar, R(T)> + Ebar * dE_A(T) + Wbar * W(T) with respect to the
         five amplitude arrays, and optionally to the DF factors B [naux, n, n]
         and the two Fock matrices [n, n]: (Tbar, Bbar, fa_bar, fb_bar), absent
-        ones None.  precision PREC_FP64 differentiates on the FP64 CUDA cores;
+        ones None.  precision PREC_FP64 differentiates in FP64;
         a tensor-core precision runs the ladder and G-pass contractions of
         both sweeps on the tensor cores with that operand split."""
         t = self.torch

@@ -1028,7 +1028,10 @@ extern "C" dcsd_status dcsd_solve(dcsd_ctx* h, const dcsd_solve_opts* o, int mem
     // solve stops at the rounding noise of its BF16X6 residuals, and a change
     // of 1e-16 in the amplitudes flips BF16 roundings that feed back: with
     // another order the converged amplitudes moved by up to 6e-9 of their
-    // norm at (8, 90, 270).  The FP64 solve, its reference, keeps the order too.
+    // norm at (8, 90, 270).  The FP64 solve does not need this (it converges on
+    // its own residual): it keeps the order so that the two differ by the
+    // MIXED path alone, and pays for it with 0.4 s an iteration at
+    // (10, 120, 360), where a residual by modular GEMMs takes 0.023.
     const FmaChain chain(c, true);
     std::vector<double> Bm(16 * 16, 0.0);
     int nhist = 0, next = 0;

@@ -430,7 +430,7 @@ dcsd_status copy_dev(Ctx* c, double* dst, const double* src, size_t n);
 dcsd_status zero_dev(Ctx* c, double* dst, size_t n);
 inline bool recording(const Ctx* c) { return c->rec; }
 // ladder R2 += sum_cd t2 (ac|bd) by einsum chunks over a (integrals never
-// stored beyond a chunk); nsplit 0: FP64 CUDA cores, else tensor cores with
+// stored beyond a chunk); nsplit 0: FP64, else tensor cores with
 // that many operand splits.  One tape entry while recording; compute false
 // writes only that entry (a caller that produces the values another way).
 dcsd_status ladder64(Ctx* c, const TV& t2, const TV& Bvv, const TV& R2, double* chunkbuf, long chunk,

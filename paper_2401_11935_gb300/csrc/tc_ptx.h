@@ -83,11 +83,10 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 // One lane of a warp whose 32 lanes are all here.  The code that issues TMA
-// and MMAs is guarded by this, not by a lane number: it tells the compiler that
-// one thread is active, and it then emits the instructions, whose operands are
-// warp-uniform, without a loop over the active lanes around each.  With a lane
-// number a k-step of four MMAs and its commit took at least 540 clocks to issue
-// whatever its width; with 64 columns it now takes 393.
+// and MMAs is guarded by this, not by a lane number: as PTX defines it, it
+// names one leader of a converged warp.  Timed with a lane number, a k-step of
+// four MMAs and its commit took at least 540 clocks whatever its width; with
+// 64 columns it now takes 393.
 __device__ __forceinline__ bool elect_one() {
     uint32_t r;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r)::"memory");

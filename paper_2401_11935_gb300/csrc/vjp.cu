@@ -91,7 +91,7 @@ dcsd_status zero_dev(Ctx* c, double* dst, size_t n) {
     return DCSD_OK;
 }
 
-// one contraction on the engine of a precision: nsplit 0 FP64 CUDA cores,
+// one contraction on the engine of a precision: nsplit 0 FP64,
 // otherwise tensor cores with nsplit operand splits
 static dcsd_status contract(Ctx* c, int nsplit, const char* spec, double alpha, const TV& A, const TV& B,
                             double beta, const TV& C) {
