@@ -110,7 +110,7 @@ struct AdjRegion {
 
 struct CrtEngine;
 constexpr long kGemm64Counters = 4096;
-constexpr size_t kGraphNodes = 4096;  // launches of a recorded graph at most
+constexpr int kGraphLaunches = 4096;  // launches of a recorded graph at most
 constexpr int kGraphAttempts = 4;  // recordings of one argument set that may fail
 
 // Memory that a launch reads or writes, for the dependencies of recorded launches
@@ -211,6 +211,7 @@ struct Ctx {
     std::vector<Graph> graphs;
     cudaStream_t capture = nullptr;   // recording stream (the user's may be the legacy stream)
     Dag* dag = nullptr;               // set while recording (see DagOp)
+    long long record_end = 0;         // value of launches at which a recording is given up
     // intermediates of one residual in buffers of their own, taken one after
     // the other, so that independent launches do not wait for a shared buffer
     // (allocated for small systems)
@@ -540,6 +541,10 @@ inline dcsd_status launch_check(Ctx* c, const char* what) {
         return DCSD_ERR_CUDA;
     }
     c->launches++;
+    if (c->dag && c->launches > c->record_end) {  // (graph_record gives the recording up)
+        c->err = "too many launches to record";
+        return DCSD_ERR_CUDA;
+    }
     return DCSD_OK;
 }
 

@@ -154,3 +154,29 @@ def test_replayed_reverse_sweeps_equal_first_calls(P, dims):
         if k in (5, 9):
             same(sweep(eng, SWEEPS[0], 4), x6, 1e-5)
     eng.close()
+
+
+def test_thousands_of_launches_are_not_recorded(P):
+    """An FP64 residual whose ladder takes one virtual row at a time: more
+    launches than a graph may hold.  Recording is given up, nothing is
+    allocated, and every call makes the same launches."""
+    import torch
+    s = make_system((2, 500, 8), seed=15)
+    T = random_amplitudes(s, seed=16, scale1=0.02, scale2=0.02)
+    eng = P.Engine.from_system(s)
+    Td = eng.to_device(T)
+    from paper_2401_11935_gb300 import _lib as L
+    count, free, first = [], [], None
+    for _ in range(3):
+        n0 = L.load().dcsd_kernel_launches(eng.ctx)
+        R, W, dE = eng.residual(Td, precision=0)
+        torch.cuda.synchronize()
+        count.append(L.load().dcsd_kernel_launches(eng.ctx) - n0)
+        free.append(torch.cuda.mem_get_info()[0])
+        out = [x.cpu().numpy() for x in R] + [np.array([W, dE])]
+        first = first or out
+        _same(out, first, 0)
+        del R
+    eng.close()
+    assert count[0] == count[1] == count[2] > 4096, count
+    assert free[1] == free[2], free
