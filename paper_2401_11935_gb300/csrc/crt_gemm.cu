@@ -29,7 +29,7 @@
 // 23.6 -> 0.91 ms, of which GEMM 0.33 (1.46 PFLOP/s of BF16), residues 0.38,
 // norms 0.18; (2196, 14884, 360) 19.2 -> 0.98 ms, of which GEMM 0.43 (short
 // k) and output 0.41; (1464, 1464, 1464) 5.18 -> 0.20 ms.  The whole FP64
-// residual at (10, 120, 360): 445 -> 23.0 ms, of which the patch takes 1.4
+// residual at (10, 120, 360): 445 -> 23.0 ms, of which the patch takes 1.7
 // (0.28 ms of a contraction whose i = j columns are zero in one operand where
 // the other is largest); before the sums of magnitudes and the patch, with 15
 // moduli, 21.1 ms.  Operands that fall by 12 decades along k, against each
