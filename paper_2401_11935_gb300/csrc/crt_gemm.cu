@@ -970,7 +970,13 @@ static dcsd_status make_map(Ctx* c, CUtensorMap* map, const uint16_t* p, long ro
 bool crt_ready(Ctx* c) {
     CrtEngine* e = c->crt;
     if (!e) return false;
-    if (!e->ws && !e->refused && !c->dag) {  // (nothing can be allocated while launches are recorded)
+    if (!e->ws && !e->refused) {
+        // (nothing can be allocated while the caller or graph_record captures the stream)
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            return false;
+        }
         if (cudaMalloc((void**)&e->ws, e->want) == cudaSuccess) {
             e->bytes = e->want;
         } else {

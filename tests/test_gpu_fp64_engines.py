@@ -220,3 +220,39 @@ def test_modular_sums_at_the_integers_bounds(ctx, K):
         assert float(va) == va and float(vb) == vb
         c = _run(ctx, 2, np.full((130, K), float(va)), np.full((24, K), float(vb)), 1.0, 0.0, np.zeros((130, 24)))
         assert (c == float(va * vb * K)).all()
+
+
+@pytest.mark.parametrize("warm", [False, True])
+def test_contraction_under_capture(warm):
+    """Captured by the caller: the workspace of the modular engine is not
+    allocated there, so a context that does not have it yet records the CUDA
+    cores' launches."""
+    import torch
+    import paper_2401_11935_gb300 as P
+    from paper_2401_11935_gb300 import _lib as L
+    from synth import make_system
+    rng = np.random.default_rng(4)
+    a, b = rng.normal(size=(500, 300)), rng.normal(size=(700, 300))
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        A, B = torch.tensor(a).cuda(), torch.tensor(b).cuda()
+        C = torch.zeros(500, 700, dtype=torch.float64, device="cuda")
+        eng = P.Engine.from_system(make_system((2, 40, 12), seed=3))
+        # (loads the kernels of both engines)
+        other = P.Engine.from_system(make_system((2, 40, 12), seed=3))
+        for engine in (1, 2):
+            L.dcsd_einsum_device(other.ctx, engine, "mk,nk->mn", 1.0, A, B, 0.0, C)
+        if warm:
+            L.dcsd_einsum_device(eng.ctx, 0, "mk,nk->mn", 1.0, A, B, 0.0, C)
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            L.dcsd_einsum_device(eng.ctx, 0, "mk,nk->mn", 1.0, A, B, 0.0, C)
+        C.zero_()
+        graph.replay()
+        stream.synchronize()
+    del graph
+    c = C.cpu().numpy()
+    eng.close()
+    other.close()
+    assert (np.abs(c - _exact(a, b)) <= _bounds(a, b, 1.0, np.zeros(c.shape), 0.0)[1]).all()
