@@ -209,6 +209,7 @@ struct Ctx {
         int failures = 0;             // recordings that failed since the state changed
     };
     std::vector<Graph> graphs;
+    bool plain_tc = false;            // tensor-core residuals launch by launch (see residual_prepare)
     cudaStream_t capture = nullptr;   // recording stream (the user's may be the legacy stream)
     Dag* dag = nullptr;               // set while recording (see DagOp)
     long long record_end = 0;         // value of launches at which a recording is given up

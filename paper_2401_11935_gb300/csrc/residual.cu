@@ -717,17 +717,20 @@ static int residual_key(const Ctx* c, int ref, int method, int prec) {
     return ((ref * 8 + method) * 8 + prec) * 2 + (chain ? 1 : 0);
 }
 
-// The classic ladder packs B for one split at a time, so a recording of one
-// precision would not outlive a call of another: there every launch is made
-static bool residual_records(const Ctx* c, int prec) { return prec == DCSD_PREC_FP64 || !tc_repacks(c); }
-
 dcsd_status residual_run(Ctx* c, int ref, int method, int prec) {
-    if (!residual_records(c, prec)) return residual_union(c, ref, method, prec);
+    if (c->plain_tc && prec != DCSD_PREC_FP64) return residual_union(c, ref, method, prec);
     return graph_run(c, residual_key(c, ref, method, prec), [=]() { return residual_union(c, ref, method, prec); });
 }
 
 void residual_prepare(Ctx* c, int prec, bool chain) {
-    if (c->rec || c->trace || c->prof_on || !residual_records(c, prec)) return;
+    if (c->rec || c->trace || c->prof_on) return;
+    // The classic ladder packs B for one split at a time, so a recording of one
+    // precision does not outlive a call of another, and the next would record
+    // again: in a reserved context these calls stay launch by launch
+    if (prec != DCSD_PREC_FP64 && tc_repacks(c)) {
+        c->plain_tc = true;
+        return;
+    }
     const FmaChain order(c, chain);
     for (int method = DCSD_CCSD; method <= DCSD_FR_DCSD_T; ++method)
         for (int ref = 0; ref < 2; ++ref) {

@@ -221,13 +221,14 @@ def test_modular_workspace_is_given_back(P):
     eng.close()
 
 
-@pytest.mark.parametrize("precision", [0, 1, 3, 4])
-def test_reserved_contexts_record_nothing_later(P, precision):
+@pytest.mark.parametrize("precision,ladder", [(0, "1"), (1, "1"), (3, "1"), (4, "1"), (3, "0")])
+def test_reserved_contexts_record_nothing_later(P, monkeypatch, precision, ladder):
     """After a reservation, repeated residuals of every method and reference,
     energies and solves leave the device's free memory as it is (a graph
     recorded by one of them would take 2 to 8 MB)."""
     import torch
     from paper_2401_11935_gb300 import _lib as L
+    monkeypatch.setenv("DCSD_LADDER_SA", ladder)
     s = make_system((4, 20, 60), seed=5)
     precs = [1, 4] if precision == 3 else [precision]
 
