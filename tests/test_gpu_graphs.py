@@ -69,47 +69,76 @@ def test_ladder_block_edges(P, dims, prec, tol):
     assert max(float(np.abs(a - b).max()) for a, b in zip(R[:5], R0[:5])) < tol * rmax
 
 
+FULL_DEVICE = """
+import time
+import numpy as np
+import torch
+import paper_2401_11935_gb300 as P
+from synth import make_system, random_amplitudes
+s = make_system((4, 20, 60), seed=11)
+T = random_amplitudes(s, seed=20, scale1=0.02, scale2=0.02)
+eng = P.Engine.from_system(s)
+Td = eng.to_device(T)
+Rd = eng.to_device(T)
+
+times = []
+
+def run():
+    out = []
+    for m, r in ((0, 0), (0, 1), (1, 0), (1, 1)):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        R, W, dE = eng.residual(Td, ref=r, method=m, precision=0, out=Rd)
+        torch.cuda.synchronize()
+        times.append(time.perf_counter() - t0)
+        out.append([x.cpu().numpy() for x in R] + [np.array([W, dE])])
+    return out
+
+def best():  # (of enough calls that no attempt to record is left)
+    t = []
+    for _ in range(12):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        eng.residual(Td, ref=0, method=0, precision=0, out=Rd)
+        torch.cuda.synchronize()
+        t.append(time.perf_counter() - t0)
+    return min(t)
+
+outs = [run()]  # launch by launch; loads the kernels
+plain = min(times)
+filler = []
+for size in (2 ** 30, 2 ** 24, 2 ** 20):  # (up to 1 MB torch takes 2 MB from the device, above that 20 MB at least)
+    while True:
+        try:
+            filler.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+        except torch.OutOfMemoryError:
+            break
+outs.append(run())
+best()
+filler.clear()
+torch.cuda.empty_cache()
+outs.append(run())
+eng.residual(Td, ref=0, method=0, precision=4)  # (new buffers: recorded residuals are dropped)
+fast = best()
+outs.append(run())
+for out in outs[1:]:
+    for xs, ys in zip(out, outs[0]):
+        for x, y in zip(xs, ys):
+            assert np.linalg.norm(x - y) <= 1e-13 * max(1.0, np.linalg.norm(y))
+assert fast < 0.75 * plain, (fast, plain)
+print("recorded", fast, plain)
+"""
+
+
 def test_recording_without_memory_is_tried_again(P):
     """No room for the recorded graphs: the calls run launch by launch and are
-    right; with memory free again the following ones are recorded (a graph
-    at this size takes 4 to 8 MB)."""
-    import torch
-    s = make_system((4, 20, 60), seed=11)
-    T = random_amplitudes(s, seed=20, scale1=0.02, scale2=0.02)
-    eng = P.Engine.from_system(s)
-    Td = eng.to_device(T)
-    keys = [(m, r) for m in (0, 1) for r in (0, 1)]
-
-    def run():
-        out = {}
-        for m, r in keys:
-            R, W, dE = eng.residual(Td, ref=r, method=m, precision=0)
-            out[m, r] = [x.cpu().numpy() for x in R] + [np.array([W, dE])]
-        torch.cuda.synchronize()
-        return out
-
-    first = run()  # launch by launch; loads the kernels
-    filler = []
-    try:
-        for size in (2 ** 30, 2 ** 24, 2 ** 21):
-            while True:
-                try:
-                    free = torch.cuda.mem_get_info()[0]
-                    filler.append(torch.empty(max(size, (free - size) // size * size), dtype=torch.uint8, device="cuda"))
-                except torch.OutOfMemoryError:
-                    break
-        full = run()
-    finally:
-        filler.clear()
-        torch.cuda.empty_cache()
-    torch.cuda.synchronize()
-    before = torch.cuda.mem_get_info()[0]
-    again = run()
-    assert before - torch.cuda.mem_get_info()[0] >= 2 ** 22
-    for out in (full, again, run()):
-        for k in keys:
-            _same(out[k], first[k], 0)
-    eng.close()
+    right; with memory free again the following ones are recorded.  What is
+    seen is the time of a call, 0.5 ms against 1.3; in a process of its own,
+    because the driver keeps memory of earlier graphs."""
+    import subprocess
+    import sys
+    r = subprocess.run([sys.executable, "-c", FULL_DEVICE], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "recorded" in r.stdout, r.stderr[-2000:]
 
 
 # (amplitudes, cotangents or None, Ebar, Wbar): every input changes from call to call
